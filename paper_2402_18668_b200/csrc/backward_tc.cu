@@ -697,43 +697,6 @@ __global__ void __launch_bounds__(kThreadsB, 1)
 }
 
 namespace {
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn encode_fn_b() {
-    static EncodeTiledFn fn = nullptr;
-    if (!fn) {
-        void* ptr = nullptr;
-        cudaDriverEntryPointQueryResult qres;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &qres) == cudaSuccess &&
-            qres == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn>(ptr);
-    }
-    return fn;
-}
-// [BH][L][width] bf16, box = [1][128][box_w] (box_w may exceed width: the rest is zero-filled)
-bool make_map_b(CUtensorMap* m, const void* base, int BH, int L, int width, int box_w, int box_rows,
-                CUtensorMapSwizzle sw) {
-    EncodeTiledFn enc = encode_fn_b();
-    if (!enc) return false;
-    cuuint64_t dims[3] = {(cuuint64_t)width, (cuuint64_t)L, (cuuint64_t)BH};
-    cuuint64_t strides[2] = {(cuuint64_t)width * 2, (cuuint64_t)L * width * 2};
-    cuuint32_t box[3] = {(cuuint32_t)box_w, (cuuint32_t)box_rows, 1};
-    cuuint32_t estr[3] = {1, 1, 1};
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-}  // namespace
-
-// the same map for the other tensor-core kernels of the library
-bool make_rows_map_bf16(CUtensorMap* m, const void* base, int BH, int L, int width, int box_w, int box_rows,
-                        CUtensorMapSwizzle sw) {
-    return make_map_b(m, base, BH, L, width, box_w, box_rows, sw);
-}
-
-namespace {
 // Block-wise path, between the passes.  state_scan_kernel: the per-block states of
 // block_state_tc_kernel summed over the blocks before (suffix = 0) or after (suffix = 1) each
 // block, as bf16 [BH x nblk][dvw][160] (tensor-core operand, transposed as the state kernel holds it) and fp32 row
@@ -832,11 +795,11 @@ based_status launch_dvb(const void* q, const void* k, const void* v, const void*
     // own tiles: 128 rows; looped tiles: 64 rows (and LTK rows for the dk/dv pass)
     CUtensorMap tq, tk, tv, tg, tk64, tv64, tqL, tgL, tdv;
     const CUtensorMapSwizzle s64 = CU_TENSOR_MAP_SWIZZLE_64B, s128 = CU_TENSOR_MAP_SWIZZLE_128B;
-    if (!make_map_b(&tq, q, BH, L, df, 32, kTile, s64) || !make_map_b(&tk, k, BH, L, df, 32, kTile, s64) ||
-        !make_map_b(&tv, v, BH, L, dvr, 64, kTile, s128) || !make_map_b(&tg, g, BH, L, dvr, 64, kTile, s128) ||
-        !make_map_b(&tk64, k, BH, L, df, 32, 64, s64) || !make_map_b(&tv64, v, BH, L, dvr, 64, 64, s128) ||
-        !make_map_b(&tqL, q, BH, L, df, 32, LTK, s64) || !make_map_b(&tgL, g, BH, L, dvr, 64, LTK, s128) ||
-        !make_map_b(&tdv, dv, BH, L, dvr, 64, kTile, s128))
+    if (!make_rows_map_bf16(&tq, q, BH, L, df, 32, kTile, s64) || !make_rows_map_bf16(&tk, k, BH, L, df, 32, kTile, s64) ||
+        !make_rows_map_bf16(&tv, v, BH, L, dvr, 64, kTile, s128) || !make_rows_map_bf16(&tg, g, BH, L, dvr, 64, kTile, s128) ||
+        !make_rows_map_bf16(&tk64, k, BH, L, df, 32, 64, s64) || !make_rows_map_bf16(&tv64, v, BH, L, dvr, 64, 64, s128) ||
+        !make_rows_map_bf16(&tqL, q, BH, L, df, 32, LTK, s64) || !make_rows_map_bf16(&tgL, g, BH, L, dvr, 64, LTK, s128) ||
+        !make_rows_map_bf16(&tdv, dv, BH, L, dvr, 64, kTile, s128))
         return BASED_ERR_CUDA;
     BParams p{};
     if (error_word_ptr(&p.err) != BASED_OK) return BASED_ERR_CUDA;
@@ -863,7 +826,7 @@ based_status launch_dvb(const void* q, const void* k, const void* v, const void*
         const BlockWs w = block_ws(ws, BH, L, dvr, nblk);
         CUtensorMap tst;
         // the block states lie transposed, [BH x nblk][d_v][160]: boxes of 32 features x all value columns
-        if (!make_map_b(&tst, w.st, BH * nblk, dvr, 160, 32, 64 * BCfg<DV, kModeDkDv, LTK>::kVB, s64)) return BASED_ERR_CUDA;
+        if (!make_rows_map_bf16(&tst, w.st, BH * nblk, dvr, 160, 32, 64 * BCfg<DV, kModeDkDv, LTK>::kVB, s64)) return BASED_ERR_CUDA;
         if (out == nullptr && !numerator_only) {
             // the centre of the merged pass: the forward output, recomputed
             st = launch_prefill_tc(q, k, v, w.out, nullptr, nullptr, BH, L, dvr, 0, w.fwd, stream);
@@ -894,7 +857,7 @@ based_status launch_dvb(const void* q, const void* k, const void* v, const void*
             // 32-row looped tiles: the accumulators then fit 256 tensor-memory columns and two CTAs share an SM, which
             // hides the fixed latency of these short-lived CTAs (273 -> 220 us for the pass at B8 H16 L4096)
             CUtensorMap tq32, tg32;
-            if (!make_map_b(&tq32, q, BH, L, df, 32, 32, s64) || !make_map_b(&tg32, g, BH, L, dvr, 64, 32, s128)) return BASED_ERR_CUDA;
+            if (!make_rows_map_bf16(&tq32, q, BH, L, df, 32, 32, s64) || !make_rows_map_bf16(&tg32, g, BH, L, dvr, 64, 32, s128)) return BASED_ERR_CUDA;
             return launch_pass<DV, kModeDkDv, 32, true>(tk, tv, tq32, tg32, p, grid, "backward_tc_kernel<dkdv, blocks>", stream, &tst,
                                                         &tdv);
         }
@@ -924,8 +887,8 @@ based_status launch_quadratic_forward_tc(const void* q, const void* k, const voi
                                          int d_feat, int d_v, int numerator_only, cudaStream_t stream) {
     CUtensorMap tq, tk64, tv64, tout;
     const CUtensorMapSwizzle s64 = CU_TENSOR_MAP_SWIZZLE_64B, s128 = CU_TENSOR_MAP_SWIZZLE_128B;
-    if (!make_map_b(&tq, q, BH, L, d_feat, 32, kTile, s64) || !make_map_b(&tk64, k, BH, L, d_feat, 32, 64, s64) ||
-        !make_map_b(&tv64, v, BH, L, d_v, 64, 64, s128) || !make_map_b(&tout, out, BH, L, d_v, 64, kTile, s128))
+    if (!make_rows_map_bf16(&tq, q, BH, L, d_feat, 32, kTile, s64) || !make_rows_map_bf16(&tk64, k, BH, L, d_feat, 32, 64, s64) ||
+        !make_rows_map_bf16(&tv64, v, BH, L, d_v, 64, 64, s128) || !make_rows_map_bf16(&tout, out, BH, L, d_v, 64, kTile, s128))
         return BASED_ERR_CUDA;
     BParams p{};
     if (error_word_ptr(&p.err) != BASED_OK) return BASED_ERR_CUDA;

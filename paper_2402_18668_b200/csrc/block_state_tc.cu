@@ -38,9 +38,6 @@
 namespace based {
 using namespace sm100;
 
-bool make_rows_map_bf16(CUtensorMap* m, const void* base, int BH, int L, int width, int box_w, int box_rows,
-                        CUtensorMapSwizzle sw);
-
 namespace {
 constexpr int kTok = 128;          // tokens per step
 constexpr int kThreadsR = 288;     // eight row warps (two threads per token: half of its features each), one issuer warp

@@ -25,10 +25,6 @@
 namespace based {
 using namespace sm100;
 
-// [BH][L][width] bf16 tensor map with a [1][box_rows][box_w] box (defined with the backward kernels)
-bool make_rows_map_bf16(CUtensorMap* m, const void* base, int BH, int L, int width, int box_w, int box_rows,
-                        CUtensorMapSwizzle sw);
-
 namespace {
 constexpr int kFB = 128;           // feature rows per CTA (accumulator lanes)
 constexpr int kTB = 64;            // tokens per step (K extent of one MMA burst)

@@ -1432,35 +1432,6 @@ __global__ void __launch_bounds__(kThreads, 1)
 // --------------------------------------------------------------------------------- host side
 namespace {
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_fn() {
-    static EncodeTiledFn fn = nullptr;
-    if (!fn) {
-        void* ptr = nullptr;
-        cudaDriverEntryPointQueryResult qres;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &qres) == cudaSuccess &&
-            qres == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn>(ptr);
-    }
-    return fn;
-}
-
-// [BH][L][width] bf16, box = [1][128][box_w]
-bool make_map(CUtensorMap* m, const void* base, int BH, int L, int width, int box_w, CUtensorMapSwizzle sw) {
-    EncodeTiledFn enc = encode_fn();
-    if (!enc) return false;
-    cuuint64_t dims[3] = {(cuuint64_t)width, (cuuint64_t)L, (cuuint64_t)BH};
-    cuuint64_t strides[2] = {(cuuint64_t)width * 2, (cuuint64_t)L * width * 2};
-    cuuint32_t box[3] = {(cuuint32_t)box_w, (cuuint32_t)kC, 1};
-    cuuint32_t estr[3] = {1, 1, 1};
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 #ifdef BASED_TRACE
 unsigned long long* g_trace = nullptr;
 #endif
@@ -1570,10 +1541,10 @@ based_status launch_dv(const void* q, const void* k, const void* v, void* out, f
                        int dv, int flags, float* ws, const SegPlan plan, cudaStream_t stream) {
     using C = Cfg<DV>;
     CUtensorMap tq, tk, tv, to;
-    if (!make_map(&tq, q, BH, L, kDFeat, kDFeat, CU_TENSOR_MAP_SWIZZLE_32B) ||
-        !make_map(&tk, k, BH, L, kDFeat, kDFeat, CU_TENSOR_MAP_SWIZZLE_32B) ||
-        !make_map(&tv, v, BH, L, dv, 64, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_map(&to, out, BH, L, dv, 64, CU_TENSOR_MAP_SWIZZLE_128B))
+    if (!make_rows_map_bf16(&tq, q, BH, L, kDFeat, kDFeat, kC, CU_TENSOR_MAP_SWIZZLE_32B) ||
+        !make_rows_map_bf16(&tk, k, BH, L, kDFeat, kDFeat, kC, CU_TENSOR_MAP_SWIZZLE_32B) ||
+        !make_rows_map_bf16(&tv, v, BH, L, dv, 64, kC, CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_rows_map_bf16(&to, out, BH, L, dv, 64, kC, CU_TENSOR_MAP_SWIZZLE_128B))
         return BASED_ERR_CUDA;
     Params p{};         // (every field the kernel may read has a value: pad is read on every path)
     p.kv_abi = kv;
@@ -1795,8 +1766,8 @@ static based_status launch_state_dv(const void* k, const void* v, float* kv, flo
     using C = Cfg<DV>;
     const SegPlan plan = prefill_tc_state_plan(BH, L);
     CUtensorMap tk, tv;
-    if (!make_map(&tk, k, BH, L, kDFeat, kDFeat, CU_TENSOR_MAP_SWIZZLE_32B) ||
-        !make_map(&tv, v, BH, L, dv, 64, CU_TENSOR_MAP_SWIZZLE_128B))
+    if (!make_rows_map_bf16(&tk, k, BH, L, kDFeat, kDFeat, kC, CU_TENSOR_MAP_SWIZZLE_32B) ||
+        !make_rows_map_bf16(&tv, v, BH, L, dv, 64, kC, CU_TENSOR_MAP_SWIZZLE_128B))
         return BASED_ERR_CUDA;
     Params p{};
     p.ws = ws;

@@ -7,6 +7,12 @@
 #include <stdint.h>
 
 namespace based {
+
+// tensor map of a bf16 [BH][L][width] array with a [1][box_rows][box_w] box (box_w may exceed width: the rest is
+// zero-filled on load and clipped on store); false if the encoder refuses (tensor_map.cu)
+bool make_rows_map_bf16(CUtensorMap* m, const void* base, int BH, int L, int width, int box_w, int box_rows,
+                        CUtensorMapSwizzle sw);
+
 namespace sm100 {
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {

@@ -450,33 +450,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (warp == kWarpMma) tmem_dealloc(tb, 512);
 }
 
-namespace {
-
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-bool make_map(CUtensorMap* m, const void* base, int BH, int L, int box_rows) {
-    static EncodeTiledFn enc = nullptr;
-    if (!enc) {
-        void* ptr = nullptr;
-        cudaDriverEntryPointQueryResult qres;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &qres) != cudaSuccess ||
-            qres != cudaDriverEntryPointSuccess)
-            return false;
-        enc = reinterpret_cast<EncodeTiledFn>(ptr);
-    }
-    cuuint64_t dims[3] = {(cuuint64_t)kHD, (cuuint64_t)L, (cuuint64_t)BH};
-    cuuint64_t strides[2] = {(cuuint64_t)kHD * 2, (cuuint64_t)L * kHD * 2};
-    cuuint32_t box[3] = {(cuuint32_t)kHD, (cuuint32_t)box_rows, 1};
-    cuuint32_t estr[3] = {1, 1, 1};
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-}  // namespace
-
 bool swa_tc_supported(int window) { return window >= 1 && window <= 128; }
 
 template <int PAD>
@@ -485,8 +458,10 @@ static based_status launch_swa_pad(const void* q, const void* k, const void* v, 
     using C = SwaCfg<PAD>;
     CUtensorMap tq, tk, tv, to;
     constexpr int kv_rows = PAD == 64 ? C::kKeys : kQT;      // rows of one K / V load
-    if (!make_map(&tq, q, BH, L, kQT) || !make_map(&tk, k, BH, L, kv_rows) || !make_map(&tv, v, BH, L, kv_rows) ||
-        !make_map(&to, out, BH, L, kQT))
+    const CUtensorMapSwizzle s128 = CU_TENSOR_MAP_SWIZZLE_128B;
+    if (!make_rows_map_bf16(&tq, q, BH, L, kHD, kHD, kQT, s128) || !make_rows_map_bf16(&tk, k, BH, L, kHD, kHD, kv_rows, s128) ||
+        !make_rows_map_bf16(&tv, v, BH, L, kHD, kHD, kv_rows, s128) ||
+        !make_rows_map_bf16(&to, out, BH, L, kHD, kHD, kQT, s128))
         return BASED_ERR_CUDA;
     SwaParams p;
     if (error_word_ptr(&p.err) != BASED_OK) return BASED_ERR_CUDA;

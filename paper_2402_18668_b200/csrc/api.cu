@@ -85,7 +85,7 @@ const char* based_status_string(based_status s) {
 
 size_t based_prefill_workspace_bytes(int B, int H, int L, int d_feat, int d_v, based_dtype io) {
     if (B <= 0 || H <= 0 || L <= 0 || d_feat != kDFeat || !dv_ok(d_v)) return 0;
-    if (io != BASED_BF16) return 0;            // the fp32 path keeps its state in registers
+    if (io != BASED_BF16) return 0;            // the fp32 path keeps its states on chip
     const long long BH = (long long)B * H;
     if (BH > kHeadSlab) {
         const size_t a = prefill_tc_workspace_bytes((int)kHeadSlab, L, d_v);
@@ -140,8 +140,8 @@ static based_status prefill_impl(const void* q, const void* k, const void* v, vo
     if (io == BASED_BF16)
         return launch_prefill_tc(q, k, v, out, kv_state, z_state, B * H, L, d_v, flags, workspace,
                                  static_cast<cudaStream_t>(cuda_stream), fit ? workspace_bytes : ~(size_t)0);
-    return launch_prefill_simt(q, k, v, out, kv_state, z_state, B * H, L, d_v, io, flags,
-                               static_cast<cudaStream_t>(cuda_stream));
+    return launch_prefill_f32(q, k, v, out, kv_state, z_state, B * H, L, d_v, flags,
+                              static_cast<cudaStream_t>(cuda_stream));
 }
 
 based_status based_prefill(const void* q, const void* k, const void* v, void* out, float* kv_state, float* z_state,

@@ -82,8 +82,9 @@ based_status preload_generation_step();
 // full (273-row) state -> symmetric (153-row) state, or back
 based_status launch_state_convert(const float* kv_in, const float* z_in, float* kv_out, float* z_out, int BH,
                                   int d_v, bool to_sym, cudaStream_t stream);
-based_status launch_prefill_simt(const void* q, const void* k, const void* v, void* out, float* kv, float* z,
-                                 int BH, int L, int d_v, based_dtype io, int flags, cudaStream_t stream);
+// fp32 io (prefill_f32.cu)
+based_status launch_prefill_f32(const void* q, const void* k, const void* v, void* out, float* kv, float* z, int BH,
+                                int L, int d_v, int flags, cudaStream_t stream);
 // bf16 tensor-core prefill (tcgen05); workspace holds partial states of sequence segments.  prefill_tc_workspace_bytes
 // is what the fastest plan needs; workspace_limit = the bytes behind `workspace`: a call given less takes the fastest
 // plan that fits (fewer segments per head, in the end none: the plain loop and the recompute mode need no workspace).

@@ -443,8 +443,10 @@ static based_status prefill_backward(const void* q, const void* k, const void* v
         return launch_prefill_backward_tc(q, k, v, out, dout, dq, dk, dv, static_cast<float*>(workspace), B * H, L,
                                           d_feat, d_v, (flags & BASED_NUMERATOR_ONLY) ? 1 : 0,
                                           static_cast<cudaStream_t>(cuda_stream));
-    return launch_prefill_backward(q, k, v, dout, dq, dk, dv, static_cast<float*>(workspace), B * H, L, d_v, io,
-                                   (flags & BASED_NUMERATOR_ONLY) ? 1 : 0, static_cast<cudaStream_t>(cuda_stream));
+    auto in = [](const void* p) { return static_cast<const float*>(p); };
+    return launch_prefill_backward_f32(in(q), in(k), in(v), in(dout), static_cast<float*>(dq), static_cast<float*>(dk),
+                                       static_cast<float*>(dv), static_cast<float*>(workspace), B * H, L, d_v,
+                                       (flags & BASED_NUMERATOR_ONLY) ? 1 : 0, static_cast<cudaStream_t>(cuda_stream));
 }
 
 based_status based_prefill_backward(const void* q, const void* k, const void* v, const void* dout, void* dq,

@@ -1,0 +1,407 @@
+// based_prefill_backward for fp32 io (d' = 16): gradients of the causal Taylor linear attention (definition form, left-hand
+// side of Eq. (2) of Sec. 4.1).  The paper gives no backward algorithm; this is the chain rule on the definition, evaluated
+// tile by tile in the quadratic ("attention") form with fp32 FMAs (bf16 / tf32 operands cannot meet fp32's tolerance):
+//
+//   y_i = N_i / D_i,  N_i = sum_{j<=i} w_ij v_j,  D_i = sum_{j<=i} w_ij + eps,  w_ij = 1 + s/4 + s^2/32,
+//   s = q_i.k_j;  with G_i the gradient of the loss with respect to y_i:
+//   a_i = G_i / D_i,  b_i = -(G_i.y_i) / D_i = -(G_i.N_i) / D_i^2,  ds_ij = (a_i.v_j + b_i)(1/4 + s_ij/16),
+//   dq_i = sum_{j<=i} ds_ij k_j,   dk_j = sum_{i>=j} ds_ij q_i,   dv_j = sum_{i>=j} w_ij a_i.
+//
+// Two launches over 64 x 64 tiles of (own, looped) rows, one CTA of 128 threads per own tile:
+//   dq       own = queries, loops over the key tiles j <= i.  Row statistics and dq in one sweep: with m_i = G_i.v_i,
+//            X_i = sum_j w'_ij (G_i.v_j - m_i) k_j and Y_i = sum_j w'_ij k_j, w' = 1/4 + s/16,
+//            dq_i = X_i / D_i + (m_i / D_i + b_i) Y_i needs neither D_i nor b_i while the keys are swept (any m_i gives the
+//            same sum; this one is exact for the first row, where the two terms of ds cancel).
+//   dk, dv   own = keys, loops over the query tiles i >= j.
+// A thread holds 8 x 4 pairs of s and G.v in registers, a warp 16 own rows; what a warp needs of its own weights for the
+// products over the looped rows (X, Y, dk, dv) goes through shared memory of its own, in tiles laid out along the
+// summation index.  Lanes 2n and 2n + 1 differ in the own rows only: a 128-bit load whose neighbouring lanes share an
+// address costs two passes, four otherwise.  Few tiles: the CTAs of a cluster share one own tile's loop, and their sums
+// are added through distributed shared memory in a fixed order.
+// Measured against three sweeps of 4 x 8 pairs per thread on scalar shared-memory loads: B2 H16 L1024 d_v64 1050 -> 424 us,
+// B1 H2 L1024 d_v64 56 us with eight CTAs per own tile.  Bound: the fp32 pipe at a third of its rate (135 us of FMAs); two
+// CTAs of four warps fit an SM, and a tile's loads and its products take turns in each.
+#include <cooperative_groups.h>
+
+#include "common.cuh"
+
+namespace based {
+
+namespace {
+namespace cg = cooperative_groups;
+
+constexpr int kT = 64;             // tile edge
+constexpr int kBT = 128;           // threads: 4 warps of 16 own rows
+constexpr int kP = 68;             // row pitch of tiles with 64 entries per row
+constexpr int kMaxSplit = 8;       // CTAs of a cluster that share an own tile
+
+template <int DV, bool KEYS>
+struct BwdSmem {
+    static constexpr int kCols = (DV + 63) / 64 * 64;
+    static constexpr int kWide = kCols + 4;
+    float an[kDFeat * kP];         // own q (keys pass: k), transposed [16][68]
+    float aw[DV * kP];             // own dout (v), transposed [DV][68]
+    float bn[kDFeat * kP];         // looped k (q), transposed
+    float bw[DV * kP];             // looped v (dout), transposed
+    float rn[kT * kDFeat];         // looped k (q) as it lies, row t at place of(t)
+    float rw[KEYS ? kT * kWide : 4];    // looped dout as it lies
+    float p[2][4][kT * 16];        // per warp: two weights of (looped row at place of(t), own row)
+    float2 st[kT];                 // keys pass: (1 / D, b) of the looped queries
+    float m[kT];
+};
+// place of looped row t where four consecutive rows belong to one thread: spreads those over the banks
+__device__ __forceinline__ int place_of(int t) { return (t & 3) * 16 + (t >> 2); }
+
+__device__ __forceinline__ float4 lds4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+
+// 64 rows of W values (a multiple of 16) of a row-major array, transposed -> [W][68]; rows from nt on are zero.
+// nat: the rows as they lie too, at pitch natp (of: at place_of(t))
+template <int W>
+__device__ __forceinline__ void load_tile(float* dst, float* nat, int natp, bool of, const float* __restrict__ src, int nt,
+                                          int warp, int lane) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int t = (lane & 7) + 8 * warp + 32 * h;
+        float4 x[W / 16];
+#pragma unroll
+        for (int i = 0; i < W / 16; ++i) {
+            x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (t < nt) x[i] = __ldg(reinterpret_cast<const float4*>(src + (size_t)t * W) + (lane >> 3) + 4 * i);
+        }
+#pragma unroll
+        for (int i = 0; i < W / 16; ++i) {
+            const int c = 4 * ((lane >> 3) + 4 * i);
+            dst[(c + 0) * kP + t] = x[i].x;
+            dst[(c + 1) * kP + t] = x[i].y;
+            dst[(c + 2) * kP + t] = x[i].z;
+            dst[(c + 3) * kP + t] = x[i].w;
+            if (nat) *reinterpret_cast<float4*>(&nat[(of ? place_of(t) : t) * natp + c]) = x[i];
+        }
+    }
+}
+
+// s[i][j] += sum_k a[k][row i] b[k][4 co + j]
+template <int K>
+__device__ __forceinline__ void pair_product(float (&s)[8][4], const float* a, const float* b) {
+#pragma unroll 4
+    for (int k = 0; k < K; ++k) {
+        const float4 x0 = lds4(a + k * kP), x1 = lds4(a + k * kP + 8), y = lds4(b + k * kP);
+        const float xs[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w}, ys[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) s[i][j] = fmaf(xs[i], ys[j], s[i][j]);
+    }
+}
+// acc[i][d] += sum over this lane group's 16 looped rows of p[row][4 rg + i] n[row][8 dg + d]
+__device__ __forceinline__ void narrow_product(float (&acc)[4][8], const float* p, const float* n, int ks, int rg, int dg) {
+#pragma unroll 4
+    for (int u = 0; u < 16; ++u) {
+        const int r = u * 4 + ks;
+        const float4 x = lds4(p + r * 16 + rg * 4), y0 = lds4(n + r * 16 + dg * 8), y1 = lds4(n + r * 16 + dg * 8 + 4);
+        const float xs[4] = {x.x, x.y, x.z, x.w}, ys[8] = {y0.x, y0.y, y0.z, y0.w, y1.x, y1.y, y1.z, y1.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int d = 0; d < 8; ++d) acc[i][d] = fmaf(xs[i], ys[d], acc[i][d]);
+    }
+}
+// sums over the four lane groups ks (lane bits 3, 4)
+__device__ __forceinline__ void narrow_reduce(float (&acc)[4][8]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int d = 0; d < 8; ++d) {
+            acc[i][d] += __shfl_xor_sync(0xffffffffu, acc[i][d], 8);
+            acc[i][d] += __shfl_xor_sync(0xffffffffu, acc[i][d], 16);
+        }
+}
+}  // namespace
+
+// KEYS = false: dq and the statistics.  KEYS = true: dk and dv.  grid (tiles, heads, CTAs per tile)
+template <int DV, bool KEYS>
+__global__ void __launch_bounds__(kBT)
+    backward_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v,
+                        const float* __restrict__ g, float2* stats, float* __restrict__ dx, float* __restrict__ dv, int L,
+                        int numerator_only) {
+    using S = BwdSmem<DV, KEYS>;
+    constexpr int NV = S::kCols / 64;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    S& s = *reinterpret_cast<S*>(smem_raw);
+    cg::cluster_group cluster = cg::this_cluster();
+    const int ntile = gridDim.x, nsplit = gridDim.z, rank = blockIdx.z;
+    const int own = KEYS ? blockIdx.x : ntile - 1 - blockIdx.x;      // longest loops first
+    const size_t head = blockIdx.y;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int ro = lane & 1, co = lane >> 1;                         // pair tile: own rows row0 + {0..3, 8..11}, looped 4 co + j
+    const int row0 = warp * 16 + ro * 4;
+    const int dg = lane & 1, rg = (lane >> 1) & 3, ks = lane >> 3;   // narrow products
+    const size_t hn = head * (size_t)L * kDFeat, hw = head * (size_t)L * DV;
+    const float* own_n = (KEYS ? k : q) + hn;
+    const float* own_w = (KEYS ? v : g) + hw;
+    const float* loop_n = (KEYS ? q : k) + hn;
+    const float* loop_w = (KEYS ? g : v) + hw;
+    const int n_own = min(kT, L - own * kT);
+
+    load_tile<kDFeat>(s.an, nullptr, 0, false, own_n + (size_t)own * kT * kDFeat, n_own, warp, lane);
+    load_tile<DV>(s.aw, nullptr, 0, false, own_w + (size_t)own * kT * DV, n_own, warp, lane);
+    float m[8];
+    if (!KEYS) {
+        // the centre m_i: two threads per row
+        float x = 0.f;
+        const int t = tid >> 1;
+        if (t < n_own && !numerator_only) {
+            const float4* gr = reinterpret_cast<const float4*>(g + hw + (size_t)(own * kT + t) * DV);
+            const float4* vr = reinterpret_cast<const float4*>(v + hw + (size_t)(own * kT + t) * DV);
+#pragma unroll 8
+            for (int c = tid & 1; c < DV / 4; c += 2) {
+                const float4 a = __ldg(gr + c), b = __ldg(vr + c);
+                x = fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, x))));
+            }
+        }
+        x += __shfl_xor_sync(0xffffffffu, x, 1);
+        if ((tid & 1) == 0) s.m[t] = x;
+        __syncwarp();                                                // a warp's rows are its own
+#pragma unroll
+        for (int i = 0; i < 8; ++i) m[i] = s.m[row0 + (i >> 2) * 8 + (i & 3)];
+    }
+
+    float n1[4][8], n2[KEYS ? 1 : 4][8];             // X and Y, or dk
+    float den[8], num[8];                            // row sums of w and w G.v (dq pass)
+    float wide[KEYS ? 8 : 1][KEYS ? 4 * NV : 1];     // dv
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int d = 0; d < 8; ++d) {
+            n1[i][d] = 0.f;
+            if (!KEYS) n2[i][d] = 0.f;
+        }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        den[i] = num[i] = 0.f;
+        if (KEYS)
+#pragma unroll
+            for (int c = 0; c < 4 * NV; ++c) wide[i][c] = 0.f;
+    }
+
+    float* p1 = s.p[0][warp];
+    float* p2 = s.p[1][warp];
+    const int first = KEYS ? own : 0, last = KEYS ? ntile - 1 : own;
+    for (int tile = first + rank; tile <= last; tile += nsplit) {
+        const int n_loop = min(kT, L - tile * kT);
+        __syncthreads();                             // the tile before is read
+        load_tile<kDFeat>(s.bn, s.rn, kDFeat, true, loop_n + (size_t)tile * kT * kDFeat, n_loop, warp, lane);
+        load_tile<DV>(s.bw, KEYS ? s.rw : nullptr, S::kWide, false, loop_w + (size_t)tile * kT * DV, n_loop, warp, lane);
+        if (KEYS && tid < kT)
+            s.st[tid] = tid < n_loop ? stats[head * (size_t)L + tile * kT + tid] : make_float2(0.f, 0.f);
+        __syncthreads();
+
+        float sc[8][4], gv[8][4];
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) sc[i][j] = gv[i][j] = 0.f;
+        pair_product<kDFeat>(sc, s.an + row0, s.bn + 4 * co);
+        pair_product<DV>(gv, s.aw + row0, s.bw + 4 * co);
+
+        const bool diag = tile == own;
+        float2 st[4];
+        if (KEYS)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) st[j] = s.st[4 * co + j];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            float a[8], b[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int r = row0 + (i >> 2) * 8 + (i & 3), c = 4 * co + j;
+                const bool live = !diag || (KEYS ? r <= c : c <= r);
+                const float x = sc[i][j];
+                const float w = live ? fmaf(x, fmaf(x, 0.03125f, 0.25f), 1.0f) : 0.f;
+                const float w1 = live ? fmaf(x, 0.0625f, 0.25f) : 0.f;
+                if (KEYS) {
+                    a[i] = fmaf(gv[i][j], st[j].x, st[j].y) * w1;
+                    b[i] = w * st[j].x;
+                } else {
+                    den[i] += w;
+                    num[i] = fmaf(w, gv[i][j], num[i]);
+                    a[i] = w1 * (gv[i][j] - m[i]);
+                    b[i] = w1;
+                }
+            }
+            const int at = (j * 16 + co) * 16 + ro * 4;              // place_of(4 co + j)
+            *reinterpret_cast<float4*>(p1 + at) = make_float4(a[0], a[1], a[2], a[3]);
+            *reinterpret_cast<float4*>(p1 + at + 8) = make_float4(a[4], a[5], a[6], a[7]);
+            *reinterpret_cast<float4*>(p2 + at) = make_float4(b[0], b[1], b[2], b[3]);
+            *reinterpret_cast<float4*>(p2 + at + 8) = make_float4(b[4], b[5], b[6], b[7]);
+        }
+        __syncwarp();
+        narrow_product(n1, p1, s.rn, ks, rg, dg);
+        if constexpr (!KEYS) {
+            narrow_product(n2, p2, s.rn, ks, rg, dg);
+        } else {
+            // dv rows row0 + ..., columns 64 c + 4 co + e
+#pragma unroll 4
+            for (int t = 0; t < kT; ++t) {
+                const float* pr = p2 + place_of(t) * 16 + ro * 4;
+                const float4 x0 = lds4(pr), x1 = lds4(pr + 8);
+                const float xs[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+#pragma unroll
+                for (int c = 0; c < NV; ++c) {
+                    const float4 y = lds4(&s.rw[t * S::kWide + 64 * c + 4 * co]);
+                    const float ys[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) wide[i][4 * c + e] = fmaf(xs[i], ys[e], wide[i][4 * c + e]);
+                }
+            }
+        }
+        __syncwarp();
+    }
+
+    // ---- sums to shared memory ([64][16] each, statistics, [64][DV]; s.m lies behind them), then out, each CTA of the
+    // cluster its share of rows
+    __syncthreads();
+    float* o1 = reinterpret_cast<float*>(smem_raw);
+    float* o2 = o1 + kT * kDFeat;
+    float2* o3 = reinterpret_cast<float2*>(o2 + kT * kDFeat);
+    float* ow = o2;                                  // keys pass: dv behind dk
+    narrow_reduce(n1);
+    if constexpr (!KEYS) narrow_reduce(n2);
+    if (ks == 0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int at = (warp * 16 + rg * 4 + i) * kDFeat + dg * 8;
+            *reinterpret_cast<float4*>(o1 + at) = make_float4(n1[i][0], n1[i][1], n1[i][2], n1[i][3]);
+            *reinterpret_cast<float4*>(o1 + at + 4) = make_float4(n1[i][4], n1[i][5], n1[i][6], n1[i][7]);
+            if constexpr (!KEYS) {
+                *reinterpret_cast<float4*>(o2 + at) = make_float4(n2[i][0], n2[i][1], n2[i][2], n2[i][3]);
+                *reinterpret_cast<float4*>(o2 + at + 4) = make_float4(n2[i][4], n2[i][5], n2[i][6], n2[i][7]);
+            }
+        }
+    }
+    if constexpr (!KEYS) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int o = 2; o < 32; o <<= 1) {
+                den[i] += __shfl_xor_sync(0xffffffffu, den[i], o);
+                num[i] += __shfl_xor_sync(0xffffffffu, num[i], o);
+            }
+        if (co == 0)
+#pragma unroll
+            for (int i = 0; i < 8; ++i) o3[row0 + (i >> 2) * 8 + (i & 3)] = make_float2(den[i], num[i]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int c = 0; c < NV; ++c)
+                if (64 * c + 4 * co < DV)
+                    *reinterpret_cast<float4*>(ow + (row0 + (i >> 2) * 8 + (i & 3)) * DV + 64 * c + 4 * co) =
+                        make_float4(wide[i][4 * c], wide[i][4 * c + 1], wide[i][4 * c + 2], wide[i][4 * c + 3]);
+    }
+    if (nsplit > 1) cluster.sync();
+    else __syncthreads();
+    auto sum4 = [&](float* p) {
+        float4 x = lds4(p);
+        if (nsplit > 1) {
+            x = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int r = 0; r < nsplit; ++r) {
+                const float4 y = *reinterpret_cast<const float4*>(cluster.map_shared_rank(p, r));
+                x.x += y.x; x.y += y.y; x.z += y.z; x.w += y.w;
+            }
+        }
+        return x;
+    };
+    const int share = kT / nsplit, r0 = rank * share;
+    if constexpr (!KEYS) {
+        const int r_end = min(r0 + share, n_own);
+        for (int e = tid; e < share * 4; e += kBT) {
+            const int r = r0 + (e >> 2), d = (e & 3) * 4;
+            if (r >= r_end) continue;
+            const float4 x = sum4(o1 + r * kDFeat + d), y = sum4(o2 + r * kDFeat + d);
+            float dsum = 0.f, nsum = 0.f;
+            for (int c = 0; c < nsplit; ++c) {
+                const float2 t = nsplit > 1 ? *cluster.map_shared_rank(o3 + r, c) : o3[r];
+                dsum += t.x;
+                nsum += t.y;
+            }
+            const float inv = numerator_only ? 1.f : 1.f / (dsum + kEps);
+            const float b = numerator_only ? 0.f : -nsum * inv * inv;
+            const float c = numerator_only ? 0.f : fmaf(s.m[r], inv, b);
+            *reinterpret_cast<float4*>(dx + hn + (size_t)(own * kT + r) * kDFeat + d) =
+                make_float4(fmaf(x.x, inv, c * y.x), fmaf(x.y, inv, c * y.y), fmaf(x.z, inv, c * y.z), fmaf(x.w, inv, c * y.w));
+            if (d == 0) stats[head * (size_t)L + own * kT + r] = make_float2(inv, b);
+        }
+    } else {
+        const int r_end = min(r0 + share, n_own);
+        for (int e = tid; e < share * 4; e += kBT) {
+            const int r = r0 + (e >> 2), d = (e & 3) * 4;
+            if (r < r_end)
+                *reinterpret_cast<float4*>(dx + hn + (size_t)(own * kT + r) * kDFeat + d) = sum4(o1 + r * kDFeat + d);
+        }
+        for (int e = tid; e < share * (DV / 4); e += kBT) {
+            const int r = r0 + e / (DV / 4), d = e % (DV / 4) * 4;
+            if (r < r_end) *reinterpret_cast<float4*>(dv + hw + (size_t)(own * kT + r) * DV + d) = sum4(ow + r * DV + d);
+        }
+    }
+    if (nsplit > 1) cluster.sync();                  // no CTA leaves while another reads its sums
+}
+
+namespace {
+template <int DV, bool KEYS>
+based_status launch_pass(const float* q, const float* k, const float* v, const float* g, float2* stats, float* dx, float* dv,
+                         int BH, int L, int numerator_only, cudaStream_t stream) {
+    const int smem = (int)sizeof(BwdSmem<DV, KEYS>);
+    {
+        static bool configured[64] = {};
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return BASED_ERR_CUDA;
+        std::lock_guard<std::mutex> lock(setup_mutex());
+        if (!configured[dev]) {
+            if (cudaFuncSetAttribute(backward_f32_kernel<DV, KEYS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
+                cudaSuccess)
+                return BASED_ERR_CUDA;
+            configured[dev] = true;
+        }
+    }
+    const int ntile = (L + kT - 1) / kT;
+    int nsplit = 1;                                  // two CTAs fit an SM
+    while (nsplit < kMaxSplit && 2 * nsplit <= ntile && (long long)BH * ntile * 2 * nsplit <= 2 * 148) nsplit *= 2;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(ntile, BH, nsplit);
+    cfg.blockDim = dim3(kBT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 1;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = nsplit;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, backward_f32_kernel<DV, KEYS>, q, k, v, g, stats, dx, dv, L, numerator_only);
+    note_launch();
+    const based_status st = check_launch("backward_f32_kernel");
+    return e == cudaSuccess ? st : BASED_ERR_CUDA;
+}
+template <int DV>
+based_status launch_dv(const float* q, const float* k, const float* v, const float* g, float* dq, float* dk, float* dv,
+                       float2* stats, int BH, int L, int numerator_only, cudaStream_t stream) {
+    const based_status st = launch_pass<DV, false>(q, k, v, g, stats, dq, nullptr, BH, L, numerator_only, stream);
+    if (st != BASED_OK) return st;
+    return launch_pass<DV, true>(q, k, v, g, stats, dk, dv, BH, L, numerator_only, stream);
+}
+}  // namespace
+
+based_status launch_prefill_backward_f32(const float* q, const float* k, const float* v, const float* g, float* dq, float* dk,
+                                         float* dv, float* stats, int BH, int L, int d_v, int numerator_only,
+                                         cudaStream_t stream) {
+    float2* st = reinterpret_cast<float2*>(stats);
+    if (d_v == 64) return launch_dv<64>(q, k, v, g, dq, dk, dv, st, BH, L, numerator_only, stream);
+    if (d_v == 112) return launch_dv<112>(q, k, v, g, dq, dk, dv, st, BH, L, numerator_only, stream);
+    return launch_dv<128>(q, k, v, g, dq, dk, dv, st, BH, L, numerator_only, stream);
+}
+
+}  // namespace based

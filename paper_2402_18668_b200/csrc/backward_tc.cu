@@ -1,5 +1,5 @@
 // based_prefill_backward, bf16 tensor-core path (tcgen05 / TMEM / TMA): the same three passes as
-// the fp32 path (row statistics, dq, dk + dv; see backward_simt.cu for the formulas), with every
+// the fp32 path (row statistics, dq, dk + dv; see backward_f32.cu for the formulas), with every
 // 128 x 128 tile of (query, key) pairs evaluated by tensor-core products:
 //
 //   S  = Q_i K_j^T          (K = 16)          GV = G_i V_j^T   (K = d_v; G = dout, exact in bf16)

@@ -109,9 +109,9 @@ based_status launch_swa_decode(const void* q, const void* k, const void* v, void
 based_status launch_baseconv(const void* a, const void* g, const float* h, const float* b2, void* state, void* out,
                              int B, int N, int C, int width, bool step, based_dtype io, cudaStream_t stream);
 // backward of the linear attention (fp32 FMA, quadratic form); stats: [BH, L] float2 scratch
-based_status launch_prefill_backward(const void* q, const void* k, const void* v, const void* g, void* dq, void* dk,
-                                     void* dv, float* stats, int BH, int L, int d_v, based_dtype io,
-                                     int numerator_only, cudaStream_t stream);
+based_status launch_prefill_backward_f32(const float* q, const float* k, const float* v, const float* g, float* dq, float* dk,
+                                         float* dv, float* stats, int BH, int L, int d_v, int numerator_only,
+                                         cudaStream_t stream);
 // feature dimensions 8, 24, 32 (fp32 FMA, definition form); state layout [1 + d' + d'^2, d_v]
 // outputs_done: out has been written already (tensor-core forward), only the state is still to do
 based_status launch_prefill_generic(const void* q, const void* k, const void* v, void* out, float* kv, float* z,

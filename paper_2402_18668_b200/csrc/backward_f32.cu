@@ -19,8 +19,10 @@
 // address costs two passes, four otherwise.  Few tiles: the CTAs of a cluster share one own tile's loop, and their sums
 // are added through distributed shared memory in a fixed order.
 // Measured against three sweeps of 4 x 8 pairs per thread on scalar shared-memory loads: B2 H16 L1024 d_v64 1050 -> 424 us,
-// B1 H2 L1024 d_v64 56 us with eight CTAs per own tile.  Bound: the fp32 pipe at a third of its rate (135 us of FMAs); two
-// CTAs of four warps fit an SM, and a tile's loads and its products take turns in each.
+// B1 H2 L1024 d_v64 56 us with eight CTAs per own tile; 424 -> 294 us with the longest loops of all heads first and one
+// weight at a time in shared memory.  Bound: the fp32 pipe at half its rate (135 us of FMAs there; 1050 of 2090 us at
+// B4 H16 L2048).  Three CTAs per SM (168 registers, the weights in the looped tile's place) 328 to 350 us: their spills
+// and the extra barrier cost what the third CTA hides.
 #include <cooperative_groups.h>
 
 #include "common.cuh"
@@ -45,7 +47,7 @@ struct BwdSmem {
     float bw[DV * kP];             // looped v (dout), transposed
     float rn[kT * kDFeat];         // looped k (q) as it lies, row t at place of(t)
     float rw[KEYS ? kT * kWide : 4];    // looped dout as it lies
-    float p[2][4][kT * 16];        // per warp: two weights of (looped row at place of(t), own row)
+    float p[4][kT * 16];           // per warp: a weight of (looped row at place of(t), own row)
     float2 st[kT];                 // keys pass: (1 / D, b) of the looped queries
     float m[kT];
 };
@@ -106,6 +108,12 @@ __device__ __forceinline__ void narrow_product(float (&acc)[4][8], const float* 
             for (int d = 0; d < 8; ++d) acc[i][d] = fmaf(xs[i], ys[d], acc[i][d]);
     }
 }
+// one weight of a thread's own rows and looped row 4 co + j
+__device__ __forceinline__ void store_weight(float* p, const float (&a)[8], int j, int co, int ro) {
+    float* at = p + (j * 16 + co) * 16 + ro * 4;                     // place_of(4 co + j)
+    *reinterpret_cast<float4*>(at) = make_float4(a[0], a[1], a[2], a[3]);
+    *reinterpret_cast<float4*>(at + 8) = make_float4(a[4], a[5], a[6], a[7]);
+}
 // sums over the four lane groups ks (lane bits 3, 4)
 __device__ __forceinline__ void narrow_reduce(float (&acc)[4][8]) {
 #pragma unroll
@@ -118,20 +126,20 @@ __device__ __forceinline__ void narrow_reduce(float (&acc)[4][8]) {
 }
 }  // namespace
 
-// KEYS = false: dq and the statistics.  KEYS = true: dk and dv.  grid (tiles, heads, CTAs per tile)
+// KEYS = false: dq and the statistics.  KEYS = true: dk and dv.  grid (heads x tiles, 1, CTAs per tile)
 template <int DV, bool KEYS>
-__global__ void __launch_bounds__(kBT)
+__global__ void __launch_bounds__(kBT, DV > 64 ? 1 : 2)
     backward_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v,
-                        const float* __restrict__ g, float2* stats, float* __restrict__ dx, float* __restrict__ dv, int L,
-                        int numerator_only) {
+                        const float* __restrict__ g, float2* stats, float* __restrict__ dx, float* __restrict__ dv, int heads,
+                        int L, int numerator_only) {
     using S = BwdSmem<DV, KEYS>;
     constexpr int NV = S::kCols / 64;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     S& s = *reinterpret_cast<S*>(smem_raw);
     cg::cluster_group cluster = cg::this_cluster();
-    const int ntile = gridDim.x, nsplit = gridDim.z, rank = blockIdx.z;
-    const int own = KEYS ? blockIdx.x : ntile - 1 - blockIdx.x;      // longest loops first
-    const size_t head = blockIdx.y;
+    const int nsplit = gridDim.z, rank = blockIdx.z, ntile = (L + kT - 1) / kT, turn = blockIdx.x / heads;
+    const int own = KEYS ? turn : ntile - 1 - turn;                  // longest loops of all heads first
+    const size_t head = blockIdx.x - turn * heads;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int ro = lane & 1, co = lane >> 1;                         // pair tile: own rows row0 + {0..3, 8..11}, looped 4 co + j
     const int row0 = warp * 16 + ro * 4;
@@ -184,8 +192,7 @@ __global__ void __launch_bounds__(kBT)
             for (int c = 0; c < 4 * NV; ++c) wide[i][c] = 0.f;
     }
 
-    float* p1 = s.p[0][warp];
-    float* p2 = s.p[1][warp];
+    float* p = s.p[warp];
     const int first = KEYS ? own : 0, last = KEYS ? ntile - 1 : own;
     for (int tile = first + rank; tile <= last; tile += nsplit) {
         const int n_loop = min(kT, L - tile * kT);
@@ -209,9 +216,10 @@ __global__ void __launch_bounds__(kBT)
         if (KEYS)
 #pragma unroll
             for (int j = 0; j < 4; ++j) st[j] = s.st[4 * co + j];
+        // the first weight to the warp's shared memory; the second one takes the place of the scores
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            float a[8], b[8];
+            float a[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const int r = row0 + (i >> 2) * 8 + (i & 3), c = 4 * co + j;
@@ -221,29 +229,32 @@ __global__ void __launch_bounds__(kBT)
                 const float w1 = live ? fmaf(x, 0.0625f, 0.25f) : 0.f;
                 if (KEYS) {
                     a[i] = fmaf(gv[i][j], st[j].x, st[j].y) * w1;
-                    b[i] = w * st[j].x;
+                    sc[i][j] = w * st[j].x;
                 } else {
                     den[i] += w;
                     num[i] = fmaf(w, gv[i][j], num[i]);
                     a[i] = w1 * (gv[i][j] - m[i]);
-                    b[i] = w1;
+                    sc[i][j] = w1;
                 }
             }
-            const int at = (j * 16 + co) * 16 + ro * 4;              // place_of(4 co + j)
-            *reinterpret_cast<float4*>(p1 + at) = make_float4(a[0], a[1], a[2], a[3]);
-            *reinterpret_cast<float4*>(p1 + at + 8) = make_float4(a[4], a[5], a[6], a[7]);
-            *reinterpret_cast<float4*>(p2 + at) = make_float4(b[0], b[1], b[2], b[3]);
-            *reinterpret_cast<float4*>(p2 + at + 8) = make_float4(b[4], b[5], b[6], b[7]);
+            store_weight(p, a, j, co, ro);
         }
         __syncwarp();
-        narrow_product(n1, p1, s.rn, ks, rg, dg);
+        narrow_product(n1, p, s.rn, ks, rg, dg);
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float a[8] = {sc[0][j], sc[1][j], sc[2][j], sc[3][j], sc[4][j], sc[5][j], sc[6][j], sc[7][j]};
+            store_weight(p, a, j, co, ro);
+        }
+        __syncwarp();
         if constexpr (!KEYS) {
-            narrow_product(n2, p2, s.rn, ks, rg, dg);
+            narrow_product(n2, p, s.rn, ks, rg, dg);
         } else {
             // dv rows row0 + ..., columns 64 c + 4 co + e
 #pragma unroll 4
             for (int t = 0; t < kT; ++t) {
-                const float* pr = p2 + place_of(t) * 16 + ro * 4;
+                const float* pr = p + place_of(t) * 16 + ro * 4;
                 const float4 x0 = lds4(pr), x1 = lds4(pr + 8);
                 const float xs[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
 #pragma unroll
@@ -370,7 +381,7 @@ based_status launch_pass(const float* q, const float* k, const float* v, const f
     int nsplit = 1;                                  // two CTAs fit an SM
     while (nsplit < kMaxSplit && 2 * nsplit <= ntile && (long long)BH * ntile * 2 * nsplit <= 2 * 148) nsplit *= 2;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(ntile, BH, nsplit);
+    cfg.gridDim = dim3((unsigned)BH * ntile, 1, nsplit);
     cfg.blockDim = dim3(kBT);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
@@ -381,7 +392,7 @@ based_status launch_pass(const float* q, const float* k, const float* v, const f
     attr.val.clusterDim.z = nsplit;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, backward_f32_kernel<DV, KEYS>, q, k, v, g, stats, dx, dv, L, numerator_only);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, backward_f32_kernel<DV, KEYS>, q, k, v, g, stats, dx, dv, BH, L, numerator_only);
     note_launch();
     const based_status st = check_launch("backward_f32_kernel");
     return e == cudaSuccess ? st : BASED_ERR_CUDA;

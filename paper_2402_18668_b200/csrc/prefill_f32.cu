@@ -303,11 +303,12 @@ namespace {
 int f32_segment_tokens(int L, int nseg) { return ((L + nseg - 1) / nseg + 15) / 16 * 16; }
 // Segments per head (the cluster holds all segments of both column groups, at most 16 CTAs), by a time model fitted on
 // B200, in us: outputs of a full chunk 10.5 (a chunk of up to 32 / 16 tokens 0.5 / 0.3 of that), a state update 5.5, two
-// CTAs on an SM 1.9 times one, 5 for launch and ramps, 4 + 0.3 n for the running sums of n segments.  More segments
-// shorten the chain of chunks but every chunk then updates a state twice (its segment's own sums, then the running
-// state): B1 H2 L256 d_v64 70 / 46 / 26 / 23 / 22 us with 1 / 2 / 4 / 8 / 16 segments, B2 H16 L1024 d_v64 257 / 177 / 92 /
-// 93 / 126, B8 H16 L512 d_v64 133 / 153 / 150 / 184 / 343.  The same whether the state is asked for or not: so are the
-// outputs.
+// CTAs on an SM 1.9 times one, 5 for launch and ramps, 4 + 0.3 n for the running sums of n segments, all of it once per
+// wave.  Clusters of 8 and 16 CTAs leave SMs of a GPC unused: about 104 and 96 fit one per SM.  More segments shorten the
+// chain of chunks but every chunk then updates a state twice (its segment's own sums, then the running state): B1 H2 L256
+// d_v64 70 / 46 / 26 / 23 / 22 us with 1 / 2 / 4 / 8 / 16 segments, B2 H16 L1024 d_v64 257 / 177 / 92 / 93 / 126, B8 H16
+// L512 d_v64 133 / 153 / 150 / 184 / 343, B1 H16 L700 d_v64 179 / 126 / 68 / 71 / 75.  The same whether the state is asked
+// for or not: so are the outputs.
 int f32_segments(int BH, int L, int nz) {
     int best = 1;
     double best_t = 1e30;
@@ -315,8 +316,9 @@ int f32_segments(int BH, int L, int nz) {
         const int seg = f32_segment_tokens(L, n), rest = seg % kTok, chunks = (seg + kTok - 1) / kTok;
         const double outs = seg / kTok + (rest == 0 ? 0.0 : rest <= 16 ? 0.3 : rest <= 32 ? 0.5 : 1.0);
         const double ups = n > 1 ? 2 * chunks - 1 : chunks;
-        const long long per_sm = ((long long)BH * nz * n + 147) / 148;
-        const double t = (per_sm == 1 ? 1.0 : 0.95 * (double)per_sm) * (outs * 10.5 + ups * 5.5) + 5.0 + (n > 1 ? 4.0 + 0.3 * n : 0.0);
+        const long long ctas = (long long)BH * nz * n, fit = n * nz <= 4 ? 148 : n * nz == 8 ? 104 : 96;
+        const double waves = (double)((ctas + 2 * fit - 1) / (2 * fit));
+        const double t = waves * ((ctas <= fit ? 1.0 : 1.9) * (outs * 10.5 + ups * 5.5) + 5.0 + (n > 1 ? 4.0 + 0.3 * n : 0.0));
         if (t < best_t) { best_t = t; best = n; }
     }
     return best;

@@ -1,4 +1,4 @@
-"""Builds libbased.so (CUDA, sm_100a only) in-tree with nvcc.
+"""Builds libbased.so (CUDA, sm_100a only) in-tree with nvcc, and the binding's extension with g++.
 
 ``python -m paper_2402_18668_b200.build`` or ``build()``; objects are rebuilt only
 when their source (or a header) is newer.  nvcc cross-compiles without a GPU.
@@ -16,6 +16,8 @@ CSRC = PKG / "csrc"
 INCLUDE = PKG.parent / "include"
 OBJ = PKG / "build"
 LIB = PKG / "libbased.so"
+NATIVE_SRC = PKG / "csrc_host" / "native.cpp"
+NATIVE = PKG / "_native.so"
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -33,6 +35,43 @@ def _nvcc() -> str:
 
 def sources():
     return sorted(CSRC.glob("*.cu"))
+
+
+def _native_is_stale() -> bool:
+    """Also after a change of the interpreter or of torch, whose C++ headers the extension is compiled against."""
+    stamp = OBJ / "native.stamp"
+    return (not NATIVE.exists() or not stamp.exists() or stamp.read_text() != _native_versions() or
+            NATIVE.stat().st_mtime < max(p.stat().st_mtime for p in (NATIVE_SRC, INCLUDE / "based.h")))
+
+
+def _native_versions() -> str:
+    import torch
+    return f"{sys.version_info[:3]} {torch.__version__}"
+
+
+def build_native() -> Path:
+    """_native.so: compiled against torch's headers; libbased.so is found beside it when it is loaded."""
+    import sysconfig
+
+    import torch
+    t = Path(torch.__file__).resolve().parent
+    stub = OBJ / "libbased.so"             # stands in for the library at link time: its symbols are resolved at load time
+    r = subprocess.run(["g++", "-shared", "-Wl,-soname,libbased.so", "-o", str(stub), "-x", "c", os.devnull],
+                       capture_output=True, text=True)
+    tmp = NATIVE.with_suffix(f".so.tmp{os.getpid()}")
+    if r.returncode == 0:
+        r = subprocess.run(
+            ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
+             "-isystem", str(t / "include"), "-isystem", str(t / "include" / "torch" / "csrc" / "api" / "include"),
+             "-isystem", sysconfig.get_paths()["include"], "-isystem", "/usr/local/cuda/include", "-I", str(INCLUDE),
+             str(NATIVE_SRC), "-o", str(tmp), "-L", str(t / "lib"), "-Wl,--no-as-needed", "-lc10", "-lc10_cuda", "-ltorch_cpu",
+             "-ltorch", "-ltorch_python", "-L", str(OBJ), "-l:libbased.so", "-Wl,-rpath,$ORIGIN"],
+            capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"{NATIVE_SRC.name} failed to build:\n{r.stdout}\n{r.stderr}")
+    os.replace(tmp, NATIVE)
+    (OBJ / "native.stamp").write_text(_native_versions())
+    return NATIVE
 
 
 def build(force: bool = False, verbose: bool = False) -> Path:
@@ -55,8 +94,11 @@ def build(force: bool = False, verbose: bool = False) -> Path:
         if verbose:
             sys.stderr.write(r.stderr)
 
-    with ThreadPoolExecutor(max_workers=min(8, max(1, len(jobs)))) as ex:
-        list(ex.map(compile_one, jobs))
+    native_jobs = [build_native] if force or _native_is_stale() else []
+    with ThreadPoolExecutor(max_workers=min(8, max(1, len(jobs) + len(native_jobs)))) as ex:
+        running = [ex.submit(j) for j in native_jobs] + [ex.submit(compile_one, j) for j in jobs]
+        for r in running:
+            r.result()
     objs = [OBJ / (s.stem + ".o") for s in srcs]
     if jobs or not LIB.exists() or force:
         tmp = LIB.with_suffix(f".so.tmp{os.getpid()}")

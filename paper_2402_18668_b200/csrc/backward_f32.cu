@@ -379,7 +379,7 @@ based_status launch_pass(const float* q, const float* k, const float* v, const f
     }
     const int ntile = (L + kT - 1) / kT;
     int nsplit = 1;                                  // two CTAs fit an SM
-    while (nsplit < kMaxSplit && 2 * nsplit <= ntile && (long long)BH * ntile * 2 * nsplit <= 2 * 148) nsplit *= 2;
+    while (nsplit < kMaxSplit && 2 * nsplit <= ntile && (long long)BH * ntile * 2 * nsplit <= 2 * kSMs) nsplit *= 2;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)BH * ntile, 1, nsplit);
     cfg.blockDim = dim3(kBT);

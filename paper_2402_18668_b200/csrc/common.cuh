@@ -14,6 +14,7 @@ namespace based {
 constexpr int kDFeat = 16;                              // d' of the paper
 constexpr int kD = 1 + kDFeat + kDFeat * kDFeat;        // 273 expanded features
 constexpr int kDSym = 1 + kDFeat + kDFeat * (kDFeat + 1) / 2;   // 153 features, one per unordered pair
+constexpr int kSMs = 148;                                // B200
 constexpr float kEps = 1e-12f;                          // eps of the paper's listings
 // feature-map scales: x / d'^(1/4) and x_m x_n / (sqrt(2) sqrt(d')), d' = 16
 constexpr float kLinScale = 0.5f;
@@ -48,13 +49,11 @@ __device__ __forceinline__ float phi_at(const float* x, int f) {
 
 // Symmetric feature set: index 0 the constant, 1..16 the linear terms, then the pairs m <= n in
 // row-major order of the upper triangle.  pair_of(p) returns (m, n) of pair p in [0, 136).
-__host__ __device__ __forceinline__ void pair_of(int p, int& m, int& n) {
-    m = 0;
-    while (p >= kDFeat - m) {
-        p -= kDFeat - m;
-        ++m;
-    }
-    n = m + p;
+__device__ __forceinline__ void pair_of(int p, int& m, int& n) {
+    // m = the largest with 16 m - m (m - 1) / 2 <= p, the root of a quadratic: its argument is a perfect square (and the
+    // square root exact) where p starts a row, and at least 8 below the next one elsewhere
+    m = static_cast<int>((33.f - sqrtf(1089.f - 8.f * static_cast<float>(p))) * 0.5f);
+    n = p - kDFeat * m + m * (m - 1) / 2 + m;
 }
 // row of pair (m, n), m <= n, in the symmetric layout
 __host__ __device__ constexpr int sym_pair_row(int m, int n) {

@@ -7,39 +7,69 @@
 //
 // The step is a pure stream over the fp32 state: each head's [273, d_v] block is
 // read once and written once (2 * 273 * d_v * 4 bytes per head), 0.5 flop per byte,
-// so the kernel is bounded by HBM bandwidth.  One CTA of 256 threads owns one head.
+// so the kernel is bounded by HBM bandwidth.  One CTA of 256 threads owns one head (with few heads, a cluster of CTAs).
 // A state row is covered by d_v/4 consecutive threads with one 128-bit load each, so
 // every warp instruction touches whole 512-byte (d_v=128) or two 256-byte (d_v=64)
 // rows; loads of several rows are issued before the first dependent FMA to keep
-// many bytes in flight per SM (4 CTAs per SM).
+// many bytes in flight per SM.
 #include "common.cuh"
 #include "decode.cuh"
 
 namespace based {
 
-template <int DV, typename T, bool STREAM, bool SYM>
-__global__ void __launch_bounds__(256, 4) decode_step_kernel(const T* __restrict__ q, const T* __restrict__ k,
+template <int DV, typename T, bool SYM, int PARTS, int UN, int CTAS, bool STREAM>
+__global__ void __launch_bounds__(256, CTAS) decode_step_kernel(const T* __restrict__ q, const T* __restrict__ k,
                                                           const T* __restrict__ v, float* __restrict__ kv,
                                                           float* __restrict__ z, T* __restrict__ out,
                                                           int numerator_only) {
-    decode_step_body<DV, T, STREAM, SYM>(q, k, v, kv, z, out, numerator_only, blockIdx.x);
+    decode_step_body<DV, T, SYM, PARTS, UN, STREAM>(q, k, v, kv, z, out, numerator_only, blockIdx.x / PARTS,
+                                                    blockIdx.x % PARTS);
 }
 
-template <int DV, typename T, bool SYM>
-static based_status launch_t(const void* q, const void* k, const void* v, float* kv, float* z, void* out, int BH,
-                             int num_only, cudaStream_t stream) {
-    // 96 MB: safely above what L2 (126 MB, shared with everything else) keeps from one step to the next
-    const bool streaming = (size_t)BH * (SYM ? kDSym : kD) * DV * sizeof(float) > (size_t)96 << 20;
-    if (streaming)
-        decode_step_kernel<DV, T, true, SYM><<<BH, 256, 0, stream>>>(
-            static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), kv, z, static_cast<T*>(out),
-            num_only);
-    else
-        decode_step_kernel<DV, T, false, SYM><<<BH, 256, 0, stream>>>(
-            static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), kv, z, static_cast<T*>(out),
-            num_only);
+template <int DV, typename T, bool SYM, int PARTS, int UN, int CTAS, bool STREAM>
+static based_status launch_variant(const T* q, const T* k, const T* v, float* kv, float* z, T* out, int BH, int num_only,
+                                   cudaStream_t stream) {
+    auto kern = decode_step_kernel<DV, T, SYM, PARTS, UN, CTAS, STREAM>;
+    if (PARTS == 1) {
+        kern<<<BH, 256, 0, stream>>>(q, k, v, kv, z, out, num_only);
+    } else {
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(PARTS * BH);
+        cfg.blockDim = dim3(256);
+        cfg.stream = stream;
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = PARTS;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        if (cudaLaunchKernelEx(&cfg, kern, q, k, v, kv, z, out, num_only) != cudaSuccess) {
+            note_launch();
+            check_launch("decode_step_kernel");
+            return BASED_ERR_CUDA;
+        }
+    }
     note_launch();
     return check_launch("decode_step_kernel");
+}
+
+// The variants of a step, by the number of heads (us per step on B200, replayed back to back):
+//   deep   18 rows in flight per thread, two CTAs per SM: one wave of up to 296 heads (d_v 128: 128 heads 6.0 against 6.2
+//          wide; 153 rows: 4.2 / 4.7), and again beyond one wave of wide ones (2048 heads 89.9 / 91.4, 800: 36.9 / 39.7);
+//   wide   6 rows, four CTAs per SM: one wave of up to 592 heads (592: 17.5 against 19.2 deep; 400: 12.0 / 15.3);
+//   parts  9 rows, a cluster of two or four CTAs per head (decode_parts).
+template <int DV, typename T, bool SYM>
+static based_status launch_t(const void* q_, const void* k_, const void* v_, float* kv, float* z, void* out_, int BH,
+                             int n, cudaStream_t stream) {
+    const T *q = static_cast<const T*>(q_), *k = static_cast<const T*>(k_), *v = static_cast<const T*>(v_);
+    T* out = static_cast<T*>(out_);
+    const int parts = decode_parts<DV, SYM>(BH);
+    if (parts == 4) return launch_variant<DV, T, SYM, 4, 9, 2, false>(q, k, v, kv, z, out, BH, n, stream);
+    if (parts == 2) return launch_variant<DV, T, SYM, 2, 9, 2, false>(q, k, v, kv, z, out, BH, n, stream);
+    if (decode_streams(BH, DV, SYM))
+        return launch_variant<DV, T, SYM, 1, 18, 2, true>(q, k, v, kv, z, out, BH, n, stream);
+    if (BH > 2 * kSMs && BH <= 4 * kSMs) return launch_variant<DV, T, SYM, 1, 6, 4, false>(q, k, v, kv, z, out, BH, n, stream);
+    return launch_variant<DV, T, SYM, 1, 18, 2, false>(q, k, v, kv, z, out, BH, n, stream);
 }
 
 template <int DV, bool SYM>
@@ -128,10 +158,15 @@ bool load_kernel(K kernel) {
     cudaFuncAttributes attr;
     return cudaFuncGetAttributes(&attr, kernel) == cudaSuccess;
 }
+template <int DV, typename T, bool SYM>
+bool load_decode_format() {
+    return load_kernel(decode_step_kernel<DV, T, SYM, 4, 9, 2, false>) && load_kernel(decode_step_kernel<DV, T, SYM, 2, 9, 2, false>) &&
+           load_kernel(decode_step_kernel<DV, T, SYM, 1, 18, 2, false>) && load_kernel(decode_step_kernel<DV, T, SYM, 1, 18, 2, true>) &&
+           load_kernel(decode_step_kernel<DV, T, SYM, 1, 6, 4, false>);
+}
 template <int DV, typename T>
 bool load_decode_variants() {
-    return load_kernel(decode_step_kernel<DV, T, false, false>) && load_kernel(decode_step_kernel<DV, T, true, false>) &&
-           load_kernel(decode_step_kernel<DV, T, false, true>) && load_kernel(decode_step_kernel<DV, T, true, true>);
+    return load_decode_format<DV, T, false>() && load_decode_format<DV, T, true>();
 }
 }  // namespace
 

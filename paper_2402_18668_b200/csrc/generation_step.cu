@@ -13,7 +13,7 @@
 // CTA roles by block index (256 threads each):
 //   window role: two groups of 128 threads, one head each, the code of swa_decode_kernel with a named
 //                barrier per group (swa_decode.cuh);
-//   state role:  the code of decode_step_kernel (decode.cuh).
+//   state role:  the code of decode_step_kernel (decode.cuh), with few heads shared by the CTAs of a cluster as there.
 #include "decode.cuh"
 #include "swa_decode.cuh"
 
@@ -37,17 +37,17 @@ struct GenArgs {
     int* pos_state;       // {position, ticket}
     float scale;
     unsigned int* err;
-    // dealing of the roles
-    int n_pairs;          // leading triples (window CTA, state CTA, state CTA)
+    int n_pairs;          // dealing of the roles: leading triples (window CTA, state CTA, state CTA)
     int swa_group_bytes;  // shared memory of one 128-thread window group
 };
 
-template <int DV, typename T, bool STREAM, bool SYM, int NPW>
-__global__ void __launch_bounds__(256, 4) generation_step_kernel(const GenArgs a) {
+template <int DV, typename T, bool STREAM, bool SYM, int NPW, int PARTS, int UN, int CTAS>
+__global__ void __launch_bounds__(256, CTAS) generation_step_kernel(const GenArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
     // block index -> role: the first 3 * n_pairs blocks come in triples (window, state, state); then
-    // whatever window CTAs are left, then the remaining state CTAs
-    const int i = blockIdx.x, n_swa_ctas = (a.n_swa + 1) / 2;
+    // whatever window CTAs are left, then the remaining state CTAs.  With PARTS > 1 a block of this numbering is a
+    // cluster: the parts of one state head, or that many window CTAs.
+    const int i = blockIdx.x / PARTS, part = blockIdx.x % PARTS, n_swa_ctas = ((a.n_swa + 1) / 2 + PARTS - 1) / PARTS;
     int swa_cta = -1, lin_head = -1;
     if (i < 3 * a.n_pairs) {
         const int g = i / 3, r = i - 3 * g;
@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(256, 4) generation_step_kernel(const GenArgs a
     }
     if (swa_cta >= 0) {
         const int half = threadIdx.x >> 7;
-        const int head = 2 * swa_cta + half;
+        const int head = 2 * (swa_cta * PARTS + part) + half;
         if (head < a.n_swa) {
             const T* qw = static_cast<const T*>(a.qw);
             const T* kw = static_cast<const T*>(a.kw);
@@ -77,26 +77,56 @@ __global__ void __launch_bounds__(256, 4) generation_step_kernel(const GenArgs a
                                            (size_t)head, threadIdx.x & 127, a.n_swa, smem + a.swa_group_bytes);
         }
     } else {
-        decode_step_body<DV, T, STREAM, SYM>(static_cast<const T*>(a.q), static_cast<const T*>(a.k),
-                                             static_cast<const T*>(a.v), a.kv, a.z, static_cast<T*>(a.out),
-                                             a.numerator_only, (size_t)lin_head);
+        decode_step_body<DV, T, SYM, PARTS, UN, STREAM>(static_cast<const T*>(a.q), static_cast<const T*>(a.k),
+                                                    static_cast<const T*>(a.v), a.kv, a.z, static_cast<T*>(a.out),
+                                                    a.numerator_only, (size_t)lin_head, part);
     }
 }
 
-template <int DV, typename T, bool STREAM, bool SYM, int NPW>
-based_status launch_k(const GenArgs& a, size_t smem, cudaStream_t stream) {
-    auto kern = generation_step_kernel<DV, T, STREAM, SYM, NPW>;
+// State rows in flight per thread and CTAs per SM: 18 and 2, but 6 and 4 for narrow states that stay in L2 (batch 64 x 16
+// heads, 153 rows, d_v 64: 12.2 against 13.5 us; d_v 128: 25.8 deep, 30.9 wide; batch 128: 53.8 deep, 67.6 wide, 57.6 before both).
+template <int DV, bool STREAM> struct Depth {
+    static constexpr bool kWide = DV == 64 && !STREAM;
+    static constexpr int kRows = kWide ? 6 : 18, kCtas = kWide ? 4 : 2;
+};
+
+template <int DV, typename T, bool STREAM, bool SYM, int NPW, int PARTS>
+based_status launch_k(const GenArgs& args, size_t smem, cudaStream_t stream) {
+    auto kern = generation_step_kernel<DV, T, STREAM, SYM, NPW, PARTS, (PARTS > 1 ? 9 : Depth<DV, STREAM>::kRows), Depth<DV, STREAM>::kCtas>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return BASED_ERR_CUDA;
-    const int grid = a.n_lin + (a.n_swa + 1) / 2;
-    kern<<<grid, 256, smem, stream>>>(a);
+    GenArgs a = args;
+    const int n_swa_ctas = ((a.n_swa + 1) / 2 + PARTS - 1) / PARTS;
+    a.n_pairs = n_swa_ctas < a.n_lin / 2 ? n_swa_ctas : a.n_lin / 2;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((a.n_lin + n_swa_ctas) * PARTS);
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = PARTS;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = PARTS > 1 ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a);
     note_launch();
-    return check_launch("generation_step_kernel");
+    const based_status st = check_launch("generation_step_kernel");
+    return e == cudaSuccess ? st : BASED_ERR_CUDA;
 }
 
+template <int DV, typename T, bool STREAM, bool SYM, int NPW>
+based_status launch_p(const GenArgs& a, size_t smem, cudaStream_t stream) {
+    if constexpr (!STREAM) {
+        const int parts = decode_parts<DV, SYM>(a.n_lin);
+        if (parts == 4) return launch_k<DV, T, STREAM, SYM, NPW, 4>(a, smem, stream);
+        if (parts == 2) return launch_k<DV, T, STREAM, SYM, NPW, 2>(a, smem, stream);
+    }
+    return launch_k<DV, T, STREAM, SYM, NPW, 1>(a, smem, stream);
+}
 template <int DV, typename T, bool STREAM, bool SYM>
 based_status launch_w(const GenArgs& a, size_t smem, cudaStream_t stream) {
-    return a.window <= 64 ? launch_k<DV, T, STREAM, SYM, 4>(a, smem, stream) : launch_k<DV, T, STREAM, SYM, 8>(a, smem, stream);
+    return a.window <= 64 ? launch_p<DV, T, STREAM, SYM, 4>(a, smem, stream) : launch_p<DV, T, STREAM, SYM, 8>(a, smem, stream);
 }
 template <int DV, typename T>
 based_status launch_s(const GenArgs& a, size_t smem, bool sym, bool streaming, cudaStream_t stream) {
@@ -109,8 +139,7 @@ based_status launch_d(const GenArgs& a, int d_v, bool sym, cudaStream_t stream) 
     GenArgs b = a;
     b.swa_group_bytes = (int)group;
     const size_t smem = 2 * group;
-    // as in the stand-alone decode step: evict-first accesses once the state of all heads outgrows L2
-    const bool streaming = (size_t)a.n_lin * (sym ? kDSym : kD) * d_v * sizeof(float) > (size_t)96 << 20;
+    const bool streaming = decode_streams(a.n_lin, d_v, sym);
     if (d_v == 64) return launch_s<64, T>(b, smem, sym, streaming, stream);
     if (d_v == 112) return launch_s<112, T>(b, smem, sym, streaming, stream);
     return launch_s<128, T>(b, smem, sym, streaming, stream);
@@ -118,14 +147,20 @@ based_status launch_d(const GenArgs& a, int d_v, bool sym, cudaStream_t stream) 
 }  // namespace
 
 namespace {
-template <int DV, typename T, bool STREAM, bool SYM, int NPW>
-bool load_one() {
-    auto kern = generation_step_kernel<DV, T, STREAM, SYM, NPW>;
+template <int DV, typename T, bool STREAM, bool SYM, int NPW, int PARTS>
+bool load_parts() {
+    auto kern = generation_step_kernel<DV, T, STREAM, SYM, NPW, PARTS, (PARTS > 1 ? 9 : Depth<DV, STREAM>::kRows), Depth<DV, STREAM>::kCtas>;
     cudaFuncAttributes attr;
     // the largest request a launch of this variant can make: two groups at the widest window it serves
     const size_t group = (swa_decode_smem_bytes<T>(NPW == 4 ? 64 : 128) + 127) & ~(size_t)127;
     return cudaFuncGetAttributes(&attr, kern) == cudaSuccess &&
            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * group)) == cudaSuccess;
+}
+template <int DV, typename T, bool STREAM, bool SYM, int NPW>
+bool load_one() {
+    if (!load_parts<DV, T, STREAM, SYM, NPW, 1>()) return false;
+    if constexpr (!STREAM) return load_parts<DV, T, STREAM, SYM, NPW, 2>() && load_parts<DV, T, STREAM, SYM, NPW, 4>();
+    return true;
 }
 template <int DV, typename T>
 bool load_dv() {
@@ -152,8 +187,6 @@ based_status launch_generation_step(const void* q, const void* k, const void* v,
     a.qw = qw; a.kw = kw; a.vw = vw; a.kc = kc; a.vc = vc; a.outw = outw; a.n_swa = n_swa; a.window = window;
     a.pos_state = pos_state; a.scale = scale;
     if (error_word_ptr(&a.err) != BASED_OK) return BASED_ERR_CUDA;
-    const int n_swa_ctas = (n_swa + 1) / 2;
-    a.n_pairs = n_swa_ctas < n_lin / 2 ? n_swa_ctas : n_lin / 2;
     return io == BASED_F32 ? launch_d<float>(a, d_v, sym, stream) : launch_d<__nv_bfloat16>(a, d_v, sym, stream);
 }
 

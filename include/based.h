@@ -347,6 +347,25 @@ based_status based_generation_step(const void* q, const void* k, const void* v, 
                                    void* cuda_stream);
 
 /*
+ * The same step held as a CUDA graph of one kernel node, for a loop that takes every token's inputs from a different
+ * place: based_generation_graph_step points the node at this token's inputs and launches the graph (no copies into fixed
+ * input buffers ahead of it, one launch per token).  The arguments of based_generation_graph_create are those of
+ * based_generation_step; q, k, v, qw, kw, vw are buffers that hold the inputs of the last token: a step with inputs of its
+ * own (device pointers of the same layout, 16-byte aligned, read in stream order like any launch's inputs; not overlapping
+ * another input's buffer) leaves a copy in them, a step with six NULLs runs on what they hold.  All other pointers are
+ * fixed at creation and must outlive the graph.  Creation launches nothing; call based_preload_decode first.  Steps of one
+ * graph may come from several threads; like the step's state they belong on one stream at a time.
+ */
+typedef struct based_generation_graph based_generation_graph;
+based_status based_generation_graph_create(void* q, void* k, void* v, float* kv_state, float* z_state, void* out, void* qw,
+                                           void* kw, void* vw, void* k_cache, void* v_cache, void* out_w, int B, int H,
+                                           int d_feat, int d_v, int H_w, int d_w, int window, int* pos_state,
+                                           float softmax_scale, based_dtype io, int flags, based_generation_graph** graph);
+based_status based_generation_graph_step(based_generation_graph* graph, const void* q, const void* k, const void* v,
+                                         const void* qw, const void* kw, const void* vw, void* cuda_stream);
+void based_generation_graph_destroy(based_generation_graph* graph);
+
+/*
  * The same computation as based_prefill, for callers that cannot give the library scratch
  * memory.  (The paper has no counterpart: this is a deployment convenience.)  Some hosts
  * may not allocate device memory around a call at all - a serving process that has handed

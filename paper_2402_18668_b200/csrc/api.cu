@@ -3,6 +3,8 @@
 #include <atomic>
 #include <mutex>
 #include <cstdio>
+#include <new>
+#include <vector>
 
 #include "common.cuh"
 
@@ -369,6 +371,85 @@ based_status based_generation_step(const void* q, const void* k, const void* v, 
     return launch_generation_step(q, k, v, kv_state, z_state, out, B * H, d_v, (flags & BASED_STATE_SYM) != 0,
                                   (flags & BASED_NUMERATOR_ONLY) != 0, qw, kw, vw, k_cache, v_cache, out_w, B * H_w,
                                   window, pos_state, scale, io, static_cast<cudaStream_t>(cuda_stream));
+}
+
+struct based_generation_graph {
+    cudaGraph_t graph = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    cudaGraphNode_t node = nullptr;
+    cudaKernelNodeParams params{};
+    std::vector<unsigned char> args;           // the kernel's one argument
+    void* arg_list[1] = {nullptr};
+    void* buffers[6] = {};
+    bool own_inputs = false;                   // the node points at inputs other than the buffers
+    std::mutex mu;
+};
+
+void based_generation_graph_destroy(based_generation_graph* g) {
+    if (!g) return;
+    if (g->exec) cudaGraphExecDestroy(g->exec);
+    if (g->graph) cudaGraphDestroy(g->graph);
+    delete g;
+}
+
+based_status based_generation_graph_create(void* q, void* k, void* v, float* kv_state, float* z_state, void* out, void* qw,
+                                           void* kw, void* vw, void* k_cache, void* v_cache, void* out_w, int B, int H,
+                                           int d_feat, int d_v, int H_w, int d_w, int window, int* pos_state,
+                                           float softmax_scale, based_dtype io, int flags, based_generation_graph** graph) {
+    if (!graph) return BASED_ERR_INVALID_ARG;
+    *graph = nullptr;
+    // the step itself, captured on a stream of its own, gives the node
+    cudaStream_t stream = nullptr;
+    based_generation_graph* g = new (std::nothrow) based_generation_graph;
+    if (!g) return BASED_ERR_CUDA;
+    if (cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking) != cudaSuccess) {
+        delete g;
+        return BASED_ERR_CUDA;
+    }
+    based_status st = BASED_ERR_CUDA;
+    if (cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+        st = based_generation_step(q, k, v, kv_state, z_state, out, qw, kw, vw, k_cache, v_cache, out_w, B, H, d_feat, d_v, H_w,
+                                   d_w, window, pos_state, softmax_scale, io, flags, stream);
+        if (cudaStreamEndCapture(stream, &g->graph) != cudaSuccess && st == BASED_OK) st = BASED_ERR_CUDA;
+    }
+    cudaStreamDestroy(stream);
+    size_t n = 1;
+    if (st == BASED_OK && (cudaGraphGetNodes(g->graph, &g->node, &n) != cudaSuccess || n != 1 ||
+                           cudaGraphKernelNodeGetParams(g->node, &g->params) != cudaSuccess ||
+                           cudaGraphInstantiate(&g->exec, g->graph, 0) != cudaSuccess))
+        st = BASED_ERR_CUDA;
+    if (st != BASED_OK) {
+        based_generation_graph_destroy(g);
+        return st;
+    }
+    const unsigned char* arg = static_cast<const unsigned char*>(g->params.kernelParams[0]);
+    g->args.assign(arg, arg + generation_step_args_bytes());
+    g->arg_list[0] = g->args.data();
+    g->params.kernelParams = g->arg_list;
+    g->params.extra = nullptr;
+    void* const buffers[6] = {q, k, v, qw, kw, vw};
+    for (int i = 0; i < 6; ++i) g->buffers[i] = buffers[i];
+    *graph = g;
+    return BASED_OK;
+}
+
+based_status based_generation_graph_step(based_generation_graph* g, const void* q, const void* k, const void* v, const void* qw,
+                                         const void* kw, const void* vw, void* cuda_stream) {
+    if (!g) return BASED_ERR_INVALID_ARG;
+    const void* const in[6] = {q, k, v, qw, kw, vw};
+    int given = 0;
+    for (const void* p : in) {
+        given += p != nullptr;
+        if (!aligned16(p)) return BASED_ERR_ALIGNMENT;
+    }
+    if (given != 0 && given != 6) return BASED_ERR_INVALID_ARG;
+    std::lock_guard<std::mutex> lock(g->mu);
+    if (given || g->own_inputs) {
+        generation_step_inputs(g->args.data(), in, g->buffers);
+        if (cudaGraphExecKernelNodeSetParams(g->exec, g->node, &g->params) != cudaSuccess) return BASED_ERR_CUDA;
+        g->own_inputs = given != 0;
+    }
+    return cudaGraphLaunch(g->exec, static_cast<cudaStream_t>(cuda_stream)) == cudaSuccess ? BASED_OK : BASED_ERR_CUDA;
 }
 
 static based_status baseconv_check(const void* a, const void* g, const float* h, const float* b2, const void* out,

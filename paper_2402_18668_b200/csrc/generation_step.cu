@@ -39,7 +39,14 @@ struct GenArgs {
     unsigned int* err;
     int n_pairs;          // dealing of the roles: leading triples (window CTA, state CTA, state CTA)
     int swa_group_bytes;  // shared memory of one 128-thread window group
+    void* keep[6];        // null, or where the step leaves a copy of q, k, v, qw, kw, vw
 };
+
+// head's W values of an input to the place where a copy is kept (threads of one warp)
+template <typename T, int W>
+__device__ __forceinline__ void keep_row(void* to, const void* from, size_t head, int lane) {
+    for (int i = lane; i < W; i += 32) static_cast<T*>(to)[head * W + i] = static_cast<const T*>(from)[head * W + i];
+}
 
 template <int DV, typename T, bool STREAM, bool SYM, int NPW, int PARTS, int UN, int CTAS>
 __global__ void __launch_bounds__(256, CTAS) generation_step_kernel(const GenArgs a) {
@@ -75,11 +82,23 @@ __global__ void __launch_bounds__(256, CTAS) generation_step_kernel(const GenArg
             else
                 swa_decode_body<T, NPW, 2>(qw, kw, vw, kc, vc, ow, a.window, 0, a.pos_state, a.pos_state, a.scale, a.err,
                                            (size_t)head, threadIdx.x & 127, a.n_swa, smem + a.swa_group_bytes);
+            const int warp = (threadIdx.x & 127) >> 5, lane = threadIdx.x & 31;
+            if (a.keep[3] != nullptr && warp < 3) {
+                if (warp == 0) keep_row<T, kHD>(a.keep[3], a.qw, head, lane);
+                else if (warp == 1) keep_row<T, kHD>(a.keep[4], a.kw, head, lane);
+                else keep_row<T, kHD>(a.keep[5], a.vw, head, lane);
+            }
         }
     } else {
         decode_step_body<DV, T, SYM, PARTS, UN, STREAM>(static_cast<const T*>(a.q), static_cast<const T*>(a.k),
                                                     static_cast<const T*>(a.v), a.kv, a.z, static_cast<T*>(a.out),
                                                     a.numerator_only, (size_t)lin_head, part);
+        if (a.keep[0] != nullptr && part == 0) {
+            const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+            if (warp == 0) keep_row<T, kDFeat>(a.keep[0], a.q, lin_head, lane);
+            else if (warp == 1) keep_row<T, kDFeat>(a.keep[1], a.k, lin_head, lane);
+            else if (warp == 2) keep_row<T, DV>(a.keep[2], a.v, lin_head, lane);
+        }
     }
 }
 
@@ -188,6 +207,16 @@ based_status launch_generation_step(const void* q, const void* k, const void* v,
     a.pos_state = pos_state; a.scale = scale;
     if (error_word_ptr(&a.err) != BASED_OK) return BASED_ERR_CUDA;
     return io == BASED_F32 ? launch_d<float>(a, d_v, sym, stream) : launch_d<__nv_bfloat16>(a, d_v, sym, stream);
+}
+
+size_t generation_step_args_bytes() { return sizeof(GenArgs); }
+void generation_step_inputs(void* kernel_args, const void* const* in, void* const* buffers) {
+    GenArgs& a = *static_cast<GenArgs*>(kernel_args);
+    const void** const to[6] = {&a.q, &a.k, &a.v, &a.qw, &a.kw, &a.vw};
+    for (int i = 0; i < 6; ++i) {
+        *to[i] = in[i] ? in[i] : buffers[i];
+        a.keep[i] = in[i] ? buffers[i] : nullptr;
+    }
 }
 
 }  // namespace based

@@ -317,6 +317,78 @@ PyObject* generation_step(PyObject* const* a) {
     return wrap({out, out_w});
 }
 
+struct GenerationGraph {
+    based_generation_graph* graph;
+    Tensor in[6];                              // q, k, v, qw, kw, vw: the buffers of the last token's inputs
+};
+constexpr const char* kGraphName = "based_generation_graph";
+void free_graph(PyObject* capsule) {
+    GenerationGraph* g = static_cast<GenerationGraph*>(PyCapsule_GetPointer(capsule, kGraphName));
+    if (!g) return;
+    based_generation_graph_destroy(g->graph);
+    delete g;
+}
+GenerationGraph& graph_of(PyObject* o) {
+    GenerationGraph* g = static_cast<GenerationGraph*>(PyCapsule_GetPointer(o, kGraphName));
+    if (!g) {
+        PyErr_Clear();
+        throw TypeFault("expected a generation graph");
+    }
+    return *g;
+}
+// q, k, v, kv_state, z_state, qw, kw, vw, k_cache, v_cache, pos_state, out, out_w, flags, softmax_scale (all tensors live as
+// long as the graph: the caller sees to it)
+PyObject* generation_graph(PyObject* const* a) {
+    Tensor t[13];
+    for (int i = 0; i < 13; ++i) t[i] = need(a[i], "every tensor of a generation graph");
+    const Tensor &q = t[0], &v = t[2], &kv = t[3], &z = t[4], &qw = t[5], &kc = t[8];
+    check_qkv(q, t[1], v, t[11]);
+    const int B = size(q, 0), H = size(q, 1), d_feat = size(q, 2), d_v = size(v, 2), flags = integer(a[13]);
+    check_state(kv, z, B, H, d_feat, d_v, flags, true);
+    check_caches(kc, t[9], qw, "qw");
+    const float scale = number(a[14]);
+    const based_dtype io = dtype_code(q);
+    based_generation_graph* made = nullptr;
+    const based_status st = unlocked([&] {
+        return based_generation_graph_create(ptr(q), ptr(t[1]), ptr(v), fptr(kv), fptr(z), ptr(t[11]), ptr(qw), ptr(t[6]), ptr(t[7]),
+                                             ptr(kc), ptr(t[9]), ptr(t[12]), B, H, d_feat, d_v, size(qw, 1), size(qw, 2),
+                                             size(kc, 2), static_cast<int*>(ptr(t[10])), scale, io, flags, &made);
+    });
+    check(st, "based_generation_graph_create");
+    return PyCapsule_New(new GenerationGraph{made, {q, t[1], v, qw, t[6], t[7]}}, kGraphName, free_graph);
+}
+// graph, q, k, v, qw, kw, vw -> whether the step was launched on these inputs; False: they have to be copied into the
+// buffers first (another dtype, shape or layout, or they overlap the buffers)
+PyObject* generation_graph_step(PyObject* const* a) {
+    GenerationGraph& g = graph_of(a[0]);
+    const void* p[6];
+    for (int i = 0; i < 6; ++i) {
+        const Tensor &t = tensor(a[1 + i]), &own = g.in[i];
+        if (!t.defined() || t.scalar_type() != own.scalar_type() || t.sizes() != own.sizes() || t.device() != own.device() ||
+            !t.is_contiguous() || (reinterpret_cast<uintptr_t>(t.const_data_ptr()) & 15))
+            Py_RETURN_FALSE;
+        p[i] = t.const_data_ptr();
+        for (const Tensor& b : g.in) {
+            const char *x = static_cast<const char*>(p[i]), *y = static_cast<const char*>(b.const_data_ptr());
+            if (x < y + b.nbytes() && y < x + t.nbytes()) Py_RETURN_FALSE;
+        }
+    }
+    void* stream = c10::cuda::getCurrentCUDAStream().stream();
+    const based_status st = unlocked([&] { return based_generation_graph_step(g.graph, p[0], p[1], p[2], p[3], p[4], p[5], stream); });
+    check(st, "based_generation_graph_step");
+    Py_RETURN_TRUE;
+}
+// graph: the step on what the buffers hold
+PyObject* generation_graph_replay(PyObject* const* a) {
+    GenerationGraph& g = graph_of(a[0]);
+    void* stream = c10::cuda::getCurrentCUDAStream().stream();
+    const based_status st = unlocked([&] {
+        return based_generation_graph_step(g.graph, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, stream);
+    });
+    check(st, "based_generation_graph_step");
+    Py_RETURN_NONE;
+}
+
 // a, g, h, b2, conv_state, out, step (bool), stream
 PyObject* baseconv(PyObject* const* p) {
     const Tensor &a = need(p[0], "a"), &g = need(p[1], "g"), &h = need(p[2], "h"), &b2 = need(p[3], "b2"), &state = dev(p[4]);
@@ -422,6 +494,8 @@ template <PyObject* (*F)(PyObject* const*), int N> PyMethodDef method(const char
 PyMethodDef methods[] = {method<prefill, 9>("prefill"), method<prefill_backward, 8>("prefill_backward"),
                          method<decode_step, 9>("decode_step"), method<swa, 7>("swa"), method<swa_decode, 9>("swa_decode"),
                          method<generation_step, 16>("generation_step"), method<baseconv, 8>("baseconv"),
+                         method<generation_graph, 15>("generation_graph"), method<generation_graph_step, 7>("generation_graph_step"),
+                         method<generation_graph_replay, 1>("generation_graph_replay"),
                          method<linear_attention, 4>("linear_attention"), {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 }  // namespace

@@ -7,8 +7,10 @@ linear-attention decode step (on the 273-row or the 153-row symmetric state) and
 sliding-window decode step on its rolling cache, which reads the position from device memory and
 advances it itself, and replays it once per generated token.  By default the step is the
 library's fused call (based_generation_step: one kernel node in which the two mixers' CTAs are
-dealt out in turn, so the short window step rides in the shadow of the long state stream);
-fused=False captures the two separate kernels one after the other.
+dealt out in turn, so the short window step rides in the shadow of the long state stream), and
+`step` points that node at the token's inputs instead of copying them into fixed buffers first
+(the kernel leaves the copy in them): one launch per token.  fused=False captures the two separate
+kernels one after the other behind copies of the inputs.
 
 Only plumbing lives here (static buffers, stream capture); every arithmetic step runs in the
 library's kernels.
@@ -49,23 +51,25 @@ class DecodeGraph:
         self._pos_state = torch.tensor([int(pos), 0], dtype=torch.int32, device=dev)    # {position, ticket}
         self.pos = self._pos_state[:1]
         self._scale, self._window, self._d = float(softmax_scale), window, d
-        self._stream = torch.cuda.Stream(device=dev)
-        self._graph = torch.cuda.CUDAGraph()
         # an eager warm-up pass would advance the state, so the kernels are loaded explicitly and
         # the step is captured directly (the library allocates nothing: the calls only enqueue kernels)
-        _b._check(_b.lib().based_preload_decode(), "based_preload_decode")
-        self._stream.wait_stream(torch.cuda.current_stream(dev))
-        with torch.cuda.stream(self._stream):
-            with torch.cuda.graph(self._graph, stream=self._stream):
-                self._enqueue()
-        torch.cuda.current_stream(dev).wait_stream(self._stream)
+        with torch.cuda.device(dev):
+            _b._check(_b.lib().based_preload_decode(), "based_preload_decode")
+            if fused:
+                self._native = _b.native()
+                self._graph = self._native.generation_graph(
+                    self.q, self.k, self.v, self.kv, self.z, self.qw, self.kw, self.vw, self.kc, self.vc, self._pos_state,
+                    self.out_lin, self.out_swa, _b.BASED_STATE_SYM if sym else 0, self._scale)
+                return
+            self._stream = torch.cuda.Stream(device=dev)
+            self._graph = torch.cuda.CUDAGraph()
+            self._stream.wait_stream(torch.cuda.current_stream(dev))
+            with torch.cuda.stream(self._stream):
+                with torch.cuda.graph(self._graph, stream=self._stream):
+                    self._enqueue()
+            torch.cuda.current_stream(dev).wait_stream(self._stream)
 
     def _enqueue(self):
-        if self.fused:
-            _b.based_generation_step(self.q, self.k, self.v, self.kv, self.z, self.qw, self.kw, self.vw, self.kc,
-                                     self.vc, self._pos_state, out=self.out_lin, out_w=self.out_swa,
-                                     flags=_b.BASED_STATE_SYM if self.sym else 0, softmax_scale=self._scale)
-            return
         dec = _b.based_decode_step_sym if self.sym else _b.based_decode_step
         dec(self.q, self.k, self.v, self.kv, self.z, out=self.out_lin)
         B, H, d = self.qw.shape
@@ -76,13 +80,18 @@ class DecodeGraph:
         _b._check(st, "swa_decode_step_advance")
 
     def step(self, q, k, v, qw, kw, vw):
-        """Copies the token's inputs into the graph's buffers, replays it; returns the two outputs
+        """One token; its inputs are left in the graph's buffers (q, k, v, qw, kw, vw).  Returns the two outputs
         (views of buffers that the next step overwrites)."""
+        if self.fused and self._native.generation_graph_step(self._graph, q, k, v, qw, kw, vw):
+            return self.out_lin, self.out_swa
         self.q.copy_(q); self.k.copy_(k); self.v.copy_(v)
         self.qw.copy_(qw); self.kw.copy_(kw); self.vw.copy_(vw)
-        self._graph.replay()
+        self.replay()
         return self.out_lin, self.out_swa
 
     def replay(self):
         """Replays the step on whatever the input buffers hold (benchmarks)."""
-        self._graph.replay()
+        if self.fused:
+            self._native.generation_graph_replay(self._graph)
+        else:
+            self._graph.replay()

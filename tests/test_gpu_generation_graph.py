@@ -1,0 +1,48 @@
+"""DecodeGraph.step on a token's own tensors (the graph's node is pointed at them), on ones that have to be copied first,
+and replay() on what the buffers hold: the same outputs, states and caches as the eager fused call, bit for bit."""
+import pytest
+import torch
+
+import paper_2402_18668_b200 as based
+from paper_2402_18668_b200.generation import DecodeGraph
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("B,H,d_v,window,sym", [(1, 3, 64, 16, False), (2, 16, 128, 64, True), (5, 7, 112, 100, False),
+                                                (40, 16, 128, 64, True)])
+def test_step_equals_the_eager_call(dtype, B, H, d_v, window, sym):
+    g = torch.Generator(device="cuda").manual_seed(B + d_v)
+    rnd = lambda *s, dt=dtype: torch.randn(*s, generator=g, device="cuda").to(dt)
+    kv, z = based.new_state(B, H, d_v, sym=sym)
+    kv.copy_(rnd(*kv.shape)); z.copy_(rnd(*z.shape).abs() + 5.0)
+    kc, vc = rnd(B, H, window, 64), rnd(B, H, window, 64)
+    eager = [t.clone() for t in (kv, z, kc, vc)]
+    pos = torch.tensor([window - 2, 0], dtype=torch.int32, device="cuda")
+    graph = DecodeGraph(kv, z, kc, vc, pos=window - 2, dtype=dtype, sym=sym)
+    token = None
+    for kind in ("own", "own", "strided", "replay", "own", "other dtype", "buffers", "swapped buffers", "replay"):
+        if kind == "replay":
+            got = [t.clone() for t in (graph.replay(), graph.out_lin, graph.out_swa)[1:]]
+        else:
+            token = [rnd(B, H, 16), rnd(B, H, 16), rnd(B, H, d_v), rnd(B, H, 64), rnd(B, H, 64), rnd(B, H, 64)]
+            given = token
+            if kind == "strided":
+                given = [torch.stack([t, t], dim=-1)[..., 0] for t in token]
+            elif kind == "other dtype":                    # bf16 values in the other type: the conversion is exact
+                token = [t.bfloat16().to(dtype) for t in token]
+                given = [t.to(torch.float32 if dtype == torch.bfloat16 else torch.bfloat16) for t in token]
+            elif kind == "buffers":
+                given = [graph.q, graph.k, graph.v, graph.qw, graph.kw, graph.vw]
+                token = [t.clone() for t in given]
+            elif kind == "swapped buffers":                # copied one after the other: q from k's buffer, then k from q's new one
+                given = [graph.k, graph.q, graph.v, graph.qw, graph.kw, graph.vw]
+                token = [graph.k.clone(), graph.k.clone()] + [t.clone() for t in given[2:]]
+            got = [t.clone() for t in graph.step(*given)]
+        want = based.based_generation_step(*token[:3], *eager[:2], *token[3:], *eager[2:], pos,
+                                           flags=based.BASED_STATE_SYM if sym else 0)
+        for a, b in zip(got + [kv, z, kc, vc, graph.q, graph.k, graph.v, graph.qw, graph.kw, graph.vw],
+                        list(want) + eager + token):
+            assert torch.equal(a, b), kind
+        assert int(graph.pos) == int(pos[0]) and based.based_poll_error() == based.BASED_OK

@@ -285,6 +285,12 @@ based_status baseconv_gate_step(const void* a, const void* g, const float* h, co
                                 void* out, int B, int C, int width, based_dtype io, void* cuda_stream);
 
 /*
+ * The layout change in front of the mixers: src [B,L,H,row] (a layer's projections: the heads of a token side by side)
+ * to dst [B,H,L,row].  row_bytes: bytes of one head's row, a multiple of 16; src and dst must not overlap.
+ */
+based_status based_tokens_to_heads(const void* src, void* dst, int B, int H, int L, int row_bytes, void* cuda_stream);
+
+/*
  * Loads the kernels of the generation step (based_decode_step, based_decode_step_sym,
  * swa_decode_step, swa_decode_step_at, the state conversions) into the current device's
  * context and resolves the library's device symbols, so that their first use may happen inside

@@ -32,7 +32,8 @@ EXPORTS = (
     "based_state_to_sym", "based_state_from_sym", "swa_decode_step_at", "based_preload_decode",
     "baseconv_gate_forward", "baseconv_gate_step", "based_decode_step_flags", "based_prefill_backward",
     "based_prefill_backward_workspace_bytes", "based_prefill_backward_with_out", "based_prefill_backward_block_tokens", "swa_decode_step_advance", "swa_decode_step_ragged", "based_generation_step",
-    "based_prefill_state", "based_prefill_state_workspace_bytes",
+    "based_prefill_state", "based_prefill_state_workspace_bytes", "based_generation_graph_create", "based_generation_graph_step",
+    "based_generation_graph_destroy", "based_tokens_to_heads",
 )
 
 _lib = None
@@ -103,6 +104,8 @@ def lib() -> ctypes.CDLL:
         L.baseconv_gate_forward.argtypes = [vp, vp, vp, vp, vp, i, i, i, i, i, vp]
         L.baseconv_gate_step.restype = i
         L.baseconv_gate_step.argtypes = [vp, vp, vp, vp, vp, vp, i, i, i, i, vp]
+        L.based_tokens_to_heads.restype = i
+        L.based_tokens_to_heads.argtypes = [vp, vp, i, i, i, i, vp]
         L.based_poll_error.restype = i
         L.based_poll_error.argtypes = [vp]
         L.based_status_string.restype = ctypes.c_char_p

@@ -546,6 +546,14 @@ based_status based_prefill_backward_with_out(const void* q, const void* k, const
                             workspace_bytes, cuda_stream);
 }
 
+based_status based_tokens_to_heads(const void* src, void* dst, int B, int H, int L, int row_bytes, void* cuda_stream) {
+    if (!src || !dst || src == dst || B <= 0 || H <= 0 || L <= 0 || row_bytes <= 0) return BASED_ERR_INVALID_ARG;
+    // one head of one sequence is indexed with 32 bits, heads and sequences by the grid's y and z
+    if (row_bytes % 16 || (long long)L * (row_bytes / 16) > 0x7fffffffLL || B > 65535 || H > 65535) return BASED_ERR_UNSUPPORTED;
+    if (!aligned16(src) || !aligned16(dst)) return BASED_ERR_ALIGNMENT;
+    return launch_tokens_to_heads(src, dst, B, H, L, row_bytes, static_cast<cudaStream_t>(cuda_stream));
+}
+
 based_status based_preload_decode(void) {
     unsigned int* err = nullptr;
     based_status st = error_word_ptr(&err);

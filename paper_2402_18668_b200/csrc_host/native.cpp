@@ -417,6 +417,17 @@ PyObject* baseconv(PyObject* const* p) {
 }
 
 // ---------------------------------------------------------------------------------------------- autograd
+// The output gradient as the backward pass takes it.  It usually comes back from a projection with the heads of a token
+// side by side, [B,L,H,d_v] seen as [B,H,L,d_v]: that layout has a copy kernel of its own in the library.
+Tensor heads_first(const Tensor& g, at::ScalarType dt, void* stream) {
+    if (g.is_contiguous() || g.dim() != 4 || !g.is_cuda() || g.scalar_type() != dt) return g.contiguous().to(dt);
+    const int64_t B = g.size(0), H = g.size(1), L = g.size(2), d = g.size(3);
+    if (g.stride(3) != 1 || g.stride(1) != d || g.stride(2) != H * d || (B > 1 && g.stride(0) != L * H * d)) return g.contiguous();
+    const Tensor out = at::empty({B, H, L, d}, g.options());
+    const based_status st = based_tokens_to_heads(g.const_data_ptr(), ptr(out), static_cast<int>(B), static_cast<int>(H),
+                                                  static_cast<int>(L), static_cast<int>(d * g.element_size()), stream);
+    return st == BASED_OK ? out : g.contiguous();
+}
 struct LinearAttention : torch::autograd::Function<LinearAttention> {
     static Tensor forward(torch::autograd::AutogradContext* ctx, const Tensor& q_, const Tensor& k_, const Tensor& v_, int64_t flags) {
         const Tensor q = q_.contiguous(), k = k_.contiguous(), v = v_.contiguous();
@@ -432,9 +443,9 @@ struct LinearAttention : torch::autograd::Function<LinearAttention> {
     static torch::autograd::variable_list backward(torch::autograd::AutogradContext* ctx, torch::autograd::variable_list grads) {
         const auto saved = ctx->get_saved_variables();
         const Tensor &q = saved[0], &k = saved[1], &v = saved[2], &out = saved[3];
-        const Tensor dout = grads[0].defined() ? grads[0].contiguous().to(q.scalar_type()) : at::zeros_like(v);
-        const Gradients g = backward_call(q, k, v, dout, out, static_cast<int>(ctx->saved_data["flags"].toInt()), kNone,
-                                          c10::cuda::getCurrentCUDAStream().stream());
+        void* stream = c10::cuda::getCurrentCUDAStream().stream();
+        const Tensor dout = grads[0].defined() ? heads_first(grads[0], q.scalar_type(), stream) : at::zeros_like(v);
+        const Gradients g = backward_call(q, k, v, dout, out, static_cast<int>(ctx->saved_data["flags"].toInt()), kNone, stream);
         return {g.dq, g.dk, g.dv, Tensor()};
     }
 };

@@ -125,16 +125,17 @@ static based_status prefill_impl(const void* q, const void* k, const void* v, vo
     }
     if (d_feat != kDFeat) {
         if (flags & BASED_STATE_SYM) return BASED_ERR_UNSUPPORTED;
-        // bf16 io from the empty state: outputs on the tensor cores (definition form), the state by the fp32 kernel
-        bool outputs_done = false;
+        // bf16 io from the empty state: outputs (definition form) and state on the tensor cores, side by side
         if (io == BASED_BF16 && !(flags & BASED_STATE_CONTINUE)) {
-            const based_status st =
-                launch_quadratic_forward_tc(q, k, v, out, B * H, L, d_feat, d_v, (flags & BASED_NUMERATOR_ONLY) ? 1 : 0,
-                                            static_cast<cudaStream_t>(cuda_stream));
-            if (st != BASED_OK) return st;
-            outputs_done = true;
+            cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
+            if (kv_state) {
+                const based_status st = launch_state_generic_tc(k, v, kv_state, z_state, B * H, L, d_feat, d_v, 0, stream);
+                if (st != BASED_OK) return st;
+            }
+            return launch_quadratic_forward_tc(q, k, v, out, B * H, L, d_feat, d_v, (flags & BASED_NUMERATOR_ONLY) ? 1 : 0,
+                                               kv_state != nullptr, stream);
         }
-        return launch_prefill_generic(q, k, v, out, kv_state, z_state, B * H, L, d_feat, d_v, io, flags, outputs_done,
+        return launch_prefill_generic(q, k, v, out, kv_state, z_state, B * H, L, d_feat, d_v, io, flags,
                                       static_cast<cudaStream_t>(cuda_stream));
     }
     const size_t need = based_prefill_workspace_bytes(B, H, L, d_feat, d_v, io);

@@ -75,11 +75,11 @@ template <int DV, int MODE, int LT, bool XB = false> struct BCfg {
     static constexpr uint32_t kSmem = offMisc + 2048 + 1024;                    // barriers, the block state's row sums (160 floats), m (128)
 
     // tensor memory columns: scores, dout.v products, ds (dq pass; the dk/dv pass packs in place), accumulators
-    static constexpr uint32_t colS = 0, colG = LT, colD = MODE == kModeFwd ? LT : 2 * LT;   // forward: no dout.v product
+    static constexpr uint32_t colS = 0, colG = LT, colD = MODE == kModeFwd ? 0 : 2 * LT;    // forward: no dout.v product, the weights over the scores
     static constexpr uint32_t colD2 = colD + LT / 2;                                      // second packed tile (merged pass)
     static constexpr uint32_t colAcc = MODE == kModeDq ? 2 * LT + LT / 2                  // dQ (32)
                                        : MODE == kModeDqS ? 3 * LT                        // X (32), then Y (32)
-                                       : MODE == kModeFwd ? LT + LT / 2                   // Y (64 * kVB)
+                                       : MODE == kModeFwd ? LT                            // Y (64 * kVB)
                                                           : (LT == 32 ? 96 : 2 * LT < 160 ? 160 : 2 * LT);  // dV (64 * kVB): above the block
                                        // product (160 columns), or with 32-row looped tiles above its packed monomials (80): the
                                        // product is read before the first dV product is issued
@@ -109,6 +109,7 @@ struct BParams {
     float s1, s2;                // w = 1 + s * s1 + s^2 * s2 (1 / sqrt d', 1 / (2 d'))
     // block-wise path: pairs inside a block of W tokens by tiles, the other blocks through their summed state
     int W, nblk;
+    int overlapped;              // forward: this grid runs beside the one before it, and ends after it
     const float* sv;             // [BH x nblk][160]: row sums of the block states (z, or the b-weighted sums of phi(q))
 };
 
@@ -130,6 +131,25 @@ __device__ __forceinline__ bool rows_all(bool pred) {
         : "r"((uint32_t)pred)
         : "memory");
     return r != 0;
+}
+// pairs of fp32 values in one register pair
+__device__ __forceinline__ uint64_t f32x2(float lo, float hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void split_f32x2(uint64_t v, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
 }
 // w = 1 + s / sqrt(d') + s^2 / (2 d') and its derivative, s1 = 1 / sqrt(d'), s2 = 1 / (2 d') (d' = 16: 1/4, 1/32)
 __device__ __forceinline__ float tw(float s, float s1, float s2) { return fmaf(s, fmaf(s, s2, s1), 1.0f); }
@@ -194,7 +214,7 @@ __device__ __forceinline__ void block_rows(uint32_t tb, uint32_t lane_base, cons
 // XB: the block-wise path (merged statistics + dq pass and dk/dv pass, d' = 16); tm_st: the block states,
 // transposed: [BH x nblk][d_v][160] bf16.  tm_out: the wide output (dv, or the forward output), stored by TMA.
 template <int DV, int MODE, int LT, bool XB>
-__global__ void __launch_bounds__(kThreadsB, 1)
+__global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? (DV == 64 && LT == 64 ? 4 : 2) : 1)
     backward_tc_kernel(const __grid_constant__ CUtensorMap tm_n0, const __grid_constant__ CUtensorMap tm_w0,
                        const __grid_constant__ CUtensorMap tm_n1, const __grid_constant__ CUtensorMap tm_w1,
                        const __grid_constant__ CUtensorMap tm_st, const __grid_constant__ CUtensorMap tm_out,
@@ -542,6 +562,32 @@ __global__ void __launch_bounds__(kThreadsB, 1)
             // diagonal or the end of the sequence (the others need no per-pair test)
             auto pass = [&](auto masked_tag) {
                 constexpr bool MASKED = decltype(masked_tag)::value;
+                if constexpr (MODE == kModeFwd && !MASKED) {
+                    // two pairs per instruction: w = 1 + s (s1 + s s2), its sum, and the packed weight
+                    const uint64_t k2 = f32x2(p.s2, p.s2), k1 = f32x2(p.s1, p.s1), one = f32x2(1.f, 1.f);
+                    uint64_t d0 = f32x2(den, 0.f), d1 = 0;
+#pragma unroll
+                    for (int blk = 0; blk < LT / 32; ++blk) {
+                        uint32_t sr[32], pw[16];
+                        tmem_ld32(tmem_addr(tb, lane_base, C::colS + blk * 32), sr);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) {
+                            const uint64_t s2v = f32x2(__uint_as_float(sr[2 * i]), __uint_as_float(sr[2 * i + 1]));
+                            const uint64_t w = fma_f32x2(s2v, fma_f32x2(s2v, k2, k1), one);
+                            if (i & 1) d1 = add_f32x2(d1, w);
+                            else d0 = add_f32x2(d0, w);
+                            float lo, hi;
+                            split_f32x2(w, lo, hi);
+                            pw[i] = pack_bf16x2(lo, hi);
+                        }
+                        tmem_st16(tmem_addr(tb, lane_base, C::colD + blk * 16), pw);
+                    }
+                    float a, b;
+                    split_f32x2(add_f32x2(d0, d1), a, b);
+                    den = a + b;
+                    return;
+                }
 #pragma unroll 1
                 for (int blk = 0; blk < LT / 32; ++blk) {
                     uint32_t sr[32], gr[32];
@@ -694,6 +740,9 @@ __global__ void __launch_bounds__(kThreadsB, 1)
     }
     __syncthreads();
     if (warp == 4) tmem_dealloc(tb, C::kCols);
+    // one CTA holds the grid's end back until the grid before it is complete: what follows in the stream sees both
+    if (MODE == kModeFwd && p.overlapped && blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && tid == 0)
+        asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 namespace {
@@ -740,10 +789,21 @@ based_status launch_pass(const CUtensorMap& n0, const CUtensorMap& w0, const CUt
             configured[dev] = true;
         }
     }
-    backward_tc_kernel<DV, MODE, LT, XB><<<grid, kThreadsB, C::kSmem, stream>>>(n0, w0, n1, w1, st ? *st : n0,
-                                                                               outm ? *outm : w0, p);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(kThreadsB);
+    cfg.dynamicSmemBytes = C::kSmem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = p.overlapped ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, backward_tc_kernel<DV, MODE, LT, XB>, n0, w0, n1, w1, st ? *st : n0,
+                                             outm ? *outm : w0, p);
     note_launch();
-    return check_launch(what);
+    const based_status s2 = check_launch(what);
+    return e == cudaSuccess ? s2 : BASED_ERR_CUDA;
 }
 
 // Block length of the block-wise path, or 0 for the tile path alone.  The block-wise path needs d' = 16 and the
@@ -883,8 +943,11 @@ based_status launch_dvb(const void* q, const void* k, const void* v, const void*
 
 // Forward of the definition form on the same tiles, for feature dimensions other than 16 (bf16 io,
 // empty initial state): out = (sum_j w_ij v_j) / (sum_j w_ij + eps), w = 1 + s/sqrt(d') + s^2/(2 d').
+// The weights lie over the scores, so at d_v 64 a CTA takes 128 columns of tensor memory and four share an SM, and tiles off
+// the diagonal evaluate two pairs per instruction: B4 H16 L2048 d_v64 80 -> 48 us (looped tiles of 128 rows: 47).  With the
+// state asked for it runs beside that kernel (80 + 61 us one after the other before, 48 + 40, together 74).
 based_status launch_quadratic_forward_tc(const void* q, const void* k, const void* v, void* out, int BH, int L,
-                                         int d_feat, int d_v, int numerator_only, cudaStream_t stream) {
+                                         int d_feat, int d_v, int numerator_only, bool overlapped, cudaStream_t stream) {
     CUtensorMap tq, tk64, tv64, tout;
     const CUtensorMapSwizzle s64 = CU_TENSOR_MAP_SWIZZLE_64B, s128 = CU_TENSOR_MAP_SWIZZLE_128B;
     if (!make_rows_map_bf16(&tq, q, BH, L, d_feat, 32, kTile, s64) || !make_rows_map_bf16(&tk64, k, BH, L, d_feat, 32, 64, s64) ||
@@ -895,6 +958,7 @@ based_status launch_quadratic_forward_tc(const void* q, const void* k, const voi
     p.dvo = static_cast<__nv_bfloat16*>(out);
     p.L = L;
     p.dvw = d_v;
+    p.overlapped = overlapped;
     p.numerator_only = numerator_only;
     p.df = d_feat;
     p.kdim = d_feat <= 16 ? 16 : 32;

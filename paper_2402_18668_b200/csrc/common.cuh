@@ -118,9 +118,8 @@ based_status launch_prefill_backward_f32(const float* q, const float* k, const f
                                          float* dv, float* stats, int BH, int L, int d_v, int numerator_only,
                                          cudaStream_t stream);
 // feature dimensions 8, 24, 32 (fp32 FMA, definition form); state layout [1 + d' + d'^2, d_v]
-// outputs_done: out has been written already (tensor-core forward), only the state is still to do
 based_status launch_prefill_generic(const void* q, const void* k, const void* v, void* out, float* kv, float* z,
-                                    int BH, int L, int d_feat, int d_v, based_dtype io, int flags, bool outputs_done,
+                                    int BH, int L, int d_feat, int d_v, based_dtype io, int flags,
                                     cudaStream_t stream);
 // the final state of those feature dimensions on tensor cores (bf16 io); cont: add to the state given
 based_status launch_state_generic_tc(const void* k, const void* v, float* kv, float* z, int BH, int L, int d_feat,
@@ -150,9 +149,10 @@ int backward_tc_block_tokens(int BH, int L, int d_feat, int d_v, int merged);
 based_status launch_prefill_backward_tc(const void* q, const void* k, const void* v, const void* out, const void* g,
                                         void* dq, void* dk, void* dv, float* ws, int BH, int L, int d_feat, int d_v,
                                         int numerator_only, cudaStream_t stream);
-// definition-form forward on tensor cores for d' in {8, 24, 32} (bf16 io, empty initial state)
+// definition-form forward on tensor cores for d' in {8, 24, 32} (bf16 io, empty initial state); overlapped: beside the
+// kernel before it in the stream (launch_state_generic_tc's, which lets it), whose results it does not use
 based_status launch_quadratic_forward_tc(const void* q, const void* k, const void* v, void* out, int BH, int L,
-                                         int d_feat, int d_v, int numerator_only, cudaStream_t stream);
+                                         int d_feat, int d_v, int numerator_only, bool overlapped, cudaStream_t stream);
 // load the generation-step kernels into the current context
 based_status preload_decode();
 based_status preload_swa_decode();

@@ -9,7 +9,7 @@
 //
 // The op is one pass over a, g and out: 3 elements of traffic per output element and a dozen
 // flops, so it is bound by HBM bandwidth.  A thread owns 8 consecutive channels (one 16-byte
-// piece of a bf16 row, two of an fp32 row) and walks a run of kRun tokens with the last w-1 rows
+// piece of a bf16 row, two of an fp32 row) and walks a run of up to 32 tokens with the last w-1 rows
 // of g in registers, so g is read once (plus w-1 halo rows per run, which the neighbouring run
 // has just brought into L2); a warp covers 256 consecutive channels of a row.  The loop is
 // software-pipelined: the rows of the next four tokens are in flight (kept packed, as loaded)
@@ -19,7 +19,7 @@
 namespace based {
 
 namespace {
-constexpr int kRun = 64;        // tokens per thread run
+constexpr int kMaxRun = 32;     // tokens per thread run, at most
 constexpr int kUnroll = 4;      // tokens whose loads are in flight together
 constexpr int kThreadsBC = 128;
 
@@ -80,6 +80,12 @@ template <> struct Row8<float> {
     }
 };
 
+// 8 fp32 values of a filter row or the bias
+__device__ __forceinline__ void load8(const float* p, float (&x)[8]) {
+    const float4 lo = __ldg(reinterpret_cast<const float4*>(p)), hi = __ldg(reinterpret_cast<const float4*>(p) + 1);
+    x[0] = lo.x; x[1] = lo.y; x[2] = lo.z; x[3] = lo.w; x[4] = hi.x; x[5] = hi.y; x[6] = hi.z; x[7] = hi.w;
+}
+
 // SiLU(x) = x * sigmoid(x); the fast exponential and division are exact enough for bf16 outputs,
 // fp32 io takes the accurate ones
 template <bool FAST>
@@ -92,21 +98,13 @@ template <typename T, int W>
 __global__ void __launch_bounds__(kThreadsBC) baseconv_gate_kernel(const T* __restrict__ a, const T* __restrict__ g,
                                                                    const float* __restrict__ h,
                                                                    const float* __restrict__ b2, T* __restrict__ out,
-                                                                   int N, int C) {
+                                                                   int N, int C, int run) {
     constexpr bool FAST = sizeof(T) == 2;
     const int c0 = (blockIdx.x * kThreadsBC + threadIdx.x) * 8;
     if (c0 >= C) return;
-    const int i0 = blockIdx.y * kRun;
-    const int i1 = min(N, i0 + kRun);
+    const int i0 = blockIdx.y * run;
+    const int i1 = min(N, i0 + run);
     const size_t base = (size_t)blockIdx.z * N * C + c0;
-
-    float taps[W][8], bias[8];
-#pragma unroll
-    for (int j = 0; j < W; ++j)
-#pragma unroll
-        for (int e = 0; e < 8; ++e) taps[j][e] = h[(size_t)j * C + c0 + e];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) bias[e] = b2[c0 + e];
 
     // prev[j] = g of the token j+1 steps back (zero before the sequence start)
     float prev[W > 1 ? W - 1 : 1][8];
@@ -132,6 +130,10 @@ __global__ void __launch_bounds__(kThreadsBC) baseconv_gate_kernel(const T* __re
         }
     };
     fetch(i0, gr, ar);
+    float taps[W][8], bias[8];
+#pragma unroll
+    for (int j = 0; j < W; ++j) load8(h + (size_t)j * C + c0, taps[j]);
+    load8(b2 + c0, bias);
     for (int i = i0; i < i1; i += kUnroll) {
         fetch(i + kUnroll, gn, an);
 #pragma unroll
@@ -191,10 +193,6 @@ __global__ void __launch_bounds__(kThreadsBC) baseconv_step_kernel(const T* __re
         }
     }
     float taps[W][8], bias[8];
-    auto load8 = [](const float* p, float (&x)[8]) {
-        const float4 lo = __ldg(reinterpret_cast<const float4*>(p)), hi = __ldg(reinterpret_cast<const float4*>(p) + 1);
-        x[0] = lo.x; x[1] = lo.y; x[2] = lo.z; x[3] = lo.w; x[4] = hi.x; x[5] = hi.y; x[6] = hi.z; x[7] = hi.w;
-    };
 #pragma unroll
     for (int j = 0; j < W; ++j) load8(h + (size_t)j * C + c0, taps[j]);
     load8(b2 + c0, bias);
@@ -234,9 +232,15 @@ static void launch_w(const void* a, const void* g, const float* h, const float* 
     else if (step)
         baseconv_step_kernel<T, W, 1><<<dim3(gx, B), kThreadsBC, 0, stream>>>(
             static_cast<const T*>(a), static_cast<const T*>(g), h, b2, static_cast<T*>(state), static_cast<T*>(out), B, C);
-    else
-        baseconv_gate_kernel<T, W><<<dim3(gx, (N + kRun - 1) / kRun, B), kThreadsBC, 0, stream>>>(
-            static_cast<const T*>(a), static_cast<const T*>(g), h, b2, static_cast<T*>(out), N, C);
+    else {
+        // shorter runs until the grid has a block or two for every SM (us with runs of 64 / 32 / 16 / 8 / 4 tokens:
+        // B3 N128 C5208 12.8 / 7.4 / 5.0 / 4.4 / 5.7, B2 N1024 C2048 12.9 / 7.7 / 6.4 / 6.9 / 7.1; B8 N4096 C8192
+        // 267 / 264 / 270 / 295 / 350, B4 N1024 C8192 width 4 41 / 37 / 38 / 42 / 51)
+        int run = kMaxRun;
+        while (run > 4 && (long long)gx * ((N + run - 1) / run) * B < 240) run /= 2;
+        baseconv_gate_kernel<T, W><<<dim3(gx, (N + run - 1) / run, B), kThreadsBC, 0, stream>>>(
+            static_cast<const T*>(a), static_cast<const T*>(g), h, b2, static_cast<T*>(out), N, C, run);
+    }
 }
 
 template <typename T>

@@ -453,6 +453,66 @@ __device__ __noinline__ void init_state_blocks(const float* wsh, int nprev, bool
     tmem_wait_st();
 }
 
+// The same from the caller's state alone, one of four role groups' share (blocks part, part + 4, part + 8): the loads of
+// all its blocks are in flight together, the second row of each pair of a full state in a second round.  Block by block,
+// by the state group alone, the ten blocks' load latency was 8 to 14 us of every continued call (B3 H16 L777 d_v112, 153 rows,
+// 28.4 us a call; 21.0 with the blocks shared, 19.8 with the loads together).
+template <int DV>
+__device__ __noinline__ void init_from_abi(const float* kv_abi, const float* z_abi, int dv, int abi_row0, const short2* s_abi,
+                                           uint32_t tb, int part) {
+    using C = Cfg<DV>;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t lane_base = (uint32_t)(warp & 3) * 32u;
+    const int t = ((warp & 3) << 5) + lane;
+    const bool is_z = (DV == 64) && t == 64, live = is_z || (t < C::kSLanes && t < dv);
+    const float* base = is_z ? z_abi + abi_row0 : kv_abi + (size_t)abi_row0 * dv + (live ? t : 0);
+    const size_t pitch = is_z ? 1 : dv;
+    constexpr int NB = (kF / 16 + 3) / 4;
+    float x[NB][16];
+#pragma unroll
+    for (int j = 0; j < NB; ++j)
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const int f = (part + 4 * j) * 16 + i;
+            const int a = f < kF ? s_abi[f].x : -1;
+            x[j][i] = a >= 0 && live ? base[(size_t)a * pitch] : 0.f;
+        }
+#pragma unroll
+    for (int j = 0; j < NB; ++j) {
+        const int b = part + 4 * j;
+        if (b >= kF / 16) break;
+        float y[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const int a = s_abi[b * 16 + i].y;
+            y[i] = a >= 0 && live ? base[(size_t)a * pitch] : 0.f;
+        }
+        uint32_t r[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+            r[i] = __float_as_uint(s_abi[b * 16 + i].y >= 0 ? (x[j][i] + y[i]) * kRsqrt2 : x[j][i]);
+        tmem_st16(tmem_addr(tb, lane_base, C::colS + b * 16), r);
+    }
+    if (DV == 128 && part == 3) {
+        // d_v 128: the K-state of feature t (tile 0) and of feature z1f (tile 1), column 0 of each tile
+        const int z1f = (t & 31) < 16 && (t >> 5) < 2 ? 128 + (t >> 5) * 16 + (t & 15) : -1;
+        auto z_init = [&](int f) -> float {
+            if (f < 0) return 0.f;
+            const short2 ar = s_abi[f];
+            const float* zh = z_abi + abi_row0;
+            return ar.x < 0 ? 0.f : ar.y >= 0 ? (zh[ar.x] + zh[ar.y]) * kRsqrt2 : zh[ar.x];
+        };
+        uint32_t r0[16], r1[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) r0[i] = r1[i] = 0u;
+        r0[0] = __float_as_uint(z_init(t));
+        r1[0] = __float_as_uint(z_init(z1f));
+        tmem_st16(tmem_addr(tb, lane_base, C::colZ0), r0);
+        tmem_st16(tmem_addr(tb, lane_base, C::colZ1), r1);
+    }
+    tmem_wait_st();
+}
+
 // ---- the CTA's piece of work: a head, a token range, where its initial state comes from (workspace slots
 // ws_first .. ws_first + ws_count - 1) and where its final state goes (slot ws_out, or the caller's state if
 // the piece ends its head).
@@ -564,7 +624,8 @@ __device__ __noinline__ void find_piece(Piece* piece, int* s_rest, int balanced,
     __syncthreads();
 }
 
-template <int DV, int MODE>
+// CONT: the piece starts from the caller's state (an instance of its own: what it adds stays out of the others' registers).
+template <int DV, int MODE, bool CONT = false>
 __global__ void __launch_bounds__(kThreads, 1)
     prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                       const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o,
@@ -709,13 +770,17 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     // ---- initial state from earlier pieces' slots, d_v 128 (see Cfg::kSlotScan): in the main pass behind a state pass
     // all four role groups share it
-    const bool share_init = !C::kSlotScan && MODE == kModeMain && ws_count > 0;
+    const bool share_init = CONT || (!C::kSlotScan && MODE == kModeMain && ws_count > 0);
     auto init_state = [&](int part, int nparts) {
+        if constexpr (CONT) {
+            init_from_abi<DV>(p.kv_abi, p.z_abi, p.dv, head * abi_nrows, s_abi, tb, part);
+            return;
+        }
         init_state_blocks<DV>(p.ws + (size_t)ws_first * seg_state_floats(DV), ws_count, MODE == kModeMain && ws_count > 0,
                               (!STATE_ONLY && p.continue_abi) ? p.kv_abi : nullptr, p.z_abi, p.dv, head * abi_nrows, s_abi, tb,
                               part, nparts);
     };
-    if constexpr (!C::kSlotScan) {
+    if constexpr (!C::kSlotScan || CONT) {
         if (share_init && warp < 16 && (warp >> 2) != 2) {      // row, feature and output group (parts 0, 1, 3)
             init_state(warp >> 2, 4);
             tc_fence_before();
@@ -1013,7 +1078,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const bool is_z = (DV == 64) && t == 64;
         // d_v 128: K-state features held in the two z tiles (64-row MMA: rows 0..31 in lanes 0-15, 32-47)
         const int z1f = (DV == 128 && (t & 31) < 16 && (t >> 5) < 2) ? 128 + (t >> 5) * 16 + (t & 15) : -1;
-        if constexpr (C::kSlotScan) {
+        if constexpr (C::kSlotScan && !CONT) {
             const size_t seg_stride = seg_state_floats(DV);
             const float* wsh = p.ws + (size_t)ws_first * seg_stride;      // the partial states this piece starts from
             const int dv = p.dv;                        // row pitch of the caller's state; lanes >= dv hold zeros
@@ -1444,7 +1509,7 @@ unsigned long long* g_trace = nullptr;
 // (they cannot take an SM that a CTA of the state pass still needs, all of those being resident or done by then),
 // and the one group that reads what the state pass wrote waits for its completion.  The recompute-mode kernel behind
 // whatever precedes the call: it waits right after its set-up.
-template <int DV, int MODE>
+template <int DV, int MODE, bool CONT = false>
 cudaError_t launch_dependent(dim3 grid, cudaStream_t stream, const CUtensorMap& tq, const CUtensorMap& tk,
                              const CUtensorMap& tv, const CUtensorMap& to, const Params& p) {
     cudaLaunchConfig_t cfg = {};
@@ -1457,7 +1522,7 @@ cudaError_t launch_dependent(dim3 grid, cudaStream_t stream, const CUtensorMap& 
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, prefill_tc_kernel<DV, MODE>, tq, tk, tv, to, p);
+    return cudaLaunchKernelEx(&cfg, prefill_tc_kernel<DV, MODE, CONT>, tq, tk, tv, to, p);
 }
 
 // The caller's state of a continued call, folded into the internal basis, as the first workspace slot of each head
@@ -1574,6 +1639,10 @@ based_status launch_dv(const void* q, const void* k, const void* v, void* out, f
                 cudaFuncSetAttribute(prefill_tc_kernel<DV, kModeState>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)C::kSmemBytes) != cudaSuccess ||
                 cudaFuncSetAttribute(prefill_tc_kernel<DV, kModePre>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)C::kSmemBytes) != cudaSuccess ||
+                cudaFuncSetAttribute(prefill_tc_kernel<DV, kModeMain, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)C::kSmemBytes) != cudaSuccess ||
+                cudaFuncSetAttribute(prefill_tc_kernel<DV, kModePre, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)C::kSmemBytes) != cudaSuccess)
                 return BASED_ERR_CUDA;
             configured[dev] = true;
@@ -1607,7 +1676,9 @@ based_status launch_dv(const void* q, const void* k, const void* v, void* out, f
         return check_launch("prefill_tc_kernel<balanced>");
     }
     if (nseg > 1 && recompute) {
-        if (launch_dependent<DV, kModePre>(dim3(nseg, BH), stream, tq, tk, tv, to, p) != cudaSuccess) return BASED_ERR_CUDA;
+        const cudaError_t e = p.continue_abi ? launch_dependent<DV, kModePre, true>(dim3(nseg, BH), stream, tq, tk, tv, to, p)
+                                             : launch_dependent<DV, kModePre>(dim3(nseg, BH), stream, tq, tk, tv, to, p);
+        if (e != cudaSuccess) return BASED_ERR_CUDA;
         note_launch();
         return check_launch("prefill_tc_kernel<pre>");
     }
@@ -1635,6 +1706,8 @@ based_status launch_dv(const void* q, const void* k, const void* v, void* out, f
     }
     if (nseg > 1) {
         if (launch_dependent<DV, kModeMain>(dim3(nseg, BH), stream, tq, tk, tv, to, p) != cudaSuccess) return BASED_ERR_CUDA;
+    } else if (p.continue_abi) {
+        prefill_tc_kernel<DV, kModeMain, true><<<dim3(nseg, BH), kThreads, C::kSmemBytes, stream>>>(tq, tk, tv, to, p);
     } else {
         prefill_tc_kernel<DV, kModeMain><<<dim3(nseg, BH), kThreads, C::kSmemBytes, stream>>>(tq, tk, tv, to, p);
     }

@@ -9,7 +9,7 @@
 //
 // The op is one pass over a, g and out: 3 elements of traffic per output element and a dozen
 // flops, so it is bound by HBM bandwidth.  A thread owns 8 consecutive channels (one 16-byte
-// piece of a bf16 row, two of an fp32 row) and walks a run of up to 32 tokens with the last w-1 rows
+// piece of a bf16 row, two of an fp32 row) and walks a run of up to 64 tokens with the last w-1 rows
 // of g in registers, so g is read once (plus w-1 halo rows per run, which the neighbouring run
 // has just brought into L2); a warp covers 256 consecutive channels of a row.  The loop is
 // software-pipelined: the rows of the next four tokens are in flight (kept packed, as loaded)
@@ -19,7 +19,7 @@
 namespace based {
 
 namespace {
-constexpr int kMaxRun = 32;     // tokens per thread run, at most
+constexpr int kMaxRun = 64;     // tokens per thread run, at most
 constexpr int kUnroll = 4;      // tokens whose loads are in flight together
 constexpr int kThreadsBC = 128;
 
@@ -233,11 +233,14 @@ static void launch_w(const void* a, const void* g, const float* h, const float* 
         baseconv_step_kernel<T, W, 1><<<dim3(gx, B), kThreadsBC, 0, stream>>>(
             static_cast<const T*>(a), static_cast<const T*>(g), h, b2, static_cast<T*>(state), static_cast<T*>(out), B, C);
     else {
-        // shorter runs until the grid has a block or two for every SM (us with runs of 64 / 32 / 16 / 8 / 4 tokens:
-        // B3 N128 C5208 12.8 / 7.4 / 5.0 / 4.4 / 5.7, B2 N1024 C2048 12.9 / 7.7 / 6.4 / 6.9 / 7.1; B8 N4096 C8192
-        // 267 / 264 / 270 / 295 / 350, B4 N1024 C8192 width 4 41 / 37 / 38 / 42 / 51)
+        // runs of 64 tokens (a halo of width - 1 rows each) while the last wave of blocks is a small part of the grid, 32
+        // below, shorter ones until the grid has a block or two for every SM (us with runs of 64 / 32 / 16 / 8 / 4 tokens:
+        // B3 N128 C5208 12.8 / 7.4 / 5.0 / 4.4 / 5.7, B2 N1024 C2048 12.9 / 7.7 / 6.4 / 6.9 / 7.1, B4 N1024 C8192 width 4
+        // 41 / 37 / 38 / 42 / 51; B8 N4096 C8192 267 / 264 / 270 / 295 / 350, but 276.5 / 277.8 on alternating inputs)
+        auto blocks = [&](int run) { return (long long)gx * ((N + run - 1) / run) * B; };
         int run = kMaxRun;
-        while (run > 4 && (long long)gx * ((N + run - 1) / run) * B < 240) run /= 2;
+        if (blocks(run) < 2048) run /= 2;
+        while (run > 4 && blocks(run) < 240) run /= 2;
         baseconv_gate_kernel<T, W><<<dim3(gx, (N + run - 1) / run, B), kThreadsBC, 0, stream>>>(
             static_cast<const T*>(a), static_cast<const T*>(g), h, b2, static_cast<T*>(out), N, C, run);
     }

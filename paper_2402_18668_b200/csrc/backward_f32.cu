@@ -19,13 +19,14 @@
 // address costs two passes, four otherwise.  Few tiles: the CTAs of a cluster share one own tile's loop, and their sums
 // are added through distributed shared memory in a fixed order.
 // Measured against three sweeps of 4 x 8 pairs per thread on scalar shared-memory loads: B2 H16 L1024 d_v64 1050 -> 424 us,
-// B1 H2 L1024 d_v64 56 us with eight CTAs per own tile; 424 -> 294 us with the longest loops of all heads first and one
-// weight at a time in shared memory.  Bound: the fp32 pipe at half its rate (135 us of FMAs there; 1050 of 2090 us at
-// B4 H16 L2048).  Three CTAs per SM (168 registers, the weights in the looped tile's place) 328 to 350 us: their spills
-// and the extra barrier cost what the third CTA hides.
+// B1 H2 L1024 d_v64 50 us with eight CTAs per own tile; 424 -> 294 us with the longest loops of all heads first and one
+// weight at a time in shared memory, 275 with two products per instruction (B4 H16 L2048 2090 -> 1823, of which the FMA
+// pipe needs 1050).  Bound: issue slots and latency of two CTAs of four warps per SM.  Three CTAs (168 registers, the weights
+// in the looped tile's place) 328 to 350 us: their spills and the extra barrier cost what the third CTA hides.
 #include <cooperative_groups.h>
 
 #include "common.cuh"
+#include "f32_tiles.cuh"
 
 namespace based {
 
@@ -54,8 +55,6 @@ struct BwdSmem {
 // place of looped row t where four consecutive rows belong to one thread: spreads those over the banks
 __device__ __forceinline__ int place_of(int t) { return (t & 3) * 16 + (t >> 2); }
 
-__device__ __forceinline__ float4 lds4(const float* p) { return *reinterpret_cast<const float4*>(p); }
-
 // 64 rows of W values (a multiple of 16) of a row-major array, transposed -> [W][68]; rows from nt on are zero.
 // nat: the rows as they lie too, at pitch natp (of: at place_of(t))
 template <int W>
@@ -82,30 +81,36 @@ __device__ __forceinline__ void load_tile(float* dst, float* nat, int natp, bool
     }
 }
 
-// s[i][j] += sum_k a[k][row i] b[k][4 co + j]
+// s[i / 2][j], element i % 2, += sum_k a[k][row i] b[k][4 co + j]
 template <int K>
-__device__ __forceinline__ void pair_product(float (&s)[8][4], const float* a, const float* b) {
+__device__ __forceinline__ void pair_product(float2 (&s)[4][4], const float* a, const float* b) {
 #pragma unroll 4
     for (int k = 0; k < K; ++k) {
         const float4 x0 = lds4(a + k * kP), x1 = lds4(a + k * kP + 8), y = lds4(b + k * kP);
-        const float xs[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w}, ys[4] = {y.x, y.y, y.z, y.w};
+        const float ys[4] = {y.x, y.y, y.z, y.w};
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) s[i][j] = fmaf(xs[i], ys[j], s[i][j]);
+        for (int j = 0; j < 4; ++j) {
+            fma_pair(s[0][j], x0.x, x0.y, ys[j]);
+            fma_pair(s[1][j], x0.z, x0.w, ys[j]);
+            fma_pair(s[2][j], x1.x, x1.y, ys[j]);
+            fma_pair(s[3][j], x1.z, x1.w, ys[j]);
+        }
     }
 }
-// acc[i][d] += sum over this lane group's 16 looped rows of p[row][4 rg + i] n[row][8 dg + d]
-__device__ __forceinline__ void narrow_product(float (&acc)[4][8], const float* p, const float* n, int ks, int rg, int dg) {
+// acc[i][d / 2], element d % 2, += sum over this lane group's 16 looped rows of p[row][4 rg + i] n[row][8 dg + d]
+__device__ __forceinline__ void narrow_product(float2 (&acc)[4][4], const float* p, const float* n, int ks, int rg, int dg) {
 #pragma unroll 4
     for (int u = 0; u < 16; ++u) {
         const int r = u * 4 + ks;
         const float4 x = lds4(p + r * 16 + rg * 4), y0 = lds4(n + r * 16 + dg * 8), y1 = lds4(n + r * 16 + dg * 8 + 4);
-        const float xs[4] = {x.x, x.y, x.z, x.w}, ys[8] = {y0.x, y0.y, y0.z, y0.w, y1.x, y1.y, y1.z, y1.w};
+        const float xs[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int d = 0; d < 8; ++d) acc[i][d] = fmaf(xs[i], ys[d], acc[i][d]);
+        for (int i = 0; i < 4; ++i) {
+            fma_pair(acc[i][0], y0.x, y0.y, xs[i]);
+            fma_pair(acc[i][1], y0.z, y0.w, xs[i]);
+            fma_pair(acc[i][2], y1.x, y1.y, xs[i]);
+            fma_pair(acc[i][3], y1.z, y1.w, xs[i]);
+        }
     }
 }
 // one weight of a thread's own rows and looped row 4 co + j
@@ -115,14 +120,16 @@ __device__ __forceinline__ void store_weight(float* p, const float (&a)[8], int 
     *reinterpret_cast<float4*>(at + 8) = make_float4(a[4], a[5], a[6], a[7]);
 }
 // sums over the four lane groups ks (lane bits 3, 4)
-__device__ __forceinline__ void narrow_reduce(float (&acc)[4][8]) {
+__device__ __forceinline__ void narrow_reduce(float2 (&acc)[4][4]) {
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int d = 0; d < 8; ++d) {
-            acc[i][d] += __shfl_xor_sync(0xffffffffu, acc[i][d], 8);
-            acc[i][d] += __shfl_xor_sync(0xffffffffu, acc[i][d], 16);
-        }
+        for (int d = 0; d < 4; ++d)
+#pragma unroll
+            for (int o = 8; o < 32; o <<= 1) {
+                acc[i][d].x += __shfl_xor_sync(0xffffffffu, acc[i][d].x, o);
+                acc[i][d].y += __shfl_xor_sync(0xffffffffu, acc[i][d].y, o);
+            }
 }
 }  // namespace
 
@@ -174,23 +181,23 @@ __global__ void __launch_bounds__(kBT, DV > 64 ? 1 : 2)
         for (int i = 0; i < 8; ++i) m[i] = s.m[row0 + (i >> 2) * 8 + (i & 3)];
     }
 
-    float n1[4][8], n2[KEYS ? 1 : 4][8];             // X and Y, or dk
+    float2 n1[4][4], n2[KEYS ? 1 : 4][4];            // X and Y, or dk
     float den[8], num[8];                            // row sums of w and w G.v (dq pass)
-    float wide[KEYS ? 8 : 1][KEYS ? 4 * NV : 1];     // dv
+    float2 wide[KEYS ? 4 : 1][KEYS ? 4 * NV : 1];    // dv, rows in pairs
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int d = 0; d < 8; ++d) {
-            n1[i][d] = 0.f;
-            if (!KEYS) n2[i][d] = 0.f;
+        for (int d = 0; d < 4; ++d) {
+            n1[i][d] = make_float2(0.f, 0.f);
+            if (!KEYS) n2[i][d] = make_float2(0.f, 0.f);
         }
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        den[i] = num[i] = 0.f;
-        if (KEYS)
+    for (int i = 0; i < 8; ++i) den[i] = num[i] = 0.f;
+    if (KEYS)
 #pragma unroll
-            for (int c = 0; c < 4 * NV; ++c) wide[i][c] = 0.f;
-    }
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int c = 0; c < 4 * NV; ++c) wide[i][c] = make_float2(0.f, 0.f);
 
     float* p = s.p[warp];
     const int first = KEYS ? own : 0, last = KEYS ? ntile - 1 : own;
@@ -203,13 +210,21 @@ __global__ void __launch_bounds__(kBT, DV > 64 ? 1 : 2)
             s.st[tid] = tid < n_loop ? stats[head * (size_t)L + tile * kT + tid] : make_float2(0.f, 0.f);
         __syncthreads();
 
+        float2 sc2[4][4], gv2[4][4];                 // rows in pairs
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) sc2[i][j] = gv2[i][j] = make_float2(0.f, 0.f);
+        pair_product<kDFeat>(sc2, s.an + row0, s.bn + 4 * co);
+        pair_product<DV>(gv2, s.aw + row0, s.bw + 4 * co);
         float sc[8][4], gv[8][4];
 #pragma unroll
         for (int i = 0; i < 8; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) sc[i][j] = gv[i][j] = 0.f;
-        pair_product<kDFeat>(sc, s.an + row0, s.bn + 4 * co);
-        pair_product<DV>(gv, s.aw + row0, s.bw + 4 * co);
+            for (int j = 0; j < 4; ++j) {
+                sc[i][j] = i & 1 ? sc2[i >> 1][j].y : sc2[i >> 1][j].x;
+                gv[i][j] = i & 1 ? gv2[i >> 1][j].y : gv2[i >> 1][j].x;
+            }
 
         const bool diag = tile == own;
         float2 st[4];
@@ -256,15 +271,17 @@ __global__ void __launch_bounds__(kBT, DV > 64 ? 1 : 2)
             for (int t = 0; t < kT; ++t) {
                 const float* pr = p + place_of(t) * 16 + ro * 4;
                 const float4 x0 = lds4(pr), x1 = lds4(pr + 8);
-                const float xs[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
 #pragma unroll
                 for (int c = 0; c < NV; ++c) {
                     const float4 y = lds4(&s.rw[t * S::kWide + 64 * c + 4 * co]);
                     const float ys[4] = {y.x, y.y, y.z, y.w};
 #pragma unroll
-                    for (int i = 0; i < 8; ++i)
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) wide[i][4 * c + e] = fmaf(xs[i], ys[e], wide[i][4 * c + e]);
+                    for (int e = 0; e < 4; ++e) {
+                        fma_pair(wide[0][4 * c + e], x0.x, x0.y, ys[e]);
+                        fma_pair(wide[1][4 * c + e], x0.z, x0.w, ys[e]);
+                        fma_pair(wide[2][4 * c + e], x1.x, x1.y, ys[e]);
+                        fma_pair(wide[3][4 * c + e], x1.z, x1.w, ys[e]);
+                    }
                 }
             }
         }
@@ -284,11 +301,11 @@ __global__ void __launch_bounds__(kBT, DV > 64 ? 1 : 2)
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int at = (warp * 16 + rg * 4 + i) * kDFeat + dg * 8;
-            *reinterpret_cast<float4*>(o1 + at) = make_float4(n1[i][0], n1[i][1], n1[i][2], n1[i][3]);
-            *reinterpret_cast<float4*>(o1 + at + 4) = make_float4(n1[i][4], n1[i][5], n1[i][6], n1[i][7]);
+            *reinterpret_cast<float4*>(o1 + at) = make_float4(n1[i][0].x, n1[i][0].y, n1[i][1].x, n1[i][1].y);
+            *reinterpret_cast<float4*>(o1 + at + 4) = make_float4(n1[i][2].x, n1[i][2].y, n1[i][3].x, n1[i][3].y);
             if constexpr (!KEYS) {
-                *reinterpret_cast<float4*>(o2 + at) = make_float4(n2[i][0], n2[i][1], n2[i][2], n2[i][3]);
-                *reinterpret_cast<float4*>(o2 + at + 4) = make_float4(n2[i][4], n2[i][5], n2[i][6], n2[i][7]);
+                *reinterpret_cast<float4*>(o2 + at) = make_float4(n2[i][0].x, n2[i][0].y, n2[i][1].x, n2[i][1].y);
+                *reinterpret_cast<float4*>(o2 + at + 4) = make_float4(n2[i][2].x, n2[i][2].y, n2[i][3].x, n2[i][3].y);
             }
         }
     }
@@ -310,7 +327,8 @@ __global__ void __launch_bounds__(kBT, DV > 64 ? 1 : 2)
             for (int c = 0; c < NV; ++c)
                 if (64 * c + 4 * co < DV)
                     *reinterpret_cast<float4*>(ow + (row0 + (i >> 2) * 8 + (i & 3)) * DV + 64 * c + 4 * co) =
-                        make_float4(wide[i][4 * c], wide[i][4 * c + 1], wide[i][4 * c + 2], wide[i][4 * c + 3]);
+                        i & 1 ? make_float4(wide[i >> 1][4 * c].y, wide[i >> 1][4 * c + 1].y, wide[i >> 1][4 * c + 2].y, wide[i >> 1][4 * c + 3].y)
+                              : make_float4(wide[i >> 1][4 * c].x, wide[i >> 1][4 * c + 1].x, wide[i >> 1][4 * c + 2].x, wide[i >> 1][4 * c + 3].x);
     }
     if (nsplit > 1) cluster.sync();
     else __syncthreads();

@@ -10,13 +10,16 @@
 //      the elements through all segments' shared memory and writes that share of the final state (no scratch in global
 //      memory, one launch);
 //   3. chunks of 64 tokens: out = (psi(Q) S + P V) / (psi(Q) z + rowsum P), P = (1 + s/4 + s^2/32)[j <= i] with
-//      s = q.k, then, unless it is the segment's last chunk, S += psi(K)^T V, z += sum psi(K).  A warp builds the feature
-//      rows and weights of its own 8 query rows and is the only one that reads them.
+//      s = q.k, then, unless it is the segment's last chunk, S += psi(K)^T V, z += sum psi(K).
 // With one segment there is no step 1 and 2 and every chunk of step 3 updates the state.
-// Bound: shared-memory passes and the fp32 pipe together (ncu, 296 heads x 512, d_v 64: 76 % of the shared-memory passes,
-// 49 % of the FMA pipe's cycles; per chunk and SM 28 k cycles against 13 k of FMAs); at few heads the chain of chunks.
-// Measured against one CTA per head that walked the tokens one by one: B1 H2 L256 d_v64 190 -> 22 us, B2 H16 L1024 d_v64
-// 660 -> 92 us.
+// Every operand lies along its product's summation index (f32_tiles.cuh).  Outputs: a warp owns 16 query rows and a slice of
+// the features; four slices' groups of 16 rows make a full chunk's eight warps two slices, a chunk of at most 32 (16) tokens
+// has four (eight), and the slices' sums meet in shared memory.
+// Bound: issue slots and latency (per full chunk and SM 27 k cycles, of which the FMA pipe needs 14 k; 11 k instructions per
+// scheduler, 6.6 k of them multiply-adds); at few heads the chain of steps.  Against one CTA per head that walked the tokens
+// one by one: B1 H2 L256 d_v64 190 -> 16 us, B2 H16 L1024 d_v64 660 -> 75.  An earlier form with the operands row by row
+// along the summation index (even and odd terms in one two-wide FMA) took 22 and 92: twice the shared-memory passes, and
+// chunks of 16 tokens used a quarter of the warps' rows.
 #include <cooperative_groups.h>
 
 #include "common.cuh"
@@ -30,17 +33,23 @@ namespace cg = cooperative_groups;
 constexpr int kTok = 64;           // tokens per chunk
 constexpr int kNT = 256;
 constexpr int kMaxSeg = 16;        // CTAs of the largest cluster
+constexpr int kRowT = 68;          // row pitch of tiles with 64 tokens per row
+constexpr int kRowX = 20;          // row pitch of k rows: 16 values, then 1 (0 past the end)
+constexpr int kWarpRows = 16;
 
 struct F32Smem {
-    float psi[kFeatRows * kRowT];  // psi(K)^T [160][68], or psi(Q) [64][156] whose rows are replaced by P's [64][156]
-    float st[64 * kFeat];          // state transposed: [64 columns][156 features]
+    float psi[kFeat * kRowT];      // in turn: the warps' P^T [32 keys][16 rows] each, psi(Q)^T [156][68], the slices'
+                                   // sums, psi(K) [64][160]
+    float st[kFeat * 64];          // state [156 features][64 columns]
     float z[kFeatRows];
-    float vt[64 * kRowT];          // V^T of the chunk [64 columns][68]
-    float xq[kTok * kRowX], xk[kTok * kRowX];
+    float v[kTok * 64];            // V of the chunk
+    float xq[(kDFeat + 1) * kRowT], xk[kDFeat * kRowT];      // transposed; xq: a row of ones behind
+    float kr[kTok * kRowX];        // k rows as they lie
+    float den[kTok];
     FeatTab tab;
 };
-static_assert(sizeof(F32Smem) + 1024 <= (227 * 1024) / 2, "two CTAs per SM");
-static_assert(kTok * kFeat <= kFeatRows * kRowT, "psi(Q) fits");
+static_assert(2 * (sizeof(F32Smem) + 1024) <= 228 * 1024, "two CTAs per SM");
+static_assert(kTok * kFeatRows <= kFeat * kRowT, "psi(K) fits");
 
 // The head's state in the caller's arrays, by symmetric feature f (order of based_decode_step_sym): the row itself, or the
 // rows (m, n) and (n, m) of a full state.
@@ -56,93 +65,221 @@ struct AbiState {
         a = 1 + kDFeat + m * kDFeat + n;
         b = 1 + kDFeat + n * kDFeat + m;
     }
-    static __device__ __forceinline__ float get(const float* p, size_t a, size_t b) {
-        return a == b ? p[a] : (p[a] + p[b]) * kRsqrt2;
+    static __device__ __forceinline__ float fold(float x, float y, bool two) { return two ? (x + y) * kRsqrt2 : x; }
+    __device__ __forceinline__ float4 kv_get(const FeatTab& tab, int f, int c) const {
+        int a, b;
+        rows(tab, f, a, b);
+        const float4 x = *reinterpret_cast<const float4*>(kv + (size_t)a * pitch + c);
+        const float4 y = *reinterpret_cast<const float4*>(kv + (size_t)b * pitch + c);
+        const bool two = a != b;
+        return make_float4(fold(x.x, y.x, two), fold(x.y, y.y, two), fold(x.z, y.z, two), fold(x.w, y.w, two));
     }
-    __device__ __forceinline__ void put(float* p, size_t a, size_t b, float x, bool pair) const {
+    __device__ __forceinline__ void kv_put(const FeatTab& tab, int f, int c, float4 x, bool pair) const {
+        int a, b;
+        rows(tab, f, a, b);
+        float4* pa = reinterpret_cast<float4*>(kv + (size_t)a * pitch + c);
+        float4* pb = reinterpret_cast<float4*>(kv + (size_t)b * pitch + c);
         if (!pair) {
-            p[a] = x;
+            *pa = x;
             return;
         }
-        const float half = keep ? 0.5f * (p[a] - p[b]) : 0.f;
-        p[a] = fmaf(x, kRsqrt2, half);
-        p[b] = fmaf(x, kRsqrt2, -half);
+        float4 h = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (keep) {
+            const float4 u = *pa, w = *pb;
+            h = make_float4(0.5f * (u.x - w.x), 0.5f * (u.y - w.y), 0.5f * (u.z - w.z), 0.5f * (u.w - w.w));
+        }
+        *pa = make_float4(fmaf(x.x, kRsqrt2, h.x), fmaf(x.y, kRsqrt2, h.y), fmaf(x.z, kRsqrt2, h.z), fmaf(x.w, kRsqrt2, h.w));
+        *pb = make_float4(fmaf(x.x, kRsqrt2, -h.x), fmaf(x.y, kRsqrt2, -h.y), fmaf(x.z, kRsqrt2, -h.z), fmaf(x.w, kRsqrt2, -h.w));
     }
-    __device__ __forceinline__ float kv_get(const FeatTab& tab, int f, int c) const {
+    __device__ __forceinline__ void kv_put(const FeatTab& tab, int f, int c, float4 x) const {
         int a, b;
         rows(tab, f, a, b);
-        return get(kv + c, (size_t)a * pitch, (size_t)b * pitch);
-    }
-    __device__ __forceinline__ void kv_put(const FeatTab& tab, int f, int c, float x) const {
-        int a, b;
-        rows(tab, f, a, b);
-        put(kv + c, (size_t)a * pitch, (size_t)b * pitch, x, a != b);
+        kv_put(tab, f, c, x, a != b);
     }
     __device__ __forceinline__ float z_get(const FeatTab& tab, int f) const {
         int a, b;
         rows(tab, f, a, b);
-        return get(z, a, b);
+        return fold(z[a], z[b], a != b);
     }
     __device__ __forceinline__ void z_put(const FeatTab& tab, int f, float x) const {
         int a, b;
         rows(tab, f, a, b);
-        put(z, a, b, x, a != b);
+        if (a == b) {
+            z[a] = x;
+            return;
+        }
+        const float half = keep ? 0.5f * (z[a] - z[b]) : 0.f;
+        z[a] = fmaf(x, kRsqrt2, half);
+        z[b] = fmaf(x, kRsqrt2, -half);
     }
 };
 
-// outputs of up to 8 NI tokens of a chunk; everything but the state, V^T and the k rows is the warp's own
-template <int NI>
+// up to 64 rows of 16 values, transposed -> [16][68]; rows past nt are zero.  rows: as they lie too, element 16 1 on real rows
+__device__ __forceinline__ void load_x(float* dst, float* rows, const float* __restrict__ src, int nt, int tid) {
+    const int t = tid >> 2, p = tid & 3;
+    const bool live = t < nt;
+    const float4 x = live ? __ldg(reinterpret_cast<const float4*>(src + (size_t)t * kDFeat) + p) : make_float4(0.f, 0.f, 0.f, 0.f);
+    dst[(4 * p + 0) * kRowT + t] = x.x;
+    dst[(4 * p + 1) * kRowT + t] = x.y;
+    dst[(4 * p + 2) * kRowT + t] = x.z;
+    dst[(4 * p + 3) * kRowT + t] = x.w;
+    if (rows) {
+        *reinterpret_cast<float4*>(&rows[t * kRowX + 4 * p]) = x;
+        if (p == 0) rows[t * kRowX + kDFeat] = live ? 1.f : 0.f;
+    }
+}
+// 64 tokens x 64 columns of a row-major array; tokens past nt and columns past ncol (a multiple of 4) are zero
+__device__ __forceinline__ void load_v(float* dst, const float* __restrict__ src, int pitch, int ncol, int nt, int tid) {
+    float4 x[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int t = (tid >> 4) + 16 * i, c = (tid & 15) * 4;
+        x[i] = t < nt && c < ncol ? __ldg(reinterpret_cast<const float4*>(src + (size_t)t * pitch + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) *reinterpret_cast<float4*>(&dst[((tid >> 4) + 16 * i) * 64 + (tid & 15) * 4]) = x[i];
+}
+
+// acc (rows in pairs: row0 + {0..3, 8..11}, columns 4 co + j) += sum_{k < n} a[k][row] b[k][column]
+__device__ __forceinline__ void tile_product(float2 (&acc)[4][4], const float* a, int pa, const float* b, int pb, int n) {
+#pragma unroll 4
+    for (int k = 0; k < n; ++k, a += pa, b += pb) {
+        const float4 x0 = lds4(a), x1 = lds4(a + 8), y = lds4(b);
+        const float ys[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            fma_pair(acc[0][j], x0.x, x0.y, ys[j]);
+            fma_pair(acc[1][j], x0.z, x0.w, ys[j]);
+            fma_pair(acc[2][j], x1.x, x1.y, ys[j]);
+            fma_pair(acc[3][j], x1.z, x1.w, ys[j]);
+        }
+    }
+}
+// state tile of a thread, features 8 fg + 2 i + {0, 1} (i < 4) and 128 + 2 fg + {0, 1} (i = 4), columns 4 cg + j:
+// += sum_{t < nt} psi(K)[t][feature] V[t][column]
+__device__ __forceinline__ void state_product(float2 (&acc)[5][4], const float* psi, const float* v, int nt, int fg, int cg) {
+    const float *a = psi + 8 * fg, *a2 = psi + 128 + 2 * fg, *b = v + 4 * cg;
+#pragma unroll 2
+    for (int t = 0; t < nt; ++t, a += kFeatRows, a2 += kFeatRows, b += 64) {
+        const float4 x0 = lds4(a), x1 = lds4(a + 4), y = lds4(b);
+        const float2 x2 = *reinterpret_cast<const float2*>(a2);
+        const float ys[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            fma_pair(acc[0][j], x0.x, x0.y, ys[j]);
+            fma_pair(acc[1][j], x0.z, x0.w, ys[j]);
+            fma_pair(acc[2][j], x1.x, x1.y, ys[j]);
+            fma_pair(acc[3][j], x1.z, x1.w, ys[j]);
+            fma_pair(acc[4][j], x2.x, x2.y, ys[j]);
+        }
+    }
+}
+
+// Outputs of a chunk of nt <= 16 NR tokens; ends with a barrier.  Warp w: rows 16 (w % NR), slice w / NR of 8 / NR.
+template <int NR>
 __device__ __forceinline__ void chunk_outputs(F32Smem& s, float* __restrict__ o, int d_v, int ncol, int nt, bool numerator_only,
-                                              int warp, int lane) {
-    psi_rows<NI>(s.psi, s.xq, s.tab, warp, lane);
-    // weights of the rows warp + 8 i and the keys lane + 32 j
-    float2 acc[NI][2];
-    float p[NI][2], den[NI];
+                                              int tid) {
+    constexpr int KS = 8 / NR;
+    const int warp = tid >> 5, lane = tid & 31, ro = lane & 1, co = lane >> 1;
+    const int rg = warp % NR, ks = warp / NR, row0 = rg * kWarpRows + ro * 4;
+    float2 acc[4][4];
+    float den[8];
 #pragma unroll
-    for (int i = 0; i < NI; ++i) acc[i][0] = acc[i][1] = make_float2(0.f, 0.f);
-    rows_product<NI, kRowX, kRowX>(acc, s.xq, s.xk, kDFeat, warp, lane);
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int i = 0; i < NI; ++i) {
+        for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) den[i] = 0.f;
+    // in-chunk part: 32 keys per slice (a chunk of more than 32 tokens has two slices of keys), weights in the warp's own
+    // place, [key][16 rows]
+    if (32 * ks < nt) {
+        float* pw = s.psi + warp * (32 * kWarpRows);
+        float2 p[4][2];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) p[i][0] = p[i][1] = make_float2(0.f, 0.f);
+#pragma unroll 4
+        for (int k = 0; k < kDFeat; ++k) {
+            const float4 x0 = lds4(&s.xq[k * kRowT + row0]), x1 = lds4(&s.xq[k * kRowT + row0 + 8]);
+            const float2 y = *reinterpret_cast<const float2*>(&s.xk[k * kRowT + 32 * ks + 2 * co]);
+            fma_pair(p[0][0], x0.x, x0.y, y.x); fma_pair(p[0][1], x0.x, x0.y, y.y);
+            fma_pair(p[1][0], x0.z, x0.w, y.x); fma_pair(p[1][1], x0.z, x0.w, y.y);
+            fma_pair(p[2][0], x1.x, x1.y, y.x); fma_pair(p[2][1], x1.x, x1.y, y.y);
+            fma_pair(p[3][0], x1.z, x1.w, y.x); fma_pair(p[3][1], x1.z, x1.w, y.y);
+        }
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
-            const float x = acc[i][j].x + acc[i][j].y;
-            p[i][j] = lane + 32 * j <= warp + 8 * i ? fmaf(x, fmaf(x, 0.03125f, 0.25f), 1.0f) : 0.f;
-            acc[i][j] = make_float2(0.f, 0.f);
+            float w[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const float x = i & 1 ? p[i >> 1][j].y : p[i >> 1][j].x;
+                const int row = row0 + (i >> 2) * 8 + (i & 3), key = 32 * ks + 2 * co + j;
+                w[i] = key <= row ? fmaf(x, fmaf(x, 0.03125f, 0.25f), 1.0f) : 0.f;
+                den[i] += w[i];
+            }
+            float* at = pw + (2 * co + j) * kWarpRows + ro * 4;
+            *reinterpret_cast<float4*>(at) = make_float4(w[0], w[1], w[2], w[3]);
+            *reinterpret_cast<float4*>(at + 8) = make_float4(w[4], w[5], w[6], w[7]);
         }
-        den[i] = p[i][0] + p[i][1];
+        __syncwarp();
+        // no key behind the warp's last row counts
+        tile_product(acc, pw + ro * 4, kWarpRows, s.v + 32 * ks * 64 + 4 * co, 64,
+                     min(32, max(0, min(nt, (rg + 1) * kWarpRows) - 32 * ks)));
     }
-    __syncwarp();
-    rows_product<NI, kFeat, kFeat>(acc, s.psi, s.st, kFeat, warp, lane);
-    // cross-chunk denominator
+    __syncthreads();                                 // P is read: psi(Q)^T takes its place
+    for (int e = tid; e < kFeat * (NR * 4); e += kNT) {
+        // four tokens of a feature; consecutive lanes: consecutive features
+        const int t = e / kFeat * 4, f = e % kFeat;
+        const float4 a = lds4(&s.xq[(s.tab.mn[f] & 255) * kRowT + t]), b = lds4(&s.xq[(s.tab.mn[f] >> 8) * kRowT + t]);
+        const float c = s.tab.scale[f];
+        *reinterpret_cast<float4*>(&s.psi[f * kRowT + t]) = make_float4(c * a.x * b.x, c * a.y * b.y, c * a.z * b.z, c * a.w * b.w);
+    }
+    __syncthreads();
+    const int f0 = ks * kFeat / KS, f1 = (ks + 1) * kFeat / KS;
+    tile_product(acc, s.psi + f0 * kRowT + row0, kRowT, s.st + f0 * 64 + 4 * co, 64, f1 - f0);
+    for (int f = f0 + co; f < f1; f += 16) {
+        const float4 x0 = lds4(&s.psi[f * kRowT + row0]), x1 = lds4(&s.psi[f * kRowT + row0 + 8]);
+        const float zf = s.z[f];
+        den[0] = fmaf(x0.x, zf, den[0]); den[1] = fmaf(x0.y, zf, den[1]); den[2] = fmaf(x0.z, zf, den[2]); den[3] = fmaf(x0.w, zf, den[3]);
+        den[4] = fmaf(x1.x, zf, den[4]); den[5] = fmaf(x1.y, zf, den[5]); den[6] = fmaf(x1.z, zf, den[6]); den[7] = fmaf(x1.w, zf, den[7]);
+    }
 #pragma unroll
-    for (int u = 0; u < kTF; ++u) {
-        const int f = lane + 32 * u;
-        if (f < kFeat) {
-            const float zf = s.z[f];
+    for (int i = 0; i < 8; ++i)
 #pragma unroll
-            for (int i = 0; i < NI; ++i) den[i] = fmaf(s.psi[(warp + 8 * i) * kFeat + f], zf, den[i]);
+        for (int x = 2; x < 32; x <<= 1) den[i] += __shfl_xor_sync(0xffffffffu, den[i], x);
+    __syncthreads();                                 // psi(Q)^T is read: the slices' sums take its place
+    float* red = s.psi + (ks - 1) * (NR * kWarpRows * 64);
+    float* red_den = s.psi + (KS - 1) * (NR * kWarpRows * 64);
+    if (ks > 0) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int row = row0 + (i >> 2) * 8 + (i & 3);
+            *reinterpret_cast<float4*>(&red[row * 64 + 4 * co]) =
+                i & 1 ? make_float4(acc[i >> 1][0].y, acc[i >> 1][1].y, acc[i >> 1][2].y, acc[i >> 1][3].y)
+                      : make_float4(acc[i >> 1][0].x, acc[i >> 1][1].x, acc[i >> 1][2].x, acc[i >> 1][3].x);
+            if (co == 0) red_den[(ks - 1) * (NR * kWarpRows) + row] = den[i];
         }
     }
-    __syncwarp();                                    // psi(Q) is read: P takes its place
+    __syncthreads();
+    if (ks == 0) {
 #pragma unroll
-    for (int i = 0; i < NI; ++i) {
-        den[i] = warp_sum(den[i]);
-        s.psi[(warp + 8 * i) * kFeat + lane] = p[i][0];
-        s.psi[(warp + 8 * i) * kFeat + lane + 32] = p[i][1];
-    }
-    __syncwarp();
-    rows_product<NI, kFeat, kRowT>(acc, s.psi, s.vt, (nt + 3) & ~3, warp, lane);
+        for (int i = 0; i < 8; ++i) {
+            const int row = row0 + (i >> 2) * 8 + (i & 3);
+            float4 x = i & 1 ? make_float4(acc[i >> 1][0].y, acc[i >> 1][1].y, acc[i >> 1][2].y, acc[i >> 1][3].y)
+                             : make_float4(acc[i >> 1][0].x, acc[i >> 1][1].x, acc[i >> 1][2].x, acc[i >> 1][3].x);
+            float d = den[i];
 #pragma unroll
-    for (int i = 0; i < NI; ++i) {
-        const int t = warp + 8 * i;
-        if (t >= nt) continue;
-        const float d = numerator_only ? 1.f : den[i] + kEps;
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const int c = lane + 32 * j;
-            if (c < ncol) o[(size_t)t * d_v + c] = (acc[i][j].x + acc[i][j].y) / d;
+            for (int r = 0; r < KS - 1; ++r) {
+                const float4 y = lds4(&s.psi[r * (NR * kWarpRows * 64) + row * 64 + 4 * co]);
+                x.x += y.x; x.y += y.y; x.z += y.z; x.w += y.w;
+                d += red_den[r * (NR * kWarpRows) + row];
+            }
+            if (row < nt && 4 * co < ncol) {
+                d = numerator_only ? 1.f : d + kEps;
+                *reinterpret_cast<float4*>(&o[(size_t)row * d_v + 4 * co]) = make_float4(x.x / d, x.y / d, x.z / d, x.w / d);
+            }
         }
     }
+    __syncthreads();                                 // the slices' sums are read
 }
 }  // namespace
 
@@ -156,7 +293,8 @@ __global__ void __launch_bounds__(kNT, 2)
     const int cluster_row = blockIdx.z * nseg;
     const size_t head = blockIdx.y;
     const int col0 = blockIdx.z * ncol;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int fg = (tid >> 5) * 2 + (lane & 1), cgr = lane >> 1;     // state tile (state_product)
     const int t_begin = min(rank * seg, L), t_end = min(t_begin + seg, L);
     const bool cont = (flags & BASED_STATE_CONTINUE) != 0, numerator_only = (flags & BASED_NUMERATOR_ONLY) != 0;
     AbiState abi;
@@ -172,68 +310,89 @@ __global__ void __launch_bounds__(kNT, 2)
     float* oh = out + head * (size_t)L * d_v + col0;
 
     fill_feat_tab(s.tab, tid);
+    if (tid < kRowT) s.xq[kDFeat * kRowT + tid] = 1.f;
     __syncthreads();
 
-    // a chunk's contribution to the state tile of a thread: features lane + 32 i, columns 8 warp + j
-    auto chunk_state = [&](float2 (&acc)[kTF][8], int nt) {
-        psi_transposed(s.psi, s.xk, s.tab, nt, tid);
-        __syncthreads();
-        state_update(acc, s.psi, s.vt, nt, warp, lane);
+    float2 acc[5][4];
+    auto clear = [&] {
+#pragma unroll
+        for (int i = 0; i < 5; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
     };
-    float zsum = 0.f;                                // thread f < 160: z of feature f
+    // a chunk's contribution to the state tile; psi(K) is left in place for z
+    auto chunk_state = [&](int nt) {
+        // a lane's five features of every eighth token
+#pragma unroll
+        for (int i = 0; i < kFeatRows / 32; ++i) {
+            const int f = lane + 32 * i;
+            const float *xm = s.kr + (s.tab.mn[f] & 255), *xn = s.kr + (s.tab.mn[f] >> 8);
+            const float c = s.tab.scale[f];
+#pragma unroll
+            for (int u = 0; u < kTok / 8; ++u) {
+                const int t = (tid >> 5) + 8 * u;
+                if (8 * u < nt) s.psi[t * kFeatRows + f] = c * xm[t * kRowX] * xn[t * kRowX];
+            }
+        }
+        __syncthreads();
+        state_product(acc, s.psi, s.v, nt, fg, cgr);
+    };
+    auto chunk_z = [&](int nt) {                     // thread f < 160
+        float a[4] = {0.f, 0.f, 0.f, 0.f};           // (rows past nt up to the next eight are zero)
+        for (int t = 0; t < nt; t += 8)
+#pragma unroll
+            for (int u = 0; u < 8; ++u) a[u & 3] += s.psi[(t + u) * kFeatRows + tid];
+        return (a[0] + a[1]) + (a[2] + a[3]);
+    };
+    // the state tile's elements: feature, columns 4 cgr .. + 3
+    auto each_row = [&](auto fn) {
+#pragma unroll
+        for (int i = 0; i < 5; ++i)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int f = (i < 4 ? 8 * fg + 2 * i : 128 + 2 * fg) + h;
+                if (f < kFeat)
+                    fn(f, h ? make_float4(acc[i][0].y, acc[i][1].y, acc[i][2].y, acc[i][3].y)
+                            : make_float4(acc[i][0].x, acc[i][1].x, acc[i][2].x, acc[i][3].x));
+            }
+    };
     if (nseg > 1) {
         // ---- step 1: this segment's own state (the last one's is needed for the final state only)
-        float2 acc[kTF][8];
-#pragma unroll
-        for (int i = 0; i < kTF; ++i)
-#pragma unroll
-            for (int j = 0; j < 8; ++j) acc[i][j] = make_float2(0.f, 0.f);
+        clear();
+        float zsum = 0.f;                            // thread f < 160: z of feature f
         const float zc = cont && rank == 0 && tid < kDSym ? abi.z_get(s.tab, tid) : 0.f;
         if (rank < nseg - 1 || kv != nullptr) {
             for (int t0 = t_begin; t0 < t_end; t0 += kTok) {
                 const int nt = min(kTok, t_end - t0);
-                load_x(s.xk, kh + (size_t)t0 * kDFeat, nt, tid);
-                load_vt(s.vt, vh + (size_t)t0 * d_v, d_v, ncol, nt, tid);
+                load_x(s.xk, s.kr, kh + (size_t)t0 * kDFeat, nt, tid);
+                load_v(s.v, vh + (size_t)t0 * d_v, d_v, ncol, nt, tid);
                 __syncthreads();
-                chunk_state(acc, nt);
-                if (tid < kFeatRows) zsum += row_sum(s.psi, tid, nt);
+                chunk_state(nt);
+                if (tid < kFeatRows) zsum += chunk_z(nt);
                 __syncthreads();
             }
         }
-#pragma unroll
-        for (int i = 0; i < kTF; ++i) {
-            const int f = lane + 32 * i;
-            if (f < kFeat)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) s.st[(warp * 8 + j) * kFeat + f] = acc[i][j].x + acc[i][j].y;
-        }
+        each_row([&](int f, float4 x) { *reinterpret_cast<float4*>(&s.st[f * 64 + 4 * cgr]) = x; });
         if (tid < kFeatRows) s.z[tid] = zsum;
         cluster.sync();
 
-        // ---- step 2: running sums over the segments, four features of a column per thread; consecutive lanes take
-        // consecutive columns, so the caller's state is read and written in whole rows
-        for (int e = rank * kNT + tid; e < 64 * (kFeat / 4); e += nseg * kNT) {
-            const int c = e & 63, f = (e >> 6) * 4;
-            float4* mine = reinterpret_cast<float4*>(&s.st[c * kFeat + f]);
+        // ---- step 2: running sums over the segments, four columns of a feature per thread
+        for (int e = rank * kNT + tid; e < kFeat * 16; e += nseg * kNT) {
+            const int f = e >> 4, c = (e & 15) * 4;
+            float4* mine = reinterpret_cast<float4*>(&s.st[f * 64 + c]);
             float4 x[kMaxSeg];
 #pragma unroll
             for (int r = 0; r < kMaxSeg; ++r)
                 if (r < nseg) x[r] = *cluster.map_shared_rank(mine, cluster_row + r);
-            float run[4] = {0.f, 0.f, 0.f, 0.f};
-            if (cont && c < ncol)
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (f + u < kDSym) run[u] = abi.kv_get(s.tab, f + u, c);
+            const bool real = f < kDSym && c < ncol;
+            float4 run = cont && real ? abi.kv_get(s.tab, f, c) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
             for (int r = 0; r < kMaxSeg; ++r)
                 if (r < nseg) {
-                    *cluster.map_shared_rank(mine, cluster_row + r) = make_float4(run[0], run[1], run[2], run[3]);
-                    run[0] += x[r].x; run[1] += x[r].y; run[2] += x[r].z; run[3] += x[r].w;
+                    *cluster.map_shared_rank(mine, cluster_row + r) = run;
+                    run.x += x[r].x; run.y += x[r].y; run.z += x[r].z; run.w += x[r].w;
                 }
-            if (kv != nullptr && c < ncol)
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (f + u < kDSym) abi.kv_put(s.tab, f + u, c, run[u]);
+            if (kv != nullptr && real) abi.kv_put(s.tab, f, c, run);
         }
         if (rank == 0 && tid < kFeatRows) {
             float x[kMaxSeg], run = zc;
@@ -250,9 +409,10 @@ __global__ void __launch_bounds__(kNT, 2)
         }
         cluster.sync();
     } else {
-        for (int e = tid; e < 64 * kFeat; e += kNT) {
-            const int c = e & 63, f = e >> 6;
-            s.st[c * kFeat + f] = cont && f < kDSym && c < ncol ? abi.kv_get(s.tab, f, c) : 0.f;
+        for (int e = tid; e < kFeat * 16; e += kNT) {
+            const int f = e >> 4, c = (e & 15) * 4;
+            *reinterpret_cast<float4*>(&s.st[f * 64 + c]) =
+                cont && f < kDSym && c < ncol ? abi.kv_get(s.tab, f, c) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
         if (tid < kFeatRows) s.z[tid] = cont && tid < kDSym ? abi.z_get(s.tab, tid) : 0.f;
         // column group 0 writes the K-state that the other one reads
@@ -262,37 +422,31 @@ __global__ void __launch_bounds__(kNT, 2)
     // ---- step 3: outputs, chunk by chunk
     for (int t0 = t_begin; t0 < t_end; t0 += kTok) {
         const int nt = min(kTok, t_end - t0);
-        load_x(s.xq, qh + (size_t)t0 * kDFeat, nt, tid);
-        load_x(s.xk, kh + (size_t)t0 * kDFeat, nt, tid);
-        load_vt(s.vt, vh + (size_t)t0 * d_v, d_v, ncol, nt, tid);
+        load_x(s.xq, nullptr, qh + (size_t)t0 * kDFeat, nt, tid);
+        load_x(s.xk, s.kr, kh + (size_t)t0 * kDFeat, nt, tid);
+        load_v(s.v, vh + (size_t)t0 * d_v, d_v, ncol, nt, tid);
         __syncthreads();
         float* o = oh + (size_t)t0 * d_v;
-        if (nt > 32) chunk_outputs<8>(s, o, d_v, ncol, nt, numerator_only, warp, lane);
-        else if (nt > 16) chunk_outputs<4>(s, o, d_v, ncol, nt, numerator_only, warp, lane);
-        else chunk_outputs<2>(s, o, d_v, ncol, nt, numerator_only, warp, lane);
+        if (nt > 32) chunk_outputs<4>(s, o, d_v, ncol, nt, numerator_only, tid);
+        else if (nt > 16) chunk_outputs<2>(s, o, d_v, ncol, nt, numerator_only, tid);
+        else chunk_outputs<1>(s, o, d_v, ncol, nt, numerator_only, tid);
         if (t0 + kTok >= t_end && (nseg > 1 || kv == nullptr)) break;   // nobody reads the state after this chunk
-        __syncthreads();                             // P and the state are read
-        float2 acc[kTF][8];
-#pragma unroll
-        for (int i = 0; i < kTF; ++i)
-#pragma unroll
-            for (int j = 0; j < 8; ++j) acc[i][j] = make_float2(0.f, 0.f);
-        chunk_state(acc, nt);
-#pragma unroll
-        for (int i = 0; i < kTF; ++i) {
-            const int f = lane + 32 * i;
-            if (f < kFeat)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) s.st[(warp * 8 + j) * kFeat + f] += acc[i][j].x + acc[i][j].y;
-        }
-        if (tid < kFeatRows) s.z[tid] += row_sum(s.psi, tid, nt);
+        clear();
+        chunk_state(nt);
+        each_row([&](int f, float4 x) {
+            float4* p = reinterpret_cast<float4*>(&s.st[f * 64 + 4 * cgr]);
+            float4 y = *p;
+            y.x += x.x; y.y += x.y; y.z += x.z; y.w += x.w;
+            *p = y;
+        });
+        if (tid < kFeatRows) s.z[tid] += chunk_z(nt);
         __syncthreads();
     }
 
     if (nseg == 1 && kv != nullptr) {
-        for (int e = tid; e < 64 * kDSym; e += kNT) {
-            const int c = e & 63, f = e >> 6;
-            if (c < ncol) abi.kv_put(s.tab, f, c, s.st[c * kFeat + f]);
+        for (int e = tid; e < kDSym * 16; e += kNT) {
+            const int f = e >> 4, c = (e & 15) * 4;
+            if (c < ncol) abi.kv_put(s.tab, f, c, lds4(&s.st[f * 64 + c]));
         }
         if (blockIdx.z == 0 && tid < kDSym) abi.z_put(s.tab, tid, s.z[tid]);
     }
@@ -302,23 +456,26 @@ namespace {
 // whole groups of 16 tokens, so that every segment but the last ends on a tile edge of the products
 int f32_segment_tokens(int L, int nseg) { return ((L + nseg - 1) / nseg + 15) / 16 * 16; }
 // Segments per head (the cluster holds all segments of both column groups, at most 16 CTAs), by a time model fitted on
-// B200, in us: outputs of a full chunk 10.5 (a chunk of up to 32 / 16 tokens 0.5 / 0.3 of that), a state update 5.5, two
-// CTAs on an SM 1.9 times one, 5 for launch and ramps, 4 + 0.3 n for the running sums of n segments, all of it once per
-// wave.  Clusters of 8 and 16 CTAs leave SMs of a GPC unused: about 104 and 96 fit one per SM.  More segments shorten the
-// chain of chunks but every chunk then updates a state twice (its segment's own sums, then the running state): B1 H2 L256
-// d_v64 70 / 46 / 26 / 23 / 22 us with 1 / 2 / 4 / 8 / 16 segments, B2 H16 L1024 d_v64 257 / 177 / 92 / 93 / 126, B8 H16
-// L512 d_v64 133 / 153 / 150 / 184 / 343, B1 H16 L700 d_v64 179 / 126 / 68 / 71 / 75.  The same whether the state is asked
-// for or not: so are the outputs.
+// B200, in us: outputs of a full chunk 9.3 (a chunk of up to 32 / 16 tokens 6.8 / 6), a state update 4.9 (3.8 / 3.5), 3 for
+// launch and ramps, 3 + 0.1 n for the running sums of n segments; two CTAs on an SM 1.8 times one, more in proportion.
+// Clusters of 8 and 16 CTAs leave SMs of a GPC unused: about 104 and 96 CTAs fit one per SM, and many waves take 1.15 and
+// 1.4 times as long.  More segments shorten the chain of chunks but every chunk then updates a state twice (its segment's
+// own sums, then the running state).  Measured with 1 / 2 / 4 / 8 / 16 segments: B1 H2 L256 d_v64 60 / 39 / 20 / 17 / 16,
+// B2 H16 L1024 d_v64 229 / 154 / 78 / 75 / 80, B8 H16 L512 d_v64 117 / 130 / 121 / 118 / 201, B1 H16 L700 d_v64 159 / 111 /
+// 57 / 55 / 47.  The same whether the state is asked for or not: so are the outputs.
 int f32_segments(int BH, int L, int nz) {
     int best = 1;
     double best_t = 1e30;
     for (int n = 1; n * nz <= kMaxSeg; n *= 2) {
-        const int seg = f32_segment_tokens(L, n), rest = seg % kTok, chunks = (seg + kTok - 1) / kTok;
-        const double outs = seg / kTok + (rest == 0 ? 0.0 : rest <= 16 ? 0.3 : rest <= 32 ? 0.5 : 1.0);
-        const double ups = n > 1 ? 2 * chunks - 1 : chunks;
-        const long long ctas = (long long)BH * nz * n, fit = n * nz <= 4 ? 148 : n * nz == 8 ? 104 : 96;
-        const double waves = (double)((ctas + 2 * fit - 1) / (2 * fit));
-        const double t = waves * ((ctas <= fit ? 1.0 : 1.9) * (outs * 10.5 + ups * 5.5) + 5.0 + (n > 1 ? 4.0 + 0.3 * n : 0.0));
+        const int seg = f32_segment_tokens(L, n), full = seg / kTok, rest = seg % kTok;
+        const double outs = full * 9.3 + (rest == 0 ? 0.0 : rest <= 16 ? 6.0 : rest <= 32 ? 6.8 : 9.3);
+        const double ups = full * 4.9 + (rest == 0 ? 0.0 : rest <= 16 ? 3.5 : rest <= 32 ? 3.8 : 4.9);
+        const double last = rest == 0 ? 4.9 : rest <= 16 ? 3.5 : rest <= 32 ? 3.8 : 4.9;
+        const int cl = n * nz;
+        const double ctas = (double)BH * cl, fit = cl <= 4 ? 148 : cl == 8 ? 104 : 96;
+        const double many = ctas / 148 * (cl <= 4 ? 1.0 : cl == 8 ? 1.15 : 1.4);
+        const double load = ctas <= fit ? 1.0 : many > 1.8 ? many : 1.8;
+        const double t = load * (outs + (n > 1 ? 2 * ups - last : ups)) + 3.0 + (n > 1 ? 3.0 + 0.1 * n : 0.0);
         if (t < best_t) { best_t = t; best = n; }
     }
     return best;

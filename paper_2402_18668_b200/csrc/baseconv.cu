@@ -177,6 +177,7 @@ __global__ void __launch_bounds__(kThreadsBC) baseconv_step_kernel(const T* __re
                                                                    const float* __restrict__ h,
                                                                    const float* __restrict__ b2, T* __restrict__ state,
                                                                    T* __restrict__ out, int B, int C) {
+    enter_dependent();
     constexpr bool FAST = sizeof(T) == 2;
     const int c0 = (blockIdx.x * kThreadsBC + threadIdx.x) * 8;
     if (c0 >= C) return;
@@ -225,12 +226,17 @@ template <typename T, int W>
 static void launch_w(const void* a, const void* g, const float* h, const float* b2, void* state, void* out, int B,
                      int N, int C, bool step, cudaStream_t stream) {
     const int gx = (C / 8 + kThreadsBC - 1) / kThreadsBC;
-    // four sequences per thread once that still gives every SM a block
+    static std::atomic<bool> split[3][64];
+    prefer_l1(baseconv_step_kernel<T, W, 4>, 0, split[0]);       // (a preference only: the launch reports what fails)
+    prefer_l1(baseconv_step_kernel<T, W, 1>, 0, split[1]);
+    prefer_l1(baseconv_gate_kernel<T, W>, 0, split[2]);
+    // a step is a dependent launch: its blocks come in while the kernel ahead drains (behind the other mixers' steps at batch
+    // 128 1.0 us less a token; back to back with itself 0.5 more); four sequences per thread once that still gives every SM a block
     if (step && gx * ((B + 3) / 4) >= kSMs)
-        baseconv_step_kernel<T, W, 4><<<dim3(gx, (B + 3) / 4), kThreadsBC, 0, stream>>>(
+        launch_ex(baseconv_step_kernel<T, W, 4>, dim3(gx, (B + 3) / 4), dim3(kThreadsBC), 0, 1, true, stream,
             static_cast<const T*>(a), static_cast<const T*>(g), h, b2, static_cast<T*>(state), static_cast<T*>(out), B, C);
     else if (step)
-        baseconv_step_kernel<T, W, 1><<<dim3(gx, B), kThreadsBC, 0, stream>>>(
+        launch_ex(baseconv_step_kernel<T, W, 1>, dim3(gx, B), dim3(kThreadsBC), 0, 1, true, stream,
             static_cast<const T*>(a), static_cast<const T*>(g), h, b2, static_cast<T*>(state), static_cast<T*>(out), B, C);
     else {
         // runs of 64 tokens (a halo of width - 1 rows each) while the last wave of blocks is a small part of the grid, 32

@@ -31,6 +31,52 @@ std::mutex& setup_mutex();
 void note_launch();                                     // ++launch counter
 based_status check_launch(const char* what);            // cudaGetLastError -> status
 
+// Launch, PARTS > 1 CTAs per cluster; dependent: with programmatic stream serialization, so that the grid's CTAs may be
+// scheduled once every CTA of the grid ahead in the stream has signalled (griddepcontrol.launch_dependents) or left.  The
+// kernel itself waits (enter_dependent) before it touches what that grid reads or writes; behind a kernel that never signals
+// such a launch behaves like a plain one.
+template <typename... P, typename... A>
+cudaError_t launch_ex(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, int cluster, bool dependent, cudaStream_t stream,
+                      const A&... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute at[2]{};
+    int n = 0;
+    if (dependent) {
+        at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        at[n].id = cudaLaunchAttributeClusterDimension;
+        at[n].val.clusterDim.x = cluster;
+        at[n].val.clusterDim.y = 1;
+        at[n++].val.clusterDim.z = 1;
+    }
+    cfg.attrs = at;
+    cfg.numAttrs = n;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+// Splits an SM's 256 KB between L1 and shared memory for a kernel that streams through L1: loads in flight take L1 lines, and
+// without a preference a kernel runs with whatever split the one before it left (decode step, 2048 heads, d_v 128: 91 us
+// with a quarter for shared memory or no preference alone, 113 with all of it).  Once per kernel and device.
+template <typename K>
+cudaError_t prefer_l1(K kernel, int shared_percent, std::atomic<bool> (&done)[64]) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess || dev < 0 || dev >= 64) return e != cudaSuccess ? e : cudaErrorInvalidDevice;
+    if (done[dev].load(std::memory_order_acquire)) return cudaSuccess;
+    const cudaError_t f = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, shared_percent);
+    if (f == cudaSuccess) done[dev].store(true, std::memory_order_release);
+    return f;
+}
+__device__ __forceinline__ void enter_dependent() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 template <typename T> __device__ __forceinline__ float to_f32(T x);
 template <> __device__ __forceinline__ float to_f32<float>(float x) { return x; }
 template <> __device__ __forceinline__ float to_f32<__nv_bfloat16>(__nv_bfloat16 x) { return __bfloat162float(x); }

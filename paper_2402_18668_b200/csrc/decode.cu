@@ -22,6 +22,7 @@ __global__ void __launch_bounds__(256, CTAS) decode_step_kernel(const T* __restr
                                                           const T* __restrict__ v, float* __restrict__ kv,
                                                           float* __restrict__ z, T* __restrict__ out,
                                                           int numerator_only) {
+    enter_dependent();
     decode_step_body<DV, T, SYM, PARTS, UN, STREAM>(q, k, v, kv, z, out, numerator_only, blockIdx.x / PARTS,
                                                     blockIdx.x % PARTS);
 }
@@ -30,27 +31,14 @@ template <int DV, typename T, bool SYM, int PARTS, int UN, int CTAS, bool STREAM
 static based_status launch_variant(const T* q, const T* k, const T* v, float* kv, float* z, T* out, int BH, int num_only,
                                    cudaStream_t stream) {
     auto kern = decode_step_kernel<DV, T, SYM, PARTS, UN, CTAS, STREAM>;
-    if (PARTS == 1) {
-        kern<<<BH, 256, 0, stream>>>(q, k, v, kv, z, out, num_only);
-    } else {
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(PARTS * BH);
-        cfg.blockDim = dim3(256);
-        cfg.stream = stream;
-        cudaLaunchAttribute attr{};
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = PARTS;
-        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        if (cudaLaunchKernelEx(&cfg, kern, q, k, v, kv, z, out, num_only) != cudaSuccess) {
-            note_launch();
-            check_launch("decode_step_kernel");
-            return BASED_ERR_CUDA;
-        }
-    }
+    static std::atomic<bool> split[64];
+    if (prefer_l1(kern, 25, split) != cudaSuccess) return BASED_ERR_CUDA;
+    // a dependent launch: its CTAs come in while the kernel ahead drains (16 heads 6.3 -> 4.8 us a call, 2048 heads 91.3 ->
+    // 89.5; with the window's step behind it, a pair of calls 103.7 -> 100.1)
+    const cudaError_t e = launch_ex(kern, dim3(PARTS * BH), dim3(256), 0, PARTS, true, stream, q, k, v, kv, z, out, num_only);
     note_launch();
-    return check_launch("decode_step_kernel");
+    const based_status st = check_launch("decode_step_kernel");
+    return e == cudaSuccess ? st : BASED_ERR_CUDA;
 }
 
 // The variants of a step, by the number of heads (us per step on B200, replayed back to back):

@@ -107,6 +107,9 @@ __global__ void __launch_bounds__(256, CTAS) generation_step_kernel(const GenArg
 template <int DV, bool STREAM> struct Depth {
     static constexpr bool kWide = DV == 64 && !STREAM;
     static constexpr int kRows = kWide ? 6 : 18, kCtas = kWide ? 4 : 2;
+    // percent of an SM's 256 KB for shared memory, the rest is L1 for the loads in flight (batch 128, d_v 128, 153 rows:
+    // 100 / 80 / 60 / 50 / 40 % 68.8 / 55.2 / 54.1 / 53.9 / 57.9 us; batch 64, d_v 64, 273 rows: 25.3 / 21.3 / 22.6 / 22.6 / 27.1)
+    static constexpr int kShared = kWide ? 80 : 50;
 };
 
 template <int DV, typename T, bool STREAM, bool SYM, int NPW, int PARTS>
@@ -114,6 +117,8 @@ based_status launch_k(const GenArgs& args, size_t smem, cudaStream_t stream) {
     auto kern = generation_step_kernel<DV, T, STREAM, SYM, NPW, PARTS, (PARTS > 1 ? 9 : Depth<DV, STREAM>::kRows), Depth<DV, STREAM>::kCtas>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return BASED_ERR_CUDA;
+    static std::atomic<bool> split[64];
+    if (prefer_l1(kern, Depth<DV, STREAM>::kShared, split) != cudaSuccess) return BASED_ERR_CUDA;
     GenArgs a = args;
     const int n_swa_ctas = ((a.n_swa + 1) / 2 + PARTS - 1) / PARTS;
     a.n_pairs = n_swa_ctas < a.n_lin / 2 ? n_swa_ctas : a.n_lin / 2;

@@ -391,6 +391,10 @@ static based_status decode_t(const void* q, const void* k, const void* v, float*
     const T* qq = static_cast<const T*>(q);
     const T* kk = static_cast<const T*>(k);
     const T* vv = static_cast<const T*>(v);
+    static std::atomic<bool> split[2][64];
+    if (prefer_l1(generic_decode_kernel<T, DV, true>, 25, split[0]) != cudaSuccess ||
+        prefer_l1(generic_decode_kernel<T, DV, false>, 25, split[1]) != cudaSuccess)
+        return BASED_ERR_CUDA;
     if (streaming) generic_decode_kernel<T, DV, true><<<BH, 256, 0, stream>>>(qq, kk, vv, kv, z, static_cast<T*>(out), df, num_only);
     else generic_decode_kernel<T, DV, false><<<BH, 256, 0, stream>>>(qq, kk, vv, kv, z, static_cast<T*>(out), df, num_only);
     note_launch();

@@ -24,6 +24,7 @@ swa_decode_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __r
                   T* __restrict__ vc, T* __restrict__ out, int window, int pos_arg,
                   const int* pos_dev, int* pos_adv, float scale, unsigned int* __restrict__ error_word, int pos_group) {
     extern __shared__ __align__(128) unsigned char smem[];
+    enter_dependent();
     swa_decode_body<T, NPW, 1>(q, k, v, kc, vc, out, window, pos_arg, pos_dev, pos_adv, scale, error_word, blockIdx.x,
                                threadIdx.x, (int)gridDim.x, smem, pos_group);
 }
@@ -38,11 +39,16 @@ static based_status launch_n(const void* q, const void* k, const void* v, void* 
                                  (int)smem) != cudaSuccess)
             return BASED_ERR_CUDA;
     }
-    swa_decode_kernel<T, NPW><<<BH, 32 * kWarps, smem, stream>>>(static_cast<const T*>(q), static_cast<const T*>(k),
-                                                          static_cast<const T*>(v), static_cast<T*>(kc),
-                                                          static_cast<T*>(vc), static_cast<T*>(out), window, pos,
-                                                          pos_dev, pos_adv, scale, err, pos_group);
+    // a dependent launch: its CTAs come in while the kernel ahead drains (a pair of calls with the recurrent step at batch 128
+    // 103.7 -> 102.2 us, at batch 4 9.9 -> 9.6)
+    const cudaError_t e = launch_ex(swa_decode_kernel<T, NPW>, dim3(BH), dim3(32 * kWarps), smem, 1, true, stream, static_cast<const T*>(q),
+                                    static_cast<const T*>(k), static_cast<const T*>(v), static_cast<T*>(kc), static_cast<T*>(vc),
+                                    static_cast<T*>(out), window, pos, pos_dev, pos_adv, scale, err, pos_group);
     note_launch();
+    if (e != cudaSuccess) {
+        check_launch("swa_decode_kernel");
+        return BASED_ERR_CUDA;
+    }
     return check_launch("swa_decode_kernel");
 }
 

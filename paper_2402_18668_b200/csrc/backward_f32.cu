@@ -396,8 +396,12 @@ based_status launch_pass(const float* q, const float* k, const float* v, const f
         }
     }
     const int ntile = (L + kT - 1) / kT;
-    int nsplit = 1;                                  // two CTAs fit an SM
-    while (nsplit < kMaxSplit && 2 * nsplit <= ntile && (long long)BH * ntile * 2 * nsplit <= 2 * kSMs) nsplit *= 2;
+    // CTAs per own tile: as many as one wave of two per SM has room for, and two up to twice that, where one per tile leaves
+    // a second wave of few (1 / 2 / 4 CTAs, us: 256 tiles of B1 H16 L1024 192 / 156 / 180, 224 of B2 H16 L390 87 / 83 / 103,
+    // 512 of B4 H16 L512 151 / 176 / 232, 64 of B1 H8 L512 86 / 51 / 37)
+    const long long tiles = (long long)BH * ntile;
+    int nsplit = 1;
+    while (nsplit < kMaxSplit && 2 * nsplit <= ntile && tiles * 2 * nsplit <= (nsplit == 1 ? 4 : 2) * kSMs) nsplit *= 2;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)BH * ntile, 1, nsplit);
     cfg.blockDim = dim3(kBT);

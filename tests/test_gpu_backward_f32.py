@@ -13,7 +13,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("d_v,BH,L", [(64, 1, 63), (64, 2, 65), (64, 2, 128), (112, 3, 129), (128, 2, 257), (64, 1, 700),
-                                      (64, 150, 130), (128, 80, 200)])
+                                      (64, 150, 130), (128, 80, 200), (64, 32, 513), (128, 74, 256),
+                                      (64, 75, 256)])
 @pytest.mark.parametrize("flags", [0, based.BASED_NUMERATOR_ONLY])
 def test_backward_f32_tiles(d_v, BH, L, flags):
     w = wl.Workload("bwd32", 1, BH, L, 16, d_v, "f32", 1.0)

@@ -109,6 +109,7 @@ struct BParams {
     float s1, s2;                // w = 1 + s * s1 + s^2 * s2 (1 / sqrt d', 1 / (2 d'))
     // block-wise path: pairs inside a block of W tokens by tiles, the other blocks through their summed state
     int W, nblk;
+    int heads, by_length;        // by_length: the longest loops of all heads first, else head by head
     int overlapped;              // forward: this grid runs beside the one before it, and ends after it
     const float* sv;             // [BH x nblk][160]: row sums of the block states (z, or the b-weighted sums of phi(q))
 };
@@ -233,8 +234,9 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? (DV == 64 && LT 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int ntiles = (p.L + kTile - 1) / kTile;
     // own tile: the longest loops first (dq, statistics: last query tiles; dk/dv: first key tiles)
-    const int own = MODE == kModeDkDv ? blockIdx.x : ntiles - 1 - blockIdx.x;
-    const int head = blockIdx.y;
+    const int turn = p.by_length ? blockIdx.x / p.heads : blockIdx.x % ntiles;
+    const int head = p.by_length ? blockIdx.x - turn * p.heads : blockIdx.x / ntiles;
+    const int own = MODE == kModeDkDv ? turn : ntiles - 1 - turn;
     const int r0 = own * kTile;
     // looped tiles (LT rows each): keys 0 .. end of the own tile, or queries from the own tile's first row on
     // block-wise path: the loop stays inside the own tile's block of W tokens; the blocks before it (queries) or
@@ -741,7 +743,7 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? (DV == 64 && LT 
     __syncthreads();
     if (warp == 4) tmem_dealloc(tb, C::kCols);
     // one CTA holds the grid's end back until the grid before it is complete: what follows in the stream sees both
-    if (MODE == kModeFwd && p.overlapped && blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && tid == 0)
+    if (MODE == kModeFwd && p.overlapped && blockIdx.x == gridDim.x - 1 && tid == 0)
         asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
@@ -808,22 +810,25 @@ based_status launch_pass(const CUtensorMap& n0, const CUtensorMap& w0, const CUt
 
 // Block length of the block-wise path, or 0 for the tile path alone.  The block-wise path needs d' = 16 and the
 // statistics in one sweep (the forward output, or the numerator-only form); its cost grows with L where the tile
-// path's grows with L^2, and the lengths below are where it starts to win on B200 (128 heads, d_v 64: 101 against
-// 117 us at L = 768; d_v 128: 191 against 213 us at L = 1024; 32 heads, d_v 128: 129 against 134 us at L = 1536).
-// Blocks of 256 tokens are the fastest from there on (B8 H16 L4096 d_v128: 613 / 582 / 661 us at 128 / 256 / 512),
-// except with few heads at d_v 128, where every block's state costs a CTA of its own.
-// A caller without the forward output gets it recomputed into the workspace first (one forward pass, 23 us at B4 H16
-// L2048 d_v64, 83 us at B8 H16 L4096 d_v128), from somewhat longer sequences on.
+// path's grows with L^2.  Tiles / blocks of 256 tokens on B200, us, around the lines below:
+//   128 heads: d_v 64 L 768 73 / 82, L 1024 112 / 105; d_v 128 L 768 106 / 109, L 1024 157 / 142
+//   16 heads: d_v 64 L 768 31 / 39, L 1024 39 / 39, L 1536 54 / 45; d_v 128 L 1280 50 / 59, L 1536 58 / 62, L 2048 79 / 63
+//   32 heads: d_v 64 L 1280 56 / 70, L 1536 69 / 74, L 2048 99 / 83; d_v 128 L 1536 84 / 105, L 2048 126 / 115
+// Below 64 heads one CTA per head and block sums the states, and a second short wave of those costs as much as a full one:
+// there the line lies later once the blocks are more than one wave (24 heads are not at L 1536: 62 / 48, 69 / 65).
+// With them at d_v 128 blocks of 512 tokens are the faster from 64 k rows on (256 / 512 tokens: 16 heads L 8192 217 / 206,
+// L 16384 403 / 381, 32 heads L 4096 216 / 202; 8 heads L 4096 64 / 79, L 8192 117 / 116; 2 heads L 16384 73 / 83).
+// A caller without the forward output gets it recomputed into the workspace first (one forward pass, 20 us at B4 H16
+// L2048 d_v64, 83 us at B8 H16 L4096 d_v128), from somewhat longer sequences on (64 heads and more: d_v 64 96 heads L 1024
+// 93 / 103, L 1280 130 / 125, d_v 128 64 heads L 1024 94 / 108, L 1280 131 / 134, 128 heads L 1280 256 / 202).
 int backward_block_len(int L, int df, bool merged, int d_v, int BH) {
     if (df != 16) return 0;
-    if (!merged) {
-        if (d_v == 64) return L >= 1024 ? 256 : 0;
-        if (BH >= 64) return L >= 1536 ? 256 : 0;
-        return L >= 4096 ? 512 : L >= 2048 ? 256 : 0;
-    }
-    if (d_v == 64) return L >= 768 ? 256 : 0;
-    if (BH >= 64) return L >= 1024 ? 256 : 0;
-    return L >= 4096 ? 512 : L >= 1536 ? 256 : 0;
+    int from;
+    if (BH >= 64) from = !merged ? 1280 : d_v == 64 ? 768 : 1024;
+    else if (BH * ((L + 255) / 256) > kSMs) from = 2048;
+    else from = d_v == 64 ? (merged ? 768 : 1024) : 1536;
+    if (L < from) return 0;
+    return BH < 64 && d_v != 64 && L >= 4096 && (long long)BH * L >= 65536 ? 512 : 256;
 }
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 struct BlockWs {
@@ -846,6 +851,13 @@ BlockWs block_ws(float* ws, int BH, int L, int dvr, int nblk) {
     w.bytes = off;
     return w;
 }
+
+// Tile passes: whether the longest loops of all heads start first, for an even end and long loops beside short ones on an SM.
+// Head by head the last heads' long loops start when the other SMs have run dry: the forward at B4 H16 L2048 d' 24 d_v 64 took
+// 50 us against 39, at B4 H16 L16384 d_v 128, where the looped tiles of all heads are 300 MB and do not stay in L2, 3609
+// against 3390; the backward at the first 230 against 187, at B2 H16 L1000 d_v 128 (256 CTAs) 63 against 49.  With a CTA or
+// less per SM there is nothing to even out: head by head 18.5 against 19.4 (B1 H8 L300, d' 16).
+int long_loops_first(int BH, int L) { return (long long)BH * ((L + kTile - 1) / kTile) > kSMs; }
 
 template <int DV>
 based_status launch_dvb(const void* q, const void* k, const void* v, const void* out, const void* g, void* dq, void* dk,
@@ -877,7 +889,9 @@ based_status launch_dvb(const void* q, const void* k, const void* v, const void*
     p.kdim = df <= 16 ? 16 : 32;
     p.s1 = 1.0f / sqrtf((float)df);
     p.s2 = 0.5f / (float)df;
-    const dim3 grid((L + kTile - 1) / kTile, BH);
+    const dim3 grid((unsigned)((L + kTile - 1) / kTile) * BH);
+    p.heads = BH;
+    p.by_length = long_loops_first(BH, L);
     based_status st;
     const int W = backward_block_len(L, df, out != nullptr || numerator_only, dvr, BH);
     if (W > 0) {
@@ -894,6 +908,7 @@ based_status launch_dvb(const void* q, const void* k, const void* v, const void*
             p.o_raw = w.out;
         }
         p.W = W;
+        p.by_length = 0;                             // loops of one length
         p.nblk = nblk;
         p.sv = w.sv;
         // With many heads one CTA per head walks the blocks and writes the running sums; with few, one CTA per head
@@ -944,8 +959,9 @@ based_status launch_dvb(const void* q, const void* k, const void* v, const void*
 // Forward of the definition form on the same tiles, for feature dimensions other than 16 (bf16 io,
 // empty initial state): out = (sum_j w_ij v_j) / (sum_j w_ij + eps), w = 1 + s/sqrt(d') + s^2/(2 d').
 // The weights lie over the scores, so at d_v 64 a CTA takes 128 columns of tensor memory and four share an SM, and tiles off
-// the diagonal evaluate two pairs per instruction: B4 H16 L2048 d_v64 80 -> 48 us (looped tiles of 128 rows: 47).  With the
-// state asked for it runs beside that kernel (80 + 61 us one after the other before, 48 + 40, together 74).
+// the diagonal evaluate two pairs per instruction: B4 H16 L2048 d_v64 80 -> 48 us (looped tiles of 128 rows: 47), 38 with the
+// longest loops first.  With the state asked for it runs beside that kernel (38 + 40 us alone, together 64; 80 + 61 one after
+// the other before).
 based_status launch_quadratic_forward_tc(const void* q, const void* k, const void* v, void* out, int BH, int L,
                                          int d_feat, int d_v, int numerator_only, bool overlapped, cudaStream_t stream) {
     CUtensorMap tq, tk64, tv64, tout;
@@ -964,7 +980,9 @@ based_status launch_quadratic_forward_tc(const void* q, const void* k, const voi
     p.kdim = d_feat <= 16 ? 16 : 32;
     p.s1 = 1.0f / sqrtf((float)d_feat);
     p.s2 = 0.5f / (float)d_feat;
-    const dim3 grid((L + kTile - 1) / kTile, BH);
+    const dim3 grid((unsigned)((L + kTile - 1) / kTile) * BH);
+    p.heads = BH;
+    p.by_length = long_loops_first(BH, L);
     if (d_v == 64) return launch_pass<64, kModeFwd, 64>(tq, tq, tk64, tv64, p, grid, "quadratic forward (tc)", stream, nullptr, &tout);
     return launch_pass<128, kModeFwd, 64>(tq, tq, tk64, tv64, p, grid, "quadratic forward (tc)", stream, nullptr, &tout);
 }

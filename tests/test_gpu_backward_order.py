@@ -44,7 +44,8 @@ def test_tile_passes_in_either_order(d_feat, d_v, BH, L, with_out):
 
 
 @pytest.mark.parametrize("d_v,BH,L,tokens", [(64, 19, 2047, 0), (64, 19, 2048, 256), (64, 18, 2000, 256), (128, 63, 2047, 0),
-                                             (112, 24, 2049, 256), (128, 16, 4096, 512), (128, 15, 4100, 256)])
+                                             (112, 24, 2049, 256), (128, 16, 4096, 512), (128, 15, 4100, 256),
+                                             (64, 74, 800, 256), (64, 75, 1281, 256), (112, 74, 1100, 256), (128, 75, 1024, 256)])
 def test_lines_of_the_blockwise_path(d_v, BH, L, tokens):
     assert based.lib().based_prefill_backward_block_tokens(1, BH, L, 16, d_v, 1, 0, 1) == tokens
     _check(*_inputs(BH, L, 16, d_v), True)

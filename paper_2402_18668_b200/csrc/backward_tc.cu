@@ -152,9 +152,11 @@ __device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
     return r;
 }
-// w = 1 + s / sqrt(d') + s^2 / (2 d') and its derivative, s1 = 1 / sqrt(d'), s2 = 1 / (2 d') (d' = 16: 1/4, 1/32)
-__device__ __forceinline__ float tw(float s, float s1, float s2) { return fmaf(s, fmaf(s, s2, s1), 1.0f); }
-__device__ __forceinline__ float tdw(float s, float s1, float s2) { return fmaf(s, 2.0f * s2, s1); }
+__device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
 
 // Block-wise path, one row thread: T (160 fp32 columns of tensor memory, from column 0) holds the product of the
 // row's wide operand with a block state in the monomial basis of block_state_tc_kernel
@@ -163,50 +165,93 @@ __device__ __forceinline__ float tdw(float s, float s1, float s2) { return fmaf(
 //     den += mono(q_i) . z,  en += mono(q_i) . T,  gx = J^T (T - m_i z),  gy = J^T z      (J = d mono / d q_i)
 //   key row (dk/dv pass): T_f = (R v_j)_f, sv = R_b:  gx = J^T (T + R_b); the monomials of k_j go back to tensor
 //     memory as packed bf16 (80 columns from column 0, over the columns already read): the A operand of dV += mono(K) R
+// Two features per instruction: f, f + 1 (f even) are x_m x_n and x_(m+1) x_(n+1), m even; where n is odd the pair's second
+// factors and the sums that go to them lie across two words, in arrays of their own (xo; gxo, gyo).
 template <bool KEYS>
 __device__ __forceinline__ void block_rows(uint32_t tb, uint32_t lane_base, const float (&x)[16], const float* sv,
                                            float m_own, float& den, float& en, float (&gx)[16], float (&gy)[16]) {
+    uint64_t xe[8], xo[8], gxe[8], gxo[8], gye[8], gyo[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        xe[i] = f32x2(x[2 * i], x[2 * i + 1]);
+        xo[i] = f32x2(x[2 * i + 1], x[(2 * i + 2) & 15]);
+        gxe[i] = gxo[i] = gye[i] = gyo[i] = 0;
+    }
+    const uint64_t negm = f32x2(-m_own, -m_own);
+    uint64_t den2 = f32x2(den, 0.f), en2 = f32x2(en, 0.f);
 #pragma unroll
     for (int blk = 0; blk < 5; ++blk) {
-        uint32_t tr[32];
+        uint32_t tr[32], pk[16];
         tmem_ld32(tmem_addr(tb, lane_base, blk * 32), tr);
         tmem_wait_ld();
-        float mono[32];
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-            const int f = blk * 32 + i;
-            const int m = f < 16 ? f : f < 144 ? ((f - 16) & 15) : f < 152 ? f - 144 : -1;
-            const int n = f < 16 ? -1 : f < 144 ? ((m + ((f - 16) >> 4)) & 15) : f < 152 ? m + 8 : -1;
-            mono[i] = 0.f;
-            if (f <= 152) {
-                const float xm = m >= 0 ? x[m] : 1.0f, xn = n >= 0 ? x[n] : 1.0f;
-                mono[i] = xm * xn;
-                const float a = __uint_as_float(tr[i]), zf = sv[f];
-                const float bq = KEYS ? a + zf : fmaf(-m_own, zf, a);
-                if (!KEYS) {
-                    den = fmaf(mono[i], zf, den);
-                    en = fmaf(mono[i], a, en);
+        for (int i = 0; i < 16; ++i) {
+            const int f = blk * 32 + 2 * i;
+            const int m = f < 16 ? f : f < 144 ? ((f - 16) & 15) : f - 144;
+            const int n = f < 16 ? -1 : f < 144 ? ((m + ((f - 16) >> 4)) & 15) : m + 8;
+            if (KEYS) pk[i] = 0u;
+            if (f > 152) continue;
+            const ulonglong2 z4 = *reinterpret_cast<const ulonglong2*>(sv + (f & ~3));       // broadcast: four row sums
+            const uint64_t z = f & 2 ? z4.y : z4.x;
+            const uint64_t a = f32x2(__uint_as_float(tr[2 * i]), __uint_as_float(tr[2 * i + 1]));
+            if (f == 152) {                                  // the constant
+                float z0, z1;
+                split_f32x2(z, z0, z1);
+                if (KEYS) pk[i] = pack_bf16x2(1.0f, 0.f);
+                else {
+                    den2 = add_f32x2(den2, f32x2(z0, 0.f));
+                    en2 = add_f32x2(en2, f32x2(__uint_as_float(tr[2 * i]), 0.f));
                 }
-                if (m >= 0 && n < 0) {
-                    gx[m] += bq;
-                    if (!KEYS) gy[m] += zf;
-                } else if (m >= 0 && m != n) {
-                    gx[m] = fmaf(xn, bq, gx[m]);
-                    gx[n] = fmaf(xm, bq, gx[n]);
-                    if (!KEYS) { gy[m] = fmaf(xn, zf, gy[m]); gy[n] = fmaf(xm, zf, gy[n]); }
-                } else if (m >= 0) {
-                    gx[m] = fmaf(2.0f * xm, bq, gx[m]);
-                    if (!KEYS) gy[m] = fmaf(2.0f * xm, zf, gy[m]);
+                continue;
+            }
+            const uint64_t xm = xe[m / 2], xn = n < 0 ? 0 : n & 1 ? xo[n / 2] : xe[n / 2];
+            const uint64_t mono = n < 0 ? xm : mul_f32x2(xm, xn);
+            const uint64_t bq = KEYS ? add_f32x2(a, z) : fma_f32x2(negm, z, a);
+            if (KEYS) {
+                float lo, hi;
+                split_f32x2(mono, lo, hi);
+                pk[i] = pack_bf16x2(lo, hi);
+            } else {
+                den2 = fma_f32x2(mono, z, den2);
+                en2 = fma_f32x2(mono, a, en2);
+            }
+            uint64_t& gm = gxe[m / 2];
+            uint64_t& hm = gye[m / 2];
+            if (n < 0) {
+                gm = add_f32x2(gm, bq);
+                if (!KEYS) hm = add_f32x2(hm, z);
+            } else {                                         // (m = n: both terms)
+                uint64_t& gn = n & 1 ? gxo[n / 2] : gxe[n / 2];
+                uint64_t& hn = n & 1 ? gyo[n / 2] : gye[n / 2];
+                gm = fma_f32x2(xn, bq, gm);
+                gn = fma_f32x2(xm, bq, gn);
+                if (!KEYS) {
+                    hm = fma_f32x2(xn, z, hm);
+                    hn = fma_f32x2(xm, z, hn);
                 }
             }
         }
-        if (KEYS) {
-            uint32_t pk[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) pk[i] = pack_bf16x2(mono[2 * i], mono[2 * i + 1]);
-            tmem_st16(tmem_addr(tb, lane_base, blk * 16), pk);
-        }
+        if (KEYS) tmem_st16(tmem_addr(tb, lane_base, blk * 16), pk);
     }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        float a, b, c, d;
+        split_f32x2(gxe[i], a, b);
+        split_f32x2(gxo[(i + 7) & 7], c, d);                 // .. 2 i - 1, 2 i
+        gx[2 * i] = a + d;
+        split_f32x2(gxo[i], c, d);
+        gx[2 * i + 1] = b + c;
+        split_f32x2(gye[i], a, b);
+        split_f32x2(gyo[(i + 7) & 7], c, d);
+        gy[2 * i] = a + d;
+        split_f32x2(gyo[i], c, d);
+        gy[2 * i + 1] = b + c;
+    }
+    float a, b;
+    split_f32x2(den2, a, b);
+    den = a + b;
+    split_f32x2(en2, a, b);
+    en = a + b;
 }
 }  // namespace
 
@@ -227,7 +272,7 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? (DV == 64 && LT 
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::offMisc);
     uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(bars + bNum);
     volatile uint32_t* abort_flag = tmem_base_s + 1;
-    float2* s_b = reinterpret_cast<float2*>(smem + C::offB);
+    float* s_b = reinterpret_cast<float*>(smem + C::offB);
     float* s_sv = reinterpret_cast<float*>(smem + C::offMisc + 256);
     float* s_m = reinterpret_cast<float*>(smem + C::offMisc + 1024);
 
@@ -533,8 +578,6 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? (DV == 64 && LT 
                         x[c * 8 + 2 * i + 1] = fv.y;
                     }
                 }
-#pragma unroll
-                for (int i = 0; i < 16; ++i) { gx[i] = 0.f; gy[i] = 0.f; }
                 block_rows<MODE == kModeDkDv>(tb, lane_base, x, s_sv, m_own, den, en, gx, gy);
                 // the sums start the accumulators that the loop's products add to: X and Y, or dK
                 uint32_t o[16], zero[16];
@@ -553,100 +596,111 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? (DV == 64 && LT 
                 mbar_arrive(&bars[bX1]);
             }
         }
+        const uint64_t k1 = f32x2(p.s1, p.s1), k2 = f32x2(p.s2, p.s2), k22 = f32x2(2.0f * p.s2, 2.0f * p.s2), one = f32x2(1.f, 1.f);
+        const uint64_t negm = f32x2(-m_own, -m_own), own_d = f32x2(st_own.x, st_own.x), own_b = f32x2(st_own.y, st_own.y);
+        uint64_t den2 = f32x2(den, 0.f), en2 = f32x2(en, 0.f);
+        // the packed tiles of 32 columns, in place of columns already read
+        auto packed_out = [&](int blk, const uint32_t (&pw)[16], const uint32_t (&pd)[16]) {
+            if (MODE == kModeDq || MODE == kModeDqS) tmem_st16(tmem_addr(tb, lane_base, C::colD + blk * 16), pd);
+            if (MODE == kModeDqS) tmem_st16(tmem_addr(tb, lane_base, C::colD2 + blk * 16), pw);
+            if (MODE == kModeFwd) tmem_st16(tmem_addr(tb, lane_base, C::colD + blk * 16), pw);
+            if (MODE == kModeDkDv) {
+                tmem_st16(tmem_addr(tb, lane_base, C::colS + blk * 16), pw);
+                tmem_st16(tmem_addr(tb, lane_base, C::colG + blk * 16), pd);
+            }
+        };
         for (int it = 0; it < nloop && ok; ++it) {
             const int c0 = (first + it) * LT;                // first row of the looped tile (columns of the accumulators)
-            if (MODE == kModeDkDv && t < LT)                 // (1/D, b) of the looped queries
-                s_b[(it & 1) * LT + t] = c0 + t < p.L ? p.stats_in[(size_t)head * p.L + c0 + t] : make_float2(0.f, 0.f);
+            if (MODE == kModeDkDv && t < LT) {               // 1/D and b of the looped queries
+                const float2 st = c0 + t < p.L ? p.stats_in[(size_t)head * p.L + c0 + t] : make_float2(0.f, 0.f);
+                s_b[(it & 1) * 2 * LT + t] = st.x;
+                s_b[(it & 1) * 2 * LT + LT + t] = st.y;
+            }
             ok = rows_all(mbar_wait(&bars[bMma], it & 1, abort_flag));
             if (!ok) break;
             tc_fence_after();
-            // one pass over the tile's LT accumulator columns of this row; MASKED: the tile touches the
-            // diagonal or the end of the sequence (the others need no per-pair test)
-            auto pass = [&](auto masked_tag) {
+            // one pass over the tile's LT accumulator columns of this row, 32 at a time and two pairs per instruction.  The
+            // warp's 32 rows meet 32 columns on one of three ways: all pairs live, none (zeros, nothing read), or some
+            // (MASKED: on the diagonal or at the end of the sequence).
+            auto pass = [&](auto masked_tag, int blk) {
                 constexpr bool MASKED = decltype(masked_tag)::value;
-                if constexpr (MODE == kModeFwd && !MASKED) {
-                    // two pairs per instruction: w = 1 + s (s1 + s s2), its sum, and the packed weight
-                    const uint64_t k2 = f32x2(p.s2, p.s2), k1 = f32x2(p.s1, p.s1), one = f32x2(1.f, 1.f);
-                    uint64_t d0 = f32x2(den, 0.f), d1 = 0;
+                uint32_t sr[32], gr[32];
+                tmem_ld32(tmem_addr(tb, lane_base, C::colS + blk * 32), sr);
+                if (MODE != kModeFwd) tmem_ld32(tmem_addr(tb, lane_base, C::colG + blk * 32), gr);
+                tmem_wait_ld();
+                uint32_t pw[16], pd[16];
 #pragma unroll
-                    for (int blk = 0; blk < LT / 32; ++blk) {
-                        uint32_t sr[32], pw[16];
-                        tmem_ld32(tmem_addr(tb, lane_base, C::colS + blk * 32), sr);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) {
-                            const uint64_t s2v = f32x2(__uint_as_float(sr[2 * i]), __uint_as_float(sr[2 * i + 1]));
-                            const uint64_t w = fma_f32x2(s2v, fma_f32x2(s2v, k2, k1), one);
-                            if (i & 1) d1 = add_f32x2(d1, w);
-                            else d0 = add_f32x2(d0, w);
-                            float lo, hi;
-                            split_f32x2(w, lo, hi);
-                            pw[i] = pack_bf16x2(lo, hi);
-                        }
-                        tmem_st16(tmem_addr(tb, lane_base, C::colD + blk * 16), pw);
+                for (int i = 0; i < 16; ++i) {
+                    const uint64_t sv = f32x2(__uint_as_float(sr[2 * i]), __uint_as_float(sr[2 * i + 1]));
+                    const uint64_t gv = MODE == kModeFwd ? 0 : f32x2(__uint_as_float(gr[2 * i]), __uint_as_float(gr[2 * i + 1]));
+                    // pair (query, key): own row is the query except in the dk/dv pass
+                    bool live0 = true, live1 = true;
+                    if (MASKED) {
+                        const int col = c0 + blk * 32 + 2 * i;
+                        live0 = MODE == kModeDkDv ? (row <= col && col < p.L) : col <= row;
+                        live1 = MODE == kModeDkDv ? (row <= col + 1 && col + 1 < p.L) : col + 1 <= row;
                     }
-                    float a, b;
-                    split_f32x2(add_f32x2(d0, d1), a, b);
-                    den = a + b;
-                    return;
-                }
-#pragma unroll 1
-                for (int blk = 0; blk < LT / 32; ++blk) {
-                    uint32_t sr[32], gr[32];
-                    tmem_ld32(tmem_addr(tb, lane_base, C::colS + blk * 32), sr);
-                    if (MODE != kModeFwd) tmem_ld32(tmem_addr(tb, lane_base, C::colG + blk * 32), gr);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) {
-                        const int col = c0 + blk * 32 + i;
-                        const float s = __uint_as_float(sr[i]), gvv = MODE == kModeFwd ? 0.f : __uint_as_float(gr[i]);
-                        // pair (query, key): own row is the query except in the dk/dv pass
-                        const bool live = !MASKED || (MODE == kModeDkDv ? (row <= col && col < p.L) : (col <= row));
-                        float w = live ? tw(s, p.s1, p.s2) : 0.f;
-                        float ds = 0.f;
-                        if (MODE == kModeFwd) {
-                            den += w;
-                        } else if (MODE == kModeStats) {
-                            den += w;
-                            en = fmaf(w, gvv, en);
-                        } else if (MODE == kModeDqS) {
-                            den += w;
-                            en = fmaf(w, gvv, en);
-                            w = live ? tdw(s, p.s1, p.s2) : 0.f;         // second tile: w'
-                            ds = w * (gvv - m_own);          // first tile: w' (gv - m)
-                        } else {
-                            const float2 stq = MODE == kModeDq ? st_own : s_b[(it & 1) * LT + blk * 32 + i];
-                            ds = live ? fmaf(gvv, stq.x, stq.y) * tdw(s, p.s1, p.s2) : 0.f;
-                            w *= stq.x;                      // dv_j = sum_i (w_ij / D_i) G_i
-                        }
-                        sr[i] = __float_as_uint(w);
-                        gr[i] = __float_as_uint(ds);
-                    }
-                    uint32_t pw[16], pd[16];
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        pw[i] = pack_bf16x2(__uint_as_float(sr[2 * i]), __uint_as_float(sr[2 * i + 1]));
-                        pd[i] = pack_bf16x2(__uint_as_float(gr[2 * i]), __uint_as_float(gr[2 * i + 1]));
-                    }
-                    if (MODE == kModeDq) tmem_st16(tmem_addr(tb, lane_base, C::colD + blk * 16), pd);
+                    auto masked = [&](uint64_t v) {
+                        if (!MASKED) return v;
+                        float lo, hi;
+                        split_f32x2(v, lo, hi);
+                        return f32x2(live0 ? lo : 0.f, live1 ? hi : 0.f);
+                    };
+                    // w = 1 + s / sqrt(d') + s^2 / (2 d') and its derivative
+                    uint64_t w = 0, dw = 0, ds = 0;
+                    if (MODE != kModeDq) w = masked(fma_f32x2(sv, fma_f32x2(sv, k2, k1), one));
+                    if (MODE == kModeDq || MODE == kModeDqS || MODE == kModeDkDv) dw = masked(fma_f32x2(sv, k22, k1));
+                    if (MODE == kModeFwd || MODE == kModeStats || MODE == kModeDqS) den2 = add_f32x2(den2, w);
+                    if (MODE == kModeStats || MODE == kModeDqS) en2 = fma_f32x2(w, gv, en2);
                     if (MODE == kModeDqS) {
-                        tmem_st16(tmem_addr(tb, lane_base, C::colD + blk * 16), pd);
-                        tmem_st16(tmem_addr(tb, lane_base, C::colD2 + blk * 16), pw);
+                        ds = mul_f32x2(dw, add_f32x2(gv, negm));             // first tile: w' (gv - m); second: w'
+                        w = dw;
                     }
-                    if (MODE == kModeFwd) tmem_st16(tmem_addr(tb, lane_base, C::colD + blk * 16), pw);
+                    if (MODE == kModeDq) ds = mul_f32x2(fma_f32x2(gv, own_d, own_b), dw);
                     if (MODE == kModeDkDv) {
-                        tmem_st16(tmem_addr(tb, lane_base, C::colS + blk * 16), pw);   // in place: columns already read
-                        tmem_st16(tmem_addr(tb, lane_base, C::colG + blk * 16), pd);
+                        const int c = (it & 1) * 2 * LT + blk * 32 + 2 * i;
+                        const uint64_t qd = *reinterpret_cast<const uint64_t*>(s_b + c);
+                        ds = mul_f32x2(fma_f32x2(gv, qd, *reinterpret_cast<const uint64_t*>(s_b + LT + c)), dw);
+                        w = mul_f32x2(w, qd);                // dv_j = sum_i (w_ij / D_i) G_i
                     }
+                    float lo, hi;
+                    split_f32x2(w, lo, hi);
+                    pw[i] = pack_bf16x2(lo, hi);
+                    split_f32x2(ds, lo, hi);
+                    pd[i] = pack_bf16x2(lo, hi);
                 }
+                packed_out(blk, pw, pd);
             };
-            // uniform over the CTA: every pair of the tile is live
-            const bool all_live = MODE == kModeDkDv ? (r0 + kTile - 1 <= c0 && c0 + LT <= p.L) : (c0 + LT - 1 <= r0);
-            if (all_live) pass(std::false_type{});
-            else pass(std::true_type{});
+            if (MODE == kModeFwd && c0 + LT <= r0) {         // two column groups in flight (63 -> 60 us at B4 H16 L2048 d_v 128)
+#pragma unroll
+                for (int blk = 0; blk < LT / 32; ++blk) pass(std::false_type{}, blk);
+            } else
+#pragma unroll 1
+            for (int blk = 0; blk < LT / 32; ++blk) {
+                const int cb = c0 + blk * 32, rw = r0 + warp * 32;
+                const bool dead = MODE == kModeDkDv ? cb < rw : cb > rw;
+                const bool some = cb == rw || (MODE == kModeDkDv && cb + 32 > p.L);
+                if (dead) {
+                    uint32_t z[16];
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) z[i] = 0u;
+                    packed_out(blk, z, z);
+                } else if (some) {
+                    pass(std::true_type{}, blk);
+                } else {
+                    pass(std::false_type{}, blk);
+                }
+            }
             if (MODE != kModeStats) tmem_wait_st();
             tc_fence_before();
             mbar_arrive(&bars[bAlu]);
+        }
+        {
+            float a, b;
+            split_f32x2(den2, a, b);
+            den = a + b;
+            split_f32x2(en2, a, b);
+            en = a + b;
         }
         if (MODE != kModeStats) ok = rows_all(ok && mbar_wait(&bars[bFinal], 0, abort_flag));
         tc_fence_after();

@@ -11,7 +11,7 @@ from parity import TOL_BF16, assert_state_close, row_err
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("d_feat,d_v", [(8, 64), (24, 64), (24, 112), (32, 128)])
+@pytest.mark.parametrize("d_feat,d_v", [(8, 64), (24, 64), (24, 112), (32, 128), (32, 64), (8, 128)])
 @pytest.mark.parametrize("BH,L", [(1, 1), (3, 64), (2, 129), (5, 300), (200, 193), (64, 1500)])
 def test_outputs_and_state_side_by_side(d_feat, d_v, BH, L):
     w = wl.Workload("beside", 1, BH, L, d_feat, d_v, "bf16", 0.5, decode_steps=1)

@@ -62,14 +62,20 @@ template <int DV, int MODE, int LT, bool XB = false> struct BCfg {
     static constexpr int kVB = (DV + 63) / 64;           // 64-column blocks of a [rows][DV] tile (112 -> 2, second partly zero)
     static constexpr uint32_t kWide = kVB * kTile * 128; // own tile: [128][64 * kVB] bf16 in SWIZZLE_128B blocks
     static constexpr uint32_t kNarrowL = LT * 64, kWideL = kVB * LT * 128;       // looped tiles
-    // shared memory: resident narrow + wide tile, two stages of (narrow + wide), (1/D, b) of two stages, barriers
+    // shared memory: resident narrow + wide tile, stages of (narrow + wide), (1/D, b) of two stages, barriers
     static constexpr uint32_t offResN = 0, offResW = offResN + kQKTile;
+    // The next tile's scores are issued as soon as this tile's are read, where tensor memory holds the packed tiles beside the
+    // scores: B2 H16 L1000 d_v 128 46.5 -> 44.5 us, B1 H8 L300 d_v 64 16.8 -> 16.3 per backward call.  Not where it takes
+    // looped tiles of 32 rows (dk/dv at d_v 64: 31 -> 35 at B2 H8 L700, the own tile is read from shared memory twice as often)
+    // or of 64 for 128 (dk/dv at d_v 128: 44 -> 54), and not where loops are two to four tiles (block-wise: no gain).
+    static constexpr bool kEarly = !XB && MODE != kModeFwd && MODE != kModeDkDv;
+    static constexpr int kNSt = kEarly ? 3 : 2;          // stages
     static constexpr uint32_t offStage = offResW + kWide, kStage = kNarrowL + kWideL;
     // a block state, transposed: [64 * kVB value columns][160 features] bf16 in five SWIZZLE_64B blocks of 32 features
     // (block-wise path); it lies from the second stage on, so that the first looped tile loads beside it
     static constexpr uint32_t kStateBlk = kVB * 64 * 64;
     static constexpr uint32_t kStateTile = 5 * kStateBlk;
-    static constexpr uint32_t kStageArea = (XB && kStage + kStateTile > 2 * kStage) ? kStage + kStateTile : 2 * kStage;
+    static constexpr uint32_t kStageArea = (XB && kStage + kStateTile > kNSt * kStage) ? kStage + kStateTile : kNSt * kStage;
     static constexpr uint32_t offB = offStage + kStageArea;
     static constexpr uint32_t offMisc = offB + 2 * LT * 8;
     static constexpr uint32_t kSmem = offMisc + 2048 + 1024;                    // barriers, the block state's row sums (160 floats), m (128)
@@ -93,7 +99,7 @@ template <int DV, int MODE, int LT, bool XB = false> struct BCfg {
     static constexpr uint32_t kCols = kColsUsed <= 128 ? 128 : kColsUsed <= 256 ? 256 : 512;
     static_assert(kColsUsed <= 512, "tensor memory budget");
 };
-enum { bRes = 0, bFull0, bFull1, bMma, bAlu, bFinal, bXs, bX0, bX1, bNum };
+enum { bRes = 0, bFull0, bFull1, bFull2, bMma, bRead, bAlu, bAcc, bFinal, bXs, bX0, bX1, bNum };
 
 struct BParams {
     const __nv_bfloat16* g_raw;  // dout and the forward output as plain pointers [BH, L, dvw] (merged pass)
@@ -293,8 +299,9 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? (DV == 64 && LT 
     const int nloop = last - first + 1;
 
     if (tid == 0) {
-        mbar_init(&bars[bRes], 1); mbar_init(&bars[bFull0], 1); mbar_init(&bars[bFull1], 1);
-        mbar_init(&bars[bMma], 1); mbar_init(&bars[bAlu], 128); mbar_init(&bars[bFinal], 1);
+        mbar_init(&bars[bRes], 1); mbar_init(&bars[bFull0], 1); mbar_init(&bars[bFull1], 1); mbar_init(&bars[bFull2], 1);
+        mbar_init(&bars[bMma], 1); mbar_init(&bars[bRead], 128); mbar_init(&bars[bAlu], 128);
+        mbar_init(&bars[bAcc], 1); mbar_init(&bars[bFinal], 1);
         mbar_init(&bars[bXs], 1); mbar_init(&bars[bX0], 1); mbar_init(&bars[bX1], 128);
         *abort_flag = 0;
         fence_mbar_init();
@@ -323,8 +330,8 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? (DV == 64 && LT 
             const uint32_t lead = elect_one();
             const uint32_t aResN = smem_u32(smem + C::offResN), aResW = smem_u32(smem + C::offResW);
             auto load_stage = [&](int it) {
-                if (!lead) return;
-                const int s = it & 1;
+                if (!lead || it >= nloop) return;
+                const int s = it % C::kNSt;
                 uint8_t* st = smem + C::offStage + s * C::kStage;
                 const int row = (first + it) * LT;
                 mbar_arrive_expect_tx(&bars[bFull0 + s], C::kStage);
@@ -349,7 +356,7 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? (DV == 64 && LT 
                                 head * p.nblk + blk);
             }
             }
-            load_stage(0);
+            for (int i = 0; i < (cross ? 1 : C::kNSt); ++i) load_stage(i);     // (the block state lies over the others)
             ok = mbar_wait(&bars[bRes], 0, abort_flag);
             if (cross && ok) {
                 const uint32_t aSt = smem_u32(smem + C::offStage + C::kStage);
@@ -387,15 +394,12 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? (DV == 64 && LT 
                     if (ok) ok = mbar_wait(&bars[bX1], 0, abort_flag);     // the rows have read T: the scores may overwrite it
                     tc_fence_after();
                 }
-                // the state tile's stages are loaded again after the first iteration's products (in-order pipe)
             }
-            for (int it = 0; it < nloop && ok; ++it) {
-                const int s = it & 1;
-                const uint32_t aN = smem_u32(smem + C::offStage + s * C::kStage), aW = aN + C::kNarrowL;
-                ok = mbar_wait(&bars[bFull0 + s], (it >> 1) & 1, abort_flag);
-                if (!ok) break;
+            // scores and dout.v products of a looped tile: rows = own tile, columns = looped tile
+            auto scores = [&](int it) -> bool {
+                const uint32_t aN = smem_u32(smem + C::offStage + (it % C::kNSt) * C::kStage), aW = aN + C::kNarrowL;
+                if (!mbar_wait(&bars[bFull0 + it % C::kNSt], (it / C::kNSt) & 1, abort_flag)) return false;
                 tc_fence_after();
-                // scores: rows = own tile, columns = looped tile
                 mma_ss_w<false>(lead, tb + C::colS, desc_lo(dN) + (aResN >> 4), desc_hi(dN), desc_lo(dN) + (aN >> 4),
                                  desc_hi(dN), iS);
                 if (p.kdim > 16)                             // feature dimensions 24 and 32: second K-step
@@ -414,10 +418,28 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? (DV == 64 && LT 
                                         desc_lo(dWL) + (aW >> 4) + offL, desc_hi(dWL), iS);
                 }
                 mma_commit_w(lead, &bars[bMma]);
-                // once these products are done, so are the previous iteration's (in-order pipe): its stage is free
-                ok = mbar_wait(&bars[bMma], it & 1, abort_flag);
-                if (!ok) break;
-                if (it + 1 < nloop) load_stage(it + 1);
+                return true;
+            };
+            if (C::kEarly && ok) ok = scores(0);
+            for (int it = 0; it < nloop && ok; ++it) {
+                const int s = it % C::kNSt;
+                const uint32_t aN = smem_u32(smem + C::offStage + s * C::kStage), aW = aN + C::kNarrowL;
+                if (!C::kEarly) {
+                    // once these products are done, so are the previous iteration's (in-order pipe): its stage is free, and
+                    // after the first one's those that the block state lay over
+                    ok = scores(it) && mbar_wait(&bars[bMma], it & 1, abort_flag);
+                    if (!ok) break;
+                    if (it > 0 || cross) load_stage(it + 1);
+                } else {
+                    // the rows have read this tile's scores: the next tile's are formed while they work on them
+                    if (it + 1 < nloop) ok = mbar_wait(&bars[bRead], it & 1, abort_flag) && scores(it + 1);
+                    // the stage of the tile before is free once its last products are done (statistics: its scores, which the
+                    // rows have read)
+                    if (it > 0 && ok) ok = MODE == kModeStats || mbar_wait(&bars[bAcc], (it - 1) & 1, abort_flag);
+                    if (!ok) break;
+                    if (it > 0) load_stage(it - 1 + C::kNSt);
+                }
+                if (MODE == kModeStats) continue;
                 ok = mbar_wait(&bars[bAlu], it & 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
@@ -476,6 +498,7 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? (DV == 64 && LT 
                         }
                     }
                 }
+                if (C::kEarly) mma_commit_w(lead, &bars[bAcc]);
             }
             if (ok) mma_commit_w(lead, &bars[bFinal]);
         }
@@ -609,6 +632,14 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? (DV == 64 && LT 
                 tmem_st16(tmem_addr(tb, lane_base, C::colG + blk * 16), pd);
             }
         };
+        // after the tile's last tensor-memory load: the next tile's scores may overwrite these
+        auto have_read = [&](int blk) {
+            if (C::kEarly && blk == LT / 32 - 1) {
+                tc_fence_before();
+                mbar_arrive(&bars[bRead]);
+            }
+        };
+        bool packed_ok = true;
         for (int it = 0; it < nloop && ok; ++it) {
             const int c0 = (first + it) * LT;                // first row of the looped tile (columns of the accumulators)
             if (MODE == kModeDkDv && t < LT) {               // 1/D and b of the looped queries
@@ -616,9 +647,16 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? (DV == 64 && LT 
                 s_b[(it & 1) * 2 * LT + t] = st.x;
                 s_b[(it & 1) * 2 * LT + LT + t] = st.y;
             }
-            ok = rows_all(mbar_wait(&bars[bMma], it & 1, abort_flag));
+            ok = rows_all(packed_ok && mbar_wait(&bars[bMma], it & 1, abort_flag));
             if (!ok) break;
             tc_fence_after();
+            // the packed tiles are free once the products of the tile before are done
+            auto may_pack = [&]() {
+                if (C::kEarly && MODE != kModeStats && it > 0) {
+                    packed_ok = __all_sync(~0u, mbar_wait(&bars[bAcc], (it - 1) & 1, abort_flag)) && packed_ok;
+                    tc_fence_after();
+                }
+            };
             // one pass over the tile's LT accumulator columns of this row, 32 at a time and two pairs per instruction.  The
             // warp's 32 rows meet 32 columns on one of three ways: all pairs live, none (zeros, nothing read), or some
             // (MASKED: on the diagonal or at the end of the sequence).
@@ -628,6 +666,7 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? (DV == 64 && LT 
                 tmem_ld32(tmem_addr(tb, lane_base, C::colS + blk * 32), sr);
                 if (MODE != kModeFwd) tmem_ld32(tmem_addr(tb, lane_base, C::colG + blk * 32), gr);
                 tmem_wait_ld();
+                have_read(blk);
                 uint32_t pw[16], pd[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i) {
@@ -669,6 +708,7 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? (DV == 64 && LT 
                     split_f32x2(ds, lo, hi);
                     pd[i] = pack_bf16x2(lo, hi);
                 }
+                if (blk == 0) may_pack();
                 packed_out(blk, pw, pd);
             };
             if (MODE == kModeFwd && c0 + LT <= r0) {         // two column groups in flight (63 -> 60 us at B4 H16 L2048 d_v 128)
@@ -684,6 +724,8 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? (DV == 64 && LT 
                     uint32_t z[16];
 #pragma unroll
                     for (int i = 0; i < 16; ++i) z[i] = 0u;
+                    have_read(blk);
+                    if (blk == 0) may_pack();
                     packed_out(blk, z, z);
                 } else if (some) {
                     pass(std::true_type{}, blk);
@@ -691,9 +733,11 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? (DV == 64 && LT 
                     pass(std::false_type{}, blk);
                 }
             }
-            if (MODE != kModeStats) tmem_wait_st();
-            tc_fence_before();
-            mbar_arrive(&bars[bAlu]);
+            if (MODE != kModeStats) {
+                tmem_wait_st();
+                tc_fence_before();
+                mbar_arrive(&bars[bAlu]);
+            }
         }
         {
             float a, b;
@@ -702,7 +746,7 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? (DV == 64 && LT 
             split_f32x2(en2, a, b);
             en = a + b;
         }
-        if (MODE != kModeStats) ok = rows_all(ok && mbar_wait(&bars[bFinal], 0, abort_flag));
+        if (MODE != kModeStats) ok = rows_all(ok && packed_ok && mbar_wait(&bars[bFinal], 0, abort_flag));
         tc_fence_after();
         // tcgen05.ld is a warp-collective: every lane takes part, only the stores depend on the row
         const bool store = ok && row < p.L;

@@ -266,7 +266,7 @@ __device__ __forceinline__ void block_rows(uint32_t tb, uint32_t lane_base, cons
 // XB: the block-wise path (merged statistics + dq pass and dk/dv pass, d' = 16); tm_st: the block states,
 // transposed: [BH x nblk][d_v][160] bf16.  tm_out: the wide output (dv, or the forward output), stored by TMA.
 template <int DV, int MODE, int LT, bool XB>
-__global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? (DV == 64 && LT == 64 ? 4 : 2) : 1)
+__global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd && DV == 64 && LT == 64 ? 4 : 2)
     backward_tc_kernel(const __grid_constant__ CUtensorMap tm_n0, const __grid_constant__ CUtensorMap tm_w0,
                        const __grid_constant__ CUtensorMap tm_n1, const __grid_constant__ CUtensorMap tm_w1,
                        const __grid_constant__ CUtensorMap tm_st, const __grid_constant__ CUtensorMap tm_out,
@@ -536,23 +536,37 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? (DV == 64 && LT 
             }
             ok = rows_all(mbar_wait(&bars[bRes], 0, abort_flag));
 #pragma unroll
-            for (int i = 0; i < NI; ++i) {
-                const int pc = i * 32 + lane;
-                const int rr = warp * 32 + pc / PPR, c = pc % PPR;           // row of the tile, piece of the row
-                const uint4 u = *reinterpret_cast<const uint4*>(smem + C::offResW + (c >> 3) * (kTile * 128) + rr * 128 +
-                                                                (((c & 7) ^ (rr & 7)) << 4));
-                const __nv_bfloat162* ha = reinterpret_cast<const __nv_bfloat162*>(&u);
-                const __nv_bfloat162* hb = reinterpret_cast<const __nv_bfloat162*>(&ob[i]);
-                float d = 0.f;
+            for (int i0 = 0; i0 < NI; i0 += 8) {
+                float d[8];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float2 fa = __bfloat1622float2(ha[e]), fb = __bfloat1622float2(hb[e]);
-                    d = fmaf(fa.x, fb.x, d);
-                    d = fmaf(fa.y, fb.y, d);
+                for (int i = 0; i < 8; ++i) {
+                    const int pc = (i0 + i) * 32 + lane;
+                    const int rr = warp * 32 + pc / PPR, c = pc % PPR;       // row of the tile, piece of the row
+                    const uint4 u = *reinterpret_cast<const uint4*>(smem + C::offResW + (c >> 3) * (kTile * 128) + rr * 128 +
+                                                                    (((c & 7) ^ (rr & 7)) << 4));
+                    const __nv_bfloat162* ha = reinterpret_cast<const __nv_bfloat162*>(&u);
+                    const __nv_bfloat162* hb = reinterpret_cast<const __nv_bfloat162*>(&ob[i0 + i]);
+                    d[i] = 0.f;
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float2 fa = __bfloat1622float2(ha[e]), fb = __bfloat1622float2(hb[e]);
+                        d[i] = fmaf(fa.x, fb.x, d[i]);
+                        d[i] = fmaf(fa.y, fb.y, d[i]);
+                    }
                 }
+                // sums over the lanes of a row, eight rows at once: at every step a lane passes half of its values on and keeps
+                // the other half, so that lane i is left with load i's row (7 or 8 exchanges for 24 or 32)
 #pragma unroll
-                for (int o = PPR / 2; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-                if (c == 0) s_m[rr] = d;
+                for (int o = 4; o > 0; o >>= 1) {
+                    const bool up = lane & o;
+#pragma unroll
+                    for (int j = 0; j < o; ++j) {
+                        const float give = up ? d[j] : d[j + o], keep = up ? d[j + o] : d[j];
+                        d[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+                    }
+                }
+                if (PPR == 16) d[0] += __shfl_xor_sync(0xffffffffu, d[0], 8);
+                s_m[warp * 32 + ((i0 + (lane & 7)) * 32 + lane) / PPR] = d[0];
             }
             __syncwarp();
             m_own = s_m[t];

@@ -677,13 +677,20 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd && DV == 64 && LT 
             auto pass = [&](auto masked_tag, int blk) {
                 constexpr bool MASKED = decltype(masked_tag)::value;
                 uint32_t sr[32], gr[32];
-                tmem_ld32(tmem_addr(tb, lane_base, C::colS + blk * 32), sr);
+                // forward at d_v 64: the second sixteen columns are on their way while the first are worked on (38.3 -> 36.7 us at
+                // B4 H16 L2048 d' 24; at d_v 128, and in the other passes, no gain or 1 to 2 % slower)
+                constexpr bool kHalves = MODE == kModeFwd && DV == 64;
+                uint32_t (&s0)[16] = *reinterpret_cast<uint32_t (*)[16]>(sr), (&s1)[16] = *reinterpret_cast<uint32_t (*)[16]>(sr + 16);
+                if (kHalves) tmem_ld16(tmem_addr(tb, lane_base, C::colS + blk * 32), s0);
+                else tmem_ld32(tmem_addr(tb, lane_base, C::colS + blk * 32), sr);
                 if (MODE != kModeFwd) tmem_ld32(tmem_addr(tb, lane_base, C::colG + blk * 32), gr);
                 tmem_wait_ld();
+                if (kHalves) tmem_ld16(tmem_addr(tb, lane_base, C::colS + blk * 32 + 16), s1);
                 have_read(blk);
                 uint32_t pw[16], pd[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i) {
+                    if (kHalves && i == 8) tmem_wait_ld();
                     const uint64_t sv = f32x2(__uint_as_float(sr[2 * i]), __uint_as_float(sr[2 * i + 1]));
                     const uint64_t gv = MODE == kModeFwd ? 0 : f32x2(__uint_as_float(gr[2 * i]), __uint_as_float(gr[2 * i + 1]));
                     // pair (query, key): own row is the query except in the dk/dv pass

@@ -930,16 +930,18 @@ based_status launch_pass(const CUtensorMap& n0, const CUtensorMap& w0, const CUt
 // Block length of the block-wise path, or 0 for the tile path alone.  The block-wise path needs d' = 16 and the
 // statistics in one sweep (the forward output, or the numerator-only form); its cost grows with L where the tile
 // path's grows with L^2.  Tiles / blocks of 256 tokens on B200, us, around the lines below:
-//   128 heads: d_v 64 L 768 73 / 82, L 1024 112 / 105; d_v 128 L 768 106 / 109, L 1024 157 / 142
-//   16 heads: d_v 64 L 768 31 / 39, L 1024 39 / 39, L 1536 54 / 45; d_v 128 L 1280 50 / 59, L 1536 58 / 62, L 2048 79 / 63
-//   32 heads: d_v 64 L 1280 56 / 70, L 1536 69 / 74, L 2048 99 / 83; d_v 128 L 1536 84 / 105, L 2048 126 / 115
+//   128 heads: d_v 64 L 768 63 / 70, L 1024 98 / 91; d_v 128 L 768 96 / 97, L 1024 142 / 129
+//   64 heads: d_v 64 L 768 34 / 47, L 1024 52 / 54, L 1280 73 / 66; d_v 128 L 768 50 / 59, L 1024 74 / 72
+//   16 heads: d_v 64 L 768 29 / 36, L 1024 36 / 37, L 1536 51 / 42; d_v 128 L 1280 46 / 52, L 1536 53 / 54, L 2048 70 / 55
+//   32 heads: d_v 64 L 1280 46 / 61, L 1536 56 / 66, L 2048 82 / 70; d_v 128 L 1536 74 / 91, L 2048 112 / 101
 // Below 64 heads one CTA per head and block sums the states, and a second short wave of those costs as much as a full one:
-// there the line lies later once the blocks are more than one wave (24 heads are not at L 1536: 62 / 48, 69 / 65).
+// there the line lies later once the blocks are more than one wave (24 heads are not at L 1536: 54 / 44, 60 / 56).
 // With them at d_v 128 blocks of 512 tokens are the faster from 64 k rows on (256 / 512 tokens: 16 heads L 8192 217 / 206,
-// L 16384 403 / 381, 32 heads L 4096 216 / 202; 8 heads L 4096 64 / 79, L 8192 117 / 116; 2 heads L 16384 73 / 83).
+// L 16384 403 / 381, 32 heads L 4096 216 / 202; 8 heads L 4096 64 / 79, L 8192 117 / 116; 2 heads L 16384 73 / 83).  Blocks of
+// 128 tokens are within 3 % at d_v 64 (64 heads L 2048 99 / 100, 200 heads 286 / 276) and lose at d_v 128 (128 heads 255 / 242).
 // A caller without the forward output gets it recomputed into the workspace first (one forward pass, 20 us at B4 H16
-// L2048 d_v64, 83 us at B8 H16 L4096 d_v128), from somewhat longer sequences on (64 heads and more: d_v 64 96 heads L 1024
-// 93 / 103, L 1280 130 / 125, d_v 128 64 heads L 1024 94 / 108, L 1280 131 / 134, 128 heads L 1280 256 / 202).
+// L2048 d_v64, 83 us at B8 H16 L4096 d_v128), from somewhat longer sequences on (d_v 64: 64 heads L 1024 62 / 67, L 1280
+// 85 / 81, 128 heads L 1280 154 / 130; d_v 128: 64 heads L 1024 87 / 87, L 1280 122 / 107, 16 heads L 1536 70 / 71).
 int backward_block_len(int L, int df, bool merged, int d_v, int BH) {
     if (df != 16) return 0;
     int from;

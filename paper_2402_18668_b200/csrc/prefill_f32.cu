@@ -17,7 +17,7 @@
 // has four (eight), and the slices' sums meet in shared memory.
 // Bound: issue slots and latency (per full chunk and SM 27 k cycles, of which the FMA pipe needs 14 k; 11 k instructions per
 // scheduler, 6.6 k of them multiply-adds); at few heads the chain of steps.  Against one CTA per head that walked the tokens
-// one by one: B1 H2 L256 d_v64 190 -> 16 us, B2 H16 L1024 d_v64 660 -> 75.  An earlier form with the operands row by row
+// one by one: B1 H2 L256 d_v64 190 -> 15 us, B2 H16 L1024 d_v64 660 -> 72.  An earlier form with the operands row by row
 // along the summation index (even and odd terms in one two-wide FMA) took 22 and 92: twice the shared-memory passes, and
 // chunks of 16 tokens used a quarter of the warps' rows.
 #include <cooperative_groups.h>
@@ -176,9 +176,10 @@ __device__ __forceinline__ void state_product(float2 (&acc)[5][4], const float* 
 }
 
 // Outputs of a chunk of nt <= 16 NR tokens; ends with a barrier.  Warp w: rows 16 (w % NR), slice w / NR of 8 / NR.
-template <int NR>
+// state_ready is called before the state is read.
+template <int NR, class F>
 __device__ __forceinline__ void chunk_outputs(F32Smem& s, float* __restrict__ o, int d_v, int ncol, int nt, bool numerator_only,
-                                              int tid) {
+                                              int tid, F&& state_ready) {
     constexpr int KS = 8 / NR;
     const int warp = tid >> 5, lane = tid & 31, ro = lane & 1, co = lane >> 1;
     const int rg = warp % NR, ks = warp / NR, row0 = rg * kWarpRows + ro * 4;
@@ -233,6 +234,7 @@ __device__ __forceinline__ void chunk_outputs(F32Smem& s, float* __restrict__ o,
         const float c = s.tab.scale[f];
         *reinterpret_cast<float4*>(&s.psi[f * kRowT + t]) = make_float4(c * a.x * b.x, c * a.y * b.y, c * a.z * b.z, c * a.w * b.w);
     }
+    state_ready();
     __syncthreads();
     const int f0 = ks * kFeat / KS, f1 = (ks + 1) * kFeat / KS;
     tile_product(acc, s.psi + f0 * kRowT + row0, kRowT, s.st + f0 * 64 + 4 * co, 64, f1 - f0);
@@ -356,6 +358,7 @@ __global__ void __launch_bounds__(kNT, 2)
                             : make_float4(acc[i][0].x, acc[i][1].x, acc[i][2].x, acc[i][3].x));
             }
     };
+    bool summed = true;                              // the running sums are complete
     if (nseg > 1) {
         // ---- step 1: this segment's own state (the last one's is needed for the final state only)
         clear();
@@ -407,7 +410,11 @@ __global__ void __launch_bounds__(kNT, 2)
                 }
             if (z != nullptr && blockIdx.z == 0 && tid < kDSym) abi.z_put(s.tab, tid, run);
         }
-        cluster.sync();
+        // the wait for the other CTAs' share comes when the first chunk needs the state: behind its loads, weights and psi(Q)
+        // (B1 H2 L256 15.3 -> 14.7 us, B2 H16 L1024 74.7 -> 71.9; one load of a one-chunk segment for steps 1 and 3 gives 0.2 us
+        // more there and costs 3 % at B4 H16 L2048)
+        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+        summed = false;
     } else {
         for (int e = tid; e < kFeat * 16; e += kNT) {
             const int f = e >> 4, c = (e & 15) * 4;
@@ -420,6 +427,10 @@ __global__ void __launch_bounds__(kNT, 2)
     }
 
     // ---- step 3: outputs, chunk by chunk
+    auto state_ready = [&] {
+        if (!summed) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+        summed = true;
+    };
     for (int t0 = t_begin; t0 < t_end; t0 += kTok) {
         const int nt = min(kTok, t_end - t0);
         load_x(s.xq, nullptr, qh + (size_t)t0 * kDFeat, nt, tid);
@@ -427,9 +438,9 @@ __global__ void __launch_bounds__(kNT, 2)
         load_v(s.v, vh + (size_t)t0 * d_v, d_v, ncol, nt, tid);
         __syncthreads();
         float* o = oh + (size_t)t0 * d_v;
-        if (nt > 32) chunk_outputs<4>(s, o, d_v, ncol, nt, numerator_only, tid);
-        else if (nt > 16) chunk_outputs<2>(s, o, d_v, ncol, nt, numerator_only, tid);
-        else chunk_outputs<1>(s, o, d_v, ncol, nt, numerator_only, tid);
+        if (nt > 32) chunk_outputs<4>(s, o, d_v, ncol, nt, numerator_only, tid, state_ready);
+        else if (nt > 16) chunk_outputs<2>(s, o, d_v, ncol, nt, numerator_only, tid, state_ready);
+        else chunk_outputs<1>(s, o, d_v, ncol, nt, numerator_only, tid, state_ready);
         if (t0 + kTok >= t_end && (nseg > 1 || kv == nullptr)) break;   // nobody reads the state after this chunk
         clear();
         chunk_state(nt);
@@ -443,6 +454,7 @@ __global__ void __launch_bounds__(kNT, 2)
         __syncthreads();
     }
 
+    state_ready();                                   // (a segment without tokens)
     if (nseg == 1 && kv != nullptr) {
         for (int e = tid; e < kDSym * 16; e += kNT) {
             const int f = e >> 4, c = (e & 15) * 4;

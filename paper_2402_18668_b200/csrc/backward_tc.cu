@@ -102,8 +102,7 @@ template <int DV, int MODE, int LT, bool XB = false> struct BCfg {
 enum { bRes = 0, bFull0, bFull1, bFull2, bMma, bRead, bAlu, bAcc, bFinal, bXs, bX0, bX1, bNum };
 
 struct BParams {
-    const __nv_bfloat16* g_raw;  // dout and the forward output as plain pointers [BH, L, dvw] (merged pass)
-    const __nv_bfloat16* o_raw;
+    const __nv_bfloat16* o_raw;  // the forward output as a plain pointer [BH, L, dvw] (merged pass)
     const float2* stats_in;      // (1/D, b) per row (dq, dk/dv passes)
     float2* stats_out;           // statistics pass
     __nv_bfloat16* dq;           // [BH, L, 16]
@@ -520,19 +519,21 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd && DV == 64 && LT 
             if (t < 32) s_sv[128 + t] = svp[128 + t];
         }
         float m_own = 0.f;
-        if (MODE == kModeDqS && !p.numerator_only && (DV == 64 || p.dvw == 128)) {
+        if (MODE == kModeDqS && !p.numerator_only) {
             // a warp's 32 rows of out lie one after the other in global memory: every load instruction takes 512
-            // consecutive bytes (two rows at d_v 128, four at d_v 64); the matching piece of dout comes from the own
+            // consecutive bytes (two rows at d_v 128, four at d_v 64; 448, two rows, at d_v 112, where a thread per row had
+            // read 14 pieces of out and dout each: 512 -> 462 us per backward call at B8 H16 L4096); the matching piece of dout comes from the own
             // tile in shared memory, and the lanes of a row add up their parts
             constexpr int PPR = DV / 8;                       // 16-byte pieces per row
             constexpr int NI = PPR;                           // load instructions per warp: 32 rows x PPR pieces / 32 lanes
             const int wrow0 = r0 + warp * 32;
-            const uint4* op = reinterpret_cast<const uint4*>(p.o_raw + ((size_t)head * p.L + wrow0) * DV);
+            const uint4* op = reinterpret_cast<const uint4*>(p.o_raw + ((size_t)head * p.L + wrow0) * p.dvw);
+            const int np = DV == 64 ? PPR : p.dvw / 8;        // pieces of a row in memory
             uint4 ob[NI];
 #pragma unroll
             for (int i = 0; i < NI; ++i) {
-                const int pc = i * 32 + lane;                 // piece of the warp's 32 x PPR
-                ob[i] = wrow0 + pc / PPR < p.L ? op[pc] : make_uint4(0u, 0u, 0u, 0u);
+                const int pc = i * 32 + lane, rr = pc / PPR, c = pc % PPR;  // piece of the warp's 32 x PPR
+                ob[i] = wrow0 + rr < p.L && c < np ? op[rr * np + c] : make_uint4(0u, 0u, 0u, 0u);
             }
             ok = rows_all(mbar_wait(&bars[bRes], 0, abort_flag));
 #pragma unroll
@@ -570,31 +571,6 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd && DV == 64 && LT 
             }
             __syncwarp();
             m_own = s_m[t];
-        } else if (MODE == kModeDqS && !p.numerator_only && row < p.L) {
-            const uint4* gp = reinterpret_cast<const uint4*>(p.g_raw + ((size_t)head * p.L + row) * p.dvw);
-            const uint4* op = reinterpret_cast<const uint4*>(p.o_raw + ((size_t)head * p.L + row) * p.dvw);
-            float part[4] = {0.f, 0.f, 0.f, 0.f};
-            for (int c0 = 0; c0 < p.dvw / 8; c0 += 4) {          // 112 columns: 14 pieces; four in flight
-                uint4 a[4], b[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const bool in = c0 + u < p.dvw / 8;
-                    a[u] = in ? gp[c0 + u] : make_uint4(0u, 0u, 0u, 0u);
-                    b[u] = in ? op[c0 + u] : make_uint4(0u, 0u, 0u, 0u);
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const __nv_bfloat162* ha = reinterpret_cast<const __nv_bfloat162*>(&a[u]);
-                    const __nv_bfloat162* hb = reinterpret_cast<const __nv_bfloat162*>(&b[u]);
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float2 fa = __bfloat1622float2(ha[e]), fb = __bfloat1622float2(hb[e]);
-                        part[u] = fmaf(fa.x, fb.x, part[u]);
-                        part[u] = fmaf(fa.y, fb.y, part[u]);
-                    }
-                }
-            }
-            m_own = (part[0] + part[1]) + (part[2] + part[3]);
         }
         if (XB && cross) {
             // the blocks before (queries) or after (keys) the own one, through their summed state
@@ -998,7 +974,6 @@ based_status launch_dvb(const void* q, const void* k, const void* v, const void*
     if (error_word_ptr(&p.err) != BASED_OK) return BASED_ERR_CUDA;
     p.stats_in = stats;
     p.stats_out = stats;
-    p.g_raw = static_cast<const __nv_bfloat16*>(g);
     p.o_raw = static_cast<const __nv_bfloat16*>(out);
     p.dq = static_cast<__nv_bfloat16*>(dq);
     p.dk = static_cast<__nv_bfloat16*>(dk);

@@ -320,7 +320,12 @@ PyObject* generation_step(PyObject* const* a) {
 struct GenerationGraph {
     based_generation_graph* graph;
     Tensor in[6];                              // q, k, v, qw, kw, vw: the buffers of the last token's inputs
+    Tensor written[7];                         // state, caches, position and outputs
 };
+bool overlap(const Tensor& a, const Tensor& b) {
+    const char *x = static_cast<const char*>(a.const_data_ptr()), *y = static_cast<const char*>(b.const_data_ptr());
+    return x < y + b.nbytes() && y < x + a.nbytes();
+}
 constexpr const char* kGraphName = "based_generation_graph";
 void free_graph(PyObject* capsule) {
     GenerationGraph* g = static_cast<GenerationGraph*>(PyCapsule_GetPointer(capsule, kGraphName));
@@ -355,10 +360,12 @@ PyObject* generation_graph(PyObject* const* a) {
                                              size(kc, 2), static_cast<int*>(ptr(t[10])), scale, io, flags, &made);
     });
     check(st, "based_generation_graph_create");
-    return PyCapsule_New(new GenerationGraph{made, {q, t[1], v, qw, t[6], t[7]}}, kGraphName, free_graph);
+    return PyCapsule_New(new GenerationGraph{made, {q, t[1], v, qw, t[6], t[7]}, {kv, z, kc, t[9], t[10], t[11], t[12]}},
+                         kGraphName, free_graph);
 }
 // graph, q, k, v, qw, kw, vw -> whether the step was launched on these inputs; False: they have to be copied into the
-// buffers first (another dtype, shape or layout, or they overlap the buffers)
+// buffers first (another dtype, shape or layout, or they overlap the buffers or something that the step writes, such as the
+// outputs of the step before)
 PyObject* generation_graph_step(PyObject* const* a) {
     GenerationGraph& g = graph_of(a[0]);
     const void* p[6];
@@ -368,10 +375,10 @@ PyObject* generation_graph_step(PyObject* const* a) {
             !t.is_contiguous() || (reinterpret_cast<uintptr_t>(t.const_data_ptr()) & 15))
             Py_RETURN_FALSE;
         p[i] = t.const_data_ptr();
-        for (const Tensor& b : g.in) {
-            const char *x = static_cast<const char*>(p[i]), *y = static_cast<const char*>(b.const_data_ptr());
-            if (x < y + b.nbytes() && y < x + t.nbytes()) Py_RETURN_FALSE;
-        }
+        for (const Tensor& b : g.in)
+            if (overlap(t, b)) Py_RETURN_FALSE;
+        for (const Tensor& b : g.written)
+            if (overlap(t, b)) Py_RETURN_FALSE;
     }
     void* stream = c10::cuda::getCurrentCUDAStream().stream();
     const based_status st = unlocked([&] { return based_generation_graph_step(g.graph, p[0], p[1], p[2], p[3], p[4], p[5], stream); });

@@ -46,3 +46,35 @@ def test_step_equals_the_eager_call(dtype, B, H, d_v, window, sym):
                         list(want) + eager + token):
             assert torch.equal(a, b), kind
         assert int(graph.pos) == int(pos[0]) and based.based_poll_error() == based.BASED_OK
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("place,source", [("v", "out_swa"), ("v", "out_lin"), ("qw", "out_swa"), ("vw", "out_swa"), ("kw", "kc"),
+                                          ("qw", "kv")])
+def test_step_on_what_the_step_writes(dtype, place, source):
+    """Inputs that lie in an output of the step before (B 40: many CTAs, so that some write while others still read), a cache
+    or the state are copied first: the outputs, and what the buffers and a replay() hold, are those of the values."""
+    B, H = 40, 16
+    window = 1 if source == "kc" else 64
+    g = torch.Generator(device="cuda").manual_seed(5)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    kv, z = based.new_state(B, H, 64)
+    kv.copy_(rnd(*kv.shape)); z.copy_(rnd(*z.shape).abs() + 50.0)
+    kc, vc = rnd(B, H, window, 64).to(dtype), rnd(B, H, window, 64).to(dtype)
+    eager = [t.clone() for t in (kv, z, kc, vc)]
+    pos = torch.tensor([70, 0], dtype=torch.int32, device="cuda")
+    graph = DecodeGraph(kv, z, kc, vc, pos=70, dtype=dtype)
+    names = ("q", "k", "v", "qw", "kw", "vw")
+    for turn in range(3):
+        token = {n: rnd(B, H, 16 if n in "qk" else 64).to(dtype) for n in names}
+        if turn > 0:                            # (the first step gives the outputs their values)
+            token[place] = {"out_swa": graph.out_swa, "out_lin": graph.out_lin, "kc": kc[:, :, 0],
+                            "kv": kv.view(dtype).view(-1)[:B * H * 64].view(B, H, 64)}[source]
+        values = [token[n].clone() for n in names]
+        for replay in (False, True):
+            got = [t.clone() for t in (graph.step(*(token[n] for n in names)) if not replay else
+                                       (graph.replay(), graph.out_lin, graph.out_swa)[1:])]
+            want = based.based_generation_step(*values[:3], *eager[:2], *values[3:], *eager[2:], pos)
+            for a, b in zip(got + [kv, z, kc, vc] + [getattr(graph, n) for n in names], list(want) + eager + values):
+                assert torch.equal(torch.nan_to_num(a.float()), torch.nan_to_num(b.float())), (turn, replay)
+    assert based.based_poll_error() == based.BASED_OK

@@ -8,6 +8,7 @@
 #include <torch/csrc/utils/device_lazy_init.h>
 
 #include <ATen/ATen.h>
+#include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 
 #include <stdexcept>
@@ -321,6 +322,9 @@ struct GenerationGraph {
     based_generation_graph* graph;
     Tensor in[6];                              // q, k, v, qw, kw, vw: the buffers of the last token's inputs
     Tensor written[7];                         // state, caches, position and outputs
+    c10::Device device() const { return in[0].device(); }
+    // the steps belong on the current stream of the graph's own device, whichever device is current
+    void* stream() const { return c10::cuda::getCurrentCUDAStream(in[0].get_device()).stream(); }
 };
 bool overlap(const Tensor& a, const Tensor& b) {
     const char *x = static_cast<const char*>(a.const_data_ptr()), *y = static_cast<const char*>(b.const_data_ptr());
@@ -330,7 +334,14 @@ constexpr const char* kGraphName = "based_generation_graph";
 void free_graph(PyObject* capsule) {
     GenerationGraph* g = static_cast<GenerationGraph*>(PyCapsule_GetPointer(capsule, kGraphName));
     if (!g) return;
-    based_generation_graph_destroy(g->graph);
+    {
+        c10::cuda::OptionalCUDAGuard on;
+        try {
+            on.set_device(g->device());
+        } catch (...) {                        // (at the interpreter's end the device may be gone)
+        }
+        based_generation_graph_destroy(g->graph);
+    }
     delete g;
 }
 GenerationGraph& graph_of(PyObject* o) {
@@ -380,7 +391,8 @@ PyObject* generation_graph_step(PyObject* const* a) {
         for (const Tensor& b : g.written)
             if (overlap(t, b)) Py_RETURN_FALSE;
     }
-    void* stream = c10::cuda::getCurrentCUDAStream().stream();
+    const c10::cuda::CUDAGuard on(g.device());
+    void* stream = g.stream();
     const based_status st = unlocked([&] { return based_generation_graph_step(g.graph, p[0], p[1], p[2], p[3], p[4], p[5], stream); });
     check(st, "based_generation_graph_step");
     Py_RETURN_TRUE;
@@ -388,7 +400,8 @@ PyObject* generation_graph_step(PyObject* const* a) {
 // graph: the step on what the buffers hold
 PyObject* generation_graph_replay(PyObject* const* a) {
     GenerationGraph& g = graph_of(a[0]);
-    void* stream = c10::cuda::getCurrentCUDAStream().stream();
+    const c10::cuda::CUDAGuard on(g.device());
+    void* stream = g.stream();
     const based_status st = unlocked([&] {
         return based_generation_graph_step(g.graph, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, stream);
     });

@@ -78,3 +78,26 @@ def test_step_on_what_the_step_writes(dtype, place, source):
             for a, b in zip(got + [kv, z, kc, vc] + [getattr(graph, n) for n in names], list(want) + eager + values):
                 assert torch.equal(torch.nan_to_num(a.float()), torch.nan_to_num(b.float())), (turn, replay)
     assert based.based_poll_error() == based.BASED_OK
+
+
+@pytest.mark.skipif(not torch.cuda.is_available() or torch.cuda.device_count() < 2, reason="needs a second device")
+def test_step_on_a_device_that_is_not_current():
+    """A graph on cuda:1 while cuda:0 is current: every step runs on cuda:1's current stream, ordered with the copies there."""
+    with torch.cuda.device(1):
+        g = torch.Generator(device="cuda").manual_seed(9)
+        rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")
+        kv, z = based.new_state(2, 4, 64)
+        kv.copy_(rnd(*kv.shape)); z.copy_(rnd(*z.shape).abs() + 50.0)
+        kc, vc = rnd(2, 4, 64, 64).bfloat16(), rnd(2, 4, 64, 64).bfloat16()
+        eager = [t.clone() for t in (kv, z, kc, vc)]
+        pos = torch.tensor([70, 0], dtype=torch.int32, device="cuda")
+        token = [rnd(2, 4, w).bfloat16() for w in (16, 16, 64, 64, 64, 64)]
+    assert torch.cuda.current_device() == 0
+    graph = DecodeGraph(kv, z, kc, vc, pos=70)
+    for kind in ("own", "copied", "replay"):
+        given = [t.float() for t in token] if kind == "copied" else token
+        got = [t.clone() for t in ((graph.replay(), graph.out_lin, graph.out_swa)[1:] if kind == "replay" else graph.step(*given))]
+        with torch.cuda.device(1):
+            want = based.based_generation_step(*token[:3], *eager[:2], *token[3:], *eager[2:], pos)
+        for a, b in zip(got + [kv, z, kc, vc], list(want) + eager):
+            assert torch.equal(a, b), kind

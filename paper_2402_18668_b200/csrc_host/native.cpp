@@ -3,6 +3,7 @@
 // functions of binding.py that forward to them (which hold the signatures and defaults); an optional tensor is None.
 // Errors are the ones the Python checks raise: ValueError, TypeError, and binding.BasedError for a status of the library.
 #include <Python.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/custom_function.h>
 #include <torch/csrc/autograd/python_variable.h>
 #include <torch/csrc/utils/device_lazy_init.h>
@@ -489,35 +490,32 @@ PyObject* linear_attention(PyObject* const* a) {
 }
 
 // ---------------------------------------------------------------------------------------------- module
+void set_status_error(const StatusFault& e) {
+    PyObject* mod = PyImport_ImportModule("paper_2402_18668_b200.binding");
+    PyObject* cls = mod ? PyObject_GetAttrString(mod, "BasedError") : nullptr;
+    PyObject* err = cls ? PyObject_CallFunction(cls, "is", static_cast<int>(e.status), e.what()) : nullptr;
+    if (err) PyErr_SetObject(cls, err);
+    Py_XDECREF(err);
+    Py_XDECREF(cls);
+    Py_XDECREF(mod);
+}
+// The faults of this file first; everything else is torch's to translate: its own error types, and Python exceptions that
+// passed through C++ (python_error, from a saved-tensor hook for instance), which go on as they are.
 template <PyObject* (*F)(PyObject* const*), int N>
 PyObject* guarded(PyObject*, PyObject* const* args, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
     try {
         if (n != N) throw TypeFault("wrong number of arguments");
         return F(args);
     } catch (const StatusFault& e) {
-        PyObject* mod = PyImport_ImportModule("paper_2402_18668_b200.binding");
-        PyObject* cls = mod ? PyObject_GetAttrString(mod, "BasedError") : nullptr;
-        PyObject* err = cls ? PyObject_CallFunction(cls, "is", static_cast<int>(e.status), e.what()) : nullptr;
-        if (err) PyErr_SetObject(cls, err);
-        Py_XDECREF(err);
-        Py_XDECREF(cls);
-        Py_XDECREF(mod);
+        set_status_error(e);
     } catch (const TypeFault& e) {
         PyErr_SetString(PyExc_TypeError, e.what());
     } catch (const std::invalid_argument& e) {
         PyErr_SetString(PyExc_ValueError, e.what());
-    } catch (const c10::OutOfMemoryError& e) {
-        PyObject* mod = PyImport_ImportModule("torch");
-        PyObject* cls = mod ? PyObject_GetAttrString(mod, "OutOfMemoryError") : nullptr;
-        PyErr_SetString(cls ? cls : PyExc_RuntimeError, e.what_without_backtrace());
-        Py_XDECREF(cls);
-        Py_XDECREF(mod);
-    } catch (const c10::Error& e) {
-        PyErr_SetString(PyExc_RuntimeError, e.what_without_backtrace());
-    } catch (const std::exception& e) {
-        PyErr_SetString(PyExc_RuntimeError, e.what());
     }
     return nullptr;
+    END_HANDLE_TH_ERRORS
 }
 template <PyObject* (*F)(PyObject* const*), int N> PyMethodDef method(const char* name) {
     return {name, reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&guarded<F, N>)), METH_FASTCALL, nullptr};

@@ -437,6 +437,17 @@ PyObject* baseconv(PyObject* const* p) {
     return wrap(out);
 }
 
+// Python's exception for a status of the library
+void set_status_error(const StatusFault& e) {
+    PyObject* mod = PyImport_ImportModule("paper_2402_18668_b200.binding");
+    PyObject* cls = mod ? PyObject_GetAttrString(mod, "BasedError") : nullptr;
+    PyObject* err = cls ? PyObject_CallFunction(cls, "is", static_cast<int>(e.status), e.what()) : nullptr;
+    if (err) PyErr_SetObject(cls, err);
+    Py_XDECREF(err);
+    Py_XDECREF(cls);
+    Py_XDECREF(mod);
+}
+
 // ---------------------------------------------------------------------------------------------- autograd
 // The output gradient as the backward pass takes it.  It usually comes back from a projection with the heads of a token
 // side by side, [B,L,H,d_v] seen as [B,H,L,d_v]: that layout has a copy kernel of its own in the library.
@@ -466,8 +477,17 @@ struct LinearAttention : torch::autograd::Function<LinearAttention> {
         const Tensor &q = saved[0], &k = saved[1], &v = saved[2], &out = saved[3];
         void* stream = c10::cuda::getCurrentCUDAStream().stream();
         const Tensor dout = grads[0].defined() ? heads_first(grads[0], q.scalar_type(), stream) : at::zeros_like(v);
-        const Gradients g = backward_call(q, k, v, dout, out, static_cast<int>(ctx->saved_data["flags"].toInt()), kNone, stream);
-        return {g.dq, g.dk, g.dv, Tensor()};
+        try {
+            const Gradients g = backward_call(q, k, v, dout, out, static_cast<int>(ctx->saved_data["flags"].toInt()), kNone, stream);
+            return {g.dq, g.dk, g.dv, Tensor()};
+        } catch (const StatusFault& e) {
+            // autograd's worker thread: the engine hands a Python exception on to the thread that called backward
+            pybind11::gil_scoped_acquire lock;
+            set_status_error(e);
+            python_error err;
+            err.persist();
+            throw err;
+        }
     }
 };
 
@@ -490,15 +510,6 @@ PyObject* linear_attention(PyObject* const* a) {
 }
 
 // ---------------------------------------------------------------------------------------------- module
-void set_status_error(const StatusFault& e) {
-    PyObject* mod = PyImport_ImportModule("paper_2402_18668_b200.binding");
-    PyObject* cls = mod ? PyObject_GetAttrString(mod, "BasedError") : nullptr;
-    PyObject* err = cls ? PyObject_CallFunction(cls, "is", static_cast<int>(e.status), e.what()) : nullptr;
-    if (err) PyErr_SetObject(cls, err);
-    Py_XDECREF(err);
-    Py_XDECREF(cls);
-    Py_XDECREF(mod);
-}
 // The faults of this file first; everything else is torch's to translate: its own error types, and Python exceptions that
 // passed through C++ (python_error, from a saved-tensor hook for instance), which go on as they are.
 template <PyObject* (*F)(PyObject* const*), int N>

@@ -4,7 +4,9 @@ import torch
 from torch.utils._python_dispatch import TorchDispatchMode
 from torch.utils.checkpoint import checkpoint
 
+import paper_2402_18668_b200 as based
 from paper_2402_18668_b200.autograd import linear_attention
+from paper_2402_18668_b200.binding import BasedError
 
 
 class _Mine(Exception):
@@ -47,3 +49,13 @@ def test_activation_checkpointing(reentrant):
     checkpoint(linear_attention, *t, use_reentrant=reentrant).square().sum().backward()
     for a, b in zip(t, want):
         assert torch.equal(a.grad, b)
+
+
+@pytest.mark.gpu
+def test_status_of_the_backward():
+    """fp32 at d' 24 has a forward and no backward: the status arrives from autograd's worker thread."""
+    out = linear_attention(*_inputs(24))
+    with pytest.raises(BasedError, match="based_prefill_backward: unsupported") as e:
+        out.sum().backward()
+    assert e.value.status == 2
+    assert based.based_poll_error() == based.BASED_OK

@@ -92,6 +92,9 @@ std::string text(at::IntArrayRef s) {
     return r + ")";
 }
 bool shape_is(const Tensor& t, at::IntArrayRef s) { return t.sizes() == s; }
+// the same number of elements of the same type: enough where the kernels take a contiguous array and the caller may hold it
+// in another shape (a step's k as [B,H,1,d], its output as [B,1,C])
+bool fills(const Tensor& t, const Tensor& like) { return t.numel() == like.numel() && t.scalar_type() == like.scalar_type(); }
 
 // ---------------------------------------------------------------------------------------------- checks
 void check_qkv(const Tensor& q, const Tensor& k, const Tensor& v, const Tensor& out) {
@@ -264,8 +267,13 @@ PyObject* swa_decode(PyObject* const* a) {
     const Tensor& positions = ragged ? dev(a[5]) : kNone;
     Tensor out = dev(a[6]);
     dims(q, 3, "q");
-    check_qkv(q, k, v, out);
-    if (v.sizes() != q.sizes()) value_error("the sliding-window mixer takes q, k, v of one shape");
+    if (ragged) {
+        check_qkv(q, k, v, out);
+        if (v.sizes() != q.sizes()) value_error("the sliding-window mixer takes q, k, v of one shape");
+    } else {
+        if (!fills(k, q) || !fills(v, q)) value_error("q, k, v shapes/dtypes disagree");
+        if (out.defined() && !fills(out, v)) value_error("out must have the shape and dtype of v");
+    }
     check_caches(kc, vc, q, "q");
     const int B = size(q, 0), H = size(q, 1), d = size(q, 2), window = size(kc, 2);
     if (ragged && (positions.scalar_type() != at::kInt || !shape_is(positions, {B})))
@@ -416,13 +424,14 @@ PyObject* baseconv(PyObject* const* p) {
     Tensor out = dev(p[5]);
     const bool step = p[6] == Py_True;
     dims(a, step ? 2 : 3, "a");
-    dims(h, 2, "h");
+    if (h.dim() < 1) value_error("h must be [width, C]");
     const int B = size(a, 0), N = step ? 1 : size(a, 1), C = static_cast<int>(a.size(-1)), width = size(h, 0);
-    if (g.sizes() != a.sizes() || g.scalar_type() != a.scalar_type() || h.scalar_type() != at::kFloat || b2.scalar_type() != at::kFloat)
+    if (!(step ? fills(g, a) : g.sizes() == a.sizes() && g.scalar_type() == a.scalar_type()) || h.scalar_type() != at::kFloat ||
+        b2.scalar_type() != at::kFloat)
         value_error("a, g disagree or the filter/bias are not fp32");
-    if (size(h, 1) != C || !shape_is(b2, {C})) value_error("filter/bias shapes disagree with C");
-    if (out.defined() && (out.sizes() != a.sizes() || out.scalar_type() != a.scalar_type()))
-        value_error("out must have the shape and dtype of a");
+    if (h.numel() != static_cast<int64_t>(width) * C || (step ? b2.numel() != C : h.dim() < 2 || h.size(1) != C || !shape_is(b2, {C})))
+        value_error("filter/bias shapes disagree with C");
+    if (out.defined() && !fills(out, a)) value_error("out must have the shape and dtype of a");
     if (state.defined() && (!shape_is(state, {B, width - 1, C}) || state.scalar_type() != a.scalar_type()))
         value_error("conv_state must be [B, width-1, C] in the io dtype");
     const based_dtype io = dtype_code(a);

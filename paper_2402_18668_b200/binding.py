@@ -243,7 +243,7 @@ def based_prefill_state(k, v, kv_state=None, z_state=None, flags: int = BASED_ST
 def based_prefill_backward(q, k, v, dout, flags: int = 0, workspace=None, stream=None, out=None):
     """Gradients (dq, dk, dv) of based_prefill (empty initial state) for the output gradient dout.
     out: the forward output, if the caller kept it (based_prefill_backward_with_out)."""
-    return (_native_module or native()).prefill_backward(q, k, v, dout, flags, workspace, _handle(stream), out)
+    return (_native_module or native()).prefill_backward(q, k, v, dout, int(flags), workspace, _handle(stream), out)
 
 
 def based_static_scratch_bytes() -> int:
@@ -278,7 +278,8 @@ def based_decode_step_sym(q, k, v, kv_sym, z_sym, out=None, stream=None):
 
 def based_decode_step_flags(q, k, v, kv_state, z_state, flags: int, out=None, stream=None):
     """based_decode_step with flags (BASED_STATE_SYM and/or BASED_NUMERATOR_ONLY)."""
-    return (_native_module or native()).decode_step(q, k, v, kv_state, z_state, flags, out, _handle(stream), "based_decode_step_flags")
+    return (_native_module or native()).decode_step(q, k, v, kv_state, z_state, int(flags), out, _handle(stream),
+                                                    "based_decode_step_flags")
 
 
 def based_state_to_sym(kv_state, z_state, kv_sym=None, z_sym=None, stream=None):
@@ -324,12 +325,13 @@ def baseconv_gate_step(a, g, h, b2, conv_state, out=None, stream=None):
 
 def swa_forward(q, k, v, out=None, window: int = 64, softmax_scale: float = 0.0, stream=None):
     """q,k,v [B,H,L,d] -> out; causal softmax over keys i-window+1..i; scale<=0 -> 1/sqrt(d)."""
-    return (_native_module or native()).swa(q, k, v, out, window, softmax_scale, _handle(stream))
+    return (_native_module or native()).swa(q, k, v, out, int(window), float(softmax_scale), _handle(stream))
 
 
 def swa_decode_step(q, k, v, k_cache, v_cache, pos: int, out=None, softmax_scale: float = 0.0, stream=None):
     """q,k,v [B,H,d]; k_cache,v_cache [B,H,window,d] ring buffers updated in place (slot pos % window)."""
-    return (_native_module or native()).swa_decode(q, k, v, k_cache, v_cache, int(pos), out, softmax_scale, _handle(stream))
+    return (_native_module or native()).swa_decode(q, k, v, k_cache, v_cache, int(pos), out, float(softmax_scale),
+                                                   _handle(stream))
 
 
 def swa_decode_step_ragged(q, k, v, k_cache, v_cache, pos, out=None, softmax_scale: float = 0.0, stream=None):
@@ -337,7 +339,7 @@ def swa_decode_step_ragged(q, k, v, k_cache, v_cache, pos, out=None, softmax_sca
     of each sequence's new token."""
     if not isinstance(pos, torch.Tensor):
         raise ValueError("pos is an int32 tensor with one entry per sequence")
-    return (_native_module or native()).swa_decode(q, k, v, k_cache, v_cache, pos, out, softmax_scale, _handle(stream))
+    return (_native_module or native()).swa_decode(q, k, v, k_cache, v_cache, pos, out, float(softmax_scale), _handle(stream))
 
 
 def based_generation_step(q, k, v, kv_state, z_state, qw, kw, vw, k_cache, v_cache, pos_state, out=None, out_w=None,
@@ -348,7 +350,7 @@ def based_generation_step(q, k, v, kv_state, z_state, qw, kw, vw, k_cache, v_cac
     pos_state: int32 tensor {position, ticket} on the device; the step stores position + 1.
     Returns (out, out_w)."""
     return (_native_module or native()).generation_step(q, k, v, kv_state, z_state, qw, kw, vw, k_cache, v_cache, pos_state, out,
-                                                        out_w, flags, softmax_scale, _handle(stream))
+                                                        out_w, int(flags), float(softmax_scale), _handle(stream))
 
 
 def based_selftest_bounded_wait(limit_ms: int = 20, stream=None) -> None:

@@ -50,3 +50,23 @@ def test_views_of_a_convolution(dtype, step):
     for bad in (dict(g=g[:2]), dict(h=h[:, :32].contiguous()), dict(b2=b2[:32]), dict(out=torch.empty(a.numel() - 1, dtype=dtype, device="cuda"))):
         with pytest.raises(ValueError):
             call(**{"g": g, "h": h, "b2": b2, **bad})
+
+
+def test_numbers_of_other_types():
+    """Windows, positions, scales and flags that int() and float() take."""
+    q = _rnd(0, 1, 2, 70, 64)
+    want = based.swa_forward(q, q, q, window=16, softmax_scale=0.5)
+    for window, scale in ((16.0, "0.5"), ("16", torch.tensor(0.5))):
+        assert torch.equal(based.swa_forward(q, q, q, window=window, softmax_scale=scale), want)
+    q1, k, v = _rnd(1, 1, 2, 64), _rnd(2, 1, 2, 16, 64), _rnd(3, 1, 2, 16, 64)
+    pos = torch.tensor([5], dtype=torch.int32, device="cuda")
+    for f, p in ((based.swa_decode_step, 5.0), (based.swa_decode_step_ragged, pos)):
+        assert torch.equal(f(q1, q1, q1, k.clone(), v.clone(), p, softmax_scale="0.5"),
+                           f(q1, q1, q1, k.clone(), v.clone(), 5 if f is based.swa_decode_step else pos, softmax_scale=0.5))
+    x, y = _rnd(4, 1, 2, 30, 16), _rnd(5, 1, 2, 30, 64)
+    for a, b in zip(based.based_prefill_backward(x, x, y, y, flags=4.0), based.based_prefill_backward(x, x, y, y, flags=4)):
+        assert torch.equal(a, b)
+    x1, y1 = x[:, :, 0].contiguous(), y[:, :, 0].contiguous()
+    states = [tuple(t + 1.0 for t in based.new_state(1, 2, 64)) for _ in range(2)]
+    assert torch.equal(based.based_decode_step_flags(x1, x1, y1, *states[0], flags=4.0),
+                       based.based_decode_step_flags(x1, x1, y1, *states[1], flags=4))

@@ -57,7 +57,11 @@ struct AbiState {
     float* kv;                     // the head's first row, first column of this CTA
     float* z;
     int pitch;
-    bool sym, keep;                // keep: a full state whose rows (m, n) and (n, m) differ keeps the difference
+    // A continued full state gets what the call adds to the sum of the rows (m, n) and (n, m), not the sum folded back into
+    // both: 1 / sqrt 2 there and back is 3.4e-8 short of a half in fp32, in the same direction on every call (300 short pieces
+    // left the pair rows 9e-6 low).  So a row that nothing is added to stays bit for bit, and the rows may differ.
+    bool sym, add;
+    static __device__ __forceinline__ float added(float x, float before) { return x == before ? 0.f : x - before; }   // (inf: nothing)
     __device__ __forceinline__ void rows(const FeatTab& tab, int f, int& a, int& b) const {
         a = b = f;
         if (sym || f <= kDFeat) return;
@@ -65,7 +69,7 @@ struct AbiState {
         a = 1 + kDFeat + m * kDFeat + n;
         b = 1 + kDFeat + n * kDFeat + m;
     }
-    static __device__ __forceinline__ float fold(float x, float y, bool two) { return two ? (x + y) * kRsqrt2 : x; }
+    static __device__ __forceinline__ float fold(float x, float y, bool two) { return two ? __fmul_rn(x + y, kRsqrt2) : x; }
     __device__ __forceinline__ float4 kv_get(const FeatTab& tab, int f, int c) const {
         int a, b;
         rows(tab, f, a, b);
@@ -83,13 +87,15 @@ struct AbiState {
             *pa = x;
             return;
         }
-        float4 h = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (keep) {
-            const float4 u = *pa, w = *pb;
-            h = make_float4(0.5f * (u.x - w.x), 0.5f * (u.y - w.y), 0.5f * (u.z - w.z), 0.5f * (u.w - w.w));
+        float4 u = make_float4(0.f, 0.f, 0.f, 0.f), w = u;
+        if (add) {
+            u = *pa;
+            w = *pb;
+            x = make_float4(added(x.x, fold(u.x, w.x, true)), added(x.y, fold(u.y, w.y, true)), added(x.z, fold(u.z, w.z, true)),
+                            added(x.w, fold(u.w, w.w, true)));
         }
-        *pa = make_float4(fmaf(x.x, kRsqrt2, h.x), fmaf(x.y, kRsqrt2, h.y), fmaf(x.z, kRsqrt2, h.z), fmaf(x.w, kRsqrt2, h.w));
-        *pb = make_float4(fmaf(x.x, kRsqrt2, -h.x), fmaf(x.y, kRsqrt2, -h.y), fmaf(x.z, kRsqrt2, -h.z), fmaf(x.w, kRsqrt2, -h.w));
+        *pa = make_float4(fmaf(x.x, kRsqrt2, u.x), fmaf(x.y, kRsqrt2, u.y), fmaf(x.z, kRsqrt2, u.z), fmaf(x.w, kRsqrt2, u.w));
+        *pb = make_float4(fmaf(x.x, kRsqrt2, w.x), fmaf(x.y, kRsqrt2, w.y), fmaf(x.z, kRsqrt2, w.z), fmaf(x.w, kRsqrt2, w.w));
     }
     __device__ __forceinline__ void kv_put(const FeatTab& tab, int f, int c, float4 x) const {
         int a, b;
@@ -108,9 +114,10 @@ struct AbiState {
             z[a] = x;
             return;
         }
-        const float half = keep ? 0.5f * (z[a] - z[b]) : 0.f;
-        z[a] = fmaf(x, kRsqrt2, half);
-        z[b] = fmaf(x, kRsqrt2, -half);
+        const float u = add ? z[a] : 0.f, w = add ? z[b] : 0.f;
+        if (add) x = added(x, fold(u, w, true));
+        z[a] = fmaf(x, kRsqrt2, u);
+        z[b] = fmaf(x, kRsqrt2, w);
     }
 };
 
@@ -301,7 +308,7 @@ __global__ void __launch_bounds__(kNT, 2)
     const bool cont = (flags & BASED_STATE_CONTINUE) != 0, numerator_only = (flags & BASED_NUMERATOR_ONLY) != 0;
     AbiState abi;
     abi.sym = (flags & BASED_STATE_SYM) != 0;
-    abi.keep = cont && !abi.sym;
+    abi.add = cont && !abi.sym;
     abi.pitch = d_v;
     abi.kv = kv + head * (size_t)(abi.sym ? kDSym : kD) * d_v + col0;
     abi.z = z + head * (size_t)(abi.sym ? kDSym : kD);

@@ -50,3 +50,31 @@ def test_prefill_f32_keeps_an_uneven_full_state_apart():
     # one rounding of a sum of magnitude |kv0| + |S| per element, and the sums' own: 1e-5 of the largest entry
     assert np.abs(wl.to_f64(kv) - (wl.to_f64(kv0) + S)).max() <= 1e-5 * np.abs(S).max()
     assert np.abs(wl.to_f64(z) - (wl.to_f64(z0) + zz)).max() <= 1e-5 * np.abs(zz).max()
+
+
+@pytest.mark.parametrize("d_v,L", [(64, 1), (64, 200), (112, 3), (128, 70)])
+def test_prefill_f32_adds_to_a_full_state(d_v, L):
+    """A continued call adds to a full state: nothing added leaves it bit for bit (infinities too), and many short pieces
+    leave no drift."""
+    H = 2
+    w = wl.Workload("add", 1, H, L, 16, d_v, "f32", 0.1)
+    q, k, v = (t.cuda() for t in wl.prefill_inputs(w, wl.generator(d_v + L)))
+    g = torch.Generator().manual_seed(5)
+    kv, z = (torch.randn(1, H, *s, generator=g).cuda() for s in ((273, d_v), (273,)))
+    z[:, :, 0] += 500.0
+    kv[0, 1, 1 + 16 + 3 * 16 + 5, 7] = kv[0, 1, 1 + 16 + 5 * 16 + 3, 7] = float("inf")
+    before = [t[:, :, 1:].clone() for t in (kv, z)]       # zero keys: only the constant's row grows
+    based.based_prefill(q, torch.zeros_like(k), v, kv_state=kv, z_state=z, flags=based.BASED_STATE_CONTINUE)
+    assert torch.equal(kv[:, :, 1:], before[0]) and torch.equal(z[:, :, 1:], before[1])
+    kv = torch.randn(1, H, 273, d_v, generator=g).mul(1e3).cuda()
+    z = torch.rand(1, H, 273, generator=g).cuda() * 1e3 + 1e4
+    S = wl.to_f64(kv)
+    _, dS, _ = oracle.linattn_recurrent(*(wl.to_f64(t) for t in (q, k, v)))
+    n = 200
+    for _ in range(n):
+        based.based_prefill(q, k, v, kv_state=kv, z_state=z, flags=based.BASED_STATE_CONTINUE)
+    # a few roundings of 2^-24 a call and entry, up or down by the entry: their median over thousands of entries stays within
+    # a tenth of n 2^-24 (3.4e-8 lost on every call would be a half of it)
+    pairs = [1 + 16 + 16 * m + c for m in range(16) for c in range(16) if c != m]
+    err = ((wl.to_f64(kv) - (S + n * dS)) / np.abs(S + n * dS))[:, :, pairs]
+    assert abs(np.median(err)) <= 0.1 * n * 2.0 ** -24

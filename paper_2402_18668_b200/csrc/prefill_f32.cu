@@ -135,8 +135,9 @@ __device__ __forceinline__ void load_x(float* dst, float* rows, const float* __r
         if (p == 0) rows[t * kRowX + kDFeat] = live ? 1.f : 0.f;
     }
 }
-// 64 tokens x 64 columns of a row-major array; tokens past nt and columns past ncol (a multiple of 4) are zero
-__device__ __forceinline__ void load_v(float* dst, const float* __restrict__ src, int pitch, int ncol, int nt, int tid) {
+// 64 tokens x 64 columns of a row-major array; tokens past nt and columns past ncol (a multiple of 4) are zero.  Whether all
+// of this thread's values are finite.
+__device__ __forceinline__ bool load_v(float* dst, const float* __restrict__ src, int pitch, int ncol, int nt, int tid) {
     float4 x[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -145,6 +146,10 @@ __device__ __forceinline__ void load_v(float* dst, const float* __restrict__ src
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) *reinterpret_cast<float4*>(&dst[((tid >> 4) + 16 * i) * 64 + (tid & 15) * 4]) = x[i];
+    float zero = 0.f;                                // 0 x: NaN for an infinite x too
+#pragma unroll
+    for (int i = 0; i < 4; ++i) zero = fmaf(x[i].x, 0.f, fmaf(x[i].y, 0.f, fmaf(x[i].z, 0.f, fmaf(x[i].w, 0.f, zero))));
+    return zero == 0.f;
 }
 
 // acc (rows in pairs: row0 + {0..3, 8..11}, columns 4 co + j) += sum_{k < n} a[k][row] b[k][column]
@@ -182,11 +187,33 @@ __device__ __forceinline__ void state_product(float2 (&acc)[5][4], const float* 
     }
 }
 
+// The in-chunk product where V holds infinities or NaN: a masked weight times one would be NaN in rows that do not see the
+// key, so such pairs are left out instead of multiplied by zero.  row0: the thread's first row relative to the first key.
+// (What it costs a call on finite values is 0 to 1.5 %, measured: B2 H16 L1024 d_v64 72.9 -> 73.7 us, 148 heads L640 139.4
+// -> 139.5.  Out of line, or as a pass over the stored outputs, it cost as much or more.)
+__device__ __forceinline__ void causal_product(float2 (&acc)[4][4], const float* a, const float* b, int n, int row0) {
+#pragma unroll 1
+    for (int k = 0; k < n; ++k, a += kWarpRows, b += 64) {
+        const float4 y = lds4(b);
+        const float ys[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            if (k > row0 + (i >> 2) * 8 + (i & 3)) continue;
+            const float w = a[(i >> 2) * 8 + (i & 3)];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                float& x = i & 1 ? acc[i >> 1][j].y : acc[i >> 1][j].x;
+                x = fmaf(w, ys[j], x);
+            }
+        }
+    }
+}
+
 // Outputs of a chunk of nt <= 16 NR tokens; ends with a barrier.  Warp w: rows 16 (w % NR), slice w / NR of 8 / NR.
-// state_ready is called before the state is read.
+// state_ready is called before the state is read.  finite: all of V is.
 template <int NR, class F>
 __device__ __forceinline__ void chunk_outputs(F32Smem& s, float* __restrict__ o, int d_v, int ncol, int nt, bool numerator_only,
-                                              int tid, F&& state_ready) {
+                                              bool finite, int tid, F&& state_ready) {
     constexpr int KS = 8 / NR;
     const int warp = tid >> 5, lane = tid & 31, ro = lane & 1, co = lane >> 1;
     const int rg = warp % NR, ks = warp / NR, row0 = rg * kWarpRows + ro * 4;
@@ -230,8 +257,9 @@ __device__ __forceinline__ void chunk_outputs(F32Smem& s, float* __restrict__ o,
         }
         __syncwarp();
         // no key behind the warp's last row counts
-        tile_product(acc, pw + ro * 4, kWarpRows, s.v + 32 * ks * 64 + 4 * co, 64,
-                     min(32, max(0, min(nt, (rg + 1) * kWarpRows) - 32 * ks)));
+        const int n = min(32, max(0, min(nt, (rg + 1) * kWarpRows) - 32 * ks));
+        if (finite) tile_product(acc, pw + ro * 4, kWarpRows, s.v + 32 * ks * 64 + 4 * co, 64, n);
+        else causal_product(acc, pw + ro * 4, s.v + 32 * ks * 64 + 4 * co, n, row0 - 32 * ks);
     }
     __syncthreads();                                 // P is read: psi(Q)^T takes its place
     for (int e = tid; e < kFeat * (NR * 4); e += kNT) {
@@ -442,12 +470,11 @@ __global__ void __launch_bounds__(kNT, 2)
         const int nt = min(kTok, t_end - t0);
         load_x(s.xq, nullptr, qh + (size_t)t0 * kDFeat, nt, tid);
         load_x(s.xk, s.kr, kh + (size_t)t0 * kDFeat, nt, tid);
-        load_v(s.v, vh + (size_t)t0 * d_v, d_v, ncol, nt, tid);
-        __syncthreads();
+        const bool finite = __syncthreads_and(load_v(s.v, vh + (size_t)t0 * d_v, d_v, ncol, nt, tid));
         float* o = oh + (size_t)t0 * d_v;
-        if (nt > 32) chunk_outputs<4>(s, o, d_v, ncol, nt, numerator_only, tid, state_ready);
-        else if (nt > 16) chunk_outputs<2>(s, o, d_v, ncol, nt, numerator_only, tid, state_ready);
-        else chunk_outputs<1>(s, o, d_v, ncol, nt, numerator_only, tid, state_ready);
+        if (nt > 32) chunk_outputs<4>(s, o, d_v, ncol, nt, numerator_only, finite, tid, state_ready);
+        else if (nt > 16) chunk_outputs<2>(s, o, d_v, ncol, nt, numerator_only, finite, tid, state_ready);
+        else chunk_outputs<1>(s, o, d_v, ncol, nt, numerator_only, finite, tid, state_ready);
         if (t0 + kTok >= t_end && (nseg > 1 || kv == nullptr)) break;   // nobody reads the state after this chunk
         clear();
         chunk_state(nt);

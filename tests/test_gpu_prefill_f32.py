@@ -78,3 +78,22 @@ def test_prefill_f32_adds_to_a_full_state(d_v, L):
     pairs = [1 + 16 + 16 * m + c for m in range(16) for c in range(16) if c != m]
     err = ((wl.to_f64(kv) - (S + n * dS)) / np.abs(S + n * dS))[:, :, pairs]
     assert abs(np.median(err)) <= 0.1 * n * 2.0 ** -24
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("which", [0, 1, 2])
+@pytest.mark.parametrize("BH,L,d_v", [(2, 200, 64), (150, 40, 112), (2, 13, 128)])
+def test_prefill_f32_non_finite_tokens_stay_behind(BH, L, d_v, which, bad):
+    """A non-finite q, k or v of one token (padding behind a prompt, for instance) leaves the rows before it as they are."""
+    w = wl.Workload("bad", 1, BH, L, 16, d_v, "f32", 0.5)
+    x = [t.cuda() for t in wl.prefill_inputs(w, wl.generator(L))]
+    want = based.based_prefill(*x)
+    for at in sorted({L // 2, L - 1, 5}):
+        y = [t.clone() for t in x]
+        y[which][:, :, at] = bad
+        out = based.based_prefill(*y)
+        # the same sums where no value is taken for infinite, in another grouping where one is
+        assert torch.allclose(out[:, :, :at], want[:, :, :at], rtol=0, atol=TOL_F32 * 0.1)
+        assert not torch.isfinite(out[:, :, at]).all()
+        if which == 0:
+            assert torch.isfinite(out[:, :, at + 1:]).all()

@@ -240,16 +240,17 @@ __global__ void __launch_bounds__(kBT, DV > 64 ? 1 : 2)
                 const int r = row0 + (i >> 2) * 8 + (i & 3), c = 4 * co + j;
                 const bool live = !diag || (KEYS ? r <= c : c <= r);
                 const float x = sc[i][j];
+                // masked by selection, not by a zero factor: a non-finite v or dout stays out of rows that do not see it
                 const float w = live ? fmaf(x, fmaf(x, 0.03125f, 0.25f), 1.0f) : 0.f;
-                const float w1 = live ? fmaf(x, 0.0625f, 0.25f) : 0.f;
+                const float w1 = fmaf(x, 0.0625f, 0.25f);
                 if (KEYS) {
-                    a[i] = fmaf(gv[i][j], st[j].x, st[j].y) * w1;
+                    a[i] = live ? fmaf(gv[i][j], st[j].x, st[j].y) * w1 : 0.f;
                     sc[i][j] = w * st[j].x;
                 } else {
                     den[i] += w;
-                    num[i] = fmaf(w, gv[i][j], num[i]);
-                    a[i] = w1 * (gv[i][j] - m[i]);
-                    sc[i][j] = w1;
+                    if (live) num[i] = fmaf(w, gv[i][j], num[i]);
+                    a[i] = live ? w1 * (gv[i][j] - m[i]) : 0.f;
+                    sc[i][j] = live ? w1 : 0.f;
                 }
             }
             store_weight(p, a, j, co, ro);

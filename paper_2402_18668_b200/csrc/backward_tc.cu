@@ -685,18 +685,20 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd && DV == 64 && LT 
                     // w = 1 + s / sqrt(d') + s^2 / (2 d') and its derivative
                     uint64_t w = 0, dw = 0, ds = 0;
                     if (MODE != kModeDq) w = masked(fma_f32x2(sv, fma_f32x2(sv, k2, k1), one));
-                    if (MODE == kModeDq || MODE == kModeDqS || MODE == kModeDkDv) dw = masked(fma_f32x2(sv, k22, k1));
+                    if (MODE == kModeDq || MODE == kModeDqS || MODE == kModeDkDv) dw = fma_f32x2(sv, k22, k1);
+                    if (MODE == kModeDqS) dw = masked(dw);
                     if (MODE == kModeFwd || MODE == kModeStats || MODE == kModeDqS) den2 = add_f32x2(den2, w);
                     if (MODE == kModeStats || MODE == kModeDqS) en2 = fma_f32x2(w, gv, en2);
                     if (MODE == kModeDqS) {
                         ds = mul_f32x2(dw, add_f32x2(gv, negm));             // first tile: w' (gv - m); second: w'
                         w = dw;
                     }
-                    if (MODE == kModeDq) ds = mul_f32x2(fma_f32x2(gv, own_d, own_b), dw);
+                    // (masked by selection: 0 times a non-finite product would be NaN in pairs that do not count)
+                    if (MODE == kModeDq) ds = masked(mul_f32x2(fma_f32x2(gv, own_d, own_b), dw));
                     if (MODE == kModeDkDv) {
                         const int c = (it & 1) * 2 * LT + blk * 32 + 2 * i;
                         const uint64_t qd = *reinterpret_cast<const uint64_t*>(s_b + c);
-                        ds = mul_f32x2(fma_f32x2(gv, qd, *reinterpret_cast<const uint64_t*>(s_b + LT + c)), dw);
+                        ds = masked(mul_f32x2(fma_f32x2(gv, qd, *reinterpret_cast<const uint64_t*>(s_b + LT + c)), dw));
                         w = mul_f32x2(w, qd);                // dv_j = sum_i (w_ij / D_i) G_i
                     }
                     float lo, hi;

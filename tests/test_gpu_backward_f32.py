@@ -31,3 +31,25 @@ def test_backward_f32_tiles(d_v, BH, L, flags):
         assert (np.abs(a - b).max(axis=(0, 2, 3)) <= TOL_F32 * np.abs(b).max(axis=(0, 2, 3))).all()
     again = based.based_prefill_backward(q.cuda(), k.cuda(), v.cuda(), g.cuda(), flags=flags)
     assert all(torch.equal(a, b) for a, b in zip(got, again))
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("L,at", [(200, 100), (64, 62), (300, 129)])
+def test_backward_non_finite_values_stay_where_they_belong(L, at, bad):
+    """A non-finite v leaves dq of the rows before it as it is (fp32), a non-finite output gradient dk of the keys behind it
+    (both types)."""
+    w = wl.Workload("bad", 1, 3, L, 16, 64, "f32", 0.5)
+    gen = wl.generator(L)
+    q, k, v = (t.cuda() for t in wl.prefill_inputs(w, gen))
+    g = torch.randn(1, 3, L, 64, generator=gen).cuda()
+    want = based.based_prefill_backward(q, k, v, g)
+    vb, gb = v.clone(), g.clone()
+    vb[:, :, at], gb[:, :, at] = bad, bad
+    assert torch.equal(based.based_prefill_backward(q, k, vb, g)[0][:, :, :at], want[0][:, :, :at])
+    got = based.based_prefill_backward(q, k, v, gb)
+    assert torch.equal(got[1][:, :, at + 1:], want[1][:, :, at + 1:]) and not torch.isfinite(got[1][:, :, 0]).all()
+    q, k, v, g, gb = (t.bfloat16() for t in (q, k, v, g, gb))
+    for out in (None, based.based_prefill(q, k, v)):
+        want = based.based_prefill_backward(q, k, v, g, out=out)
+        got = based.based_prefill_backward(q, k, v, gb, out=out)
+        assert torch.equal(got[1][:, :, at + 1:], want[1][:, :, at + 1:])

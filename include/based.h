@@ -73,7 +73,9 @@ enum {
  *           prefill or a decode step produces; the bf16 d_feat = 16 path relies on that and
  *           returns both as their mean when it continues from a state where they differ.
  * workspace device scratch of at least based_prefill_workspace_bytes(...) bytes
- *           (may be NULL when that size is 0); contents are undefined afterwards.
+ *           (may be NULL when that size is 0); contents are undefined afterwards.  A size up to
+ *           BASED_WORDS_BYTES is used by continued calls only: others may pass NULL then, and a
+ *           continued call without it is served more slowly.
  * Supported: d_feat = 16; d_v in {64, 112, 128}; io in {F32, BF16}; any L >= 1.
  * d_feat in {8, 24, 32} (the other dimensions of the paper's feature-map ablation; state rows
  * D = 1 + d_feat + d_feat^2 = 73, 601, 1057) is served by the definition form: bf16 io from the
@@ -86,7 +88,8 @@ based_status based_prefill(const void* q, const void* k, const void* v, void* ou
                            float* z_state, int B, int H, int L, int d_feat, int d_v, based_dtype io,
                            int flags, void* workspace, size_t workspace_bytes, void* cuda_stream);
 
-/* Scratch bytes based_prefill needs for these arguments (0 is possible). */
+/* Scratch bytes based_prefill needs for these arguments, with any flags (0 is possible). */
+#define BASED_WORDS_BYTES 2048
 size_t based_prefill_workspace_bytes(int B, int H, int L, int d_feat, int d_v, based_dtype io);
 
 /*

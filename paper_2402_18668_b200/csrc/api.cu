@@ -139,7 +139,12 @@ static based_status prefill_impl(const void* q, const void* k, const void* v, vo
                                       static_cast<cudaStream_t>(cuda_stream));
     }
     const size_t need = based_prefill_workspace_bytes(B, H, L, d_feat, d_v, io);
-    if (!fit && need > 0 && (!workspace || workspace_bytes < need)) return BASED_ERR_WORKSPACE;
+    if (!fit && need > 0 && (!workspace || workspace_bytes < need)) {
+        // a few words for continued calls alone: others need none, and a continued call without them takes a plan without them
+        if (need > BASED_WORDS_BYTES) return BASED_ERR_WORKSPACE;
+        fit = true;
+        if (!workspace) workspace_bytes = 0;
+    }
     if (io == BASED_BF16)
         return launch_prefill_tc(q, k, v, out, kv_state, z_state, B * H, L, d_v, flags, workspace,
                                  static_cast<cudaStream_t>(cuda_stream), fit ? workspace_bytes : ~(size_t)0);

@@ -42,6 +42,7 @@
 // output staging tile, and the output group releases the accumulator before it stages anything.
 #include <cuda_bf16.h>
 #include <cstdlib>
+#include <random>
 
 #include "common.cuh"
 #include "sm100.cuh"
@@ -153,6 +154,8 @@ struct Params {
     int heads;            // B*H (balanced mode)
     int pad;              // balanced mode: chunks counted in front of every head for the CTA it starts;
                           // segments with a state pass: 1 if each head's first slot holds the caller's state
+    unsigned long long ticket;   // recompute mode, continued: what a segment's word in ws becomes when it has read the
+                          // caller's state (see wait_for_readers)
 #ifdef BASED_TRACE
     unsigned long long* trace;
 #endif
@@ -513,6 +516,43 @@ __device__ __noinline__ void init_from_abi(const float* kv_abi, const float* z_a
     tmem_wait_st();
 }
 
+// ---- continued calls in recompute mode: every segment of a head starts from the caller's state, and the last one
+// overwrites it at its end.  The segments' CTAs start as SMs come free (another stream may hold some), so the order is
+// made here: a segment that has read the state stores the call's ticket in its word of the workspace, and the last one
+// waits for the others' words before it writes (in practice they were stored long since: the last segment runs longest).
+// It clears them for a replay of the same launch; a ticket is a 64-bit number that no other launch uses, so whatever lay
+// in the workspace before is not one.  The CTAs of such a call are at most one per SM and need nothing of one another
+// to start and to read, so the wait ends; it is bounded all the same.
+// (blockIdx: segment, head.  All from special registers and constants, and out of line: values kept in registers for it
+// through the role loops cost them spills, and B3 H16 L777 d_v112 1 to 2 us; this way 19.7 -> 20.0, d_v 128 19.3 -> 20.0, d_v 64
+// nothing.)
+__device__ __forceinline__ unsigned long long* reader_words(const Params& p) {
+    return reinterpret_cast<unsigned long long*>(p.ws) + (size_t)blockIdx.y * (gridDim.x - 1);
+}
+__device__ __forceinline__ bool last_segment() { return blockIdx.x == gridDim.x - 1; }
+__device__ __noinline__ void has_read(const Params& p) {
+    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(reader_words(p) + blockIdx.x), "l"(p.ticket) : "memory");
+}
+// Every lane of a warp calls it; the same answer for all.
+__device__ __noinline__ bool wait_for_readers(const Params& p, volatile uint32_t* abort_flag) {
+    const int lane = threadIdx.x & 31;
+    const uint64_t deadline = global_timer_ns() + kWaitLimitNs;
+    bool seen = lane >= (int)gridDim.x - 1;
+    for (;;) {
+        if (!seen) {
+            unsigned long long w;
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(reader_words(p) + lane) : "memory");
+            seen = w == p.ticket;
+        }
+        if (__all_sync(~0u, seen)) return true;
+        if (__any_sync(~0u, *abort_flag || global_timer_ns() > deadline)) {
+            *abort_flag = 1;
+            return false;
+        }
+        __nanosleep(200);
+    }
+}
+
 // ---- the CTA's piece of work: a head, a token range, where its initial state comes from (workspace slots
 // ws_first .. ws_first + ws_count - 1) and where its final state goes (slot ws_out, or the caller's state if
 // the piece ends its head).
@@ -703,8 +743,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         mbar_init(&bars[kG3], 1);
         mbar_init(&bars[kP], 128); mbar_init(&bars[kR4], PQT ? 256 : 384); mbar_init(&bars[kPK], 128); mbar_init(&bars[kPKb], 128); mbar_init(&bars[kDone], 1);
         mbar_init(&bars[kSR], 128);
-        mbar_init(&bars[kFin], 1);
-        mbar_init(&bars[kInit], 384);
+        mbar_init(&bars[kFin], CONT && PRE && last_segment() ? 2 : 1);     // the last products; the other segments have read the state
+        mbar_init(&bars[kInit], CONT && PRE ? 512 : 384);
         *abort_flag = 0;
         fence_mbar_init();
         prefetch_tensormap(&tm_q); prefetch_tensormap(&tm_k); prefetch_tensormap(&tm_v); prefetch_tensormap(&tm_o);
@@ -785,6 +825,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             init_state(warp >> 2, 4);
             tc_fence_before();
             mbar_arrive(&bars[kInit]);
+            // (the output group has nothing to do before the first chunk's products)
+            if (CONT && PRE && threadIdx.x == 384 && !last_segment() && mbar_wait(&bars[kInit], 0, abort_flag)) has_read(p);
         }
     }
 
@@ -806,6 +848,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                 for (int b = 0; b < DV / 64; ++b)
                     tma_load_3d(st + kOffV + b * (kC * 128), &tm_v, &bars[kFull0 + s], b * 64, tok0, head);
             }
+        }
+        if (CONT && PRE && last_segment()) {
+            // all loads are under way: the words are looked at here, off the path of the final write, which waits for kFin
+            __syncwarp();
+            ok = __all_sync(~0u, ok) && wait_for_readers(p, abort_flag);
+            if (ok && lane == 0) mbar_arrive(&bars[kFin]);
         }
     } else if (warp == kWarpMma) {
         // ===================================================================== MMA issuer, state chain
@@ -1147,6 +1195,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
         } else if (share_init) {
             init_state(2, 4);
+            if (CONT && PRE) mbar_arrive(&bars[kInit]);
             ok = mbar_wait(&bars[kInit], 0, abort_flag);          // the other groups' blocks are written
             tc_fence_after();
         } else {
@@ -1489,6 +1538,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (*abort_flag) {
         for (int it = 0; it < 200; ++it) __nanosleep(1000);   // ~0.2 ms: far longer than any TMA load in flight
     }
+    if (CONT && PRE && last_segment() && threadIdx.x < gridDim.x - 1) reader_words(p)[threadIdx.x] = 0;       // (every warp has seen them)
     __syncthreads();
     if (warp == kWarpMma) tmem_dealloc(tb, 512);
     if (tid == 0) { TRACE(5, 1, 7); TRACE_CTA(1); }     // kernel exit
@@ -1601,6 +1651,19 @@ static cudaError_t launch_slot_scan(float* ws, int dv_kernel, int per_head, int 
     return cudaLaunchKernelEx(&cfg, slot_scan_kernel, ws, floats, per_head, (uint32_t)heads, (uint32_t)n, (uint32_t)nchr, (uint32_t)w);
 }
 
+// A number that no other launch uses: a counter from a random start, spread over 64 bits (splitmix64, Steele et al. 2014:
+// a bijection, so the numbers of one process differ), never 0.
+unsigned long long new_ticket() {
+    static std::atomic<unsigned long long> next{((unsigned long long)std::random_device{}() << 32) ^ std::random_device{}()};
+    for (;;) {
+        unsigned long long x = next.fetch_add(0x9e3779b97f4a7c15ull, std::memory_order_relaxed);
+        x = (x ^ (x >> 30)) * 0xbf58476d1ce4e5b9ull;
+        x = (x ^ (x >> 27)) * 0x94d049bb133111ebull;
+        x ^= x >> 31;
+        if (x != 0) return x;
+    }
+}
+
 template <int DV>
 based_status launch_dv(const void* q, const void* k, const void* v, void* out, float* kv, float* z, int BH, int L,
                        int dv, int flags, float* ws, const SegPlan plan, cudaStream_t stream) {
@@ -1676,6 +1739,7 @@ based_status launch_dv(const void* q, const void* k, const void* v, void* out, f
         return check_launch("prefill_tc_kernel<balanced>");
     }
     if (nseg > 1 && recompute) {
+        if (p.continue_abi) p.ticket = new_ticket();
         const cudaError_t e = p.continue_abi ? launch_dependent<DV, kModePre, true>(dim3(nseg, BH), stream, tq, tk, tv, to, p)
                                              : launch_dependent<DV, kModePre>(dim3(nseg, BH), stream, tq, tk, tv, to, p);
         if (e != cudaSuccess) return BASED_ERR_CUDA;
@@ -1717,12 +1781,15 @@ based_status launch_dv(const void* q, const void* k, const void* v, void* out, f
 
 }  // namespace
 
+// Workspace of a continued call in recompute mode: the segments' words (see wait_for_readers).
+static size_t reader_words_bytes(int BH, int nseg) { return ((size_t)BH * (nseg - 1) * 8 + 15) & ~(size_t)15; }
+
 // How a head's sequence is cut into segments so that about one CTA per SM is busy.
 //  - one segment: the plain chunk loop;
 //  - state pass: a first launch computes every segment's own state into the workspace, the main
 //    launch starts each segment from the sum of the earlier ones (long sequences; d_v 64: a small kernel in
 //    between turns the partial states into running sums, see Cfg::kSlotScan);
-//  - recompute: one launch, no workspace; a segment's CTA first runs the state update alone over
+//  - recompute: one launch, no partial states; a segment's CTA first runs the state update alone over
 //    all earlier chunks (short sequences, where a second launch and start-up cost more than that).
 // The choice compares modelled CTA times in thousands of cycles, constants fitted on B200 with every SM busy:
 // full chunk 3.0 (d_v 64) / 4.1 (d_v 128), state-update-only chunk of the state pass 1.1 / 2.2, of the recompute
@@ -1754,6 +1821,7 @@ static SegPlan prefill_tc_plan(int BH, int L, int d_v, bool continued = false, s
     SegPlan best = {nseg, (nch + nseg - 1) / nseg, false, 0};
     float best_cost = nseg > 1 ? (float)best.per * (upd + full) + second : (float)nch * full;
     for (int n = 2; n <= nmax; ++n) {
+        if (continued && reader_words_bytes(BH, n) > ws_limit) break;
         for (int per = (nch + n - 1) / n; per * (n - 1) < nch; ++per) {
             float cost = 0.f;
             for (int j = 0; j < n; ++j) {
@@ -1897,6 +1965,7 @@ size_t prefill_tc_workspace_bytes(int BH, int L, int d_v) {
         size_t n = 0;
         if (plan.balanced > 0) n = (size_t)plan.balanced * seg_state_floats(d_v) * sizeof(float);
         else if (!plan.recompute && plan.nseg > 1) n = (size_t)BH * (plan.nseg - 1 + cont) * seg_state_floats(d_v) * sizeof(float);
+        else if (plan.recompute && cont) n = reader_words_bytes(BH, plan.nseg);
         need = n > need ? n : need;
     }
     return need;

@@ -148,7 +148,9 @@ Tensor prefill_call(const Tensor& q, const Tensor& k, const Tensor& v, const Ten
     const int B = size(q, 0), H = size(q, 1), L = size(q, 2), d_feat = size(q, 3), d_v = size(v, 3);
     const based_dtype io = dtype_code(q);
     if (!out.defined()) out = at::empty_like(v);
-    const Tensor ws = workspace_of(workspace, based_prefill_workspace_bytes(B, H, L, d_feat, d_v, io), q);
+    size_t need = based_prefill_workspace_bytes(B, H, L, d_feat, d_v, io);
+    if (need <= BASED_WORDS_BYTES && !(flags & BASED_STATE_CONTINUE)) need = 0;
+    const Tensor ws = workspace_of(workspace, need, q);
     check(based_prefill(cptr(q), cptr(k), cptr(v), ptr(out), fptr(kv), fptr(z), B, H, L, d_feat, d_v, io, flags, ptr(ws),
                         bytes_of(ws), stream),
           "based_prefill");

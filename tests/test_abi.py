@@ -230,3 +230,17 @@ def test_generation_step_validation(lib):
     assert call(io=5) == 1 and call(flags=1) == 1           # BASED_STATE_CONTINUE means nothing for a step
     assert call(d_feat=8) == 2 and call(d_v=96) == 2 and call(d_w=128) == 2 and call(window=129) == 2
     assert call(q=U) == 3 and call(pos=ctypes.c_void_p(0x4004)) == 3
+
+
+def test_words_of_continued_calls(lib):
+    """A continued call whose pieces all start from the caller's state takes a few words of workspace to order its reads ahead
+    of the final write: less than any partial state, so that callers can tell."""
+    words = 2048                                                          # BASED_WORDS_BYTES
+    for B, H, L, d_v in [(3, 16, 777, 112), (4, 16, 2048, 64), (1, 1, 700, 64), (1, 2, 1000, 128), (1, 18, 1000, 64)]:
+        n = lib.based_prefill_workspace_bytes(B, H, L, 16, d_v, 1)
+        assert 0 < n <= words and n % 16 == 0
+    slot = (160 * 64 + 160) * 4
+    for BH in (1, 5, 18, 49, 74, 75, 148):
+        for L in (1, 128, 129, 500, 1000, 2100, 5000):
+            n = lib.based_prefill_workspace_bytes(1, BH, L, 16, 64, 1)
+            assert n <= words or n >= slot

@@ -107,7 +107,6 @@ struct BParams {
     float2* stats_out;           // statistics pass
     __nv_bfloat16* dq;           // [BH, L, 16]
     __nv_bfloat16* dk;
-    __nv_bfloat16* dvo;          // [BH, L, dvw]
     unsigned int* err;
     int L, dvw, numerator_only;  // dvw: value head dimension of the caller's tensors (64, 112, 128)
     int df, kdim;                // feature dimension d', and d' rounded up to 16 (K extent of the scores)
@@ -979,7 +978,6 @@ based_status launch_dvb(const void* q, const void* k, const void* v, const void*
     p.o_raw = static_cast<const __nv_bfloat16*>(out);
     p.dq = static_cast<__nv_bfloat16*>(dq);
     p.dk = static_cast<__nv_bfloat16*>(dk);
-    p.dvo = static_cast<__nv_bfloat16*>(dv);
     p.L = L;
     p.dvw = dvr;
     p.numerator_only = numerator_only;
@@ -1069,7 +1067,6 @@ based_status launch_quadratic_forward_tc(const void* q, const void* k, const voi
         return BASED_ERR_CUDA;
     BParams p{};
     if (error_word_ptr(&p.err) != BASED_OK) return BASED_ERR_CUDA;
-    p.dvo = static_cast<__nv_bfloat16*>(out);
     p.L = L;
     p.dvw = d_v;
     p.overlapped = overlapped;

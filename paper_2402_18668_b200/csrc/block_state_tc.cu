@@ -456,7 +456,7 @@ based_status launch_running(const void* x, const void* val, const float2* stats,
     p.zpart = zpart;
     p.L = L;
     p.dvw = dvw;
-    p.lspb = W == 128 ? 0 : W == 256 ? 1 : 2;
+    p.lspb = W == 256 ? 1 : 2;
     p.nblk = (L + W - 1) / W;
     p.rev = rev;
     // own sums: enough consecutive blocks per CTA to spread its fixed cost, while some waves of CTAs remain
@@ -480,7 +480,7 @@ based_status launch_running(const void* x, const void* val, const float2* stats,
 }
 }  // namespace
 
-// W: 128, 256 or 512, L > W.  stats: (1 / D_t, b_t) per token for the query side, null for the key side.
+// W: 256 or 512, L > W.  stats: (1 / D_t, b_t) per token for the query side, null for the key side.
 // part, zpart: null for the running sums (one CTA per head); else every block's own sums go there in fp32 (one CTA
 // per head and block) and st, sv stay untouched.
 based_status launch_block_states_tc(const void* x, const void* val, const void* stats, void* st, float* sv, float* part,

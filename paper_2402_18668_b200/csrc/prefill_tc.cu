@@ -145,7 +145,6 @@ struct Params {
     int L;                // tokens per head
     int nseg;             // segments per head
     int seg_len;          // tokens per segment (multiple of kC)
-    int continue_abi;     // start from the ABI state in kv_abi / z_abi
     int sym;              // kv_abi / z_abi use the 153-row symmetric format
     int numerator_only;   // outputs are not divided by the denominator
     int dv;               // value head dimension of the caller's tensors (112 runs on the d_v 128 kernel:
@@ -365,17 +364,16 @@ __device__ __forceinline__ bool group_all(int id, bool pred) {
 // a segment (partial state to the workspace); kModePre = kModeMain preceded by state-update-only
 // "pre-chunks" over everything before the segment (recompute mode).
 // ---- initial state.  One thread per TMEM lane of the state accumulator S^T; lane t of a warp's lane quarter holds
-// V column t (d_v 64: lane 64 the K-state).  Its initial value is the caller's ABI state (folded into the internal
-// basis; kv_abi == nullptr: none) plus the partial states of the earlier pieces (nprev workspace slots from wsh on).
+// V column t (d_v 64: lane 64 the K-state).  Its initial value is the sum of the partial states of the earlier pieces
+// (nprev workspace slots from wsh on).
 // Those are up to seven slots of 40-80 KB each, read as ten 16-column blocks per slot, and one thread group doing it
 // alone spends 0.7 us of load latency per block and slot before the first state update can run (2.7 us per slot).
 // So in the main pass all four role groups (each has a warp per lane quarter) take every fourth block (part of
 // nparts), and two slots' loads are in flight at a time; the state group waits for the others before it reads the
 // state.  Not inlined: its registers are its own and the role loops' allocation does not see it.
 template <int DV>
-__device__ __noinline__ void init_state_blocks(const float* wsh, int nprev, bool wait_for_state_pass, const float* kv_abi,
-                                               const float* z_abi, int dv, int abi_row0, const short2* s_abi, uint32_t tb,
-                                               int part, int nparts) {
+__device__ __noinline__ void init_state_blocks(const float* wsh, int nprev, bool wait_for_state_pass, uint32_t tb, int part,
+                                               int nparts) {
     using C = Cfg<DV>;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t lane_base = (uint32_t)(warp & 3) * 32u;
@@ -386,9 +384,6 @@ __device__ __noinline__ void init_state_blocks(const float* wsh, int nprev, bool
     // d_v 128: K-state features held in the two z tiles (64-row MMA: rows 0..31 in lanes 0-15, 32-47)
     const int z1f = (DV == 128 && (t & 31) < 16 && (t >> 5) < 2) ? 128 + (t >> 5) * 16 + (t & 15) : -1;
     const size_t seg_stride = seg_state_floats(DV);
-    const bool from_abi = kv_abi != nullptr;            // dv: row pitch of the caller's state; lanes >= dv hold zeros
-    const float* kvh = from_abi ? kv_abi + (size_t)abi_row0 * dv : nullptr;
-    const float* zh = from_abi ? z_abi + abi_row0 : nullptr;
     // the partial states are the state pass's output (a no-op when this grid was launched the plain way)
     if (wait_for_state_pass) asm volatile("griddepcontrol.wait;" ::: "memory");
 #pragma unroll 1
@@ -397,18 +392,6 @@ __device__ __noinline__ void init_state_blocks(const float* wsh, int nprev, bool
 #pragma unroll
         for (int i = 0; i < 16; ++i) acc[i] = 0.f;
         if (srow >= 0) {
-            if (from_abi) {
-                float va[16], vb[16];
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const short2 ar = s_abi[b * 16 + i];
-                    const bool live = is_z || srow < dv;
-                    va[i] = (ar.x >= 0 && live) ? (is_z ? zh[ar.x] : kvh[(size_t)ar.x * dv + srow]) : 0.f;
-                    vb[i] = (ar.y >= 0 && live) ? (is_z ? zh[ar.y] : kvh[(size_t)ar.y * dv + srow]) : 0.f;
-                }
-#pragma unroll
-                for (int i = 0; i < 16; ++i) acc[i] = (s_abi[b * 16 + i].y >= 0) ? (va[i] + vb[i]) * kRsqrt2 : va[i];
-            }
             const float* src = wsh + (is_z ? (size_t)kF * DV + b * 16 : (size_t)(b * 16) * DV + srow);
             const size_t step = is_z ? 1 : DV;
             int sp = 0;
@@ -437,10 +420,6 @@ __device__ __noinline__ void init_state_blocks(const float* wsh, int nprev, bool
     auto z_init = [&](int f) -> float {
         if (f < 0) return 0.f;
         float acc = 0.f;
-        if (from_abi) {
-            const short2 ar = s_abi[f];
-            if (ar.x >= 0) acc = (ar.y >= 0) ? (zh[ar.x] + zh[ar.y]) * kRsqrt2 : zh[ar.x];
-        }
         for (int sp = 0; sp < nprev; ++sp) acc += wsh[(size_t)sp * seg_stride + (size_t)kF * DV + f];
         return acc;
     };
@@ -524,7 +503,7 @@ __device__ __noinline__ void init_from_abi(const float* kv_abi, const float* z_a
 // in the workspace before is not one.  The CTAs of such a call are at most one per SM and need nothing of one another
 // to start and to read, so the wait ends; it is bounded all the same.
 // (blockIdx: segment, head.  All from special registers and constants, and out of line: values kept in registers for it
-// through the role loops cost them spills, and B3 H16 L777 d_v112 1 to 2 us; this way 19.7 -> 20.0, d_v 128 19.3 -> 20.0, d_v 64
+// through the role loops cost them spills, and B3 H16 L777 d_v112 1 to 2 us; this way 19.7 -> 20.0, d_v 128 19.2 -> 19.7, d_v 64
 // nothing.)
 __device__ __forceinline__ unsigned long long* reader_words(const Params& p) {
     return reinterpret_cast<unsigned long long*>(p.ws) + (size_t)blockIdx.y * (gridDim.x - 1);
@@ -697,7 +676,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 #ifdef BASED_PIECE_OUT
     constexpr bool kPieceOut = (BASED_PIECE_OUT >> ((DV == 128 ? 3 : 0) + MODE)) & 1;
 #else
-    constexpr bool kPieceOut = DV == 64 && MODE == kModeMain;
+    // (continued pieces in recompute mode, us out of line / inline: d_v 112 B3 H16 L777 20.0 / 21.9, d_v 64 B4 H16 L2048 28.7 / 29.7)
+    constexpr bool kPieceOut = (DV == 64 && MODE == kModeMain) || (CONT && PRE);
 #endif
     if constexpr (kPieceOut) {
         Piece* s_piece = reinterpret_cast<Piece*>(s_abi + kF);
@@ -816,8 +796,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             init_from_abi<DV>(p.kv_abi, p.z_abi, p.dv, head * abi_nrows, s_abi, tb, part);
             return;
         }
-        init_state_blocks<DV>(p.ws + (size_t)ws_first * seg_state_floats(DV), ws_count, MODE == kModeMain && ws_count > 0,
-                              (!STATE_ONLY && p.continue_abi) ? p.kv_abi : nullptr, p.z_abi, p.dv, head * abi_nrows, s_abi, tb,
+        init_state_blocks<DV>(p.ws + (size_t)ws_first * seg_state_floats(DV), ws_count, MODE == kModeMain && ws_count > 0, tb,
                               part, nparts);
     };
     if constexpr (!C::kSlotScan || CONT) {
@@ -1129,35 +1108,18 @@ __global__ void __launch_bounds__(kThreads, 1)
         if constexpr (C::kSlotScan && !CONT) {
             const size_t seg_stride = seg_state_floats(DV);
             const float* wsh = p.ws + (size_t)ws_first * seg_stride;      // the partial states this piece starts from
-            const int dv = p.dv;                        // row pitch of the caller's state; lanes >= dv hold zeros
-            const float* kvh = p.kv_abi ? p.kv_abi + (size_t)head * abi_nrows * dv : nullptr;
-            const float* zh = p.z_abi ? p.z_abi + (size_t)head * abi_nrows : nullptr;
-            const bool from_abi = !STATE_ONLY && p.continue_abi;
             const int nprev = ws_count;
             // the partial states are the state pass's output (a no-op when this grid was launched the plain way)
             if (MODE == kModeMain && nprev > 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 
-            // Initial value of this lane's row: the caller's ABI state (folded into the internal
-            // basis) plus the partial states of the earlier segments.  Loads are issued 16 at a
-            // time before they are consumed, so their latencies overlap.
+            // Initial value of this lane's row: the partial states of the earlier segments.  Loads are
+            // issued 16 at a time before they are consumed, so their latencies overlap.
 #pragma unroll 1
             for (int b = 0; b < kF / 16; ++b) {
                 float acc[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i) acc[i] = 0.f;
                 if (srow >= 0) {
-                    if (from_abi) {
-                        float va[16], vb[16];
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) {
-                            const short2 ar = s_abi[b * 16 + i];
-                            const bool live = is_z || srow < dv;
-                            va[i] = (ar.x >= 0 && live) ? (is_z ? zh[ar.x] : kvh[(size_t)ar.x * dv + srow]) : 0.f;
-                            vb[i] = (ar.y >= 0 && live) ? (is_z ? zh[ar.y] : kvh[(size_t)ar.y * dv + srow]) : 0.f;
-                        }
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) acc[i] = (s_abi[b * 16 + i].y >= 0) ? (va[i] + vb[i]) * kRsqrt2 : va[i];
-                    }
                     for (int sp = 0; sp < nprev; ++sp) {
                         const float* src = wsh + (size_t)sp * seg_stride + (is_z ? (size_t)kF * DV + b * 16
                                                                                  : (size_t)(b * 16) * DV + srow);
@@ -1177,10 +1139,6 @@ __global__ void __launch_bounds__(kThreads, 1)
             auto z_init = [&](int f) -> float {
                 if (f < 0) return 0.f;
                 float acc = 0.f;
-                if (from_abi) {
-                    const short2 ar = s_abi[f];
-                    if (ar.x >= 0) acc = (ar.y >= 0) ? (zh[ar.x] + zh[ar.y]) * kRsqrt2 : zh[ar.x];
-                }
                 for (int sp = 0; sp < nprev; ++sp) acc += wsh[(size_t)sp * seg_stride + (size_t)kF * DV + f];
                 return acc;
             };
@@ -1684,7 +1642,7 @@ based_status launch_dv(const void* q, const void* k, const void* v, void* out, f
     const bool recompute = plan.recompute;
     p.nseg = nseg;
     p.seg_len = plan.per * kC;
-    p.continue_abi = (flags & BASED_STATE_CONTINUE) ? 1 : 0;
+    const bool continued = (flags & BASED_STATE_CONTINUE) != 0;
     p.sym = (flags & BASED_STATE_SYM) ? 1 : 0;
     p.numerator_only = (flags & BASED_NUMERATOR_ONLY) ? 1 : 0;
     p.dv = dv;
@@ -1739,8 +1697,8 @@ based_status launch_dv(const void* q, const void* k, const void* v, void* out, f
         return check_launch("prefill_tc_kernel<balanced>");
     }
     if (nseg > 1 && recompute) {
-        if (p.continue_abi) p.ticket = new_ticket();
-        const cudaError_t e = p.continue_abi ? launch_dependent<DV, kModePre, true>(dim3(nseg, BH), stream, tq, tk, tv, to, p)
+        if (continued) p.ticket = new_ticket();
+        const cudaError_t e = continued ? launch_dependent<DV, kModePre, true>(dim3(nseg, BH), stream, tq, tk, tv, to, p)
                                              : launch_dependent<DV, kModePre>(dim3(nseg, BH), stream, tq, tk, tv, to, p);
         if (e != cudaSuccess) return BASED_ERR_CUDA;
         note_launch();
@@ -1748,10 +1706,9 @@ based_status launch_dv(const void* q, const void* k, const void* v, void* out, f
     }
     if (nseg > 1) {
         based_status st;
-        if (p.continue_abi) {
+        if (continued) {
             // the caller's state goes into each head's first slot (see abi_to_slot_kernel); no segment reads it itself
             p.pad = 1;
-            p.continue_abi = 0;
             abi_to_slot_kernel<DV><<<dim3(kF, BH), DV, 0, stream>>>(kv, z, ws, nseg, dv, p.sym);
             note_launch();
             st = check_launch("abi_to_slot_kernel");
@@ -1770,7 +1727,7 @@ based_status launch_dv(const void* q, const void* k, const void* v, void* out, f
     }
     if (nseg > 1) {
         if (launch_dependent<DV, kModeMain>(dim3(nseg, BH), stream, tq, tk, tv, to, p) != cudaSuccess) return BASED_ERR_CUDA;
-    } else if (p.continue_abi) {
+    } else if (continued) {
         prefill_tc_kernel<DV, kModeMain, true><<<dim3(nseg, BH), kThreads, C::kSmemBytes, stream>>>(tq, tk, tv, to, p);
     } else {
         prefill_tc_kernel<DV, kModeMain><<<dim3(nseg, BH), kThreads, C::kSmemBytes, stream>>>(tq, tk, tv, to, p);

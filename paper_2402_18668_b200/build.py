@@ -6,6 +6,7 @@ when their source (or a header) is newer.  nvcc cross-compiles without a GPU.
 from __future__ import annotations
 
 import os
+import shutil
 import subprocess
 import sys
 from concurrent.futures import ThreadPoolExecutor
@@ -31,6 +32,16 @@ def _nvcc() -> str:
         if cand and (os.path.sep not in cand or Path(cand).exists()):
             return cand
     raise RuntimeError("nvcc not found")
+
+
+def _cuda_include() -> str:
+    """The headers of the toolkit that the compiler belongs to: beside its bin folder, links followed."""
+    nvcc = Path(shutil.which(_nvcc()) or _nvcc())
+    for root in (nvcc.parent.parent, nvcc.resolve().parent.parent, Path("/usr/local/cuda")):
+        for inc in (root / "include", root / "targets" / "x86_64-linux" / "include"):
+            if (inc / "cuda_runtime_api.h").exists():
+                return str(inc)
+    raise RuntimeError(f"no CUDA headers beside {nvcc}")
 
 
 def sources():
@@ -63,7 +74,7 @@ def build_native() -> Path:
         r = subprocess.run(
             ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
              "-isystem", str(t / "include"), "-isystem", str(t / "include" / "torch" / "csrc" / "api" / "include"),
-             "-isystem", sysconfig.get_paths()["include"], "-isystem", "/usr/local/cuda/include", "-I", str(INCLUDE),
+             "-isystem", sysconfig.get_paths()["include"], "-isystem", _cuda_include(), "-I", str(INCLUDE),
              str(NATIVE_SRC), "-o", str(tmp), "-L", str(t / "lib"), "-Wl,--no-as-needed", "-lc10", "-lc10_cuda", "-ltorch_cpu",
              "-ltorch", "-ltorch_python", "-L", str(OBJ), "-l:libbased.so", "-Wl,-rpath,$ORIGIN"],
             capture_output=True, text=True)

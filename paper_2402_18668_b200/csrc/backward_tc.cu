@@ -911,6 +911,8 @@ based_status launch_pass(const CUtensorMap& n0, const CUtensorMap& w0, const CUt
 //   64 heads: d_v 64 L 768 34 / 47, L 1024 52 / 54, L 1280 73 / 66; d_v 128 L 768 50 / 59, L 1024 74 / 72
 //   16 heads: d_v 64 L 768 29 / 36, L 1024 36 / 37, L 1536 51 / 42; d_v 128 L 1280 46 / 52, L 1536 53 / 54, L 2048 70 / 55
 //   32 heads: d_v 64 L 1280 46 / 61, L 1536 56 / 66, L 2048 82 / 70; d_v 128 L 1536 74 / 91, L 2048 112 / 101
+// The line at L 768 (d_v 64) is older than these figures, which put the crossing between 768 and 1024 at 128 heads, at 1024
+// at 16 and between 1024 and 1280 at 64: from 768 up to there the tile path would be 2 to 13 us faster.
 // Below 64 heads one CTA per head and block sums the states, and a second short wave of those costs as much as a full one:
 // there the line lies later once the blocks are more than one wave (24 heads are not at L 1536: 54 / 44, 60 / 56).
 // With them at d_v 128 blocks of 512 tokens are the faster from 64 k rows on (256 / 512 tokens: 16 heads L 8192 217 / 206,
@@ -1056,8 +1058,8 @@ based_status launch_dvb(const void* q, const void* k, const void* v, const void*
 // empty initial state): out = (sum_j w_ij v_j) / (sum_j w_ij + eps), w = 1 + s/sqrt(d') + s^2/(2 d').
 // The weights lie over the scores, so at d_v 64 a CTA takes 128 columns of tensor memory and four share an SM, and tiles off
 // the diagonal evaluate two pairs per instruction: B4 H16 L2048 d_v64 80 -> 48 us (looped tiles of 128 rows: 47), 38 with the
-// longest loops first.  With the state asked for it runs beside that kernel (38 + 40 us alone, together 64; 80 + 61 one after
-// the other before).
+// longest loops first (36.7 with the scores' second half loaded ahead).  With the state asked for it is launched beside that
+// kernel, which takes 16 us alone; the call 55 (one after the other, and both kernels slower, 80 + 61 before).
 based_status launch_quadratic_forward_tc(const void* q, const void* k, const void* v, void* out, int BH, int L,
                                          int d_feat, int d_v, int numerator_only, bool overlapped, cudaStream_t stream) {
     CUtensorMap tq, tk64, tv64, tout;

@@ -20,7 +20,7 @@
 // a group's wait, write and hand-over beside them; the rows two steps ahead instead of one change nothing.  An accumulator
 // lane per feature instead, whose thread read both factors of 64 tokens from a transposed k tile, took three times the
 // shared-memory traffic and loaded the value tile once per 128 features: B4 H16 L2048 d_v 64 at d' 8 / 24 / 32 22.7 / 40.5 /
-// 56.1 us, here 12.6 / 16.1 / 27.4; d_v 128 d' 24 50 -> 27; B1 H8 L300 d' 24 8.9 -> 6.9 (with the sums stored straight from
+// 56.1 us, here 12.6 / 16.1 / 25.6; d_v 128 d' 24 50 -> 27; B1 H8 L300 d' 24 8.9 -> 6.9 (with the sums stored straight from
 // tensor memory, a state row's number per element, 24.5 and 15.1).  d' 32 in three parts of 192, two waves: 30.4.
 #include <cuda_bf16.h>
 #include <math.h>

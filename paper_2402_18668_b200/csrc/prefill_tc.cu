@@ -547,7 +547,7 @@ __device__ __noinline__ bool wait_for_readers(const Params& p, volatile uint32_t
 struct Piece { int head, seg, begin, end, first, count, out, head_end, skip; };
 // Every thread of the CTA calls it.  find_piece is the same out of line, with the result in shared memory: how this
 // arithmetic is compiled into the kernel moves the time of the role loops by several per cent either way (register
-// allocation), so each instance of the kernel takes the form that measured faster for it (Cfg::kPieceOutOfLine).
+// allocation), so each instance of the kernel takes the form that measured faster for it (kPieceOut).
 template <int MODE, bool SCAN>
 __device__ __forceinline__ void piece_of_cta(Piece& piece, int* s_rest, int balanced, int heads, int pad, int L, int seg_len, int nseg) {
     bool skip = false;

@@ -15,8 +15,8 @@
 // Every operand lies along its product's summation index (f32_tiles.cuh).  Outputs: a warp owns 16 query rows and a slice of
 // the features; four slices' groups of 16 rows make a full chunk's eight warps two slices, a chunk of at most 32 (16) tokens
 // has four (eight), and the slices' sums meet in shared memory.
-// Bound: issue slots and latency (per full chunk and SM 27 k cycles, of which the FMA pipe needs 14 k; 11 k instructions per
-// scheduler, 6.6 k of them multiply-adds); at few heads the chain of steps.  Against one CTA per head that walked the tokens
+// Bound: issue slots and latency (per full chunk and SM 28 k cycles, the FMA pipe busy in 12.6 k of them; 11 k instructions per
+// scheduler, 6.8 k of them multiply-adds); at few heads the chain of steps.  Against one CTA per head that walked the tokens
 // one by one: B1 H2 L256 d_v64 190 -> 15 us, B2 H16 L1024 d_v64 660 -> 74.  An earlier form with the operands row by row
 // along the summation index (even and odd terms in one two-wide FMA) took 22 and 92: twice the shared-memory passes, and
 // chunks of 16 tokens used a quarter of the warps' rows.

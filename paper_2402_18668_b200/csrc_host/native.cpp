@@ -521,11 +521,15 @@ PyObject* linear_attention(PyObject* const* a) {
 }
 
 // ---------------------------------------------------------------------------------------------- module
-// The faults of this file first; everything else is torch's to translate: its own error types, and Python exceptions that
-// passed through C++ (python_error, from a saved-tensor hook for instance), which go on as they are.
+// Everything but the faults of this file is torch's to translate: its own error types, and Python exceptions that passed
+// through C++ (python_error, from a saved-tensor hook for instance), which go on as they are.
+PyObject* translated(std::exception_ptr fault) {
+    HANDLE_TH_ERRORS
+    std::rethrow_exception(fault);
+    END_HANDLE_TH_ERRORS
+}
 template <PyObject* (*F)(PyObject* const*), int N>
 PyObject* guarded(PyObject*, PyObject* const* args, Py_ssize_t n) {
-    HANDLE_TH_ERRORS
     try {
         if (n != N) throw TypeFault("wrong number of arguments");
         return F(args);
@@ -535,9 +539,10 @@ PyObject* guarded(PyObject*, PyObject* const* args, Py_ssize_t n) {
         PyErr_SetString(PyExc_TypeError, e.what());
     } catch (const std::invalid_argument& e) {
         PyErr_SetString(PyExc_ValueError, e.what());
+    } catch (...) {
+        return translated(std::current_exception());
     }
     return nullptr;
-    END_HANDLE_TH_ERRORS
 }
 template <PyObject* (*F)(PyObject* const*), int N> PyMethodDef method(const char* name) {
     return {name, reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&guarded<F, N>)), METH_FASTCALL, nullptr};

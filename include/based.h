@@ -93,6 +93,14 @@ based_status based_prefill(const void* q, const void* k, const void* v, void* ou
 size_t based_prefill_workspace_bytes(int B, int H, int L, int d_feat, int d_v, based_dtype io);
 
 /*
+ * Scratch with which an fp32 call runs on the tensor cores, its operands split into three bf16 parts each (results at least
+ * as close to exact ones as fp32 multiply-adds give): based_prefill without a state (backward = 0) and the backward pass at
+ * d_v 64 (backward = 1) take that route when their workspace has this many bytes, else one that needs no scratch or
+ * based_prefill_backward_workspace_bytes.  0: there is no such route for these arguments, or it is not the faster one.
+ */
+size_t based_f32_parts_bytes(int B, int H, int L, int d_feat, int d_v, int backward);
+
+/*
  * The recurrent state of a token block without its outputs (Sec. 4.1, recurrent view):
  *   kv_state (+)= sum_j phi(k_j) v_j^T,   z_state (+)= sum_j phi(k_j)
  * exactly what based_prefill leaves in kv_state / z_state for the same k, v, flags, at about a
@@ -212,8 +220,8 @@ based_status swa_decode_step(const void* q, const void* k, const void* v, void* 
  * Supported: d_feat = 16 with io in {F32, BF16}, d_feat in {8, 24, 32} with BF16 io (w = 1 + s/sqrt(d') +
  * s^2/(2 d'), so ds_ij = (a_i . v_j + b_i)(1/sqrt(d') + q_i.k_j / d')); d_v in {64, 112, 128}.
  * Both paths evaluate the quadratic form, O(L^2) per head, on 128 x 128 (bf16 io: tcgen05 tensor
- * cores, bf16 operands, fp32 accumulation) or 64 x 64 (fp32 io: fp32 FMAs) tiles of (query, key)
- * pairs; with bf16 io and d_feat = 16 longer sequences take the block-wise path described at
+ * cores, bf16 operands, fp32 accumulation) or 64 x 64 (fp32 io: fp32 FMAs; with the scratch of
+ * based_f32_parts_bytes 128 x 64, tensor cores) tiles of (query, key) pairs; with bf16 io and d_feat = 16 longer sequences take the block-wise path described at
  * based_prefill_backward_with_out (the forward output that it needs is recomputed into the workspace:
  * one forward pass more).  Gradient outputs must not alias inputs.
  */

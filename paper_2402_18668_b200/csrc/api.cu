@@ -97,6 +97,12 @@ size_t based_prefill_workspace_bytes(int B, int H, int L, int d_feat, int d_v, b
     return prefill_tc_workspace_bytes(B * H, L, d_v);
 }
 
+size_t based_f32_parts_bytes(int B, int H, int L, int d_feat, int d_v, int backward) {
+    if (B <= 0 || H <= 0 || L <= 0 || d_feat != kDFeat || !dv_ok(d_v)) return 0;
+    const int heads = (long long)B * H > kHeadSlab ? (int)kHeadSlab : B * H;       // the largest slab of heads
+    return quadratic_f32_workspace_bytes(heads, L, d_v, backward != 0);
+}
+
 static based_status prefill_impl(const void* q, const void* k, const void* v, void* out, float* kv_state, float* z_state,
                                  int B, int H, int L, int d_feat, int d_v, based_dtype io, int flags, void* workspace,
                                  size_t workspace_bytes, void* cuda_stream, bool fit) {
@@ -148,6 +154,12 @@ static based_status prefill_impl(const void* q, const void* k, const void* v, vo
     if (io == BASED_BF16)
         return launch_prefill_tc(q, k, v, out, kv_state, z_state, B * H, L, d_v, flags, workspace,
                                  static_cast<cudaStream_t>(cuda_stream), fit ? workspace_bytes : ~(size_t)0);
+    const size_t parts = based_f32_parts_bytes(B, H, L, d_feat, d_v, 0);
+    if (!kv_state && parts > 0 && workspace && workspace_bytes >= parts) {
+        auto in = [](const void* p) { return static_cast<const float*>(p); };
+        return launch_quadratic_forward_f32(in(q), in(k), in(v), static_cast<float*>(out), workspace, B * H, L, d_v,
+                                            (flags & BASED_NUMERATOR_ONLY) ? 1 : 0, static_cast<cudaStream_t>(cuda_stream));
+    }
     return launch_prefill_f32(q, k, v, out, kv_state, z_state, B * H, L, d_v, flags,
                               static_cast<cudaStream_t>(cuda_stream));
 }
@@ -531,6 +543,11 @@ static based_status prefill_backward(const void* q, const void* k, const void* v
                                           d_feat, d_v, (flags & BASED_NUMERATOR_ONLY) ? 1 : 0,
                                           static_cast<cudaStream_t>(cuda_stream));
     auto in = [](const void* p) { return static_cast<const float*>(p); };
+    const size_t parts = based_f32_parts_bytes(B, H, L, d_feat, d_v, 1);
+    if (parts > 0 && workspace_bytes >= parts)
+        return launch_quadratic_backward_f32(in(q), in(k), in(v), in(dout), static_cast<float*>(dq), static_cast<float*>(dk),
+                                             static_cast<float*>(dv), workspace, B * H, L, (flags & BASED_NUMERATOR_ONLY) ? 1 : 0,
+                                             static_cast<cudaStream_t>(cuda_stream));
     return launch_prefill_backward_f32(in(q), in(k), in(v), in(dout), static_cast<float*>(dq), static_cast<float*>(dk),
                                        static_cast<float*>(dv), static_cast<float*>(workspace), B * H, L, d_v,
                                        (flags & BASED_NUMERATOR_ONLY) ? 1 : 0, static_cast<cudaStream_t>(cuda_stream));

@@ -163,6 +163,13 @@ based_status launch_baseconv(const void* a, const void* g, const float* h, const
 based_status launch_prefill_backward_f32(const float* q, const float* k, const float* v, const float* g, float* dq, float* dk,
                                          float* dv, float* stats, int BH, int L, int d_v, int numerator_only,
                                          cudaStream_t stream);
+// fp32 io in definition form on the tensor cores, operands in three bf16 parts (quadratic_f32_tc.cu): outputs from the empty
+// state, and the backward pass.  quadratic_f32_workspace_bytes: 0 where the other fp32 kernels are the faster
+size_t quadratic_f32_workspace_bytes(int BH, int L, int d_v, bool backward);
+based_status launch_quadratic_forward_f32(const float* q, const float* k, const float* v, float* out, void* ws, int BH, int L,
+                                          int d_v, int numerator_only, cudaStream_t stream);
+based_status launch_quadratic_backward_f32(const float* q, const float* k, const float* v, const float* g, float* dq, float* dk,
+                                           float* dv, void* ws, int BH, int L, int numerator_only, cudaStream_t stream);
 // feature dimensions 8, 24, 32 (fp32 FMA, definition form); state layout [1 + d' + d'^2, d_v]
 based_status launch_prefill_generic(const void* q, const void* k, const void* v, void* out, float* kv, float* z,
                                     int BH, int L, int d_feat, int d_v, based_dtype io, int flags,

@@ -12,6 +12,7 @@
 #include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 
+#include <algorithm>
 #include <stdexcept>
 #include <string>
 
@@ -132,6 +133,9 @@ Tensor workspace_of(const Tensor& given, size_t bytes, const Tensor& like) {
     if (bytes == 0 || (given.defined() && given.nbytes() >= bytes)) return given;
     return at::empty({static_cast<int64_t>(bytes)}, like.options().dtype(at::kByte));
 }
+// scratch that a call can do without is taken on the current stream only: on another one it could be handed out again while
+// the call still runs
+bool on_current(void* stream) { return stream == c10::cuda::getCurrentCUDAStream().stream(); }
 size_t bytes_of(const Tensor& t) { return t.defined() ? t.nbytes() : 0; }
 // the library's calls run without the interpreter lock: a launch can wait for room in the stream's queue
 template <typename F> based_status unlocked(F f) {
@@ -150,6 +154,7 @@ Tensor prefill_call(const Tensor& q, const Tensor& k, const Tensor& v, const Ten
     if (!out.defined()) out = at::empty_like(v);
     size_t need = based_prefill_workspace_bytes(B, H, L, d_feat, d_v, io);
     if (need <= BASED_WORDS_BYTES && !(flags & BASED_STATE_CONTINUE)) need = 0;
+    if (io == BASED_F32 && !kv.defined() && on_current(stream)) need = based_f32_parts_bytes(B, H, L, d_feat, d_v, 0);
     const Tensor ws = workspace_of(workspace, need, q);
     check(based_prefill(cptr(q), cptr(k), cptr(v), ptr(out), fptr(kv), fptr(z), B, H, L, d_feat, d_v, io, flags, ptr(ws),
                         bytes_of(ws), stream),
@@ -161,7 +166,9 @@ Gradients backward_call(const Tensor& q, const Tensor& k, const Tensor& v, const
                         const Tensor& workspace, void* stream) {
     const int B = size(q, 0), H = size(q, 1), L = size(q, 2), d_feat = size(q, 3), d_v = size(v, 3);
     const based_dtype io = dtype_code(q);
-    const Tensor ws = workspace_of(workspace, based_prefill_backward_workspace_bytes(B, H, L, d_v, io), q);
+    size_t need = based_prefill_backward_workspace_bytes(B, H, L, d_v, io);
+    if (io == BASED_F32 && on_current(stream)) need = std::max(need, based_f32_parts_bytes(B, H, L, d_feat, d_v, 1));
+    const Tensor ws = workspace_of(workspace, need, q);
     Gradients g{at::empty_like(q), at::empty_like(k), at::empty_like(v)};
     const based_status st =
         out.defined() ? based_prefill_backward_with_out(cptr(q), cptr(k), cptr(v), cptr(out), cptr(dout), ptr(g.dq), ptr(g.dk),

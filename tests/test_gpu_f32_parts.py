@@ -1,0 +1,91 @@
+"""fp32 forward and backward on the tensor cores (operands in three bf16 parts): lengths at the edges of the own tiles (128)
+and looped tiles (64), loops shared by one to eight CTAs, longest loops first and not, every value width, both forms."""
+import ctypes
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2402_18668_b200 as based
+from paper_2402_18668_b200 import workloads as wl
+from parity import TOL_F32, row_err
+
+pytestmark = pytest.mark.gpu
+
+# Sums of up to a few hundred products, each good to 2^-24 of its size: 2^-24 sqrt(300) = 1e-6 of a head's largest entry, a few
+# times that at the worst entry of thousands (fp32 multiply-adds pair by pair: 1 to 4e-6 on these)
+TOL = 1e-5
+
+
+def inputs(BH, L, d_v, seed):
+    w = wl.Workload("parts", 1, BH, L, 16, d_v, "f32", 1.0)
+    gen = wl.generator(seed)
+    return (*wl.prefill_inputs(w, gen), torch.randn(1, BH, L, d_v, generator=gen))
+
+
+@pytest.mark.parametrize("d_v", [64, 112, 128])
+@pytest.mark.parametrize("BH,L", [(2, 33), (1, 64), (3, 65), (2, 127), (150, 128), (2, 129), (1, 193), (80, 200), (1, 513), (40, 500)])
+@pytest.mark.parametrize("flags", [0, based.BASED_NUMERATOR_ONLY])
+def test_f32_parts(BH, L, d_v, flags):
+    q, k, v, g = inputs(BH, L, d_v, BH * 1000 + L + d_v)
+    lib, heads = based.binding.lib(), sorted({0, BH // 2, BH - 1})
+    x = [t.cuda() for t in (q, k, v, g)]
+    s = [wl.to_f64(t[:, heads]) for t in (q, k, v, g)]
+    before = based.launch_count()
+    y = based.based_prefill(*x[:3], flags=flags)
+    assert based.launch_count() - before == 2                    # parts, outputs
+    want, _, _ = oracle.linattn_quadratic(*s[:3])
+    if flags:
+        c = s[0] @ s[1].swapaxes(-1, -2)
+        want = want * np.tril(1 + c / 4 + c * c / 32).sum(-1, keepdims=True)
+    assert row_err(wl.to_f64(y[:, heads]), want) <= TOL_F32
+    assert np.abs(wl.to_f64(y[:, heads]) - want).max() <= TOL * np.abs(want).max()
+    # without scratch: the chunked kernel
+    plain = torch.empty_like(y)
+    p = lambda t: ctypes.c_void_p(t.data_ptr())
+    stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    assert lib.based_prefill(p(x[0]), p(x[1]), p(x[2]), p(plain), None, None, 1, BH, L, 16, d_v, 0, flags, None, 0, stream) == 0
+    assert row_err(wl.to_f64(plain[:, heads]), want) <= TOL_F32
+    if d_v == 64:
+        got = based.based_prefill_backward(*x, flags=flags)
+        for a, b in zip(got, oracle.linattn_backward(*s, numerator_only=bool(flags))):
+            assert np.abs(wl.to_f64(a[:, heads]) - b).max() <= TOL * np.abs(b).max()
+        assert all(torch.equal(a, b) for a, b in zip(got, based.based_prefill_backward(*x, flags=flags)))
+        # with the scratch of the call without parts
+        n = lib.based_prefill_backward_workspace_bytes(1, BH, L, 64, 0)
+        ws, old = torch.empty(n, dtype=torch.uint8, device="cuda"), [torch.empty_like(t) for t in x[:3]]
+        assert lib.based_prefill_backward(*(p(t) for t in x), *(p(t) for t in old), 1, BH, L, 16, 64, 0, flags, p(ws), n, stream) == 0
+        for a, b in zip(got, old):
+            assert (a - b).abs().max() <= 2 * TOL * b.abs().max()
+    assert based.based_poll_error() == based.BASED_OK
+
+
+@pytest.mark.parametrize("d_v", [64, 128])
+def test_f32_parts_outputs_on_sixteen_bytes(d_v):
+    """Arrays that start on a 16-byte boundary only."""
+    q, k, v, g = (t.cuda() for t in inputs(2, 150, d_v, 5))
+    off = [torch.empty(t.numel() + 4, device="cuda")[4:].view(t.shape).copy_(t) for t in (q, k, v, g)]
+    out = torch.empty(v.numel() + 4, device="cuda")[4:].view(v.shape)
+    based.based_prefill(*off[:3], out=out)
+    assert torch.equal(out, based.based_prefill(q, k, v))
+
+
+@pytest.mark.parametrize("big", [1e30, 3.4e38])
+@pytest.mark.parametrize("BH,L", [(2, 200), (150, 100)])
+def test_f32_parts_of_large_values(BH, L, big):
+    """Values whose first part is next to the largest bf16, or rounds past it, and their rows' neighbours."""
+    q, k, v, g = (t.cuda() for t in inputs(BH, L, 64, 7))
+    at = L // 2
+    vb = v.clone()
+    vb[:, :, at, 3] = big
+    want = based.based_prefill(q, k, v)
+    out = based.based_prefill(q, k, vb)
+    assert torch.allclose(out[:, :, :at], want[:, :, :at], rtol=0, atol=1e-4)
+    cols = [c for c in range(64) if c != 3]
+    assert torch.allclose(out[..., cols], want[..., cols], rtol=0, atol=1e-4)
+    w = wl.to_f64(vb[:, :1])
+    ref, _, _ = oracle.linattn_quadratic(wl.to_f64(q[:, :1]), wl.to_f64(k[:, :1]), w)
+    ok = np.abs(ref) < 1e38                                       # (a sum over D that would overflow in fp32 is infinite or NaN)
+    got = out[:, :1].double().cpu().numpy()
+    assert (np.abs(got - ref)[ok] <= 1e-4 * np.maximum(np.abs(ref), 1.0)[ok])[np.isfinite(got)[ok]].all()

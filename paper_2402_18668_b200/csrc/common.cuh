@@ -206,6 +206,9 @@ based_status launch_prefill_backward_tc(const void* q, const void* k, const void
 // kernel before it in the stream (launch_state_generic_tc's, which lets it), whose results it does not use
 based_status launch_quadratic_forward_tc(const void* q, const void* k, const void* v, void* out, int BH, int L,
                                          int d_feat, int d_v, int numerator_only, bool overlapped, cudaStream_t stream);
+// the same with two groups of row warps per CTA (quadratic_fwd_tc.cu)
+based_status launch_quadratic_groups_tc(const void* q, const void* k, const void* v, void* out, int BH, int L,
+                                        int d_feat, int d_v, int numerator_only, bool overlapped, cudaStream_t stream);
 // load the generation-step kernels into the current context
 based_status preload_decode();
 based_status preload_swa_decode();

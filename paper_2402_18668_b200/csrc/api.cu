@@ -545,7 +545,7 @@ static based_status prefill_backward(const void* q, const void* k, const void* v
     auto in = [](const void* p) { return static_cast<const float*>(p); };
     const size_t parts = based_f32_parts_bytes(B, H, L, d_feat, d_v, 1);
     if (parts > 0 && workspace_bytes >= parts)
-        return launch_quadratic_backward_f32(in(q), in(k), in(v), in(dout), static_cast<float*>(dq), static_cast<float*>(dk),
+        return launch_quadratic_backward_f32(in(q), in(k), in(v), in(dout), 0, static_cast<float*>(dq), static_cast<float*>(dk),
                                              static_cast<float*>(dv), workspace, B * H, L, (flags & BASED_NUMERATOR_ONLY) ? 1 : 0,
                                              static_cast<cudaStream_t>(cuda_stream));
     return launch_prefill_backward_f32(in(q), in(k), in(v), in(dout), static_cast<float*>(dq), static_cast<float*>(dk),
@@ -567,6 +567,25 @@ based_status based_prefill_backward_with_out(const void* q, const void* k, const
     if (!out || out == dq || out == dk || out == dv) return BASED_ERR_INVALID_ARG;
     return prefill_backward(q, k, v, out, dout, dq, dk, dv, B, H, L, d_feat, d_v, io, flags, workspace,
                             workspace_bytes, cuda_stream);
+}
+
+based_status based_prefill_backward_tokens_first(const void* q, const void* k, const void* v, const void* dout, void* dq, void* dk,
+                                                 void* dv, int B, int H, int L, int d_feat, int d_v, based_dtype io, int flags,
+                                                 void* workspace, size_t workspace_bytes, void* cuda_stream) {
+    if (!q || !k || !v || !dout || !dq || !dk || !dv || B <= 0 || H <= 0 || L <= 0) return BASED_ERR_INVALID_ARG;
+    if (flags & ~BASED_NUMERATOR_ONLY) return BASED_ERR_INVALID_ARG;
+    if (dq == q || dq == k || dk == q || dk == k || dv == v || dv == dout) return BASED_ERR_INVALID_ARG;
+    // one slab of heads, rows counted in 32 bits
+    const size_t parts = io == BASED_F32 ? based_f32_parts_bytes(B, H, L, d_feat, d_v, 1) : 0;
+    if (parts == 0 || (long long)B * H > kHeadSlab || (long long)B * H * L > 0x7fffffffLL) return BASED_ERR_UNSUPPORTED;
+    if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(dout) || !aligned16(dq) || !aligned16(dk) || !aligned16(dv) ||
+        !aligned16(workspace))
+        return BASED_ERR_ALIGNMENT;
+    if (!workspace || workspace_bytes < parts) return BASED_ERR_WORKSPACE;
+    auto in = [](const void* p) { return static_cast<const float*>(p); };
+    return launch_quadratic_backward_f32(in(q), in(k), in(v), in(dout), H, static_cast<float*>(dq), static_cast<float*>(dk),
+                                         static_cast<float*>(dv), workspace, B * H, L, (flags & BASED_NUMERATOR_ONLY) ? 1 : 0,
+                                         static_cast<cudaStream_t>(cuda_stream));
 }
 
 based_status based_tokens_to_heads(const void* src, void* dst, int B, int H, int L, int row_bytes, void* cuda_stream) {

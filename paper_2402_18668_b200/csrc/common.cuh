@@ -168,8 +168,9 @@ based_status launch_prefill_backward_f32(const float* q, const float* k, const f
 size_t quadratic_f32_workspace_bytes(int BH, int L, int d_v, bool backward);
 based_status launch_quadratic_forward_f32(const float* q, const float* k, const float* v, float* out, void* ws, int BH, int L,
                                           int d_v, int numerator_only, cudaStream_t stream);
-based_status launch_quadratic_backward_f32(const float* q, const float* k, const float* v, const float* g, float* dq, float* dk,
-                                           float* dv, void* ws, int BH, int L, int numerator_only, cudaStream_t stream);
+// dout_H: 0, or H where g lies [B, L, H, d_v]
+based_status launch_quadratic_backward_f32(const float* q, const float* k, const float* v, const float* g, int dout_H, float* dq,
+                                           float* dk, float* dv, void* ws, int BH, int L, int numerator_only, cudaStream_t stream);
 // feature dimensions 8, 24, 32 (fp32 FMA, definition form); state layout [1 + d' + d'^2, d_v]
 based_status launch_prefill_generic(const void* q, const void* k, const void* v, void* out, float* kv, float* z,
                                     int BH, int L, int d_feat, int d_v, based_dtype io, int flags,

@@ -37,6 +37,7 @@
 
 #include <mutex>
 #include <type_traits>
+#include <utility>
 
 #include "common.cuh"
 #include "sm100.cuh"
@@ -93,6 +94,8 @@ struct QParams {
     const float* m;                                  // kDq: the centres m_i = G_i.v_i, [heads][L]
     int pitch;                                       // L rounded up to whole looped tiles
     float *out_n, *out_w;                            // dq or dk; the forward output or dv
+    // dout may lie [B, L, H, d_v] (own side of kDq, looped side of kKeys): then H, and the slab's first head; else H = 0
+    int dout_H, dout_h0;
     unsigned int* err;
     int heads, L, dvw, numerator_only, by_length, nsplit;   // nsplit: CTAs of a cluster that share an own tile's loop
 };
@@ -163,6 +166,14 @@ __device__ __forceinline__ void store8(float* dst, const float (&x)[8]) {
                  : "memory");
 }
 
+// offset of a head's first row of dout and the distance of its rows
+__device__ __forceinline__ size_t dout_rows(int H, int h0, size_t head, int L, int W, int& pitch) {
+    pitch = W;
+    if (H == 0) return head * (size_t)L * W;
+    pitch = H * W;
+    const size_t g = h0 + head, b = g / H;
+    return (b * L * H + (g - b * H)) * W;
+}
 // The rows of a warp, a lane each, by plain multiply-adds, pair by pair: the narrow results (dq, dk) of lanes with need_n, the
 // wide ones (the output, dv) of those with need_w.  buf: kPlainFloats of shared memory of the warp's own, for 32 looped rows at a
 // time.
@@ -173,7 +184,10 @@ __device__ __noinline__ void plain_rows(const QParams& p, float* buf, size_t hea
     const int r = min(row, p.L - 1), W = p.dvw, L = p.L, lane = threadIdx.x & 31;
     const size_t hn = head * (size_t)L * kDFeat, hw = head * (size_t)L * W, hs = head * (size_t)p.pitch;
     const int from = MODE == kKeys ? __reduce_min_sync(~0u, r) : 0, to = MODE == kKeys ? L - 1 : __reduce_max_sync(~0u, r);
-    const float *loop_n = p.loop_n + hn, *loop_w = p.loop_w + hw;
+    int own_pitch = W, loop_pitch = W;
+    const float* own_w = MODE == kFwd ? nullptr : p.own_w + (MODE == kDq ? dout_rows(p.dout_H, p.dout_h0, head, L, W, own_pitch) : hw);
+    const float *loop_n = p.loop_n + hn,
+                *loop_w = p.loop_w + (MODE == kKeys ? dout_rows(p.dout_H, p.dout_h0, head, L, W, loop_pitch) : hw);
     float xn[kDFeat];
     auto row4 = [](float (&d)[kDFeat], const float* src) {
 #pragma unroll
@@ -202,7 +216,7 @@ __device__ __noinline__ void plain_rows(const QParams& p, float* buf, size_t hea
         }
         for (int e = lane; e < 8 * cols; e += 32) {
             const int i = e / (cols / 4), t = min(j + i, L - 1), u = 4 * (e % (cols / 4));
-            *reinterpret_cast<float4*>(buf + i * kPlainPitch + kDFeat + u) = __ldg(reinterpret_cast<const float4*>(loop_w + (size_t)t * W + c + u));
+            *reinterpret_cast<float4*>(buf + i * kPlainPitch + kDFeat + u) = __ldg(reinterpret_cast<const float4*>(loop_w + (size_t)t * loop_pitch + c + u));
         }
         if (MODE == kKeys) {
             const int t = min(j + lane, L - 1);
@@ -214,7 +228,7 @@ __device__ __noinline__ void plain_rows(const QParams& p, float* buf, size_t hea
     float den = 0.f;
     if (MODE != kFwd && __any_sync(~0u, need_n)) {
         constexpr int DV = 64;
-        const float* own = p.own_w + hw + (size_t)r * DV;
+        const float* own = own_w + (size_t)r * own_pitch;
         float m = 0.f, num = 0.f, x[kDFeat] = {}, y[kDFeat] = {};
         if (MODE == kDq && !p.numerator_only)
             for (int c = 0; c < DV; ++c) m = fmaf(own[c], loop_w[(size_t)r * DV + c], m);
@@ -290,7 +304,8 @@ __device__ __noinline__ void plain_rows(const QParams& p, float* buf, size_t hea
     }
 }
 
-// fp32 rows of W values as bf16 rows of 3 W: the first parts, the second, the third.  A block takes 1024 pieces of eight
+// fp32 rows of W values as bf16 rows of 3 W: the first parts, the second, the third.  dout is read as it comes back from a
+// projection, the heads of a token side by side: no copy ahead (5 us of a training step at B2 H16 L1024).  A block takes 1024 pieces of eight
 // values of one tensor, four per thread, all loads under way at once.
 struct SplitSet {
     const float* src[4];
@@ -299,6 +314,7 @@ struct SplitSet {
     unsigned end[4];                                 // blocks of the tensors up to and with this one
     long long total[4];                              // pieces of the tensor
     float* m;                                        // products of the third and the fourth tensor's rows (d_v 64)
+    unsigned L, H, h0;                               // the fourth tensor lies [B, L, H, W], h0 the slab's first head; H = 0: as the others
 };
 constexpr int kSplitPer = 4, kSplitBlock = 256 * kSplitPer;
 __global__ void __launch_bounds__(256) split_parts_kernel(const SplitSet s) {
@@ -309,15 +325,23 @@ __global__ void __launch_bounds__(256) split_parts_kernel(const SplitSet s) {
     const long long e0 = (long long)block * kSplitBlock, left = s.total[i] - e0;
     const long long row0 = e0 / n;
     const unsigned c0 = (unsigned)(e0 - row0 * n);
-    const float4* src = reinterpret_cast<const float4*>(s.src[i]) + 2 * e0;
+    const float4* src = reinterpret_cast<const float4*>(s.src[i]);
+    const bool strided = i == 3 && s.H != 0;
+    auto at = [&](unsigned e) -> long long {         // piece e of the block
+        if (!strided) return e0 + e;
+        const unsigned row = (unsigned)row0 + (c0 + e) / n, c = (c0 + e) % n, g = row / s.L, l = row - g * s.L;
+        const unsigned b = (s.h0 + g) / s.H, h = s.h0 + g - b * s.H;
+        return (((long long)b * s.L + l) * s.H + h) * n + c;
+    };
     uint4* dst = reinterpret_cast<uint4*>(s.dst[i]) + row0 * (3 * n);
     float4 a[kSplitPer], b[kSplitPer];
 #pragma unroll
     for (int u = 0; u < kSplitPer; ++u) {
         const unsigned e = u * 256 + threadIdx.x;
         if (e < left) {
-            a[u] = __ldg(src + 2 * e);
-            b[u] = __ldg(src + 2 * e + 1);
+            const long long from = 2 * at(e);
+            a[u] = __ldg(src + from);
+            b[u] = __ldg(src + from + 1);
         }
     }
 #pragma unroll
@@ -502,10 +526,15 @@ __global__ void __launch_bounds__(kNThreads, 1)
         const int h = (int)head;
         if (lead && n > 0) {
             mbar_arrive_expect_tx(&bars[bOwn], kOwn * 128 + (C::kBwd ? 3 * C::kOwnPart : 0));
-            tma_load_3d(smem + C::offOwnN, &tm_own_n, &bars[bOwn], 0, r0, h);
-            if (C::kBwd)
+            // (boxes of 64 rows: one map per tensor for both sides)
 #pragma unroll
-                for (int a = 0; a < 3; ++a) tma_load_3d(smem + C::offOwnW + a * C::kOwnPart, &tm_own_w, &bars[bOwn], a * DV, r0, h);
+            for (int u = 0; u < 2; ++u) {
+                tma_load_3d(smem + C::offOwnN + u * (kLT * 128), &tm_own_n, &bars[bOwn], 0, r0 + u * kLT, h);
+                if (C::kBwd)
+#pragma unroll
+                    for (int a = 0; a < 3; ++a)
+                        tma_load_3d(smem + C::offOwnW + a * C::kOwnPart + u * (kLT * 128), &tm_own_w, &bars[bOwn], a * DV, r0 + u * kLT, h);
+            }
         }
         for (int t = 0; t < n && ok; ++t) {
             const int s = t % C::kNS, row = (first + t) * kLT;
@@ -859,8 +888,10 @@ Parts parts_of(void* ws, int BH, int L, int d_v, bool backward) {
     x.bytes = off;
     return x;
 }
-based_status split_parts(const float* const (&src)[4], const Parts& x, int heads, int L, int d_v, bool centres, cudaStream_t stream) {
+based_status split_parts(const float* const (&src)[4], const Parts& x, int heads, int L, int d_v, bool centres, int dout_H, int h0,
+                         cudaStream_t stream) {
     SplitSet s{};
+    s.L = L; s.H = dout_H; s.h0 = h0;
     s.m = centres ? x.m : nullptr;
     __nv_bfloat16* const dst[4] = {x.n[0], x.n[1], x.w[0], x.w[1]};
     unsigned end = 0;
@@ -876,11 +907,11 @@ based_status split_parts(const float* const (&src)[4], const Parts& x, int heads
     note_launch();
     return check_launch("split_parts_kernel");
 }
-bool narrow_map(CUtensorMap* m, const void* base, int heads, int L, int rows) {
-    return make_rows_map_bf16(m, base, heads, L, 3 * kDFeat, 64, rows, CU_TENSOR_MAP_SWIZZLE_128B);
+bool narrow_map(CUtensorMap* m, const void* base, int heads, int L) {
+    return make_rows_map_bf16(m, base, heads, L, 3 * kDFeat, 64, kLT, CU_TENSOR_MAP_SWIZZLE_128B);
 }
-bool wide_map(CUtensorMap* m, const void* base, int heads, int L, int d_v, int rows) {
-    return make_rows_map_bf16(m, base, heads, L, 3 * d_v, 64, rows, CU_TENSOR_MAP_SWIZZLE_128B);
+bool wide_map(CUtensorMap* m, const void* base, int heads, int L, int d_v) {
+    return make_rows_map_bf16(m, base, heads, L, 3 * d_v, 64, kLT, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 }  // namespace
 
@@ -905,11 +936,11 @@ based_status launch_quadratic_forward_f32(const float* q, const float* k, const 
         p.own_n = q + h0 * hn; p.loop_n = k + h0 * hn; p.loop_w = v + h0 * hw; p.out_w = out + h0 * hw;
         p.L = L; p.dvw = d_v; p.numerator_only = numerator_only;
         const float* const src[4] = {p.own_n, p.loop_n, p.loop_w, nullptr};
-        based_status st = split_parts(src, x, p.heads, L, d_v, false, stream);
+        based_status st = split_parts(src, x, p.heads, L, d_v, false, 0, 0, stream);
         if (st != BASED_OK) return st;
         Maps m;
-        if (!narrow_map(&m.own_n, x.n[0], p.heads, L, kOwn) || !narrow_map(&m.loop_n, x.n[1], p.heads, L, kLT) ||
-            !wide_map(&m.loop_w, x.w[0], p.heads, L, d_v, kLT))
+        if (!narrow_map(&m.own_n, x.n[0], p.heads, L) || !narrow_map(&m.loop_n, x.n[1], p.heads, L) ||
+            !wide_map(&m.loop_w, x.w[0], p.heads, L, d_v))
             return BASED_ERR_CUDA;
         m.own_w = m.own_n;
         st = d_v == 64 ? launch_quadratic<64, kFwd>(m, p, stream) : launch_quadratic<128, kFwd>(m, p, stream);
@@ -918,8 +949,8 @@ based_status launch_quadratic_forward_f32(const float* q, const float* k, const 
     return BASED_OK;
 }
 
-based_status launch_quadratic_backward_f32(const float* q, const float* k, const float* v, const float* g, float* dq, float* dk,
-                                           float* dv, void* ws, int BH, int L, int numerator_only, cudaStream_t stream) {
+based_status launch_quadratic_backward_f32(const float* q, const float* k, const float* v, const float* g, int dout_H, float* dq,
+                                           float* dk, float* dv, void* ws, int BH, int L, int numerator_only, cudaStream_t stream) {
     constexpr int DV = 64;
     const Parts x = parts_of(ws, BH, L, DV, true);
     const size_t hn = (size_t)L * kDFeat, hw = (size_t)L * DV;
@@ -928,19 +959,19 @@ based_status launch_quadratic_backward_f32(const float* q, const float* k, const
         p.heads = BH - h0 < x.heads ? BH - h0 : x.heads;
         p.L = L; p.dvw = DV; p.numerator_only = numerator_only;
         p.inv = x.inv; p.b = x.b; p.m = x.m; p.pitch = (L + kLT - 1) / kLT * kLT;
-        const float* const src[4] = {q + h0 * hn, k + h0 * hn, v + h0 * hw, g + h0 * hw};
-        based_status st = split_parts(src, x, p.heads, L, DV, !numerator_only, stream);
+        p.dout_H = dout_H; p.dout_h0 = h0;
+        const float* const src[4] = {q + h0 * hn, k + h0 * hn, v + h0 * hw, dout_H ? g : g + h0 * hw};
+        based_status st = split_parts(src, x, p.heads, L, DV, !numerator_only, dout_H, h0, stream);
         if (st != BASED_OK) return st;
         Maps m;
-        if (!narrow_map(&m.own_n, x.n[0], p.heads, L, kOwn) || !wide_map(&m.own_w, x.w[1], p.heads, L, DV, kOwn) ||
-            !narrow_map(&m.loop_n, x.n[1], p.heads, L, kLT) || !wide_map(&m.loop_w, x.w[0], p.heads, L, DV, kLT))
+        if (!narrow_map(&m.own_n, x.n[0], p.heads, L) || !wide_map(&m.own_w, x.w[1], p.heads, L, DV) ||
+            !narrow_map(&m.loop_n, x.n[1], p.heads, L) || !wide_map(&m.loop_w, x.w[0], p.heads, L, DV))
             return BASED_ERR_CUDA;
         p.own_n = src[0]; p.own_w = src[3]; p.loop_n = src[1]; p.loop_w = src[2];
         p.out_n = dq + h0 * hn;
         if ((st = launch_quadratic<DV, kDq>(m, p, stream)) != BASED_OK) return st;
-        if (!narrow_map(&m.own_n, x.n[1], p.heads, L, kOwn) || !wide_map(&m.own_w, x.w[0], p.heads, L, DV, kOwn) ||
-            !narrow_map(&m.loop_n, x.n[0], p.heads, L, kLT) || !wide_map(&m.loop_w, x.w[1], p.heads, L, DV, kLT))
-            return BASED_ERR_CUDA;
+        std::swap(m.own_n, m.loop_n);
+        std::swap(m.own_w, m.loop_w);
         p.own_n = src[1]; p.own_w = src[2]; p.loop_n = src[0]; p.loop_w = src[3];
         p.out_n = dk + h0 * hn; p.out_w = dv + h0 * hw;
         if ((st = launch_quadratic<DV, kKeys>(m, p, stream)) != BASED_OK) return st;

@@ -467,12 +467,31 @@ void set_status_error(const StatusFault& e) {
 }
 
 // ---------------------------------------------------------------------------------------------- autograd
-// The output gradient as the backward pass takes it.  It usually comes back from a projection with the heads of a token
-// side by side, [B,L,H,d_v] seen as [B,H,L,d_v]: that layout has a copy kernel of its own in the library.
-Tensor heads_first(const Tensor& g, at::ScalarType dt, void* stream) {
-    if (g.is_contiguous() || g.dim() != 4 || !g.is_cuda() || g.scalar_type() != dt) return g.contiguous().to(dt);
+// An output gradient usually comes back from a projection with the heads of a token side by side, [B,L,H,d_v] seen as
+// [B,H,L,d_v].
+bool tokens_first(const Tensor& g, at::ScalarType dt) {
+    if (g.is_contiguous() || g.dim() != 4 || !g.is_cuda() || g.scalar_type() != dt) return false;
     const int64_t B = g.size(0), H = g.size(1), L = g.size(2), d = g.size(3);
-    if (g.stride(3) != 1 || g.stride(1) != d || g.stride(2) != H * d || (B > 1 && g.stride(0) != L * H * d)) return g.contiguous();
+    return g.stride(3) == 1 && g.stride(1) == d && g.stride(2) == H * d && (B == 1 || g.stride(0) == L * H * d);
+}
+// fp32 gradients of such an output gradient as it lies; undefined tensors where there is no such route
+Gradients backward_as_it_lies(const Tensor& q, const Tensor& k, const Tensor& v, const Tensor& dout, int flags, void* stream) {
+    const int B = size(q, 0), H = size(q, 1), L = size(q, 2), d_feat = size(q, 3), d_v = size(v, 3);
+    if (dout.sizes() != v.sizes() || (reinterpret_cast<uintptr_t>(dout.const_data_ptr()) & 15)) return {};
+    const size_t bytes = based_f32_parts_bytes(B, H, L, d_feat, d_v, 1);
+    if (bytes == 0) return {};
+    const Tensor ws = workspace_of(kNone, bytes, q);
+    Gradients g{at::empty_like(q), at::empty_like(k), at::empty_like(v)};
+    const based_status st = based_prefill_backward_tokens_first(cptr(q), cptr(k), cptr(v), dout.const_data_ptr(), ptr(g.dq), ptr(g.dk),
+                                                                ptr(g.dv), B, H, L, d_feat, d_v, BASED_F32, flags, ptr(ws), bytes, stream);
+    if (st == BASED_ERR_UNSUPPORTED) return {};
+    check(st, "based_prefill_backward");
+    return g;
+}
+// The output gradient as the backward pass takes it: the library has a copy kernel for that layout.
+Tensor heads_first(const Tensor& g, at::ScalarType dt, void* stream) {
+    if (!tokens_first(g, dt)) return g.contiguous().to(dt);
+    const int64_t B = g.size(0), H = g.size(1), L = g.size(2), d = g.size(3);
     const Tensor out = at::empty({B, H, L, d}, g.options());
     const based_status st = based_tokens_to_heads(g.const_data_ptr(), ptr(out), static_cast<int>(B), static_cast<int>(H),
                                                   static_cast<int>(L), static_cast<int>(d * g.element_size()), stream);
@@ -494,9 +513,15 @@ struct LinearAttention : torch::autograd::Function<LinearAttention> {
         const auto saved = ctx->get_saved_variables();
         const Tensor &q = saved[0], &k = saved[1], &v = saved[2], &out = saved[3];
         void* stream = c10::cuda::getCurrentCUDAStream().stream();
-        const Tensor dout = grads[0].defined() ? heads_first(grads[0], q.scalar_type(), stream) : at::zeros_like(v);
+        const int flags = static_cast<int>(ctx->saved_data["flags"].toInt());
         try {
-            const Gradients g = backward_call(q, k, v, dout, out, static_cast<int>(ctx->saved_data["flags"].toInt()), kNone, stream);
+            Gradients g;
+            if (grads[0].defined() && q.scalar_type() == at::kFloat && tokens_first(grads[0], at::kFloat))
+                g = backward_as_it_lies(q, k, v, grads[0], flags, stream);
+            if (!g.dq.defined()) {
+                const Tensor dout = grads[0].defined() ? heads_first(grads[0], q.scalar_type(), stream) : at::zeros_like(v);
+                g = backward_call(q, k, v, dout, out, flags, kNone, stream);
+            }
             return {g.dq, g.dk, g.dv, Tensor()};
         } catch (const StatusFault& e) {
             // autograd's worker thread: the engine hands a Python exception on to the thread that called backward

@@ -8,6 +8,7 @@ import torch
 
 import oracle
 import paper_2402_18668_b200 as based
+import paper_2402_18668_b200.autograd
 from paper_2402_18668_b200 import workloads as wl
 from parity import TOL_F32, row_err
 
@@ -89,3 +90,28 @@ def test_f32_parts_of_large_values(BH, L, big):
     ok = np.abs(ref) < 1e38                                       # (a sum over D that would overflow in fp32 is infinite or NaN)
     got = out[:, :1].double().cpu().numpy()
     assert (np.abs(got - ref)[ok] <= 1e-4 * np.maximum(np.abs(ref), 1.0)[ok])[np.isfinite(got)[ok]].all()
+
+
+def test_f32_parts_slabs_of_heads():
+    """More heads than the parts' scratch holds at a time, the output gradient as it lies and not: heads of both slabs and
+    their seam against the same heads alone."""
+    B, H, L = 2, 150, 1000
+    assert 2 * L * (2 * 96 + 2 * 384) * B * H // 2 > 256 << 20
+    g = torch.Generator(device="cuda").manual_seed(3)
+    r = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    q, k, v, dout = r(B, H, L, 16), r(B, H, L, 16), r(B, H, L, 64), r(B, L, H, 64)
+    x = [t.requires_grad_(True) for t in (q, k, v)]
+    y = based.autograd.linear_attention(*x)
+    got = torch.autograd.grad(y, x, dout.transpose(1, 2), retain_graph=True)
+    again = torch.autograd.grad(y, x, dout.transpose(1, 2).contiguous())
+    assert all(torch.equal(a, b) for a, b in zip(got, again))
+    y = y.detach().view(1, B * H, L, 64)
+    flat = [t.detach().reshape(1, B * H, L, -1) for t in (q, k, v, dout.transpose(1, 2))]
+    for h in (0, 149, 278, 279, 280, 299):
+        one = [t[:, h:h + 1].contiguous() for t in flat]
+        want = based.based_prefill(*one[:3])
+        assert (y[:, h:h + 1] - want).abs().max() <= TOL * want.abs().max()
+        for a, b in zip(got, based.based_prefill_backward(*one)):
+            a = a.reshape(1, B * H, L, -1)[:, h:h + 1]
+            assert (a - b).abs().max() <= TOL * b.abs().max()
+    assert based.based_poll_error() == based.BASED_OK

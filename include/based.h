@@ -93,12 +93,20 @@ based_status based_prefill(const void* q, const void* k, const void* v, void* ou
 size_t based_prefill_workspace_bytes(int B, int H, int L, int d_feat, int d_v, based_dtype io);
 
 /*
- * Scratch with which an fp32 call runs on the tensor cores, its operands split into three bf16 parts each (results at least
- * as close to exact ones as fp32 multiply-adds give): based_prefill without a state (backward = 0) and the backward pass at
- * d_v 64 (backward = 1) take that route when their workspace has this many bytes, else one that needs no scratch or
+ * Scratch with which an fp32 pass runs on the tensor cores, its operands split into three bf16 parts each (results at least
+ * as close to exact ones as fp32 multiply-adds give): based_prefill_f32_parts (backward = 0), and the backward pass at d_v 64
+ * (backward = 1), which takes that route when its workspace has this many bytes, else one that needs
  * based_prefill_backward_workspace_bytes.  0: there is no such route for these arguments, or it is not the faster one.
  */
 size_t based_f32_parts_bytes(int B, int H, int L, int d_feat, int d_v, int backward);
+
+/*
+ * The outputs of based_prefill from the empty state, fp32 io, that way (training's forward pass).  Rounded differently from
+ * based_prefill's, whose outputs are the same bit for bit whether the state is asked for or not.  workspace:
+ * based_f32_parts_bytes(..., 0); BASED_ERR_UNSUPPORTED where that is 0.  flags: 0 or BASED_NUMERATOR_ONLY.
+ */
+based_status based_prefill_f32_parts(const float* q, const float* k, const float* v, float* out, int B, int H, int L, int d_feat,
+                                     int d_v, int flags, void* workspace, size_t workspace_bytes, void* cuda_stream);
 
 /*
  * The recurrent state of a token block without its outputs (Sec. 4.1, recurrent view):

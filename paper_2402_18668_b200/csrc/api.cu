@@ -154,12 +154,6 @@ static based_status prefill_impl(const void* q, const void* k, const void* v, vo
     if (io == BASED_BF16)
         return launch_prefill_tc(q, k, v, out, kv_state, z_state, B * H, L, d_v, flags, workspace,
                                  static_cast<cudaStream_t>(cuda_stream), fit ? workspace_bytes : ~(size_t)0);
-    const size_t parts = based_f32_parts_bytes(B, H, L, d_feat, d_v, 0);
-    if (!kv_state && parts > 0 && workspace && workspace_bytes >= parts) {
-        auto in = [](const void* p) { return static_cast<const float*>(p); };
-        return launch_quadratic_forward_f32(in(q), in(k), in(v), static_cast<float*>(out), workspace, B * H, L, d_v,
-                                            (flags & BASED_NUMERATOR_ONLY) ? 1 : 0, static_cast<cudaStream_t>(cuda_stream));
-    }
     return launch_prefill_f32(q, k, v, out, kv_state, z_state, B * H, L, d_v, flags,
                               static_cast<cudaStream_t>(cuda_stream));
 }
@@ -169,6 +163,19 @@ based_status based_prefill(const void* q, const void* k, const void* v, void* ou
                            size_t workspace_bytes, void* cuda_stream) {
     return prefill_impl(q, k, v, out, kv_state, z_state, B, H, L, d_feat, d_v, io, flags, workspace, workspace_bytes,
                         cuda_stream, false);
+}
+
+based_status based_prefill_f32_parts(const float* q, const float* k, const float* v, float* out, int B, int H, int L, int d_feat,
+                                     int d_v, int flags, void* workspace, size_t workspace_bytes, void* cuda_stream) {
+    if (!q || !k || !v || !out || B <= 0 || H <= 0 || L <= 0) return BASED_ERR_INVALID_ARG;
+    if (flags & ~BASED_NUMERATOR_ONLY) return BASED_ERR_INVALID_ARG;
+    if (out == q || out == k || out == v) return BASED_ERR_INVALID_ARG;
+    const size_t need = based_f32_parts_bytes(B, H, L, d_feat, d_v, 0);
+    if (need == 0 || (long long)B * H > kHeadSlab) return BASED_ERR_UNSUPPORTED;
+    if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(out) || !aligned16(workspace)) return BASED_ERR_ALIGNMENT;
+    if (!workspace || workspace_bytes < need) return BASED_ERR_WORKSPACE;
+    return launch_quadratic_forward_f32(q, k, v, out, workspace, B * H, L, d_v, (flags & BASED_NUMERATOR_ONLY) ? 1 : 0,
+                                        static_cast<cudaStream_t>(cuda_stream));
 }
 
 size_t based_prefill_state_workspace_bytes(int B, int H, int L, int d_feat, int d_v, based_dtype io) {

@@ -154,7 +154,6 @@ Tensor prefill_call(const Tensor& q, const Tensor& k, const Tensor& v, const Ten
     if (!out.defined()) out = at::empty_like(v);
     size_t need = based_prefill_workspace_bytes(B, H, L, d_feat, d_v, io);
     if (need <= BASED_WORDS_BYTES && !(flags & BASED_STATE_CONTINUE)) need = 0;
-    if (io == BASED_F32 && !kv.defined() && on_current(stream)) need = based_f32_parts_bytes(B, H, L, d_feat, d_v, 0);
     const Tensor ws = workspace_of(workspace, need, q);
     check(based_prefill(cptr(q), cptr(k), cptr(v), ptr(out), fptr(kv), fptr(z), B, H, L, d_feat, d_v, io, flags, ptr(ws),
                         bytes_of(ws), stream),
@@ -497,14 +496,29 @@ Tensor heads_first(const Tensor& g, at::ScalarType dt, void* stream) {
                                                   static_cast<int>(L), static_cast<int>(d * g.element_size()), stream);
     return st == BASED_OK ? out : g.contiguous();
 }
+// the fp32 forward pass on the tensor cores; an undefined tensor where there is no such route
+Tensor forward_by_parts(const Tensor& q, const Tensor& k, const Tensor& v, int flags, void* stream) {
+    const int B = size(q, 0), H = size(q, 1), L = size(q, 2), d_feat = size(q, 3), d_v = size(v, 3);
+    const size_t bytes = based_f32_parts_bytes(B, H, L, d_feat, d_v, 0);
+    if (bytes == 0 || (flags & ~BASED_NUMERATOR_ONLY)) return {};
+    const Tensor ws = workspace_of(kNone, bytes, q);
+    Tensor out = at::empty_like(v);
+    auto in = [](const Tensor& t) { return static_cast<const float*>(t.const_data_ptr()); };
+    const based_status st = based_prefill_f32_parts(in(q), in(k), in(v), static_cast<float*>(ptr(out)), B, H, L, d_feat, d_v, flags,
+                                                    ptr(ws), bytes, stream);
+    if (st == BASED_ERR_UNSUPPORTED) return {};
+    check(st, "based_prefill");
+    return out;
+}
 struct LinearAttention : torch::autograd::Function<LinearAttention> {
     static Tensor forward(torch::autograd::AutogradContext* ctx, const Tensor& q_, const Tensor& k_, const Tensor& v_, int64_t flags) {
         const Tensor q = q_.contiguous(), k = k_.contiguous(), v = v_.contiguous();
         if (!q.is_cuda() || !k.is_cuda() || !v.is_cuda()) value_error("libbased takes CUDA tensors only (there is no CPU path)");
         dims(q, 4, "q");
         check_qkv(q, k, v, kNone);
-        const Tensor out = prefill_call(q, k, v, kNone, kNone, Tensor(), static_cast<int>(flags), kNone,
-                                        c10::cuda::getCurrentCUDAStream().stream());
+        void* stream = c10::cuda::getCurrentCUDAStream().stream();
+        Tensor out = q.scalar_type() == at::kFloat ? forward_by_parts(q, k, v, static_cast<int>(flags), stream) : Tensor();
+        if (!out.defined()) out = prefill_call(q, k, v, kNone, kNone, Tensor(), static_cast<int>(flags), kNone, stream);
         ctx->save_for_backward({q, k, v, out});
         ctx->saved_data["flags"] = flags;
         return out;

@@ -25,6 +25,20 @@ def inputs(BH, L, d_v, seed):
     return (*wl.prefill_inputs(w, gen), torch.randn(1, BH, L, d_v, generator=gen))
 
 
+def forward(q, k, v, flags=0, out=None):
+    """based_prefill_f32_parts."""
+    B, H, L, d_v = v.shape
+    lib, p = based.binding.lib(), lambda t: ctypes.c_void_p(t.data_ptr())
+    lib.based_f32_parts_bytes.restype = lib.based_prefill_workspace_bytes.restype
+    n = lib.based_f32_parts_bytes(B, H, L, 16, d_v, 0)
+    out, ws = torch.empty_like(v) if out is None else out, torch.empty(n, dtype=torch.uint8, device="cuda")
+    lib.based_prefill_f32_parts.argtypes = [ctypes.c_void_p] * 4 + [ctypes.c_int] * 6 + [ctypes.c_void_p, ctypes.c_size_t, ctypes.c_void_p]
+    st = lib.based_prefill_f32_parts(p(q), p(k), p(v), p(out), B, H, L, 16, d_v, flags, p(ws), n,
+                                     ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert st == based.BASED_OK
+    return out
+
+
 @pytest.mark.parametrize("d_v", [64, 112, 128])
 @pytest.mark.parametrize("BH,L", [(2, 33), (1, 64), (3, 65), (2, 127), (150, 128), (2, 129), (1, 193), (80, 200), (1, 513), (40, 500)])
 @pytest.mark.parametrize("flags", [0, based.BASED_NUMERATOR_ONLY])
@@ -34,20 +48,17 @@ def test_f32_parts(BH, L, d_v, flags):
     x = [t.cuda() for t in (q, k, v, g)]
     s = [wl.to_f64(t[:, heads]) for t in (q, k, v, g)]
     before = based.launch_count()
-    y = based.based_prefill(*x[:3], flags=flags)
+    y = forward(*x[:3], flags)
     assert based.launch_count() - before == 2                    # parts, outputs
+    assert torch.equal(based.autograd.linear_attention(*x[:3], numerator_only=bool(flags)), y)
     want, _, _ = oracle.linattn_quadratic(*s[:3])
     if flags:
         c = s[0] @ s[1].swapaxes(-1, -2)
         want = want * np.tril(1 + c / 4 + c * c / 32).sum(-1, keepdims=True)
     assert row_err(wl.to_f64(y[:, heads]), want) <= TOL_F32
     assert np.abs(wl.to_f64(y[:, heads]) - want).max() <= TOL * np.abs(want).max()
-    # without scratch: the chunked kernel
-    plain = torch.empty_like(y)
     p = lambda t: ctypes.c_void_p(t.data_ptr())
     stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
-    assert lib.based_prefill(p(x[0]), p(x[1]), p(x[2]), p(plain), None, None, 1, BH, L, 16, d_v, 0, flags, None, 0, stream) == 0
-    assert row_err(wl.to_f64(plain[:, heads]), want) <= TOL_F32
     if d_v == 64:
         got = based.based_prefill_backward(*x, flags=flags)
         for a, b in zip(got, oracle.linattn_backward(*s, numerator_only=bool(flags))):
@@ -68,8 +79,7 @@ def test_f32_parts_outputs_on_sixteen_bytes(d_v):
     q, k, v, g = (t.cuda() for t in inputs(2, 150, d_v, 5))
     off = [torch.empty(t.numel() + 4, device="cuda")[4:].view(t.shape).copy_(t) for t in (q, k, v, g)]
     out = torch.empty(v.numel() + 4, device="cuda")[4:].view(v.shape)
-    based.based_prefill(*off[:3], out=out)
-    assert torch.equal(out, based.based_prefill(q, k, v))
+    assert torch.equal(forward(*off[:3], out=out), forward(q, k, v))
 
 
 @pytest.mark.parametrize("big", [1e30, 3.4e38])
@@ -80,8 +90,8 @@ def test_f32_parts_of_large_values(BH, L, big):
     at = L // 2
     vb = v.clone()
     vb[:, :, at, 3] = big
-    want = based.based_prefill(q, k, v)
-    out = based.based_prefill(q, k, vb)
+    want = forward(q, k, v)
+    out = forward(q, k, vb)
     assert torch.allclose(out[:, :, :at], want[:, :, :at], rtol=0, atol=1e-4)
     cols = [c for c in range(64) if c != 3]
     assert torch.allclose(out[..., cols], want[..., cols], rtol=0, atol=1e-4)
@@ -109,9 +119,27 @@ def test_f32_parts_slabs_of_heads():
     flat = [t.detach().reshape(1, B * H, L, -1) for t in (q, k, v, dout.transpose(1, 2))]
     for h in (0, 149, 278, 279, 280, 299):
         one = [t[:, h:h + 1].contiguous() for t in flat]
-        want = based.based_prefill(*one[:3])
+        want = forward(*one[:3])
         assert (y[:, h:h + 1] - want).abs().max() <= TOL * want.abs().max()
         for a, b in zip(got, based.based_prefill_backward(*one)):
             a = a.reshape(1, B * H, L, -1)[:, h:h + 1]
             assert (a - b).abs().max() <= TOL * b.abs().max()
     assert based.based_poll_error() == based.BASED_OK
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("which", [0, 1, 2])
+@pytest.mark.parametrize("BH,L,d_v", [(2, 200, 64), (150, 40, 112), (2, 70, 128)])
+def test_f32_parts_non_finite_tokens_stay_behind(BH, L, d_v, which, bad):
+    """A non-finite q, k or v of one token leaves the rows before it as they are, and the others are non-finite where based_prefill's
+    are."""
+    x = [t.cuda() for t in inputs(BH, L, d_v, L)[:3]]
+    want = forward(*x)
+    for at in sorted({L // 2, L - 1, 5}):
+        y = [t.clone() for t in x]
+        y[which][:, :, at, 1] = bad
+        out, ref = forward(*y), based.based_prefill(*y)
+        assert torch.allclose(out[:, :, :at], want[:, :, :at], rtol=0, atol=TOL_F32 * 0.1)
+        assert torch.equal(torch.isfinite(out), torch.isfinite(ref))
+        ok = torch.isfinite(ref)
+        assert torch.allclose(out[ok], ref[ok], rtol=1e-5, atol=1e-4)

@@ -94,7 +94,8 @@ size_t based_prefill_workspace_bytes(int B, int H, int L, int d_feat, int d_v, b
 
 /*
  * Scratch with which an fp32 pass runs on the tensor cores, its operands split into three bf16 parts each (results at least
- * as close to exact ones as fp32 multiply-adds give): based_prefill_f32_parts (backward = 0), and the backward pass at d_v 64
+ * as close to exact ones as fp32 multiply-adds give, over the whole range of fp32; rows that meet values from about 1e24 on
+ * may be computed by multiply-adds after all, which takes longer): based_prefill_f32_parts (backward = 0), and the backward pass at d_v 64
  * (backward = 1), which takes that route when its workspace has this many bytes, else one that needs
  * based_prefill_backward_workspace_bytes.  0: there is no such route for these arguments, or it is not the faster one.
  */

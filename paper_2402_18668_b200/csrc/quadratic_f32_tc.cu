@@ -9,6 +9,10 @@
 //   - within a tile the small products go first: only the last four instructions meet an accumulator of full size;
 //   - no accumulator of the products of first parts lives longer than one looped tile of 64 rows: it is added to fp32
 //     registers, rounding (K = 64: 7e-8 against 1.5e-7 of fp32 multiply-adds, K = 1024: 1.0e-7 against 5.7e-7).
+// The parts are those of 2^24 x: of x below 2^-109 the third part, and further down the second, would have bits below the last
+// bf16 subnormal (v or dout of 1e-36: 2.7e-5 off).  Scores and products of dout and v carry 2^48: the polynomials' coefficients
+// take that back.  What is split again (weights times dout . v, times 1/D) is formed at 2^24 of its size, for the same
+// reason, and the results are scaled back at the end.  All of it by powers of two: nothing is rounded.
 //
 // One CTA per (head, 128 own rows), looping over tiles of 64 rows of the other side; formulas as in backward_f32.cu:
 //   kFwd   own = queries, looped = keys:   Y += W V,  W = 1 + S/4 + S^2/32, S = Q K^T
@@ -24,9 +28,9 @@
 // on only when the last of them has left the queue, so one for both let the tensor pipe run dry twice per tile: forward at B1 H2
 // L4096 55.6 -> 52.0 us); one the loads.
 //
-// Infinities, NaN and values next to the largest do not split (inf - inf is NaN), and a masked weight of zero times infinity
-// is NaN in rows that do not see the key.  Either way what comes out is not finite: such rows are computed once more with
-// plain fp32 multiply-adds, masked pairs left out (B2 H16 L1024 with a value of NaN in each head: 330 and 1000 us).
+// Infinities, NaN and values from 2^104 on do not split (inf - inf is NaN), scores or products of dout and v from 2^80 on overflow
+// at 2^48 of their size, and a masked weight of zero times infinity is NaN in rows that do not see the key.  Either way what
+// comes out is not finite: such rows are computed once more with plain fp32 multiply-adds, masked pairs left out (B2 H16 L1024 with a value of NaN in each head: 330 and 1000 us).
 //
 // Measured at B2 H16 L1024 d_v 64, against fp32 multiply-adds: forward 72 -> 28 us, backward 269 -> 80, errors in the 2-norm 0.8e-7
 // for 1.9e-7 (outputs), 1.7e-7 for 2.8e-7 (dq), 1.9e-7 for 4.1e-7 (dk), 1.4e-7 for 7.6e-7 (dv).  Per looped tile the forward takes 1250
@@ -51,6 +55,7 @@ namespace cg = cooperative_groups;
 constexpr int kOwn = 128, kLT = 64;
 constexpr int kNThreads = 480;
 constexpr int kFwd = 0, kDq = 1, kKeys = 2;
+constexpr float kUp = 0x1p24f, kDown = 0x1p-24f, kDown2 = 0x1p-48f;    // of the parts' scale; of the scale of a product of two
 // parts (a, b) of the six products, the smallest first
 __host__ __device__ constexpr int part_a(int i) { return i < 3 ? i : i == 4; }
 __host__ __device__ constexpr int part_b(int i) { return i < 3 ? 2 - i : i == 3; }
@@ -90,7 +95,8 @@ enum { bOwn = 0, bFull = 1, bEmpty = 7, bScore = 13, bWeight = 17, bSetFree = 21
 
 struct QParams {
     const float *own_n, *own_w, *loop_n, *loop_w;    // narrow and wide tensors of the own and the looped side (forward: own_w unused)
-    float *inv, *b;                                  // 1/D and b per query, [heads][pitch]: written by kDq, read by kKeys
+    float *inv, *b;                                  // kUp / D and -(G V^T's mean under the weights) per query, [heads][pitch]:
+                                                     // written by kDq, read by kKeys
     const float* m;                                  // kDq: the centres m_i = G_i.v_i, [heads][L]
     int pitch;                                       // L rounded up to whole looped tiles
     float *out_n, *out_w;                            // dq or dk; the forward output or dv
@@ -177,7 +183,7 @@ __device__ __forceinline__ size_t dout_rows(int H, int h0, size_t head, int L, i
 // The rows of a warp, a lane each, by plain multiply-adds, pair by pair: the narrow results (dq, dk) of lanes with need_n, the
 // wide ones (the output, dv) of those with need_w.  buf: kPlainFloats of shared memory of the warp's own, for 32 looped rows at a
 // time.
-constexpr int kPlainPitch = kDFeat + 64 + 4;         // narrow row, wide columns, 1/D, b
+constexpr int kPlainPitch = kDFeat + 64 + 4;         // narrow row, wide columns, 1/D, minus the mean
 constexpr int kPlainFloats = 32 * kPlainPitch;
 template <int MODE>
 __device__ __noinline__ void plain_rows(const QParams& p, float* buf, size_t head, int row, bool need_n, bool need_w) {
@@ -220,7 +226,7 @@ __device__ __noinline__ void plain_rows(const QParams& p, float* buf, size_t hea
         }
         if (MODE == kKeys) {
             const int t = min(j + lane, L - 1);
-            buf[lane * kPlainPitch + kDFeat + 64] = p.inv[hs + t];
+            buf[lane * kPlainPitch + kDFeat + 64] = p.inv[hs + t] * kDown;
             buf[lane * kPlainPitch + kDFeat + 65] = p.b[hs + t];
         }
         __syncwarp();
@@ -248,7 +254,7 @@ __device__ __noinline__ void plain_rows(const QParams& p, float* buf, size_t hea
                 }
                 const float s = dot16(xn, nj), w1 = fmaf(s, 0.0625f, 0.25f);
                 if (MODE == kKeys ? j0 + i < r : j0 + i > r) continue;
-                const float a = MODE == kDq ? w1 * (gv - m) : fmaf(gv, at[kDFeat + 64], at[kDFeat + 65]) * w1;
+                const float a = MODE == kDq ? w1 * (gv - m) : (gv + at[kDFeat + 65]) * at[kDFeat + 64] * w1;
                 if (MODE == kDq) {
                     den += weight(s);
                     num = fmaf(weight(s), gv, num);
@@ -260,14 +266,14 @@ __device__ __noinline__ void plain_rows(const QParams& p, float* buf, size_t hea
                 }
             }
         }
-        const float inv = p.numerator_only ? 1.f : 1.f / (den + kEps), b = p.numerator_only ? 0.f : -num * inv * inv;
-        const float c = p.numerator_only ? 0.f : fmaf(m, inv, b);
+        const float inv = p.numerator_only ? 1.f : 1.f / (den + kEps), mean = p.numerator_only ? 0.f : num * inv;
+        const float c = p.numerator_only ? 0.f : fmaf(m, inv, -mean * inv);
         if (need_n) {
 #pragma unroll
             for (int e = 0; e < kDFeat; ++e) p.out_n[hn + (size_t)r * kDFeat + e] = MODE == kDq ? fmaf(x[e], inv, c * y[e]) : x[e];
             if (MODE == kDq) {
-                p.inv[hs + r] = inv;
-                p.b[hs + r] = b;
+                p.inv[hs + r] = inv * kUp;
+                p.b[hs + r] = -mean;
             }
         }
     }
@@ -349,10 +355,10 @@ __global__ void __launch_bounds__(256) split_parts_kernel(const SplitSet s) {
         const unsigned e = u * 256 + threadIdx.x;
         if (e >= left) break;
         const unsigned row = (c0 + e) / n, c = c0 + e - row * n;
-        const uint64_t x[4] = {f2(a[u].x, a[u].y), f2(a[u].z, a[u].w), f2(b[u].x, b[u].y), f2(b[u].z, b[u].w)};
+        const uint64_t x[4] = {f2(a[u].x, a[u].y), f2(a[u].z, a[u].w), f2(b[u].x, b[u].y), f2(b[u].z, b[u].w)}, up = f2(kUp, kUp);
         uint32_t o[3][4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) split_pair(x[k], o[0][k], o[1][k], o[2][k]);
+        for (int k = 0; k < 4; ++k) split_pair(mul2(x[k], up), o[0][k], o[1][k], o[2][k]);
 #pragma unroll
         for (int k = 0; k < 3; ++k) dst[row * (3 * n) + c + k * n] = make_uint4(o[k][0], o[k][1], o[k][2], o[k][3]);
         if (i == 3 && s.m) {                         // eight lanes per row, rows in whole (d_v 64: eight pieces)
@@ -559,8 +565,10 @@ __global__ void __launch_bounds__(kNThreads, 1)
         const int wg = warp >> 2, row_l = tid & 127, row = r0 + row_l;
         const uint32_t lane_base = (uint32_t)(warp & 3) * 32u;
         const float m_own = MODE == kDq && row < p.L && !p.numerator_only ? p.m[head * (size_t)p.L + row] : 0.f;
-        const uint64_t k4 = f2(0.25f, 0.25f), k32 = f2(0.03125f, 0.03125f), k16 = f2(0.0625f, 0.0625f), one = f2(1.f, 1.f);
-        const uint64_t negm = f2(-m_own, -m_own);
+        // 1/4, 1/32, 1/16 of scores that are the products of two scaled operands
+        const uint64_t k4 = f2(0.25f * kDown2, 0.25f * kDown2), k32 = f2(0.03125f * kDown2 * kDown2, 0.03125f * kDown2 * kDown2);
+        const uint64_t k16 = f2(0.0625f * kDown2, 0.0625f * kDown2), one = f2(1.f, 1.f), quarter = f2(0.25f, 0.25f);
+        const uint64_t negm = f2(-m_own * kUp, -m_own * kUp), gv_scale = MODE == kDq ? f2(kDown, kDown) : f2(kDown2, kDown2);
         uint64_t den2 = 0, num2 = 0;
         for (int t = C::kBwd ? 0 : wg; t < n; t += C::kBwd ? 1 : 2) {
             const int c0 = (first + t) * kLT, rw = r0 + (int)lane_base;               // the tile's first column, the warp's first row
@@ -605,8 +613,8 @@ __global__ void __launch_bounds__(kNThreads, 1)
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
                         const uint64_t s = bits2(sr[16 * k + 2 * i], sr[16 * k + 2 * i + 1]);
-                        uint64_t wt = MODE == kDq ? fma2(s, k16, k4) : fma2(s, fma2(s, k32, k4), one);
-                        // (past the end 1/D and b are anything: masked after the products)
+                        uint64_t wt = MODE == kDq ? fma2(s, k16, quarter) : fma2(s, fma2(s, k32, k4), one);
+                        // (past the end 1/D and the mean are anything: masked after the products)
                         if (MODE == kKeys) wt = mul2(wt, *reinterpret_cast<const uint64_t*>(st + 32 * h + 16 * k + 2 * i));
                         wt = masked(wt, 8 * k + i);
                         if (MODE == kFwd) dt = add2(dt, wt);
@@ -626,16 +634,17 @@ __global__ void __launch_bounds__(kNThreads, 1)
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
                         const uint64_t s = bits2(sr[16 * k + 2 * i], sr[16 * k + 2 * i + 1]), gv = bits2(gr[2 * i], gr[2 * i + 1]);
-                        const uint64_t w1 = fma2(s, k16, k4);
+                        const uint64_t w1 = fma2(s, k16, quarter);
                         uint64_t x;
                         if (MODE == kDq) {
                             const uint64_t wt = masked(fma2(s, fma2(s, k32, k4), one), 8 * k + i);
                             dt = add2(dt, wt);
                             nt = fma2(wt, masked(gv, 8 * k + i), nt);
-                            x = mul2(w1, add2(gv, negm));
+                            x = mul2(w1, fma2(gv, gv_scale, negm));
                         } else {
                             const float* at = st + 32 * h + 16 * k + 2 * i;
-                            x = mul2(fma2(gv, *reinterpret_cast<const uint64_t*>(at), *reinterpret_cast<const uint64_t*>(at + kLT)), w1);
+                            x = mul2(mul2(w1, *reinterpret_cast<const uint64_t*>(at)),
+                                     fma2(gv, gv_scale, *reinterpret_cast<const uint64_t*>(at + kLT)));
                         }
                         split_pair(masked(x, 8 * k + i), w[0][i], w[1][i], w[2][i]);
                     }
@@ -764,28 +773,28 @@ __global__ void __launch_bounds__(kNThreads, 1)
             if (mine) {
                 if (MODE == kDq && good) {
                     const float inv = p.numerator_only ? 1.f : 1.f / (sum.x + kEps);
-                    const float b = p.numerator_only ? 0.f : -sum.y * inv * inv;
-                    const float c = p.numerator_only ? 0.f : fmaf(p.m[head * (size_t)p.L + row], inv, b);
+                    const float mean = p.numerator_only ? 0.f : sum.y * kDown2 * inv;
+                    const float c = p.numerator_only ? 0.f : fmaf(p.m[head * (size_t)p.L + row], inv, -mean * inv);
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         float o[8];
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) o[e] = fmaf(x[8 * h + e], inv, c * x[16 + 8 * h + e]);
+                        for (int e = 0; e < 8; ++e) o[e] = fmaf(x[8 * h + e] * kDown2, inv, c * (x[16 + 8 * h + e] * kDown));
                         store8(p.out_n + hn + (size_t)row * kDFeat + 8 * h, o);
                     }
-                    p.inv[hs + row] = inv;
-                    p.b[hs + row] = b;
+                    p.inv[hs + row] = inv * kUp;
+                    p.b[hs + row] = -mean;
                 } else if (MODE != kDq && good) {
                     // 1 / D in two parts: as close as a division, two multiply-adds per pair
                     const float d = sum.x + kEps, r = p.numerator_only ? 1.f : 1.f / d, r_lo = p.numerator_only ? 0.f : fmaf(-d, r, 1.f) * r;
-                    const uint64_t rr = f2(r, r), rl = f2(r_lo, r_lo);
+                    const uint64_t rr = f2(r, r), rl = f2(r_lo, r_lo), back = MODE == kFwd ? f2(kDown, kDown) : f2(kDown2, kDown2);
                     float* dst = p.out_w + hw + (size_t)row * p.dvw;
 #pragma unroll
                     for (int c = 0; c < DV; c += 8) {
                         float o[8];
 #pragma unroll
                         for (int e = 0; e < 8; e += 2) {
-                            const uint64_t y = f2(x[c + e], x[c + e + 1]);
+                            const uint64_t y = mul2(f2(x[c + e], x[c + e + 1]), back);
                             unpack2(MODE == kFwd ? fma2(y, rr, mul2(y, rl)) : y, o[e], o[e + 1]);
                         }
                         if (DV == 64 || c < p.dvw) store8(dst + c, o);
@@ -794,8 +803,9 @@ __global__ void __launch_bounds__(kNThreads, 1)
                 if (MODE == kKeys && good_n)
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
-                        const float o[8] = {x[64 + 8 * h], x[65 + 8 * h], x[66 + 8 * h], x[67 + 8 * h],
-                                            x[68 + 8 * h], x[69 + 8 * h], x[70 + 8 * h], x[71 + 8 * h]};
+                        float o[8];
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) o[e] = x[64 + 8 * h + e] * kDown2;
                         store8(p.out_n + hn + (size_t)row * kDFeat + 8 * h, o);
                     }
             }

@@ -143,3 +143,29 @@ def test_f32_parts_non_finite_tokens_stay_behind(BH, L, d_v, which, bad):
         assert torch.equal(torch.isfinite(out), torch.isfinite(ref))
         ok = torch.isfinite(ref)
         assert torch.allclose(out[ok], ref[ok], rtol=1e-5, atol=1e-4)
+
+
+# Relative to 64 bits in the 2-norm.  An operand's parts keep 24 bits and the products left out are below 2^-25 of it; with the
+# sums' own rounding 1 to 3e-7 is measured, whatever the inputs' magnitude.  Two parts in place of three would show 4e-6.
+TOL_NORM = 1e-6
+
+
+def norm_err(got, want):
+    return np.linalg.norm(wl.to_f64(got) - want) / np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("scale", [1e-30, 1e-36])
+@pytest.mark.parametrize("small", ["v", "dout", "q", "k"])
+@pytest.mark.parametrize("BH,L", [(2, 64), (3, 300), (150, 129)])
+def test_f32_parts_of_small_values(BH, L, small, scale):
+    """Parts of such values would be bf16 subnormals, or nothing, if the values were split as they are."""
+    x = dict(zip(("q", "k", "v", "dout"), inputs(BH, L, 64, L)))
+    x[small] *= scale
+    heads = sorted({0, BH // 2, BH - 1})
+    s = [wl.to_f64(t[:, heads]) for t in x.values()]
+    d = [t.cuda() for t in x.values()]
+    assert norm_err(forward(*d[:3])[:, heads], oracle.linattn_quadratic(*s[:3])[0]) <= TOL_NORM
+    for flags in (0, based.BASED_NUMERATOR_ONLY):
+        for a, b in zip(based.based_prefill_backward(*d, flags=flags), oracle.linattn_backward(*s, numerator_only=bool(flags))):
+            assert norm_err(a[:, heads], b) <= TOL_NORM
+    assert based.based_poll_error() == based.BASED_OK

@@ -100,6 +100,12 @@ def lib() -> ctypes.CDLL:
         L.based_prefill_backward_block_tokens.argtypes = [i, i, i, i, i, i, i, i]
         L.based_prefill_backward_workspace_bytes.restype = sz
         L.based_prefill_backward_workspace_bytes.argtypes = [i, i, i, i, i]
+        L.based_f32_parts_bytes.restype = sz
+        L.based_f32_parts_bytes.argtypes = [i, i, i, i, i, i]
+        L.based_prefill_f32_parts.restype = i
+        L.based_prefill_f32_parts.argtypes = [vp, vp, vp, vp, i, i, i, i, i, i, vp, sz, vp]
+        L.based_prefill_backward_tokens_first.restype = i
+        L.based_prefill_backward_tokens_first.argtypes = [vp, vp, vp, vp, vp, vp, vp, i, i, i, i, i, i, i, vp, sz, vp]
         L.baseconv_gate_forward.restype = i
         L.baseconv_gate_forward.argtypes = [vp, vp, vp, vp, vp, i, i, i, i, i, vp]
         L.baseconv_gate_step.restype = i

@@ -926,13 +926,25 @@ bool wide_map(CUtensorMap* m, const void* base, int heads, int L, int d_v) {
 }  // namespace
 
 size_t quadratic_f32_workspace_bytes(int BH, int L, int d_v, bool backward) {
-    // Forward: against the chunked kernel of prefill_f32.cu, whose time grows with L (us, this / that): L 32 7 / 9 at d_v 64, 10.3 /
-    // 9.0 at d_v 128, L 48 10.6 / 13; L 1024 14 / 21 with 2 heads, 28 / 72 with 32, 45 / 147 with 32 at d_v 128; L 4096 480 / 596
-    // with 64 heads, 902 / 924 at d_v 128; L 8192 99 / 154 with 2 heads, 404 / 393 with 16, 1906 / 1192 with 64.
-    // Backward, against backward_f32.cu (quadratic too, d_v 64): L 64 14 / 18, L 140 20 / 28, L 1024 30 / 45 with 2 heads, 79 / 269 with
-    // 32; with few heads and four tiles of 64 that one has a cluster per tile and a tile per CTA: L 200 and 256 with 2 to 8 heads 21 to
-    // 25 / 20 to 21, with 16 25 / 30.
-    if (backward ? d_v != 64 || (BH <= 8 && L > 192 && L <= 256) : L <= (d_v == 64 ? 24 : 32) || L > 4096) return 0;
+    // Forward (us, this / the chunked kernel of prefill_f32.cu, whose time grows with L alone; that one has two or three CTAs per head
+    // for 38 to 74 heads).  Short: d_v 64 L 25 to 32 7.2 / 8.5 up to 128 heads, 8.8 / 8.6 with 148, 24 / 21 with 500, then L 33 24 /
+    // 30; d_v 128 L 32 10.3 / 9.0, L 33 10.3 / 13.4, with 47 or 64 heads 11.4 / 10.9 at L 33 and 41, 10.7 / 10.8 at L 48.
+    // Between: L 1024 13.4 / 20.8 with 2 heads, 27 / 72 with 32, 45 / 146 with 32 at d_v 128.  Long: L 4096 483 / 622 with 64 heads
+    // (898 / 924 at d_v 128), L 3840 690 / 746 with 96, at d_v 128 1250 / 1497, but 1030 / 866 with 74 there; L 3000 616 / 683 with
+    // 128, L 2816 1077 / 1062 with 256, L 2432 840 / 917; L 8192 99 / 154 with 2, 404 / 393 with 16.
+    if (!backward) {
+        const bool two = d_v != 64 && BH > 37 && BH <= 74;
+        const int from = two ? 49 : d_v != 64 || BH > 128 ? 33 : 25;
+        const int to = BH <= 64 ? 4096 : two ? 3072 : BH <= 96 ? 3840 : BH <= 128 ? 2816 : 2432;
+        if (L < from || L > to) return 0;
+    } else {
+        // Backward, against backward_f32.cu (quadratic too, d_v 64): L 1 to 64 13.6 to 17 / 14.5 to 18 up to 74 heads; with more the
+        // 128 own rows of a CTA are half empty and that one's 64 are not: L 64 18.2 / 17.9 with 80 heads, 65 / 50 with 500, L 32 41 /
+        // 34 with 300.  From L 65 on 55 / 69 (300 heads, L 80), L 1024 30 / 45 with 2, 80 / 268 with 32.  That one gives a cluster a
+        // tile of 64 and a CTA one tile of its loop where heads are few: L 193 to 256 with up to 8 heads 21 to 25 / 20 to 21, with 16
+        // 25 / 30; L 449 to 512 with one 24 / 19.6, with two 24 / 26 to 28.
+        if (d_v != 64 || (L <= kLT && BH > 74) || (L > 192 && L <= 256 && BH <= 8) || (L > 448 && L <= 512 && BH == 1)) return 0;
+    }
     return parts_of(nullptr, BH, L, d_v, backward).bytes;
 }
 

@@ -207,6 +207,20 @@ def test_backward_validation(lib):
     assert w(q, k, v, o, g, dq, dk, dv, *ok, 0, ws, 8, None) == 6
 
 
+def test_lines_of_the_fp32_tensor_core_route(lib):
+    """No scratch, and so the fp32 multiply-add kernels, where those are the faster."""
+    def taken(BH, L, d_v=64, backward=0):
+        return lib.based_f32_parts_bytes(1, BH, L, 16, d_v, backward) > 0
+    for d_v, BH, first, last in [(64, 1, 25, 4096), (64, 128, 25, 2816), (64, 129, 33, 2432), (64, 64, 25, 4096), (64, 65, 25, 3840),
+                                 (64, 97, 25, 2816), (112, 2, 33, 4096), (112, 37, 33, 4096), (112, 38, 49, 4096), (128, 74, 49, 3072), (128, 75, 33, 3840), (128, 257, 33, 2432)]:
+        assert not taken(BH, first - 1, d_v) and taken(BH, first, d_v) and taken(BH, last, d_v) and not taken(BH, last + 1, d_v)
+    assert taken(74, 64, backward=1) and not taken(75, 1, backward=1) and not taken(75, 64, backward=1) and taken(75, 65, backward=1)
+    assert taken(8, 192, backward=1) and not taken(8, 193, backward=1) and not taken(8, 256, backward=1) and taken(9, 193, backward=1)
+    assert taken(1, 448, backward=1) and not taken(1, 449, backward=1) and not taken(1, 512, backward=1) and taken(2, 449, backward=1)
+    assert taken(1, 100000, backward=1) and not taken(4, 1024, 128, backward=1)
+    assert lib.based_f32_parts_bytes(1, 4, 1024, 24, 64, 0) == lib.based_f32_parts_bytes(1, 0, 1024, 16, 64, 0) == 0
+
+
 def test_binding_rejects_cpu_tensors():
     import torch
     from paper_2402_18668_b200 import binding

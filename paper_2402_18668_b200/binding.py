@@ -248,8 +248,20 @@ def based_prefill_state(k, v, kv_state=None, z_state=None, flags: int = BASED_ST
 
 def based_prefill_backward(q, k, v, dout, flags: int = 0, workspace=None, stream=None, out=None):
     """Gradients (dq, dk, dv) of based_prefill (empty initial state) for the output gradient dout.
-    out: the forward output, if the caller kept it (based_prefill_backward_with_out)."""
+    out: the forward output, if the caller kept it (based_prefill_backward_with_out).
+    workspace: used if it has based_prefill_backward_workspace_bytes.  fp32: with based_f32_parts_bytes(..., backward=True) of
+    workspace, or none given and the call on the current stream, the pass runs on the tensor cores, else on fp32
+    multiply-adds: equal up to rounding."""
     return (_native_module or native()).prefill_backward(q, k, v, dout, int(flags), workspace, _handle(stream), out)
+
+
+def based_f32_parts_bytes(B: int, H: int, L: int, d_feat: int, d_v: int, backward: bool = False) -> int:
+    """Scratch with which an fp32 pass runs on the tensor cores (0: it does not)."""
+    return int(lib().based_f32_parts_bytes(B, H, L, d_feat, d_v, int(backward)))
+
+
+def based_prefill_backward_workspace_bytes(B: int, H: int, L: int, d_v: int, io: int) -> int:
+    return int(lib().based_prefill_backward_workspace_bytes(B, H, L, d_v, io))
 
 
 def based_static_scratch_bytes() -> int:

@@ -166,7 +166,8 @@ Gradients backward_call(const Tensor& q, const Tensor& k, const Tensor& v, const
     const int B = size(q, 0), H = size(q, 1), L = size(q, 2), d_feat = size(q, 3), d_v = size(v, 3);
     const based_dtype io = dtype_code(q);
     size_t need = based_prefill_backward_workspace_bytes(B, H, L, d_v, io);
-    if (io == BASED_F32 && on_current(stream)) need = std::max(need, based_f32_parts_bytes(B, H, L, d_feat, d_v, 1));
+    // (a caller's workspace of that size is used as it is)
+    if (io == BASED_F32 && !workspace.defined() && on_current(stream)) need = std::max(need, based_f32_parts_bytes(B, H, L, d_feat, d_v, 1));
     const Tensor ws = workspace_of(workspace, need, q);
     Gradients g{at::empty_like(q), at::empty_like(k), at::empty_like(v)};
     const based_status st =

@@ -169,3 +169,25 @@ def test_f32_parts_of_small_values(BH, L, small, scale):
         for a, b in zip(based.based_prefill_backward(*d, flags=flags), oracle.linattn_backward(*s, numerator_only=bool(flags))):
             assert norm_err(a[:, heads], b) <= TOL_NORM
     assert based.based_poll_error() == based.BASED_OK
+
+
+def test_a_workspace_of_the_documented_size_is_used():
+    """Nothing but the gradients is allocated beside it; the route follows its size."""
+    x = [t.cuda() for t in inputs(4, 300, 64, 11)]
+    q, v = x[0], x[2]
+    small, large = (torch.empty(n, dtype=torch.uint8, device="cuda") for n in
+                    (based.based_prefill_backward_workspace_bytes(1, 4, 300, 64, 0), based.based_f32_parts_bytes(1, 4, 300, 16, 64, True)))
+    assert small.nbytes < large.nbytes
+
+    def call(workspace):
+        torch.cuda.synchronize()
+        torch.cuda.reset_peak_memory_stats()
+        before, launched = torch.cuda.memory_allocated(), based.launch_count()
+        g = based.based_prefill_backward(*x, workspace=workspace)
+        return g, torch.cuda.max_memory_allocated() - before - 2 * q.nbytes - v.nbytes, based.launch_count() - launched
+    (g_small, extra, launched), (g_large, extra_l, launched_l) = call(small), call(large)
+    assert extra <= 3 * 512 and launched == 2 and extra_l <= 3 * 512 and launched_l == 3
+    g_none, extra, _ = call(None)
+    assert extra >= large.nbytes and all(torch.equal(a, b) for a, b in zip(g_none, g_large))
+    for a, b in zip(g_small, g_large):
+        assert norm_err(a, wl.to_f64(b)) <= 2 * TOL_NORM

@@ -270,9 +270,9 @@ based_status based_prefill_backward_with_out(const void* q, const void* k, const
                                              size_t workspace_bytes, void* cuda_stream);
 
 /*
- * based_prefill_backward with dout as it comes back from a projection, the heads of a token side by side: [B,L,H,d_v].  fp32 io,
- * d_v 64, where based_f32_parts_bytes(..., 1) is not 0, with that many bytes of workspace; BASED_ERR_UNSUPPORTED otherwise (then
- * based_tokens_to_heads lays dout out for the other calls).
+ * based_prefill_backward with dout as it comes back from a projection, the heads of a token side by side: [B,L,H,d_v].  fp32 io
+ * and up to 65532 heads of 2^31 tokens in all; BASED_ERR_UNSUPPORTED otherwise (then based_tokens_to_heads lays dout out for the
+ * other calls).
  */
 based_status based_prefill_backward_tokens_first(const void* q, const void* k, const void* v, const void* dout, void* dq, void* dk,
                                                  void* dv, int B, int H, int L, int d_feat, int d_v, based_dtype io, int flags,

@@ -518,6 +518,21 @@ int based_prefill_backward_block_tokens(int B, int H, int L, int d_feat, int d_v
     return backward_tc_block_tokens(B * H, L, d_feat, d_v, (with_out || (flags & BASED_NUMERATOR_ONLY)) ? 1 : 0);
 }
 
+// fp32 io, one slab of heads, checked arguments; dout_H: 0, or H where dout lies [B, L, H, d_v]
+static based_status backward_f32(const void* q, const void* k, const void* v, const void* dout, int dout_H, void* dq, void* dk,
+                                 void* dv, int B, int H, int L, int d_v, int flags, void* workspace, size_t workspace_bytes,
+                                 void* cuda_stream) {
+    auto in = [](const void* p) { return static_cast<const float*>(p); };
+    auto out = [](void* p) { return static_cast<float*>(p); };
+    const int numerator_only = (flags & BASED_NUMERATOR_ONLY) ? 1 : 0;
+    const size_t parts = based_f32_parts_bytes(B, H, L, kDFeat, d_v, 1);
+    if (parts > 0 && workspace_bytes >= parts)
+        return launch_quadratic_backward_f32(in(q), in(k), in(v), in(dout), dout_H, out(dq), out(dk), out(dv), workspace, B * H, L,
+                                             numerator_only, static_cast<cudaStream_t>(cuda_stream));
+    return launch_prefill_backward_f32(in(q), in(k), in(v), in(dout), dout_H, out(dq), out(dk), out(dv), out(workspace), B * H, L,
+                                       d_v, numerator_only, static_cast<cudaStream_t>(cuda_stream));
+}
+
 static based_status prefill_backward(const void* q, const void* k, const void* v, const void* out, const void* dout,
                                      void* dq, void* dk, void* dv, int B, int H, int L, int d_feat, int d_v,
                                      based_dtype io, int flags, void* workspace, size_t workspace_bytes,
@@ -549,15 +564,7 @@ static based_status prefill_backward(const void* q, const void* k, const void* v
         return launch_prefill_backward_tc(q, k, v, out, dout, dq, dk, dv, static_cast<float*>(workspace), B * H, L,
                                           d_feat, d_v, (flags & BASED_NUMERATOR_ONLY) ? 1 : 0,
                                           static_cast<cudaStream_t>(cuda_stream));
-    auto in = [](const void* p) { return static_cast<const float*>(p); };
-    const size_t parts = based_f32_parts_bytes(B, H, L, d_feat, d_v, 1);
-    if (parts > 0 && workspace_bytes >= parts)
-        return launch_quadratic_backward_f32(in(q), in(k), in(v), in(dout), 0, static_cast<float*>(dq), static_cast<float*>(dk),
-                                             static_cast<float*>(dv), workspace, B * H, L, (flags & BASED_NUMERATOR_ONLY) ? 1 : 0,
-                                             static_cast<cudaStream_t>(cuda_stream));
-    return launch_prefill_backward_f32(in(q), in(k), in(v), in(dout), static_cast<float*>(dq), static_cast<float*>(dk),
-                                       static_cast<float*>(dv), static_cast<float*>(workspace), B * H, L, d_v,
-                                       (flags & BASED_NUMERATOR_ONLY) ? 1 : 0, static_cast<cudaStream_t>(cuda_stream));
+    return backward_f32(q, k, v, dout, 0, dq, dk, dv, B, H, L, d_v, flags, workspace, workspace_bytes, cuda_stream);
 }
 
 based_status based_prefill_backward(const void* q, const void* k, const void* v, const void* dout, void* dq,
@@ -583,16 +590,13 @@ based_status based_prefill_backward_tokens_first(const void* q, const void* k, c
     if (flags & ~BASED_NUMERATOR_ONLY) return BASED_ERR_INVALID_ARG;
     if (dq == q || dq == k || dk == q || dk == k || dv == v || dv == dout) return BASED_ERR_INVALID_ARG;
     // one slab of heads, rows counted in 32 bits
-    const size_t parts = io == BASED_F32 ? based_f32_parts_bytes(B, H, L, d_feat, d_v, 1) : 0;
-    if (parts == 0 || (long long)B * H > kHeadSlab || (long long)B * H * L > 0x7fffffffLL) return BASED_ERR_UNSUPPORTED;
+    if (io != BASED_F32 || d_feat != kDFeat || !dv_ok(d_v) || (long long)B * H > kHeadSlab || (long long)B * H * L > 0x7fffffffLL)
+        return BASED_ERR_UNSUPPORTED;
     if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(dout) || !aligned16(dq) || !aligned16(dk) || !aligned16(dv) ||
         !aligned16(workspace))
         return BASED_ERR_ALIGNMENT;
-    if (!workspace || workspace_bytes < parts) return BASED_ERR_WORKSPACE;
-    auto in = [](const void* p) { return static_cast<const float*>(p); };
-    return launch_quadratic_backward_f32(in(q), in(k), in(v), in(dout), H, static_cast<float*>(dq), static_cast<float*>(dk),
-                                         static_cast<float*>(dv), workspace, B * H, L, (flags & BASED_NUMERATOR_ONLY) ? 1 : 0,
-                                         static_cast<cudaStream_t>(cuda_stream));
+    if (!workspace || workspace_bytes < based_prefill_backward_workspace_bytes(B, H, L, d_v, io)) return BASED_ERR_WORKSPACE;
+    return backward_f32(q, k, v, dout, H, dq, dk, dv, B, H, L, d_v, flags, workspace, workspace_bytes, cuda_stream);
 }
 
 based_status based_tokens_to_heads(const void* src, void* dst, int B, int H, int L, int row_bytes, void* cuda_stream) {

@@ -57,11 +57,11 @@ struct BwdSmem {
 // place of looped row t where four consecutive rows belong to one thread: spreads those over the banks
 __device__ __forceinline__ int place_of(int t) { return (t & 3) * 16 + (t >> 2); }
 
-// 64 rows of W values (a multiple of 16) of a row-major array, transposed -> [W][68]; rows from nt on are zero.
+// 64 rows of W values (a multiple of 16) of a row-major array (LIES: `pitch` apart), transposed -> [W][68]; rows from nt on are zero.
 // nat: the rows as they lie too, at pitch natp (of: at place_of(t))
-template <int W>
+template <int W, bool LIES = false>
 __device__ __forceinline__ void load_tile(float* dst, float* nat, int natp, bool of, const float* __restrict__ src, int nt,
-                                          int warp, int lane) {
+                                          int warp, int lane, size_t pitch = W) {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int t = (lane & 7) + 8 * warp + 32 * h;
@@ -69,7 +69,7 @@ __device__ __forceinline__ void load_tile(float* dst, float* nat, int natp, bool
 #pragma unroll
         for (int i = 0; i < W / 16; ++i) {
             x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (t < nt) x[i] = __ldg(reinterpret_cast<const float4*>(src + (size_t)t * W) + (lane >> 3) + 4 * i);
+            if (t < nt) x[i] = __ldg(reinterpret_cast<const float4*>(src + (size_t)t * (LIES ? pitch : W)) + (lane >> 3) + 4 * i);
         }
 #pragma unroll
         for (int i = 0; i < W / 16; ++i) {
@@ -136,11 +136,14 @@ __device__ __forceinline__ void narrow_reduce(float2 (&acc)[4][4]) {
 }  // namespace
 
 // KEYS = false: dq and the statistics.  KEYS = true: dk and dv.  grid (heads x tiles, 1, CTAs per tile)
-template <int DV, bool KEYS>
+// LIES: dout is read as it comes back from a projection, the heads of a token side by side, [B, L, H, DV], which saves a copy and
+// its launch ahead (steps of B1 H8 L200 d_v 128 on the host 107 -> 105 us).  An instance of its own: with the distance of dout's
+// rows as an argument the others were 1 % slower.
+template <int DV, bool KEYS, bool LIES>
 __global__ void __launch_bounds__(kBT, DV > 64 ? 1 : 2)
     backward_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v,
                         const float* __restrict__ g, float2* stats, float* __restrict__ dx, float* __restrict__ dv, int heads,
-                        int L, int numerator_only) {
+                        int L, int numerator_only, int dout_H) {
     using S = BwdSmem<DV, KEYS>;
     constexpr int NV = S::kCols / 64;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -155,20 +158,22 @@ __global__ void __launch_bounds__(kBT, DV > 64 ? 1 : 2)
     const int dg = lane & 1, rg = (lane >> 1) & 3, ks = lane >> 3;   // narrow products
     const size_t hn = head * (size_t)L * kDFeat, hw = head * (size_t)L * DV;
     const float* own_n = (KEYS ? k : q) + hn;
-    const float* own_w = (KEYS ? v : g) + hw;
+    const size_t seq = LIES ? head / dout_H : 0, gw = LIES ? (seq * L * dout_H + head - seq * dout_H) * DV : hw;
+    const size_t gp = LIES ? (size_t)dout_H * DV : DV, own_p = KEYS ? DV : gp, loop_p = KEYS ? gp : DV;
+    const float* own_w = (KEYS ? v : g) + (KEYS ? hw : gw);
     const float* loop_n = (KEYS ? q : k) + hn;
-    const float* loop_w = (KEYS ? g : v) + hw;
+    const float* loop_w = (KEYS ? g : v) + (KEYS ? gw : hw);
     const int n_own = min(kT, L - own * kT);
 
     load_tile<kDFeat>(s.an, nullptr, 0, false, own_n + (size_t)own * kT * kDFeat, n_own, warp, lane);
-    load_tile<DV>(s.aw, nullptr, 0, false, own_w + (size_t)own * kT * DV, n_own, warp, lane);
+    load_tile<DV, LIES && !KEYS>(s.aw, nullptr, 0, false, own_w + (size_t)own * kT * own_p, n_own, warp, lane, own_p);
     float m[8];
     if (!KEYS) {
         // the centre m_i: two threads per row
         float x = 0.f;
         const int t = tid >> 1;
         if (t < n_own && !numerator_only) {
-            const float4* gr = reinterpret_cast<const float4*>(g + hw + (size_t)(own * kT + t) * DV);
+            const float4* gr = reinterpret_cast<const float4*>(g + gw + (size_t)(own * kT + t) * gp);
             const float4* vr = reinterpret_cast<const float4*>(v + hw + (size_t)(own * kT + t) * DV);
 #pragma unroll 8
             for (int c = tid & 1; c < DV / 4; c += 2) {
@@ -207,7 +212,7 @@ __global__ void __launch_bounds__(kBT, DV > 64 ? 1 : 2)
         const int n_loop = min(kT, L - tile * kT);
         __syncthreads();                             // the tile before is read
         load_tile<kDFeat>(s.bn, s.rn, kDFeat, true, loop_n + (size_t)tile * kT * kDFeat, n_loop, warp, lane);
-        load_tile<DV>(s.bw, KEYS ? s.rw : nullptr, S::kWide, false, loop_w + (size_t)tile * kT * DV, n_loop, warp, lane);
+        load_tile<DV, LIES && KEYS>(s.bw, KEYS ? s.rw : nullptr, S::kWide, false, loop_w + (size_t)tile * kT * loop_p, n_loop, warp, lane, loop_p);
         if (KEYS && tid < kT)
             s.st[tid] = tid < n_loop ? stats[head * (size_t)L + tile * kT + tid] : make_float2(0.f, 0.f);
         __syncthreads();
@@ -388,9 +393,9 @@ __global__ void __launch_bounds__(kBT, DV > 64 ? 1 : 2)
 }
 
 namespace {
-template <int DV, bool KEYS>
+template <int DV, bool KEYS, bool LIES>
 based_status launch_pass(const float* q, const float* k, const float* v, const float* g, float2* stats, float* dx, float* dv,
-                         int BH, int L, int numerator_only, cudaStream_t stream) {
+                         int BH, int L, int numerator_only, int dout_H, cudaStream_t stream) {
     const int smem = (int)sizeof(BwdSmem<DV, KEYS>);
     {
         static bool configured[64] = {};
@@ -398,7 +403,7 @@ based_status launch_pass(const float* q, const float* k, const float* v, const f
         if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return BASED_ERR_CUDA;
         std::lock_guard<std::mutex> lock(setup_mutex());
         if (!configured[dev]) {
-            if (cudaFuncSetAttribute(backward_f32_kernel<DV, KEYS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
+            if (cudaFuncSetAttribute(backward_f32_kernel<DV, KEYS, LIES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
                 cudaSuccess)
                 return BASED_ERR_CUDA;
             configured[dev] = true;
@@ -423,27 +428,31 @@ based_status launch_pass(const float* q, const float* k, const float* v, const f
     attr.val.clusterDim.z = nsplit;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, backward_f32_kernel<DV, KEYS>, q, k, v, g, stats, dx, dv, BH, L, numerator_only);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, backward_f32_kernel<DV, KEYS, LIES>, q, k, v, g, stats, dx, dv, BH, L, numerator_only, dout_H);
     note_launch();
     const based_status st = check_launch("backward_f32_kernel");
     return e == cudaSuccess ? st : BASED_ERR_CUDA;
 }
-template <int DV>
+template <int DV, bool LIES>
 based_status launch_dv(const float* q, const float* k, const float* v, const float* g, float* dq, float* dk, float* dv,
-                       float2* stats, int BH, int L, int numerator_only, cudaStream_t stream) {
-    const based_status st = launch_pass<DV, false>(q, k, v, g, stats, dq, nullptr, BH, L, numerator_only, stream);
+                       float2* stats, int BH, int L, int numerator_only, int dout_H, cudaStream_t stream) {
+    const based_status st = launch_pass<DV, false, LIES>(q, k, v, g, stats, dq, nullptr, BH, L, numerator_only, dout_H, stream);
     if (st != BASED_OK) return st;
-    return launch_pass<DV, true>(q, k, v, g, stats, dk, dv, BH, L, numerator_only, stream);
+    return launch_pass<DV, true, LIES>(q, k, v, g, stats, dk, dv, BH, L, numerator_only, dout_H, stream);
 }
 }  // namespace
 
-based_status launch_prefill_backward_f32(const float* q, const float* k, const float* v, const float* g, float* dq, float* dk,
-                                         float* dv, float* stats, int BH, int L, int d_v, int numerator_only,
+based_status launch_prefill_backward_f32(const float* q, const float* k, const float* v, const float* g, int dout_H, float* dq,
+                                         float* dk, float* dv, float* stats, int BH, int L, int d_v, int numerator_only,
                                          cudaStream_t stream) {
-    float2* st = reinterpret_cast<float2*>(stats);
-    if (d_v == 64) return launch_dv<64>(q, k, v, g, dq, dk, dv, st, BH, L, numerator_only, stream);
-    if (d_v == 112) return launch_dv<112>(q, k, v, g, dq, dk, dv, st, BH, L, numerator_only, stream);
-    return launch_dv<128>(q, k, v, g, dq, dk, dv, st, BH, L, numerator_only, stream);
+    auto launch = [&](auto lies) {
+        constexpr bool LIES = decltype(lies)::value;
+        float2* st = reinterpret_cast<float2*>(stats);
+        if (d_v == 64) return launch_dv<64, LIES>(q, k, v, g, dq, dk, dv, st, BH, L, numerator_only, dout_H, stream);
+        if (d_v == 112) return launch_dv<112, LIES>(q, k, v, g, dq, dk, dv, st, BH, L, numerator_only, dout_H, stream);
+        return launch_dv<128, LIES>(q, k, v, g, dq, dk, dv, st, BH, L, numerator_only, dout_H, stream);
+    };
+    return dout_H ? launch(std::true_type{}) : launch(std::false_type{});
 }
 
 }  // namespace based

@@ -160,8 +160,9 @@ based_status launch_tokens_to_heads(const void* src, void* dst, int B, int H, in
 based_status launch_baseconv(const void* a, const void* g, const float* h, const float* b2, void* state, void* out,
                              int B, int N, int C, int width, bool step, based_dtype io, cudaStream_t stream);
 // backward of the linear attention (fp32 FMA, quadratic form); stats: [BH, L] float2 scratch
-based_status launch_prefill_backward_f32(const float* q, const float* k, const float* v, const float* g, float* dq, float* dk,
-                                         float* dv, float* stats, int BH, int L, int d_v, int numerator_only,
+// dout_H: 0, or H where g lies [B, L, H, d_v]
+based_status launch_prefill_backward_f32(const float* q, const float* k, const float* v, const float* g, int dout_H, float* dq,
+                                         float* dk, float* dv, float* stats, int BH, int L, int d_v, int numerator_only,
                                          cudaStream_t stream);
 // fp32 io in definition form on the tensor cores, operands in three bf16 parts (quadratic_f32_tc.cu): outputs from the empty
 // state, and the backward pass.  quadratic_f32_workspace_bytes: 0 where the other fp32 kernels are the faster

@@ -1,5 +1,7 @@
 """fp32 backward on 64 x 64 tiles: lengths at the tile edges, own tiles shared by one to eight CTAs of a cluster (few
 heads) and not shared (many), every value width, both forms."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -53,3 +55,19 @@ def test_backward_non_finite_values_stay_where_they_belong(L, at, bad):
         want = based.based_prefill_backward(q, k, v, g, out=out)
         got = based.based_prefill_backward(q, k, v, gb, out=out)
         assert torch.equal(got[1][:, :, at + 1:], want[1][:, :, at + 1:])
+
+
+@pytest.mark.parametrize("B,H,L,d_v", [(2, 3, 65, 128), (1, 5, 257, 112), (3, 30, 40, 64), (2, 4, 200, 64), (1, 2, 1, 112), (5, 9, 130, 128)])
+@pytest.mark.parametrize("flags", [0, based.BASED_NUMERATOR_ONLY])
+def test_backward_f32_reads_dout_as_a_projection_leaves_it(B, H, L, d_v, flags):
+    """[B,L,H,d_v], on fp32 multiply-adds: the gradients of the copy [B,H,L,d_v], bit for bit."""
+    g = torch.Generator(device="cuda").manual_seed(L)
+    q, k, v, dout = (torch.randn(B, H, L, d, generator=g, device="cuda") for d in (16, 16, d_v, d_v))
+    n = based.based_prefill_backward_workspace_bytes(B, H, L, d_v, based.BASED_F32)
+    ws, got = torch.empty(n, dtype=torch.uint8, device="cuda"), [torch.empty_like(t) for t in (q, k, v)]
+    as_it_lies = dout.transpose(1, 2).contiguous()
+    p = lambda t: ctypes.c_void_p(t.data_ptr())
+    st = based.lib().based_prefill_backward_tokens_first(p(q), p(k), p(v), p(as_it_lies), *map(p, got), B, H, L, 16, d_v, based.BASED_F32,
+                                                         flags, p(ws), n, ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert st == based.BASED_OK
+    assert all(torch.equal(a, b) for a, b in zip(got, based.based_prefill_backward(q, k, v, dout, flags=flags, workspace=ws)))

@@ -148,6 +148,14 @@ struct Workspace {
         bytes = need;
     }
 };
+// the same for scratch that a call can do without: nothing where the device has no room for it
+Workspace optional_workspace(size_t bytes, const Tensor& like) {
+    try {
+        return Workspace(kNone, bytes, like);
+    } catch (const c10::OutOfMemoryError&) {
+        return Workspace(kNone, 0, like);
+    }
+}
 // scratch that a call can do without is taken on the current stream only: on another one it could be handed out again while
 // the call still runs
 bool on_current(void* stream) { return stream == c10::cuda::getCurrentCUDAStream().stream(); }
@@ -179,10 +187,11 @@ Gradients backward_call(const Tensor& q, const Tensor& k, const Tensor& v, const
                         const Tensor& workspace, void* stream) {
     const int B = size(q, 0), H = size(q, 1), L = size(q, 2), d_feat = size(q, 3), d_v = size(v, 3);
     const based_dtype io = dtype_code(q);
-    size_t need = based_prefill_backward_workspace_bytes(B, H, L, d_v, io);
+    const size_t need = based_prefill_backward_workspace_bytes(B, H, L, d_v, io);
     // (a caller's workspace of that size is used as it is)
-    if (io == BASED_F32 && !workspace.defined() && on_current(stream)) need = std::max(need, based_f32_parts_bytes(B, H, L, d_feat, d_v, 1));
-    const Workspace ws(workspace, need, q);
+    const size_t parts = io == BASED_F32 && !workspace.defined() && on_current(stream) ? based_f32_parts_bytes(B, H, L, d_feat, d_v, 1) : 0;
+    Workspace ws = optional_workspace(parts, q);
+    if (ws.bytes < need) ws = Workspace(workspace, need, q);
     Gradients g{at::empty_like(q), at::empty_like(k), at::empty_like(v)};
     const based_status st =
         out.defined() ? based_prefill_backward_with_out(cptr(q), cptr(k), cptr(v), cptr(out), cptr(dout), ptr(g.dq), ptr(g.dk),
@@ -497,7 +506,8 @@ Gradients backward_as_it_lies(const Tensor& q, const Tensor& k, const Tensor& v,
     // d_v 112 473 us for 475, 8192 of d_v 128 124 for 123)
     if (parts == 0 && static_cast<int64_t>(B) * H * L > 16384) return {};
     const size_t bytes = std::max(based_prefill_backward_workspace_bytes(B, H, L, d_v, BASED_F32), parts);
-    const Workspace ws(kNone, bytes, q);
+    const Workspace ws = optional_workspace(bytes, q);
+    if (!ws.data) return {};
     Gradients g{at::empty_like(q), at::empty_like(k), at::empty_like(v)};
     const based_status st = based_prefill_backward_tokens_first(cptr(q), cptr(k), cptr(v), dout.const_data_ptr(), ptr(g.dq), ptr(g.dk),
                                                                 ptr(g.dv), B, H, L, d_feat, d_v, BASED_F32, flags, ws.data, ws.bytes,
@@ -520,7 +530,8 @@ Tensor forward_by_parts(const Tensor& q, const Tensor& k, const Tensor& v, int f
     const int B = size(q, 0), H = size(q, 1), L = size(q, 2), d_feat = size(q, 3), d_v = size(v, 3);
     const size_t bytes = based_f32_parts_bytes(B, H, L, d_feat, d_v, 0);
     if (bytes == 0 || (flags & ~BASED_NUMERATOR_ONLY)) return {};
-    const Workspace ws(kNone, bytes, q);
+    const Workspace ws = optional_workspace(bytes, q);
+    if (!ws.data) return {};
     Tensor out = at::empty_like(v);
     auto in = [](const Tensor& t) { return static_cast<const float*>(t.const_data_ptr()); };
     const based_status st = based_prefill_f32_parts(in(q), in(k), in(v), static_cast<float*>(ptr(out)), B, H, L, d_feat, d_v, flags,

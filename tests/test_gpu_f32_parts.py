@@ -191,3 +191,40 @@ def test_a_workspace_of_the_documented_size_is_used():
     assert extra >= large.nbytes and all(torch.equal(a, b) for a, b in zip(g_none, g_large))
     for a, b in zip(g_small, g_large):
         assert norm_err(a, wl.to_f64(b)) <= 2 * TOL_NORM
+
+
+def test_f32_parts_without_room_for_the_scratch():
+    """A device with room for the results but not for the scratch: the routes that need none, as where the scratch is refused."""
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()                                      # (no large block that what follows would be cut from)
+    x = [t.cuda() for t in inputs(100, 2000, 64, 13)]
+    q, k, v, g = x
+    lies = g.transpose(1, 2).contiguous().transpose(1, 2)         # the heads of a token side by side
+    documented = torch.empty(based.based_prefill_backward_workspace_bytes(1, 100, 2000, 64, 0), dtype=torch.uint8, device="cuda")
+    want_y = based.based_prefill(q, k, v)
+    want = based.based_prefill_backward(*x, workspace=documented)
+    leaves = [t.requires_grad_(True) for t in (q, k, v)]
+    total = torch.cuda.get_device_properties(0).total_memory
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    # the results take 51 MB (forward) and 77 MB (backward, with a copy of dout 128 MB); the scratch 115 and 192 MB
+    for room, call in [(96 << 20, lambda: [based.autograd.linear_attention(q, k, v).detach()]),
+                       (176 << 20, lambda: based.based_prefill_backward(*(t.detach() for t in x)))]:
+        torch.cuda.set_per_process_memory_fraction((torch.cuda.memory_reserved() + room) / total)
+        try:
+            got = call()
+        finally:
+            torch.cuda.set_per_process_memory_fraction(1.0)
+        assert all(torch.equal(a, b) for a, b in zip(got, [want_y] if len(got) == 1 else want))
+        del got
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+    y = based.autograd.linear_attention(*leaves)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    torch.cuda.set_per_process_memory_fraction((torch.cuda.memory_reserved() + (176 << 20)) / total)
+    try:
+        got = torch.autograd.grad(y, leaves, lies)
+    finally:
+        torch.cuda.set_per_process_memory_fraction(1.0)
+    assert all(torch.equal(a, b) for a, b in zip(got, want))

@@ -18,6 +18,14 @@ pytestmark = pytest.mark.gpu
 # times that at the worst entry of thousands (fp32 multiply-adds pair by pair: 1 to 4e-6 on these)
 TOL = 1e-5
 
+# Relative to 64 bits in the 2-norm.  An operand's parts keep 24 bits and the products left out are below 2^-25 of it; with the
+# sums' own rounding 1 to 3e-7 is measured, whatever the inputs' magnitude.  Two parts in place of three would show 4e-6.
+TOL_NORM = 1e-6
+
+
+def norm_err(got, want):
+    return np.linalg.norm(wl.to_f64(got) - want) / np.linalg.norm(want)
+
 
 def inputs(BH, L, d_v, seed):
     w = wl.Workload("parts", 1, BH, L, 16, d_v, "f32", 1.0)
@@ -56,13 +64,13 @@ def test_f32_parts(BH, L, d_v, flags):
         c = s[0] @ s[1].swapaxes(-1, -2)
         want = want * np.tril(1 + c / 4 + c * c / 32).sum(-1, keepdims=True)
     assert row_err(wl.to_f64(y[:, heads]), want) <= TOL_F32
-    assert np.abs(wl.to_f64(y[:, heads]) - want).max() <= TOL * np.abs(want).max()
+    assert norm_err(y[:, heads], want) <= TOL_NORM
     p = lambda t: ctypes.c_void_p(t.data_ptr())
     stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
     if d_v == 64:
         got = based.based_prefill_backward(*x, flags=flags)
         for a, b in zip(got, oracle.linattn_backward(*s, numerator_only=bool(flags))):
-            assert np.abs(wl.to_f64(a[:, heads]) - b).max() <= TOL * np.abs(b).max()
+            assert norm_err(a[:, heads], b) <= TOL_NORM
         assert all(torch.equal(a, b) for a, b in zip(got, based.based_prefill_backward(*x, flags=flags)))
         # with the scratch of the call without parts
         n = lib.based_prefill_backward_workspace_bytes(1, BH, L, 64, 0)
@@ -95,11 +103,14 @@ def test_f32_parts_of_large_values(BH, L, big):
     assert torch.allclose(out[:, :, :at], want[:, :, :at], rtol=0, atol=1e-4)
     cols = [c for c in range(64) if c != 3]
     assert torch.allclose(out[..., cols], want[..., cols], rtol=0, atol=1e-4)
-    w = wl.to_f64(vb[:, :1])
-    ref, _, _ = oracle.linattn_quadratic(wl.to_f64(q[:, :1]), wl.to_f64(k[:, :1]), w)
-    ok = np.abs(ref) < 1e38                                       # (a sum over D that would overflow in fp32 is infinite or NaN)
-    got = out[:, :1].double().cpu().numpy()
-    assert (np.abs(got - ref)[ok] <= 1e-4 * np.maximum(np.abs(ref), 1.0)[ok])[np.isfinite(got)[ok]].all()
+    # column 3 from the value on: one term is all of it; infinite only where the sum over D would overflow in fp32
+    x = [wl.to_f64(t[:, :1]) for t in (q, k, vb)]
+    c = x[0] @ x[1].swapaxes(-1, -2)
+    weights = np.tril(1 + c / 4 + c * c / 32)
+    num = (weights @ x[2])[0, 0, at:, 3]
+    ref, got = num / weights.sum(-1)[0, 0, at:], wl.to_f64(out[:, :1])[0, 0, at:, 3]
+    fits = np.abs(num) < 0.999 * np.finfo(np.float32).max
+    assert fits.any() and (big > 1e38 or fits.all()) and (np.abs(got - ref)[fits] <= TOL * np.abs(ref)[fits]).all()
 
 
 def test_f32_parts_slabs_of_heads():
@@ -120,10 +131,9 @@ def test_f32_parts_slabs_of_heads():
     for h in (0, 149, 278, 279, 280, 299):
         one = [t[:, h:h + 1].contiguous() for t in flat]
         want = forward(*one[:3])
-        assert (y[:, h:h + 1] - want).abs().max() <= TOL * want.abs().max()
+        assert norm_err(y[:, h:h + 1], wl.to_f64(want)) <= 2 * TOL_NORM
         for a, b in zip(got, based.based_prefill_backward(*one)):
-            a = a.reshape(1, B * H, L, -1)[:, h:h + 1]
-            assert (a - b).abs().max() <= TOL * b.abs().max()
+            assert norm_err(a.reshape(1, B * H, L, -1)[:, h:h + 1], wl.to_f64(b)) <= 2 * TOL_NORM
     assert based.based_poll_error() == based.BASED_OK
 
 
@@ -143,15 +153,6 @@ def test_f32_parts_non_finite_tokens_stay_behind(BH, L, d_v, which, bad):
         assert torch.equal(torch.isfinite(out), torch.isfinite(ref))
         ok = torch.isfinite(ref)
         assert torch.allclose(out[ok], ref[ok], rtol=1e-5, atol=1e-4)
-
-
-# Relative to 64 bits in the 2-norm.  An operand's parts keep 24 bits and the products left out are below 2^-25 of it; with the
-# sums' own rounding 1 to 3e-7 is measured, whatever the inputs' magnitude.  Two parts in place of three would show 4e-6.
-TOL_NORM = 1e-6
-
-
-def norm_err(got, want):
-    return np.linalg.norm(wl.to_f64(got) - want) / np.linalg.norm(want)
 
 
 @pytest.mark.parametrize("scale", [1e-30, 1e-36])
@@ -228,3 +229,32 @@ def test_f32_parts_without_room_for_the_scratch():
     finally:
         torch.cuda.set_per_process_memory_fraction(1.0)
     assert all(torch.equal(a, b) for a, b in zip(got, want))
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("which", range(4))
+@pytest.mark.parametrize("BH,L", [(1, 64), (3, 300), (1, 1000), (150, 70)])
+@pytest.mark.parametrize("flags", [0, based.BASED_NUMERATOR_ONLY])
+def test_f32_parts_gradients_of_non_finite_tokens(BH, L, which, bad, flags):
+    """A non-finite q, k, v or dout of one token: the gradients that it does not enter are those without it, whichever way dout lies."""
+    assert based.based_f32_parts_bytes(1, BH, L, 16, 64, True) > 0
+    x = [t.cuda() for t in inputs(BH, L, 64, L)]
+    want = based.based_prefill_backward(*x, flags=flags)
+    at = torch.arange(L, device="cuda")
+    for t in sorted({L // 2, L - 1, 5}):
+        before, behind, others, none = at < t, at > t, at != t, at < 0
+        # rows of dq, dk, dv.  A query's statistics carry a bad k or v to every key at or before it, unless there are none (numerator)
+        clean = [(others, behind, behind),
+                 (before, others, others) if flags else (before, none, none),
+                 (before, others, at >= 0) if flags else (before, none, at >= 0),
+                 (others, behind, behind)][which]
+        y = [u.clone() for u in x]
+        y[which][:, :, t, 1] = bad
+        leaves = [u.clone().requires_grad_(True) for u in y[:3]]
+        lies = y[3].transpose(1, 2).contiguous().transpose(1, 2)
+        for got in (based.based_prefill_backward(*y, flags=flags),
+                    torch.autograd.grad(based.autograd.linear_attention(*leaves, numerator_only=bool(flags)), leaves, lies)):
+            for a, b, rows in zip(got, want, clean):
+                if rows.any():
+                    assert norm_err(a[:, :, rows], wl.to_f64(b[:, :, rows])) <= 2 * TOL_NORM
+    assert based.based_poll_error() == based.BASED_OK

@@ -709,7 +709,7 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd && DV == 64 && LT 
                 if (blk == 0) may_pack();
                 packed_out(blk, pw, pd);
             };
-            if (MODE == kModeFwd && c0 + LT <= r0) {         // two column groups in flight (63 -> 60 us at B4 H16 L2048 d_v 128)
+            if (MODE == kModeFwd && c0 + LT <= r0) {         // two column groups in flight (63 -> 60 us at B4 H16 L2048 d_v 128 when those ran here)
 #pragma unroll
                 for (int blk = 0; blk < LT / 32; ++blk) pass(std::false_type{}, blk);
             } else
@@ -1063,9 +1063,10 @@ based_status launch_dvb(const void* q, const void* k, const void* v, const void*
 based_status launch_quadratic_forward_tc(const void* q, const void* k, const void* v, void* out, int BH, int L,
                                          int d_feat, int d_v, int numerator_only, bool overlapped, cudaStream_t stream) {
     // Two groups of row warps on one tile after the other (quadratic_fwd_tc.cu) where that is the faster, us, that / this at d' 24: d_v
-    // 128 B4 H16 L2048 49 / 59, L4096 164 / 216; d_v 64 L2048 with 1 head 11.8 / 20.3, L1100 with 16 8.6 / 13.4, L200 5.0 / 5.9, L64
-    // 4.1 / 3.9, L2048 with 64 (1024 CTAs) 37.4 / 37.1, L8192 446 / 441; with the state beside it L128 with 64 9.3 / 8.5
-    if (d_v != 64 || (L > kTile && (long long)((L + kTile - 1) / kTile) * BH <= 2 * kSMs))
+    // 128 B4 H16 L2048 49 / 59, L4096 164 / 216, but one key tile, L33, with 1 head 4.5 / 4.4, with 150 5.8 / 5.4, with 600 12.0 / 11.6; d_v
+    // 64 L2048 with 1 head 11.8 / 20.3, L1100 with 16 8.6 / 13.4, L200 5.0 / 5.9, L64 4.1 / 3.9, L2048 with 64 (1024 CTAs) 37.4 / 37.1,
+    // L8192 446 / 441; with the state beside it L128 with 64 9.3 / 8.5
+    if (d_v != 64 ? L > 64 : L > kTile && (long long)((L + kTile - 1) / kTile) * BH <= 2 * kSMs)
         return launch_quadratic_groups_tc(q, k, v, out, BH, L, d_feat, d_v, numerator_only, overlapped, stream);
     CUtensorMap tq, tk64, tv64, tout;
     const CUtensorMapSwizzle s64 = CU_TENSOR_MAP_SWIZZLE_64B, s128 = CU_TENSOR_MAP_SWIZZLE_128B;
@@ -1085,7 +1086,8 @@ based_status launch_quadratic_forward_tc(const void* q, const void* k, const voi
     const dim3 grid((unsigned)((L + kTile - 1) / kTile) * BH);
     p.heads = BH;
     p.by_length = long_loops_first(BH, L);
-    return launch_pass<64, kModeFwd, 64>(tq, tq, tk64, tv64, p, grid, "quadratic forward (tc)", stream, nullptr, &tout);
+    if (d_v == 64) return launch_pass<64, kModeFwd, 64>(tq, tq, tk64, tv64, p, grid, "quadratic forward (tc)", stream, nullptr, &tout);
+    return launch_pass<128, kModeFwd, 64>(tq, tq, tk64, tv64, p, grid, "quadratic forward (tc)", stream, nullptr, &tout);
 }
 
 int backward_tc_block_tokens(int BH, int L, int d_feat, int d_v, int merged) {

@@ -1,6 +1,7 @@
 // based_prefill_backward for fp32 io (d' = 16): gradients of the causal Taylor linear attention (definition form, left-hand
 // side of Eq. (2) of Sec. 4.1).  The paper gives no backward algorithm; this is the chain rule on the definition, evaluated
-// tile by tile in the quadratic ("attention") form with fp32 FMAs (bf16 / tf32 operands cannot meet fp32's tolerance):
+// tile by tile in the quadratic ("attention") form with fp32 FMAs.  d_v 112 and 128, and d_v 64 where operands split into bf16
+// parts for the tensor cores (quadratic_f32_tc.cu) are not the faster or have no scratch:
 //
 //   y_i = N_i / D_i,  N_i = sum_{j<=i} w_ij v_j,  D_i = sum_{j<=i} w_ij + eps,  w_ij = 1 + s/4 + s^2/32,
 //   s = q_i.k_j;  with G_i the gradient of the loss with respect to y_i:

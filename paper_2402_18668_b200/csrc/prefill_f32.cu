@@ -1,8 +1,8 @@
 // based_prefill for fp32 io (d' = 16): causal Taylor linear attention in chunked form with fp32 FMAs, the sequence of a
 // head spread over the CTAs of one thread-block cluster.
 //
-// Tensor-core operand formats (bf16, tf32) cannot meet fp32's tolerance, so the contractions are register-tiled products
-// on the fp32 pipe (two-wide fma.rn.f32x2), fed from shared memory.  One CTA holds 64 value columns of one sequence
+// One bf16 or tf32 operand per fp32 value cannot meet fp32's tolerance (three bf16 parts can: quadratic_f32_tc.cu, training's
+// forward pass, in definition form and without a state), so the contractions are register-tiled products on the fp32 pipe (two-wide fma.rn.f32x2), fed from shared memory.  One CTA holds 64 value columns of one sequence
 // segment; the cluster's CTAs are the segments of a head in order (and, above 64 columns, its column groups):
 //   1. every segment sums its own state  S_seg = sum_j psi(k_j) v_j^T  (153 features, one per unordered pair) and z_seg,
 //      and leaves it in shared memory;

@@ -33,10 +33,11 @@
 // comes out is not finite: such rows are computed once more with plain fp32 multiply-adds, masked pairs left out (B2 H16 L1024 with a value of NaN in each head: 330 and 1000 us).
 //
 // Measured at B2 H16 L1024 d_v 64, against fp32 multiply-adds: forward 72 -> 28 us, backward 269 -> 80, errors in the 2-norm 0.8e-7
-// for 1.9e-7 (outputs), 1.7e-7 for 2.8e-7 (dq), 1.9e-7 for 4.1e-7 (dk), 1.4e-7 for 7.6e-7 (dv).  Per looped tile the forward takes 1250
-// cycles, dq 2400, dk and dv 2600.  What bounds them: an MMA with both operands in shared memory is read at 128 bytes per cycle, 48
+// for 1.9e-7 (outputs), 1.7e-7 for 2.8e-7 (dq), 1.9e-7 for 4.1e-7 (dk), 1.4e-7 for 7.6e-7 (dv).  The SMs are active for 39 k, 60 k and
+// 68 k cycles of 15.6 looped tiles each, the tensor pipe in 38, 35 and 44 % of them.  What bounds them: an MMA with both operands in shared memory is read at 128 bytes per cycle, 48
 // cycles at N = 64 where the tensor pipe needs 32, so the 30 of a tile's scores and products take 1440 cycles, those of dk and dv
-// 990.  The 256 CTAs of such a call are 1.7 waves, with some 8 k cycles of start and end each.
+// 990.  The 256 CTAs of such a call are 1.7 waves, with some 8 k cycles of start and end each.  480 threads leave 128 registers:
+// the forward for d_v 112 and 128, whose collectors hold 128 sums a thread, spills 0.9 KB, dq 0.1 KB.
 #include <cooperative_groups.h>
 
 #include <mutex>

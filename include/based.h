@@ -94,17 +94,19 @@ size_t based_prefill_workspace_bytes(int B, int H, int L, int d_feat, int d_v, b
 
 /*
  * Scratch with which an fp32 pass runs on the tensor cores, its operands split into three bf16 parts each (results at least
- * as close to exact ones as fp32 multiply-adds give, over the whole range of fp32; rows that meet values from about 1e24 on
- * may be computed by multiply-adds after all, which takes longer): based_prefill_f32_parts (backward = 0), and the backward pass at d_v 64
- * (backward = 1), which takes that route when its workspace has this many bytes, else one that needs
- * based_prefill_backward_workspace_bytes.  0: there is no such route for these arguments, or it is not the faster one.
+ * as close to exact ones as fp32 multiply-adds give, over the whole range of fp32; rows that meet values, or products of two,
+ * from about 1e24 on may be computed by multiply-adds after all, which takes longer): based_prefill_f32_parts (backward = 0), and
+ * the backward pass at d_v 64 (backward = 1), which takes that route when its workspace has this many bytes, else, with
+ * based_prefill_backward_workspace_bytes, the one of multiply-adds: the last bits of its results depend on the workspace's
+ * size.  0: there is no such route for these arguments, or it is not the faster one.
  */
 size_t based_f32_parts_bytes(int B, int H, int L, int d_feat, int d_v, int backward);
 
 /*
  * The outputs of based_prefill from the empty state, fp32 io, that way (training's forward pass).  Rounded differently from
  * based_prefill's, whose outputs are the same bit for bit whether the state is asked for or not.  workspace:
- * based_f32_parts_bytes(..., 0); BASED_ERR_UNSUPPORTED where that is 0.  flags: 0 or BASED_NUMERATOR_ONLY.
+ * based_f32_parts_bytes(..., 0); BASED_ERR_UNSUPPORTED where that is 0 or the heads are more than 65532.  flags: 0 or
+ * BASED_NUMERATOR_ONLY.
  */
 based_status based_prefill_f32_parts(const float* q, const float* k, const float* v, float* out, int B, int H, int L, int d_feat,
                                      int d_v, int flags, void* workspace, size_t workspace_bytes, void* cuda_stream);
@@ -230,8 +232,8 @@ based_status swa_decode_step(const void* q, const void* k, const void* v, void* 
  * s^2/(2 d'), so ds_ij = (a_i . v_j + b_i)(1/sqrt(d') + q_i.k_j / d')); d_v in {64, 112, 128}.
  * Both paths evaluate the quadratic form, O(L^2) per head, on 128 x 128 (bf16 io: tcgen05 tensor
  * cores, bf16 operands, fp32 accumulation) or 64 x 64 (fp32 io: fp32 FMAs; with the scratch of
- * based_f32_parts_bytes 128 x 64, tensor cores) tiles of (query, key) pairs; with bf16 io and d_feat = 16 longer sequences take the block-wise path described at
- * based_prefill_backward_with_out (the forward output that it needs is recomputed into the workspace:
+ * based_f32_parts_bytes 128 x 64, tensor cores) tiles of (query, key) pairs; with bf16 io and d_feat = 16
+ * longer sequences take the block-wise path described at based_prefill_backward_with_out (the forward output that it needs is recomputed into the workspace:
  * one forward pass more).  Gradient outputs must not alias inputs.
  */
 based_status based_prefill_backward(const void* q, const void* k, const void* v, const void* dout, void* dq,

@@ -237,7 +237,8 @@ def based_prefill_state(k, v, kv_state=None, z_state=None, flags: int = BASED_ST
     _check_state(kv_state, z_state, B, H, d_feat, d_v, flags, required=True)
     need = int(lib().based_prefill_state_workspace_bytes(B, H, L, d_feat, d_v, _dtype_code(k)))
     if need and (workspace is None or workspace.numel() * workspace.element_size() < need):
-        workspace = torch.empty(need, dtype=torch.uint8, device=k.device)
+        with torch.cuda.stream(stream):                  # (None: the current one)  memory of the call's own stream
+            workspace = torch.empty(need, dtype=torch.uint8, device=k.device)
     st = lib().based_prefill_state(_ptr(k), _ptr(v), _ptr(kv_state), _ptr(z_state), B, H, L, d_feat, d_v, _dtype_code(k),
                                    int(flags), _ptr(workspace),
                                    0 if workspace is None else workspace.numel() * workspace.element_size(),
@@ -250,8 +251,8 @@ def based_prefill_backward(q, k, v, dout, flags: int = 0, workspace=None, stream
     """Gradients (dq, dk, dv) of based_prefill (empty initial state) for the output gradient dout.
     out: the forward output, if the caller kept it (based_prefill_backward_with_out).
     workspace: used if it has based_prefill_backward_workspace_bytes.  fp32: with based_f32_parts_bytes(..., backward=True) of
-    workspace, or none given and the call on the current stream, the pass runs on the tensor cores, else on fp32
-    multiply-adds: equal up to rounding."""
+    workspace, or none given (and room for it), the pass runs on the tensor cores, else on fp32 multiply-adds: equal up to
+    rounding."""
     return (_native_module or native()).prefill_backward(q, k, v, dout, int(flags), workspace, _handle(stream), out)
 
 

@@ -129,13 +129,14 @@ void check_caches(const Tensor& kc, const Tensor& vc, const Tensor& q, const cha
 void check(based_status st, const char* where) {
     if (st != BASED_OK) throw StatusFault(st, where);
 }
-// a workspace of at least `bytes` bytes: the caller's, or a fresh one that lives as long as this object (memory of torch's
-// allocator on the current stream, as a tensor would hold it but without the tensor: 0.3 us for 0.7)
+// a workspace of at least `need` bytes: the caller's, or a fresh one that lives as long as this object (memory of torch's
+// allocator, as a tensor would hold it but without the tensor: 0.3 us for 0.7).  It belongs to the call's own stream, which may
+// be another than the current one: only what follows on that stream is given it again.
 struct Workspace {
     c10::DataPtr own;
     void* data = nullptr;
     size_t bytes = 0;
-    Workspace(const Tensor& given, size_t need, const Tensor& like) {
+    Workspace(const Tensor& given, size_t need, const Tensor& like, void* stream) {
         if (need == 0 || (given.defined() && given.nbytes() >= need)) {
             if (!given.defined()) return;
             data = given.mutable_data_ptr();
@@ -143,22 +144,22 @@ struct Workspace {
             return;
         }
         const c10::cuda::CUDAGuard on(like.device());
+        c10::cuda::OptionalCUDAStreamGuard of;
+        if (stream != c10::cuda::getCurrentCUDAStream().stream())
+            of.reset_stream(c10::cuda::getStreamFromExternal(static_cast<cudaStream_t>(stream), like.get_device()));
         own = c10::cuda::CUDACachingAllocator::get()->allocate(need);
         data = own.get();
         bytes = need;
     }
 };
 // the same for scratch that a call can do without: nothing where the device has no room for it
-Workspace optional_workspace(size_t bytes, const Tensor& like) {
+Workspace optional_workspace(size_t bytes, const Tensor& like, void* stream) {
     try {
-        return Workspace(kNone, bytes, like);
+        return Workspace(kNone, bytes, like, stream);
     } catch (const c10::OutOfMemoryError&) {
-        return Workspace(kNone, 0, like);
+        return Workspace(kNone, 0, like, stream);
     }
 }
-// scratch that a call can do without is taken on the current stream only: on another one it could be handed out again while
-// the call still runs
-bool on_current(void* stream) { return stream == c10::cuda::getCurrentCUDAStream().stream(); }
 // the library's calls run without the interpreter lock: a launch can wait for room in the stream's queue
 template <typename F> based_status unlocked(F f) {
     based_status st;
@@ -176,7 +177,7 @@ Tensor prefill_call(const Tensor& q, const Tensor& k, const Tensor& v, const Ten
     if (!out.defined()) out = at::empty_like(v);
     size_t need = based_prefill_workspace_bytes(B, H, L, d_feat, d_v, io);
     if (need <= BASED_WORDS_BYTES && !(flags & BASED_STATE_CONTINUE)) need = 0;
-    const Workspace ws(workspace, need, q);
+    const Workspace ws(workspace, need, q, stream);
     check(based_prefill(cptr(q), cptr(k), cptr(v), ptr(out), fptr(kv), fptr(z), B, H, L, d_feat, d_v, io, flags, ws.data, ws.bytes,
                         stream),
           "based_prefill");
@@ -189,9 +190,9 @@ Gradients backward_call(const Tensor& q, const Tensor& k, const Tensor& v, const
     const based_dtype io = dtype_code(q);
     const size_t need = based_prefill_backward_workspace_bytes(B, H, L, d_v, io);
     // (a caller's workspace of that size is used as it is)
-    const size_t parts = io == BASED_F32 && !workspace.defined() && on_current(stream) ? based_f32_parts_bytes(B, H, L, d_feat, d_v, 1) : 0;
-    Workspace ws = optional_workspace(parts, q);
-    if (ws.bytes < need) ws = Workspace(workspace, need, q);
+    const size_t parts = io == BASED_F32 && !workspace.defined() ? based_f32_parts_bytes(B, H, L, d_feat, d_v, 1) : 0;
+    Workspace ws = optional_workspace(parts, q, stream);
+    if (ws.bytes < need) ws = Workspace(workspace, need, q, stream);
     Gradients g{at::empty_like(q), at::empty_like(k), at::empty_like(v)};
     const based_status st =
         out.defined() ? based_prefill_backward_with_out(cptr(q), cptr(k), cptr(v), cptr(out), cptr(dout), ptr(g.dq), ptr(g.dk),
@@ -506,7 +507,7 @@ Gradients backward_as_it_lies(const Tensor& q, const Tensor& k, const Tensor& v,
     // d_v 112 473 us for 475, 8192 of d_v 128 124 for 123)
     if (parts == 0 && static_cast<int64_t>(B) * H * L > 16384) return {};
     const size_t bytes = std::max(based_prefill_backward_workspace_bytes(B, H, L, d_v, BASED_F32), parts);
-    const Workspace ws = optional_workspace(bytes, q);
+    const Workspace ws = optional_workspace(bytes, q, stream);
     if (!ws.data) return {};
     Gradients g{at::empty_like(q), at::empty_like(k), at::empty_like(v)};
     const based_status st = based_prefill_backward_tokens_first(cptr(q), cptr(k), cptr(v), dout.const_data_ptr(), ptr(g.dq), ptr(g.dk),
@@ -530,7 +531,7 @@ Tensor forward_by_parts(const Tensor& q, const Tensor& k, const Tensor& v, int f
     const int B = size(q, 0), H = size(q, 1), L = size(q, 2), d_feat = size(q, 3), d_v = size(v, 3);
     const size_t bytes = based_f32_parts_bytes(B, H, L, d_feat, d_v, 0);
     if (bytes == 0 || (flags & ~BASED_NUMERATOR_ONLY)) return {};
-    const Workspace ws = optional_workspace(bytes, q);
+    const Workspace ws = optional_workspace(bytes, q, stream);
     if (!ws.data) return {};
     Tensor out = at::empty_like(v);
     auto in = [](const Tensor& t) { return static_cast<const float*>(t.const_data_ptr()); };

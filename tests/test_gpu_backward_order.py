@@ -49,3 +49,25 @@ def test_tile_passes_in_either_order(d_feat, d_v, BH, L, with_out):
 def test_lines_of_the_blockwise_path(d_v, BH, L, tokens):
     assert based.lib().based_prefill_backward_block_tokens(1, BH, L, 16, d_v, 1, 0, 1) == tokens
     _check(*_inputs(BH, L, 16, d_v), True)
+
+
+@pytest.mark.parametrize("io", ["f32", "bf16"])
+def test_scratch_of_a_call_belongs_to_its_stream(io):
+    """Scratch of a call on another stream than the current one is not handed out on the current one, where nothing waits for that
+    call; and the results are those of the current stream."""
+    B, H, L = (2, 16, 1024) if io == "f32" else (4, 16, 2048)
+    g = torch.Generator(device="cuda").manual_seed(1)
+    dt = torch.float32 if io == "f32" else torch.bfloat16
+    q, v, dout = (torch.randn(B, H, L, d, generator=g, device="cuda").to(dt) for d in (16, 64, 64))
+    want = based.based_prefill_backward(q, q, v, dout)
+    other = torch.cuda.Stream()
+    other.wait_stream(torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    got = based.based_prefill_backward(q, q, v, dout, stream=other)
+    torch.cuda.synchronize()
+    reserved = torch.cuda.memory_reserved()
+    after = torch.empty(25 << 20, dtype=torch.uint8, device="cuda")          # (the scratch: 28 and 30 MB)
+    assert torch.cuda.memory_reserved() > reserved
+    del after
+    assert all(torch.equal(a, b) for a, b in zip(got, want))

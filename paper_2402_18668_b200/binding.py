@@ -237,7 +237,8 @@ def based_prefill_state(k, v, kv_state=None, z_state=None, flags: int = BASED_ST
     _check_state(kv_state, z_state, B, H, d_feat, d_v, flags, required=True)
     need = int(lib().based_prefill_state_workspace_bytes(B, H, L, d_feat, d_v, _dtype_code(k)))
     if need and (workspace is None or workspace.numel() * workspace.element_size() < need):
-        with torch.cuda.stream(stream):                  # (None: the current one)  memory of the call's own stream
+        own = None if stream is None else torch.cuda.ExternalStream(stream.cuda_stream, device=k.device)
+        with torch.cuda.stream(own):                     # memory of the call's own stream (None: the current one)
             workspace = torch.empty(need, dtype=torch.uint8, device=k.device)
     st = lib().based_prefill_state(_ptr(k), _ptr(v), _ptr(kv_state), _ptr(z_state), B, H, L, d_feat, d_v, _dtype_code(k),
                                    int(flags), _ptr(workspace),

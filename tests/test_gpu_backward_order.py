@@ -51,23 +51,27 @@ def test_lines_of_the_blockwise_path(d_v, BH, L, tokens):
     _check(*_inputs(BH, L, 16, d_v), True)
 
 
-@pytest.mark.parametrize("io", ["f32", "bf16"])
-def test_scratch_of_a_call_belongs_to_its_stream(io):
+@pytest.mark.parametrize("what", ["backward f32", "backward bf16", "state"])
+def test_scratch_of_a_call_belongs_to_its_stream(what):
     """Scratch of a call on another stream than the current one is not handed out on the current one, where nothing waits for that
     call; and the results are those of the current stream."""
-    B, H, L = (2, 16, 1024) if io == "f32" else (4, 16, 2048)
+    B, H, L, d_v = {"backward f32": (2, 16, 1024, 64), "backward bf16": (4, 16, 2048, 64), "state": (1, 148, 2048, 128)}[what]
     g = torch.Generator(device="cuda").manual_seed(1)
-    dt = torch.float32 if io == "f32" else torch.bfloat16
-    q, v, dout = (torch.randn(B, H, L, d, generator=g, device="cuda").to(dt) for d in (16, 64, 64))
-    want = based.based_prefill_backward(q, q, v, dout)
+    dt = torch.float32 if what == "backward f32" else torch.bfloat16
+    q, v, dout = (torch.randn(B, H, L, d, generator=g, device="cuda").to(dt) for d in (16, d_v, d_v))
+
+    def call(stream=None):
+        if what == "state":
+            return based.based_prefill_state(q, v, stream=stream)
+        return based.based_prefill_backward(q, q, v, dout, stream=stream)
+    want = call()
     other = torch.cuda.Stream()
-    other.wait_stream(torch.cuda.current_stream())
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
-    got = based.based_prefill_backward(q, q, v, dout, stream=other)
+    got = call(other)
     torch.cuda.synchronize()
     reserved = torch.cuda.memory_reserved()
-    after = torch.empty(25 << 20, dtype=torch.uint8, device="cuda")          # (the scratch: 28 and 30 MB)
+    after = torch.empty((11 if what == "state" else 25) << 20, dtype=torch.uint8, device="cuda")     # (the scratch: 12 and 28 to 30 MB)
     assert torch.cuda.memory_reserved() > reserved
     del after
     assert all(torch.equal(a, b) for a, b in zip(got, want))

@@ -70,7 +70,7 @@ template <int DV, int MODE> struct QCfg {
     static constexpr uint32_t offOwnN = 0, offOwnW = kOwn * 128, offStage = offOwnW + (kBwd ? 3 * kOwnPart : 0);
     static constexpr uint32_t kStage = kNarrow + 3 * kPart;
     static constexpr int kNS = kBwd ? 4 : DV == 64 ? 6 : 3;
-    static constexpr uint32_t offStats = offStage + kNS * kStage;      // keys pass: 1/D, then b, of a stage's queries
+    static constexpr uint32_t offStats = offStage + kNS * kStage;      // keys pass: inv, then b (QParams), of a stage's queries
     static constexpr uint32_t offSum = offStats + (MODE == kKeys ? kNS * kLT * 8 : 0);                // row sums of the two row groups
     static constexpr uint32_t offBars = offSum + 2 * kOwn * 8;
     static constexpr uint32_t kSmem = offBars + 512 + 1024;
@@ -435,7 +435,7 @@ __global__ void __launch_bounds__(kNThreads, 1)
     tc_fence_after();
     const uint32_t tb = *tmem_base_s;
     bool ok = true;
-    asm volatile("griddepcontrol.wait;" ::: "memory");                 // the parts; kKeys: 1/D and b
+    asm volatile("griddepcontrol.wait;" ::: "memory");                 // the parts; kKeys: inv and b
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     if (warp == 12 || warp == 14) {

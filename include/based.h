@@ -384,15 +384,15 @@ based_status based_generation_step(const void* q, const void* k, const void* v, 
                                    void* cuda_stream);
 
 /*
- * The same step held as a CUDA graph of one kernel node, for a loop that takes every token's inputs from a different
- * place: based_generation_graph_step points the node at this token's inputs and launches the graph (no copies into fixed
- * input buffers ahead of it, one launch per token).  The arguments of based_generation_graph_create are those of
- * based_generation_step; q, k, v, qw, kw, vw are buffers that hold the inputs of the last token: a step with inputs of its
- * own (device pointers of the same layout, 16-byte aligned, read in stream order like any launch's inputs; overlapping
- * neither another input's buffer nor anything that the step writes: the outputs, the state, the caches, the position) leaves
- * a copy in them, a step with six NULLs runs on what they hold.  All other pointers are
- * fixed at creation and must outlive the graph.  Creation launches nothing; call based_preload_decode first.  Steps of one
- * graph may come from several threads; like the step's state they belong on one stream at a time.
+ * The same step held with its arguments, for a loop that takes every token's inputs from a different place:
+ * based_generation_graph_step launches it on this token's inputs (no copies into fixed input buffers ahead of it, one launch
+ * per token).  The arguments of based_generation_graph_create are those of based_generation_step; q, k, v, qw, kw, vw are
+ * buffers that hold the inputs of the last token: a step with inputs of its own (device pointers of the same layout, 16-byte
+ * aligned, read in stream order like any launch's inputs; overlapping neither another input's buffer nor anything that the
+ * step writes: the outputs, the state, the caches, the position) leaves a copy in them, a step with six NULLs runs on what they
+ * hold.  All other pointers are fixed at creation and must outlive the graph.  Creation launches nothing; call
+ * based_preload_decode first.  Steps of one graph may come from several threads and on any streams of its device: each runs
+ * behind the one before it.  Not on a stream under capture (BASED_ERR_CUDA).
  */
 typedef struct based_generation_graph based_generation_graph;
 based_status based_generation_graph_create(void* q, void* k, void* v, float* kv_state, float* z_state, void* out, void* qw,

@@ -376,11 +376,10 @@ based_status swa_decode_step_advance(const void* q, const void* k, const void* v
                              static_cast<cudaStream_t>(cuda_stream));
 }
 
-based_status based_generation_step(const void* q, const void* k, const void* v, float* kv_state, float* z_state,
-                                   void* out, const void* qw, const void* kw, const void* vw, void* k_cache,
-                                   void* v_cache, void* out_w, int B, int H, int d_feat, int d_v, int H_w, int d_w,
-                                   int window, int* pos_state, float softmax_scale, based_dtype io, int flags,
-                                   void* cuda_stream) {
+static based_status generation_step_check(const void* q, const void* k, const void* v, const float* kv_state, const float* z_state,
+                                          const void* out, const void* qw, const void* kw, const void* vw, const void* k_cache,
+                                          const void* v_cache, const void* out_w, int B, int H, int d_feat, int d_v, int H_w, int d_w,
+                                          int window, const int* pos_state, based_dtype io, int flags) {
     if (!q || !k || !v || !kv_state || !z_state || !out || !qw || !kw || !vw || !k_cache || !v_cache || !out_w ||
         !pos_state || B <= 0 || H <= 0 || H_w <= 0 || window <= 0)
         return BASED_ERR_INVALID_ARG;
@@ -392,28 +391,41 @@ based_status based_generation_step(const void* q, const void* k, const void* v, 
         !aligned16(out) || !aligned16(qw) || !aligned16(kw) || !aligned16(vw) || !aligned16(k_cache) ||
         !aligned16(v_cache) || !aligned16(out_w) || (reinterpret_cast<uintptr_t>(pos_state) & 7u))
         return BASED_ERR_ALIGNMENT;
+    return BASED_OK;
+}
+
+based_status based_generation_step(const void* q, const void* k, const void* v, float* kv_state, float* z_state,
+                                   void* out, const void* qw, const void* kw, const void* vw, void* k_cache,
+                                   void* v_cache, void* out_w, int B, int H, int d_feat, int d_v, int H_w, int d_w,
+                                   int window, int* pos_state, float softmax_scale, based_dtype io, int flags,
+                                   void* cuda_stream) {
+    const based_status st = generation_step_check(q, k, v, kv_state, z_state, out, qw, kw, vw, k_cache, v_cache, out_w, B, H, d_feat,
+                                                  d_v, H_w, d_w, window, pos_state, io, flags);
+    if (st != BASED_OK) return st;
     const float scale = softmax_scale > 0.f ? softmax_scale : 0.125f;   // 1/sqrt(64)
     return launch_generation_step(q, k, v, kv_state, z_state, out, B * H, d_v, (flags & BASED_STATE_SYM) != 0,
                                   (flags & BASED_NUMERATOR_ONLY) != 0, qw, kw, vw, k_cache, v_cache, out_w, B * H_w,
                                   window, pos_state, scale, io, static_cast<cudaStream_t>(cuda_stream));
 }
 
+// The step's arguments, and the order of its launches.  The kernel is launched as based_generation_step's is, not as a node of
+// an instantiated graph: a dependent launch is on the SMs while the one before it drains, which graph launches, each behind
+// the end of the one before, are not (16 heads x batch 8 / 16 / 32, 153 rows, d_v 128, on states from memory: 10.5 -> 8.3,
+// 13.5 -> 10.2, 20.3 -> 16.8 us per step).  What a graph's launches give besides, an order among themselves whichever streams
+// they are on, an event behind every step keeps.
 struct based_generation_graph {
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
-    cudaGraphNode_t node = nullptr;
-    cudaKernelNodeParams params{};
-    std::vector<unsigned char> args;           // the kernel's one argument
-    void* arg_list[1] = {nullptr};
+    std::vector<unsigned char> args;           // launch_generation_args
     void* buffers[6] = {};
-    bool own_inputs = false;                   // the node points at inputs other than the buffers
+    bool own_inputs = false;                   // the arguments point at inputs other than the buffers
+    cudaEvent_t done = nullptr;                // behind the last step
+    unsigned long long last_stream = 0;        // its stream's number, which no later stream is given again
+    bool launched = false;
     std::mutex mu;
 };
 
 void based_generation_graph_destroy(based_generation_graph* g) {
     if (!g) return;
-    if (g->exec) cudaGraphExecDestroy(g->exec);
-    if (g->graph) cudaGraphDestroy(g->graph);
+    if (g->done) cudaEventDestroy(g->done);
     delete g;
 }
 
@@ -423,35 +435,25 @@ based_status based_generation_graph_create(void* q, void* k, void* v, float* kv_
                                            float softmax_scale, based_dtype io, int flags, based_generation_graph** graph) {
     if (!graph) return BASED_ERR_INVALID_ARG;
     *graph = nullptr;
-    // the step itself, captured on a stream of its own, gives the node
-    cudaStream_t stream = nullptr;
+    const based_status st = generation_step_check(q, k, v, kv_state, z_state, out, qw, kw, vw, k_cache, v_cache, out_w, B, H, d_feat,
+                                                  d_v, H_w, d_w, window, pos_state, io, flags);
+    if (st != BASED_OK) return st;
     based_generation_graph* g = new (std::nothrow) based_generation_graph;
     if (!g) return BASED_ERR_CUDA;
-    if (cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking) != cudaSuccess) {
+    const float scale = softmax_scale > 0.f ? softmax_scale : 0.125f;   // 1/sqrt(64)
+    try {
+        g->args.resize(generation_step_args_bytes());
+    } catch (const std::bad_alloc&) {
         delete g;
         return BASED_ERR_CUDA;
     }
-    based_status st = BASED_ERR_CUDA;
-    if (cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-        st = based_generation_step(q, k, v, kv_state, z_state, out, qw, kw, vw, k_cache, v_cache, out_w, B, H, d_feat, d_v, H_w,
-                                   d_w, window, pos_state, softmax_scale, io, flags, stream);
-        if (cudaStreamEndCapture(stream, &g->graph) != cudaSuccess && st == BASED_OK) st = BASED_ERR_CUDA;
-    }
-    cudaStreamDestroy(stream);
-    size_t n = 1;
-    if (st == BASED_OK && (cudaGraphGetNodes(g->graph, &g->node, &n) != cudaSuccess || n != 1 ||
-                           cudaGraphKernelNodeGetParams(g->node, &g->params) != cudaSuccess ||
-                           cudaGraphInstantiate(&g->exec, g->graph, 0) != cudaSuccess))
-        st = BASED_ERR_CUDA;
-    if (st != BASED_OK) {
+    if (make_generation_args(g->args.data(), q, k, v, kv_state, z_state, out, B * H, d_v, (flags & BASED_STATE_SYM) != 0,
+                             (flags & BASED_NUMERATOR_ONLY) != 0, qw, kw, vw, k_cache, v_cache, out_w, B * H_w, window, pos_state,
+                             scale, io) != BASED_OK ||
+        cudaEventCreateWithFlags(&g->done, cudaEventDisableTiming) != cudaSuccess) {
         based_generation_graph_destroy(g);
-        return st;
+        return BASED_ERR_CUDA;
     }
-    const unsigned char* arg = static_cast<const unsigned char*>(g->params.kernelParams[0]);
-    g->args.assign(arg, arg + generation_step_args_bytes());
-    g->arg_list[0] = g->args.data();
-    g->params.kernelParams = g->arg_list;
-    g->params.extra = nullptr;
     void* const buffers[6] = {q, k, v, qw, kw, vw};
     for (int i = 0; i < 6; ++i) g->buffers[i] = buffers[i];
     *graph = g;
@@ -468,13 +470,24 @@ based_status based_generation_graph_step(based_generation_graph* g, const void* 
         if (!aligned16(p)) return BASED_ERR_ALIGNMENT;
     }
     if (given != 0 && given != 6) return BASED_ERR_INVALID_ARG;
+    cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
+    // a stream under capture cannot take the order among the steps (nor could it take a graph launch)
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    if (cudaStreamIsCapturing(stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone ||
+        cudaStreamGetId(stream, &id) != cudaSuccess)
+        return BASED_ERR_CUDA;
     std::lock_guard<std::mutex> lock(g->mu);
     if (given || g->own_inputs) {
         generation_step_inputs(g->args.data(), in, g->buffers);
-        if (cudaGraphExecKernelNodeSetParams(g->exec, g->node, &g->params) != cudaSuccess) return BASED_ERR_CUDA;
         g->own_inputs = given != 0;
     }
-    return cudaGraphLaunch(g->exec, static_cast<cudaStream_t>(cuda_stream)) == cudaSuccess ? BASED_OK : BASED_ERR_CUDA;
+    if (g->launched && id != g->last_stream && cudaStreamWaitEvent(stream, g->done, 0) != cudaSuccess) return BASED_ERR_CUDA;
+    const based_status st = launch_generation_args(g->args.data(), stream);
+    if (st != BASED_OK) return st;
+    g->launched = true;
+    g->last_stream = id;
+    return cudaEventRecord(g->done, stream) == cudaSuccess ? BASED_OK : BASED_ERR_CUDA;
 }
 
 static based_status baseconv_check(const void* a, const void* g, const float* h, const float* b2, const void* out,

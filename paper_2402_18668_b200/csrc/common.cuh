@@ -124,10 +124,15 @@ based_status launch_generation_step(const void* q, const void* k, const void* v,
                                     const void* vw, void* kc, void* vc, void* outw, int n_swa, int window,
                                     int* pos_state, float scale, based_dtype io, cudaStream_t stream);
 based_status preload_generation_step();
-// the arguments of a captured generation_step kernel node, pointed at other inputs (null: at `buffers`, q k v qw kw vw)
-// that the step also copies into the buffers
-void generation_step_inputs(void* kernel_args, const void* const* inputs, void* const* buffers);
+// the same call kept as its arguments (generation_step_args_bytes of them) and launched again and again;
+// generation_step_inputs points them at other inputs (null: at `buffers`, q k v qw kw vw) that the step also copies into the buffers
 size_t generation_step_args_bytes();
+based_status make_generation_args(void* args, const void* q, const void* k, const void* v, float* kv, float* z, void* out,
+                                  int n_lin, int d_v, bool sym, bool numerator_only, const void* qw, const void* kw, const void* vw,
+                                  void* kc, void* vc, void* outw, int n_swa, int window, int* pos_state, float scale,
+                                  based_dtype io);
+based_status launch_generation_args(const void* args, cudaStream_t stream);
+void generation_step_inputs(void* args, const void* const* inputs, void* const* buffers);
 // full (273-row) state -> symmetric (153-row) state, or back
 based_status launch_state_convert(const float* kv_in, const float* z_in, float* kv_out, float* z_out, int BH,
                                   int d_v, bool to_sym, cudaStream_t stream);

@@ -1,16 +1,16 @@
-"""Next-token step of the mixer pair as one replayable CUDA graph.
+"""Next-token step of the mixer pair, set up once and run once per generated token.
 
 The paper runs next-token prediction under CUDA graphs (Sec. 6, "Efficiency Benchmarks"): at
 batch sizes where a decode step lasts tens of microseconds the launch overhead of separate
-calls is a visible share of it.  `DecodeGraph` captures one step of both mixers, the Taylor
+calls is a visible share of it.  `DecodeGraph` holds one step of both mixers, the Taylor
 linear-attention decode step (on the 273-row or the 153-row symmetric state) and the
 sliding-window decode step on its rolling cache, which reads the position from device memory and
-advances it itself, and replays it once per generated token.  By default the step is the
-library's fused call (based_generation_step: one kernel node in which the two mixers' CTAs are
-dealt out in turn, so the short window step rides in the shadow of the long state stream), and
-`step` points that node at the token's inputs instead of copying them into fixed buffers first
-(the kernel leaves the copy in them): one launch per token.  fused=False captures the two separate
-kernels one after the other behind copies of the inputs.
+advances it itself.  By default the step is the library's fused call (based_generation_step: one
+kernel in which the two mixers' CTAs are dealt out in turn, so the short window step rides in the
+shadow of the long state stream), held with its arguments and launched on each token's inputs
+without copying them into fixed buffers first (the kernel leaves the copy in them): one dependent
+launch per token, which is on the SMs while the one before it drains.  fused=False captures the
+two separate kernels in a CUDA graph, one after the other behind copies of the inputs.
 
 Only plumbing lives here (static buffers, stream capture); every arithmetic step runs in the
 library's kernels.

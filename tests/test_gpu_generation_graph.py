@@ -101,3 +101,41 @@ def test_step_on_a_device_that_is_not_current():
             want = based.based_generation_step(*token[:3], *eager[:2], *token[3:], *eager[2:], pos)
         for a, b in zip(got + [kv, z, kc, vc], list(want) + eager):
             assert torch.equal(a, b), kind
+
+
+@pytest.mark.parametrize("B,sym", [(2, False), (40, True)])
+def test_steps_on_streams_in_turn(B, sym):
+    """Steps of one graph on three streams in turn, without a wait between them: each runs behind the one before it."""
+    H, d_v = 16, 128
+    g = torch.Generator(device="cuda").manual_seed(B)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    kv, z = based.new_state(B, H, d_v, sym=sym)
+    kv.copy_(rnd(*kv.shape)); z.copy_(rnd(*z.shape).abs() + 50.0)
+    kc, vc = rnd(B, H, 64, 64).bfloat16(), rnd(B, H, 64, 64).bfloat16()
+    eager = [t.clone() for t in (kv, z, kc, vc)]
+    pos = torch.tensor([60, 0], dtype=torch.int32, device="cuda")
+    tokens = [[rnd(B, H, w).bfloat16() for w in (16, 16, d_v, 64, 64, 64)] for _ in range(12)]
+    graph = DecodeGraph(kv, z, kc, vc, pos=60, sym=sym)
+    streams = [torch.cuda.current_stream(), torch.cuda.Stream(), torch.cuda.Stream()]
+    torch.cuda.synchronize()
+    for i, t in enumerate(tokens):
+        with torch.cuda.stream(streams[(i * i + i // 3) % 3]):
+            graph.step(*t)
+    torch.cuda.synchronize()
+    for t in tokens:
+        want = based.based_generation_step(*t[:3], *eager[:2], *t[3:], *eager[2:], pos, flags=based.BASED_STATE_SYM if sym else 0)
+    for a, b in zip([graph.out_lin, graph.out_swa, kv, z, kc, vc], list(want) + eager):
+        assert torch.equal(a, b)
+    assert int(graph.pos) == 72 and based.based_poll_error() == based.BASED_OK
+
+
+def test_step_under_capture_is_refused():
+    kv, z = based.new_state(1, 2, 64)
+    kc = torch.zeros(1, 2, 16, 64, dtype=torch.bfloat16, device="cuda")
+    graph = DecodeGraph(kv, z, kc, torch.zeros_like(kc), pos=3)
+    token = [torch.ones(1, 2, w, dtype=torch.bfloat16, device="cuda") for w in (16, 16, 64, 64, 64, 64)]
+    with pytest.raises(Exception):
+        with torch.cuda.graph(torch.cuda.CUDAGraph()):
+            graph.step(*token)
+    graph.step(*token)
+    assert int(graph.pos) == 4

@@ -35,6 +35,14 @@ def test_prefill_f32_segments(BH, L, d_v):
     assert row_err(wl.to_f64(based.based_prefill(*first)), y_ref[:, :, :L]) <= TOL_F32      # no state asked for
 
 
+# the definition form at the edges of its tiles (16 or 32 rows, groups of 32 keys, eight groups a CTA) and of its rule, and the
+# chunked kernel on the other side of it: 2 x 2049, 16 x 900 (and continued 8 x 640, 60 x 128), 64 x 300
+@pytest.mark.parametrize("BH,L,d_v", [(1, 2048, 64), (2, 257, 112), (3, 31, 64), (3, 32, 128), (5, 513, 64), (64, 33, 64), (64, 97, 64),
+                                      (100, 16, 112), (2, 2049, 64), (16, 900, 64), (8, 640, 64), (60, 128, 64), (64, 300, 64)])
+def test_prefill_f32_either_form(BH, L, d_v):
+    test_prefill_f32_segments(BH, L, d_v)
+
+
 def test_prefill_f32_keeps_an_uneven_full_state_apart():
     """Rows (m, n) and (n, m) of a caller's state that differ: outputs use their sum, and each keeps its own value plus
     the tokens' share."""

@@ -124,7 +124,8 @@ based_status launch_generation_step(const void* q, const void* k, const void* v,
                                     const void* vw, void* kc, void* vc, void* outw, int n_swa, int window,
                                     int* pos_state, float scale, based_dtype io, cudaStream_t stream);
 based_status preload_generation_step();
-// the same call kept as its arguments (generation_step_args_bytes of them) and launched again and again;
+// the same call kept as its arguments (generation_step_args_bytes of them) and launched again and again, each launch no call of
+// based_generation_step and not counted as one;
 // generation_step_inputs points them at other inputs (null: at `buffers`, q k v qw kw vw) that the step also copies into the buffers
 size_t generation_step_args_bytes();
 based_status make_generation_args(void* args, const void* q, const void* k, const void* v, float* kv, float* z, void* out,

@@ -126,7 +126,6 @@ based_status launch_k(const GenArgs& args, size_t smem, cudaStream_t stream) {
     const int n_swa_ctas = ((a.n_swa + 1) / 2 + PARTS - 1) / PARTS;
     a.n_pairs = n_swa_ctas < a.n_lin / 2 ? n_swa_ctas : a.n_lin / 2;
     const cudaError_t e = launch_ex(kern, dim3((a.n_lin + n_swa_ctas) * PARTS), dim3(256), smem, PARTS, true, stream, a);
-    note_launch();
     const based_status st = check_launch("generation_step_kernel");
     return e == cudaSuccess ? st : BASED_ERR_CUDA;
 }
@@ -231,7 +230,9 @@ based_status launch_generation_step(const void* q, const void* k, const void* v,
     GenCall c;
     const based_status st = make_generation_args(&c, q, k, v, kv, z, out, n_lin, d_v, sym, numerator_only, qw, kw, vw, kc, vc, outw,
                                                  n_swa, window, pos_state, scale, io);
-    return st == BASED_OK ? launch_generation_args(&c, stream) : st;
+    if (st != BASED_OK) return st;
+    note_launch();
+    return launch_generation_args(&c, stream);
 }
 
 void generation_step_inputs(void* args, const void* const* in, void* const* buffers) {

@@ -495,6 +495,71 @@ __device__ __noinline__ void init_from_abi(const float* kv_abi, const float* z_a
     tmem_wait_st();
 }
 
+// ---- final state, one role group's share of its 16-feature blocks (part, part + 4, ..) in the caller's layout.  A block goes
+// through the group's own place in the phi(K) tile, which no product reads any more, so that 16-byte words of a state row leave
+// side by side and a row's number is looked up once per word: stored straight from tensor memory, an element and a lookup per
+// thread, the state cost a call 2.5 us more (B1 H8 L2048 d_v64 outputs alone 14.7 us, with a new state 18.9, now 16.1; B4 H16 L2048
+// 19.2 / 23.8 / 20.6; B8 H16 L4096 d_v128 72.0 / 76.1 / 74.8).  Inlined, behind a condition that keeps no value of its own: out of
+// line, or with the CTA's head and whether it ends it in shared memory, the role loops ahead of it took up to 8 % longer, on calls
+// without a state too (B4 H16 L2048 20.8 us), and in an instance without any of this 4 %.
+template <int DV>
+__device__ __forceinline__ void write_state(float* kv, float* z, int dv, const short2* s_abi, uint32_t tb, int part, float* stage) {
+    using C = Cfg<DV>;
+    constexpr int kQ = DV / 4, kPer = 128 / kQ;                      // 16-byte words of a row, rows per pass
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x & 127;
+    const uint32_t lane_base = (uint32_t)(warp & 3) * 32u;
+    const int t = ((warp & 3) << 5) + lane;                              // lane of S^T
+    float* rows = stage + part * (16 * DV + 16);
+    float* zs = rows + 16 * DV;
+    static_assert(4 * (16 * DV + 16) * sizeof(float) <= C::kPhiBytes, "the groups' places");
+    auto put_z = [&](int f, float v) {
+        const short2 ar = s_abi[f];
+        if (ar.x < 0) return;
+        if (ar.y >= 0) v *= kRsqrt2;
+        z[ar.x] = v;
+        if (ar.y >= 0) z[ar.y] = v;
+    };
+#pragma unroll 1
+    for (int b = part; b < kF / 16; b += 4) {
+        uint32_t r[16];
+        tmem_ld16(tmem_addr(tb, lane_base, C::colS + b * 16), r);
+        tmem_wait_ld();
+        if (t < DV) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) rows[i * DV + t] = __uint_as_float(r[i]);
+        } else if (t == DV) {                                            // d_v 64: the K-state's lane
+#pragma unroll
+            for (int i = 0; i < 16; ++i) zs[i] = __uint_as_float(r[i]);
+        }
+        group_sync(part + 2);
+        const int c = (tid % kQ) * 4;
+        if (c < dv) {
+#pragma unroll
+            for (int u = 0; u < 16 / kPer; ++u) {
+                const int i = tid / kQ + u * kPer;
+                const short2 ar = s_abi[b * 16 + i];
+                float4 v = *reinterpret_cast<const float4*>(rows + i * DV + c);
+                if (ar.y >= 0) {
+                    v.x *= kRsqrt2; v.y *= kRsqrt2; v.z *= kRsqrt2; v.w *= kRsqrt2;
+                    *reinterpret_cast<float4*>(kv + (size_t)ar.y * dv + c) = v;
+                }
+                if (ar.x >= 0) *reinterpret_cast<float4*>(kv + (size_t)ar.x * dv + c) = v;
+            }
+        }
+        if (DV == 64 && tid < 16) put_z(b * 16 + tid, zs[tid]);
+        group_sync(part + 2);                                            // the place is read
+    }
+    if (DV == 128 && part == 2) {
+        // the K-state of feature t (tile 0) and of features 128 on (tile 1: a 64-row product, lanes 0-15 and 32-47)
+        uint32_t z0, z1;
+        tmem_ld1(tmem_addr(tb, lane_base, C::colZ0), z0);
+        tmem_ld1(tmem_addr(tb, lane_base, C::colZ1), z1);
+        tmem_wait_ld();
+        put_z(t, __uint_as_float(z0));
+        if ((t & 31) < 16 && (t >> 5) < 2) put_z(128 + (t >> 5) * 16 + (t & 15), __uint_as_float(z1));
+    }
+}
+
 // ---- continued calls in recompute mode: every segment of a head starts from the caller's state, and the last one
 // overwrites it at its end.  The segments' CTAs start as SMs come free (another stream may hold some), so the order is
 // made here: a segment that has read the state stores the call's ticket in its word of the workspace, and the last one
@@ -1438,35 +1503,28 @@ __global__ void __launch_bounds__(kThreads, 1)
     // warp's lane quarter), so the four role groups share the ten 16-column blocks: the write is 140 KB per head at
     // d_v 128, a fifth of a chunk's time when one group does it alone.
     if (warp < 16) {
-        const bool write_ws = STATE_ONLY;
-        const bool write_abi = !STATE_ONLY && p.kv_abi != nullptr && head_end;
-        if (write_ws || write_abi) {
+        if constexpr (!STATE_ONLY) {
+            // (in recompute mode the piece is the CTA's place in the grid)
+            const bool write = p.kv_abi != nullptr && (PRE ? blockIdx.x == gridDim.x - 1 : head_end);
+            if (write && ok) ok = mbar_wait(&bars[kFin], 0, abort_flag);
+            tc_fence_after();
+            if (write) {
+                ok = group_all((warp >> 2) + 2, ok);                     // the group's threads meet in write_state
+                const size_t row = (size_t)(PRE ? (int)blockIdx.y : head) * (p.sym ? kDSym : kD);
+                if (ok) write_state<DV>(p.kv_abi + row * p.dv, p.z_abi + row, p.dv, s_abi, tb, warp >> 2, reinterpret_cast<float*>(sPK));
+            }
+        } else {
             const int part = warp >> 2;                                  // 0 row, 1 feature, 2 state, 3 output group
+            // without chunks there is no last MMA to wait for, and only the state group knows the state is initialised
+            const bool shared = ntot > 0;
             const int t = ((warp & 3) << 5) + lane;
             const int srow = (t < C::kSLanes) ? t : -1;
             const bool is_z = (DV == 64) && t == 64;
             const int z1f = (DV == 128 && (t & 31) < 16 && (t >> 5) < 2) ? 128 + (t >> 5) * 16 + (t & 15) : -1;
-            const int dv = p.dv;
-            // without chunks there is no last MMA to wait for, and only the state group knows the state is initialised
-            const bool shared = ntot > 0;
             if (ok && shared) ok = mbar_wait(&bars[kFin], 0, abort_flag);
             tc_fence_after();
             if (ok && (shared || part == 2)) {
                 float* wseg = p.ws + (size_t)(ws_out < 0 ? 0 : ws_out) * seg_state_floats(DV);
-                float* kvo = write_abi ? p.kv_abi + (size_t)head * abi_nrows * dv : nullptr;
-                float* zo = write_abi ? p.z_abi + (size_t)head * abi_nrows : nullptr;
-                auto put = [&](int f, float v, bool zrow, int col) {
-                    if (write_ws) {
-                        if (zrow) wseg[(size_t)kF * DV + f] = v;
-                        else wseg[(size_t)f * DV + col] = v;
-                        return;
-                    }
-                    const short2 ar = s_abi[f];
-                    if (ar.x < 0) return;
-                    if (ar.y >= 0) v *= kRsqrt2;
-                    if (zrow) { zo[ar.x] = v; if (ar.y >= 0) zo[ar.y] = v; }
-                    else if (col < dv) { kvo[(size_t)ar.x * dv + col] = v; if (ar.y >= 0) kvo[(size_t)ar.y * dv + col] = v; }
-                };
 #pragma unroll 1
                 for (int b = shared ? part : 0; b < kF / 16; b += shared ? 4 : 1) {
                     uint32_t r[16];
@@ -1474,7 +1532,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     tmem_wait_ld();
                     if (srow >= 0) {
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) put(b * 16 + i, __uint_as_float(r[i]), is_z, srow);
+                        for (int i = 0; i < 16; ++i)
+                            wseg[is_z ? (size_t)kF * DV + b * 16 + i : (size_t)(b * 16 + i) * DV + srow] = __uint_as_float(r[i]);
                     }
                 }
                 if (DV == 128 && part == 2) {
@@ -1482,8 +1541,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     tmem_ld1(tmem_addr(tb, lane_base, C::colZ0), z0);
                     tmem_ld1(tmem_addr(tb, lane_base, C::colZ1), z1);
                     tmem_wait_ld();
-                    put(t, __uint_as_float(z0), true, 0);
-                    if (z1f >= 0) put(z1f, __uint_as_float(z1), true, 0);
+                    wseg[(size_t)kF * DV + t] = __uint_as_float(z0);
+                    if (z1f >= 0) wseg[(size_t)kF * DV + z1f] = __uint_as_float(z1);
                 }
             }
         }

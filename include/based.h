@@ -281,6 +281,15 @@ based_status based_prefill_backward_tokens_first(const void* q, const void* k, c
                                                  void* workspace, size_t workspace_bytes, void* cuda_stream);
 
 /*
+ * The same for bf16 io, with the forward output, which lies [B,H,L,d_v]: based_prefill_backward_with_out on such a dout.  fp32 io
+ * and more than 65532 heads or 2^31 rows: BASED_ERR_UNSUPPORTED (then based_tokens_to_heads lays dout out for the other call).
+ */
+based_status based_prefill_backward_tokens_first_with_out(const void* q, const void* k, const void* v, const void* out,
+                                                          const void* dout, void* dq, void* dk, void* dv, int B, int H, int L,
+                                                          int d_feat, int d_v, based_dtype io, int flags, void* workspace,
+                                                          size_t workspace_bytes, void* cuda_stream);
+
+/*
  * Which path a backward call with these arguments takes: the block length W of the block-wise path, or 0
  * for the tile path (fp32 io, d_feat other than 16, short sequences).  with_out: nonzero for
  * based_prefill_backward_with_out with out non-null; without the forward output (and without

@@ -34,6 +34,7 @@ EXPORTS = (
     "based_prefill_backward_workspace_bytes", "based_prefill_backward_with_out", "based_prefill_backward_block_tokens", "swa_decode_step_advance", "swa_decode_step_ragged", "based_generation_step",
     "based_prefill_state", "based_prefill_state_workspace_bytes", "based_generation_graph_create", "based_generation_graph_step",
     "based_generation_graph_destroy", "based_tokens_to_heads", "based_f32_parts_bytes", "based_prefill_backward_tokens_first", "based_prefill_f32_parts",
+    "based_prefill_backward_tokens_first_with_out",
 )
 
 _lib = None

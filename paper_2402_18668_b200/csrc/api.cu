@@ -574,7 +574,7 @@ static based_status prefill_backward(const void* q, const void* k, const void* v
         return BASED_OK;
     }
     if (io == BASED_BF16)
-        return launch_prefill_backward_tc(q, k, v, out, dout, dq, dk, dv, static_cast<float*>(workspace), B * H, L,
+        return launch_prefill_backward_tc(q, k, v, out, dout, 0, dq, dk, dv, static_cast<float*>(workspace), B * H, L,
                                           d_feat, d_v, (flags & BASED_NUMERATOR_ONLY) ? 1 : 0,
                                           static_cast<cudaStream_t>(cuda_stream));
     return backward_f32(q, k, v, dout, 0, dq, dk, dv, B, H, L, d_v, flags, workspace, workspace_bytes, cuda_stream);
@@ -610,6 +610,25 @@ based_status based_prefill_backward_tokens_first(const void* q, const void* k, c
         return BASED_ERR_ALIGNMENT;
     if (!workspace || workspace_bytes < based_prefill_backward_workspace_bytes(B, H, L, d_v, io)) return BASED_ERR_WORKSPACE;
     return backward_f32(q, k, v, dout, H, dq, dk, dv, B, H, L, d_v, flags, workspace, workspace_bytes, cuda_stream);
+}
+
+based_status based_prefill_backward_tokens_first_with_out(const void* q, const void* k, const void* v, const void* out,
+                                                          const void* dout, void* dq, void* dk, void* dv, int B, int H, int L,
+                                                          int d_feat, int d_v, based_dtype io, int flags, void* workspace,
+                                                          size_t workspace_bytes, void* cuda_stream) {
+    if (!q || !k || !v || !out || !dout || !dq || !dk || !dv || B <= 0 || H <= 0 || L <= 0) return BASED_ERR_INVALID_ARG;
+    if (flags & ~BASED_NUMERATOR_ONLY) return BASED_ERR_INVALID_ARG;
+    if (dq == q || dq == k || dk == q || dk == k || dv == v || dv == dout || out == dq || out == dk || out == dv) return BASED_ERR_INVALID_ARG;
+    // one slab of heads, rows counted in 32 bits
+    if (io != BASED_BF16 || !(d_feat == kDFeat || df_generic(d_feat)) || !dv_ok(d_v) || (long long)B * H > kHeadSlab ||
+        (long long)B * H * L > 0x7fffffffLL)
+        return BASED_ERR_UNSUPPORTED;
+    if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(out) || !aligned16(dout) || !aligned16(dq) || !aligned16(dk) ||
+        !aligned16(dv) || !aligned16(workspace))
+        return BASED_ERR_ALIGNMENT;
+    if (!workspace || workspace_bytes < based_prefill_backward_workspace_bytes(B, H, L, d_v, io)) return BASED_ERR_WORKSPACE;
+    return launch_prefill_backward_tc(q, k, v, out, dout, H, dq, dk, dv, static_cast<float*>(workspace), B * H, L, d_feat, d_v,
+                                      (flags & BASED_NUMERATOR_ONLY) ? 1 : 0, static_cast<cudaStream_t>(cuda_stream));
 }
 
 based_status based_tokens_to_heads(const void* src, void* dst, int B, int H, int L, int row_bytes, void* cuda_stream) {

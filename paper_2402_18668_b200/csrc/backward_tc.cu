@@ -114,6 +114,7 @@ struct BParams {
     // block-wise path: pairs inside a block of W tokens by tiles, the other blocks through their summed state
     int W, nblk;
     int heads, by_length;        // by_length: the longest loops of all heads first, else head by head
+    int dout_H;                  // heads per sequence where dout lies [B, L, H, d_v]; else 0
     int overlapped;              // forward: this grid runs beside the one before it, and ends after it
     const float* sv;             // [BH x nblk][160]: row sums of the block states (z, or the b-weighted sums of phi(q))
 };
@@ -336,7 +337,8 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd && DV == 64 && LT 
                 tma_load_3d(st, &tm_n1, &bars[bFull0 + s], 0, row, head);
 #pragma unroll
                 for (int b = 0; b < C::kVB; ++b)
-                    tma_load_3d(st + C::kNarrowL + b * (LT * 128), &tm_w1, &bars[bFull0 + s], b * 64, row, head);
+                    if (MODE == kModeDkDv) tma_load_head_rows(st + C::kNarrowL + b * (LT * 128), &tm_w1, &bars[bFull0 + s], b * 64, row, head, p.dout_H);
+                    else tma_load_3d(st + C::kNarrowL + b * (LT * 128), &tm_w1, &bars[bFull0 + s], b * 64, row, head);
             };
             if (lead) {
             mbar_arrive_expect_tx(&bars[bRes], MODE == kModeFwd ? kQKTile : kQKTile + C::kWide);
@@ -344,7 +346,8 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd && DV == 64 && LT 
             if (MODE != kModeFwd) {
 #pragma unroll
                 for (int b = 0; b < C::kVB; ++b)
-                    tma_load_3d(smem + C::offResW + b * (kTile * 128), &tm_w0, &bars[bRes], b * 64, r0, head);
+                    if (MODE == kModeDkDv) tma_load_3d(smem + C::offResW + b * (kTile * 128), &tm_w0, &bars[bRes], b * 64, r0, head);
+                    else tma_load_head_rows(smem + C::offResW + b * (kTile * 128), &tm_w0, &bars[bRes], b * 64, r0, head, p.dout_H);
             }
             if (cross) {
                 mbar_arrive_expect_tx(&bars[bXs], C::kStateTile);
@@ -960,17 +963,18 @@ BlockWs block_ws(float* ws, int BH, int L, int dvr, int nblk) {
 int long_loops_first(int BH, int L) { return (long long)BH * ((L + kTile - 1) / kTile) > kSMs; }
 
 template <int DV>
-based_status launch_dvb(const void* q, const void* k, const void* v, const void* out, const void* g, void* dq, void* dk,
+based_status launch_dvb(const void* q, const void* k, const void* v, const void* out, const void* g, int dout_H, void* dq, void* dk,
                         void* dv, float* ws, int BH, int L, int df, int dvr, int numerator_only, cudaStream_t stream) {
     constexpr int LTK = (DV == 64) ? 64 : 128;       // looped tile of the dk/dv pass (d_v 128 needs all 512 columns anyway)
     float2* stats = reinterpret_cast<float2*>(ws);
     // own tiles: 128 rows; looped tiles: 64 rows (and LTK rows for the dk/dv pass)
     CUtensorMap tq, tk, tv, tg, tk64, tv64, tqL, tgL, tdv;
     const CUtensorMapSwizzle s64 = CU_TENSOR_MAP_SWIZZLE_64B, s128 = CU_TENSOR_MAP_SWIZZLE_128B;
+    auto dout_map = [&](CUtensorMap* m, int rows) { return make_head_rows_map_bf16(m, g, BH, dout_H, L, dvr, 64, rows, s128); };
     if (!make_rows_map_bf16(&tq, q, BH, L, df, 32, kTile, s64) || !make_rows_map_bf16(&tk, k, BH, L, df, 32, kTile, s64) ||
-        !make_rows_map_bf16(&tv, v, BH, L, dvr, 64, kTile, s128) || !make_rows_map_bf16(&tg, g, BH, L, dvr, 64, kTile, s128) ||
+        !make_rows_map_bf16(&tv, v, BH, L, dvr, 64, kTile, s128) || !dout_map(&tg, kTile) ||
         !make_rows_map_bf16(&tk64, k, BH, L, df, 32, 64, s64) || !make_rows_map_bf16(&tv64, v, BH, L, dvr, 64, 64, s128) ||
-        !make_rows_map_bf16(&tqL, q, BH, L, df, 32, LTK, s64) || !make_rows_map_bf16(&tgL, g, BH, L, dvr, 64, LTK, s128) ||
+        !make_rows_map_bf16(&tqL, q, BH, L, df, 32, LTK, s64) || !dout_map(&tgL, LTK) ||
         !make_rows_map_bf16(&tdv, dv, BH, L, dvr, 64, kTile, s128))
         return BASED_ERR_CUDA;
     BParams p{};
@@ -990,6 +994,7 @@ based_status launch_dvb(const void* q, const void* k, const void* v, const void*
     const dim3 grid((unsigned)((L + kTile - 1) / kTile) * BH);
     p.heads = BH;
     p.by_length = long_loops_first(BH, L);
+    p.dout_H = dout_H;
     based_status st;
     const int W = backward_block_len(L, df, out != nullptr || numerator_only, dvr, BH);
     if (W > 0) {
@@ -1013,8 +1018,9 @@ based_status launch_dvb(const void* q, const void* k, const void* v, const void*
         // and block writes the block's own sums and a scan adds them up.
         const bool running = BH >= 64;
         auto states = [&](const void* x, const void* val, const void* sts, int rev) -> based_status {
-            if (running) return launch_block_states_tc(x, val, sts, w.st, w.sv, nullptr, nullptr, BH, L, W, dvr, rev, stream);
-            based_status s2 = launch_block_states_tc(x, val, sts, w.st, w.sv, w.part, w.zpart, BH, L, W, dvr, rev, stream);
+            const int val_H = rev ? dout_H : 0;
+            if (running) return launch_block_states_tc(x, val, sts, w.st, w.sv, nullptr, nullptr, BH, val_H, L, W, dvr, rev, stream);
+            based_status s2 = launch_block_states_tc(x, val, sts, w.st, w.sv, w.part, w.zpart, BH, val_H, L, W, dvr, rev, stream);
             if (s2 != BASED_OK) return s2;
             state_scan_kernel<<<dim3((160 * dvr + 255) / 256, BH), 256, 0, stream>>>(w.part, w.zpart, w.st, w.sv, nblk, 160 * dvr, rev);
             note_launch();
@@ -1030,7 +1036,7 @@ based_status launch_dvb(const void* q, const void* k, const void* v, const void*
             // 32-row looped tiles: the accumulators then fit 256 tensor-memory columns and two CTAs share an SM, which
             // hides the fixed latency of these short-lived CTAs (273 -> 220 us for the pass at B8 H16 L4096)
             CUtensorMap tq32, tg32;
-            if (!make_rows_map_bf16(&tq32, q, BH, L, df, 32, 32, s64) || !make_rows_map_bf16(&tg32, g, BH, L, dvr, 64, 32, s128)) return BASED_ERR_CUDA;
+            if (!make_rows_map_bf16(&tq32, q, BH, L, df, 32, 32, s64) || !dout_map(&tg32, 32)) return BASED_ERR_CUDA;
             return launch_pass<DV, kModeDkDv, 32, true>(tk, tv, tq32, tg32, p, grid, "backward_tc_kernel<dkdv, blocks>", stream, &tst,
                                                         &tdv);
         }
@@ -1100,11 +1106,11 @@ size_t backward_tc_workspace_bytes(int BH, int L, int d_v) {
     return (size_t)BH * L * 2 * sizeof(float);                 // (1 / D, b) per row
 }
 
-based_status launch_prefill_backward_tc(const void* q, const void* k, const void* v, const void* out, const void* g,
+based_status launch_prefill_backward_tc(const void* q, const void* k, const void* v, const void* out, const void* g, int dout_H,
                                         void* dq, void* dk, void* dv, float* ws, int BH, int L, int d_feat, int d_v,
                                         int numerator_only, cudaStream_t stream) {
-    if (d_v == 64) return launch_dvb<64>(q, k, v, out, g, dq, dk, dv, ws, BH, L, d_feat, 64, numerator_only, stream);
-    return launch_dvb<128>(q, k, v, out, g, dq, dk, dv, ws, BH, L, d_feat, d_v, numerator_only, stream);  // 112 or 128
+    if (d_v == 64) return launch_dvb<64>(q, k, v, out, g, dout_H, dq, dk, dv, ws, BH, L, d_feat, 64, numerator_only, stream);
+    return launch_dvb<128>(q, k, v, out, g, dout_H, dq, dk, dv, ws, BH, L, d_feat, d_v, numerator_only, stream);  // 112 or 128
 }
 
 }  // namespace based

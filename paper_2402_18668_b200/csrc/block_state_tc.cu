@@ -81,6 +81,7 @@ struct RParams {
     float* zpart;
     unsigned int* err;
     int L, dvw, nblk, rev;
+    int val_H;                     // heads per sequence where the wide tensor is dout as [B, L, H, d_v]; else 0
     int lspb;                      // log2 of the steps per block
     int grp;                       // own sums: blocks per CTA (consecutive blocks of one head)
 };
@@ -166,7 +167,7 @@ __global__ void __launch_bounds__(kThreadsR, 1)
                 mbar_arrive_expect_tx(&bars[rFull0 + s], C::kVBytes);
 #pragma unroll
                 for (int b = 0; b < C::kVB; ++b)
-                    tma_load_3d(st + b * (kTok * 128), &tm_val, &bars[rFull0 + s], b * 64, tile_of(it) * kTok, head);
+                    tma_load_head_rows(st + b * (kTok * 128), &tm_val, &bars[rFull0 + s], b * 64, tile_of(it) * kTok, head, p.val_H);
             };
             for (int it = 0; it < kNSR && it < nit; ++it) load(it);
             int nblk_done = 0;                               // blocks walked so far: the accumulators alternate
@@ -442,10 +443,10 @@ __global__ void __launch_bounds__(kThreadsR, 1)
 namespace {
 template <int DV, int FN, bool KEYS>
 based_status launch_running(const void* x, const void* val, const float2* stats, void* st, float* sv, float* part,
-                            float* zpart, int BH, int L, int W, int dvw, int rev, cudaStream_t stream) {
+                            float* zpart, int BH, int val_H, int L, int W, int dvw, int rev, cudaStream_t stream) {
     using C = RCfg<DV, FN>;
     CUtensorMap tv;
-    if (!make_rows_map_bf16(&tv, val, BH, L, dvw, 64, kTok, CU_TENSOR_MAP_SWIZZLE_128B)) return BASED_ERR_CUDA;
+    if (!make_head_rows_map_bf16(&tv, val, BH, val_H, L, dvw, 64, kTok, CU_TENSOR_MAP_SWIZZLE_128B)) return BASED_ERR_CUDA;
     RParams p{};
     if (error_word_ptr(&p.err) != BASED_OK) return BASED_ERR_CUDA;
     p.x = static_cast<const __nv_bfloat16*>(x);
@@ -455,6 +456,7 @@ based_status launch_running(const void* x, const void* val, const float2* stats,
     p.part = part;
     p.zpart = zpart;
     p.L = L;
+    p.val_H = val_H;
     p.dvw = dvw;
     p.lspb = W == 256 ? 1 : 2;
     p.nblk = (L + W - 1) / W;
@@ -484,7 +486,7 @@ based_status launch_running(const void* x, const void* val, const float2* stats,
 // part, zpart: null for the running sums (one CTA per head); else every block's own sums go there in fp32 (one CTA
 // per head and block) and st, sv stay untouched.
 based_status launch_block_states_tc(const void* x, const void* val, const void* stats, void* st, float* sv, float* part,
-                                    float* zpart, int BH, int L, int W, int d_v, int rev, cudaStream_t stream) {
+                                    float* zpart, int BH, int val_H, int L, int W, int d_v, int rev, cudaStream_t stream) {
     const float2* s2 = static_cast<const float2*>(stats);
     // Two CTAs per head, each with half of the features, where both fit the chip at once: a CTA's steps are a chain that its
     // eight row warps issue at a third of the SM's rate, and shorter steps pay more than the doubled loads cost (64 heads, us
@@ -492,8 +494,8 @@ based_status launch_block_states_tc(const void* x, const void* val, const void* 
     const bool halves = !part && 2 * BH <= kSMs;
     auto go = [&](auto dv_tag, auto fn_tag, int dvw) {
         constexpr int DV = decltype(dv_tag)::value, FN = decltype(fn_tag)::value;
-        return s2 ? launch_running<DV, FN, false>(x, val, s2, st, sv, part, zpart, BH, L, W, dvw, rev, stream)
-                  : launch_running<DV, FN, true>(x, val, s2, st, sv, part, zpart, BH, L, W, dvw, rev, stream);
+        return s2 ? launch_running<DV, FN, false>(x, val, s2, st, sv, part, zpart, BH, val_H, L, W, dvw, rev, stream)
+                  : launch_running<DV, FN, true>(x, val, s2, st, sv, part, zpart, BH, val_H, L, W, dvw, rev, stream);
     };
     const std::integral_constant<int, 64> c64;
     const std::integral_constant<int, 128> c128;             // 112 or 128

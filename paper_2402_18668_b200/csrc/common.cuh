@@ -189,9 +189,10 @@ based_status launch_state_generic_tc(const void* k, const void* v, float* kv, fl
 // bf16 and sv [BH x nblk][160]: for every block of W tokens the sums over the blocks before it (rev = 0) or after it
 // (rev = 1), one CTA per head; stats: (1 / D, b) per
 // token for the query side (x = q, val = dout), null for the key side (x = k, val = v); part, zpart: null, or the
-// blocks' own sums in fp32 instead (one CTA per head and block), for state_scan_kernel
+// blocks' own sums in fp32 instead (one CTA per head and block), for state_scan_kernel; val_H: 0, or H where val lies
+// [B, L, H, d_v]
 based_status launch_block_states_tc(const void* x, const void* val, const void* stats, void* st, float* sv, float* part,
-                                    float* zpart, int BH, int L, int W, int d_v, int rev, cudaStream_t stream);
+                                    float* zpart, int BH, int val_H, int L, int W, int d_v, int rev, cudaStream_t stream);
 // the state of a token block alone (no outputs): kv (+)= sum_j phi(k_j) v_j^T, z (+)= sum_j phi(k_j)
 based_status launch_state_generic(const void* k, const void* v, float* kv, float* z, int BH, int L, int d_feat, int d_v,
                                   based_dtype io, int cont, cudaStream_t stream);
@@ -207,7 +208,8 @@ size_t backward_tc_workspace_bytes(int BH, int L, int d_v);
 // the numerator-only form)
 int backward_tc_block_tokens(int BH, int L, int d_feat, int d_v, int merged);
 // out: the forward output (may be null): with it, statistics and dq run as one sweep
-based_status launch_prefill_backward_tc(const void* q, const void* k, const void* v, const void* out, const void* g,
+// dout_H: 0, or H where g lies [B, L, H, d_v]
+based_status launch_prefill_backward_tc(const void* q, const void* k, const void* v, const void* out, const void* g, int dout_H,
                                         void* dq, void* dk, void* dv, float* ws, int BH, int L, int d_feat, int d_v,
                                         int numerator_only, cudaStream_t stream);
 // definition-form forward on tensor cores for d' in {8, 24, 32} (bf16 io, empty initial state); overlapped: beside the

@@ -51,3 +51,18 @@ def test_convolution_step_rows_per_thread(dtype, width, B, C):
     want = f(a) * x / (1 + torch.exp(-x))
     assert row_err(wl.to_f64(out), want.numpy()) <= tol_for(dtype)
     assert torch.equal(state.cpu(), torch.cat([g[:, None], st], dim=1)[:, :width - 1])
+
+
+@pytest.mark.parametrize("B,H,L,d_v", [(4, 16, 800, 64), (2, 8, 1100, 64), (4, 16, 1100, 128), (1, 8, 4200, 128), (2, 3, 129, 128),
+                                       (3, 50, 200, 64), (2, 16, 1300, 112), (4, 16, 1100, 112), (2, 3, 129, 112), (2, 1, 64, 64)])
+def test_gradients_of_dout_as_it_lies(B, H, L, d_v):
+    """bf16, block by block (a CTA per head, sums of every block with few heads, blocks of 512) and by tiles."""
+    g = torch.Generator(device="cuda").manual_seed(L)
+    q, k = ((torch.randn(B, H, L, 16, generator=g, device="cuda") * 0.5).bfloat16().requires_grad_(True) for _ in range(2))
+    v = torch.randn(B, H, L, d_v, generator=g, device="cuda").bfloat16().requires_grad_(True)
+    dout = torch.randn(B, L, H, d_v, generator=g, device="cuda").bfloat16().transpose(1, 2)
+    y = linear_attention(q, k, v)
+    want = torch.autograd.grad(y, (q, k, v), dout.contiguous(), retain_graph=True)
+    got = torch.autograd.grad(y, (q, k, v), dout)
+    assert all(torch.equal(a, c) for a, c in zip(got, want))
+    assert based.based_poll_error() == based.BASED_OK

@@ -327,6 +327,7 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd && DV == 64 && LT 
         {
             // the whole warp runs this block; one elected lane issues the MMAs, commits and loads (see mma_ss_w)
             const uint32_t lead = elect_one();
+            const int gb = p.dout_H ? head / p.dout_H : 0, gh = head - gb * p.dout_H;      // the head in the coordinates of a dout [B][L][H][d_v]
             const uint32_t aResN = smem_u32(smem + C::offResN), aResW = smem_u32(smem + C::offResW);
             auto load_stage = [&](int it) {
                 if (!lead || it >= nloop) return;
@@ -337,7 +338,7 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd && DV == 64 && LT 
                 tma_load_3d(st, &tm_n1, &bars[bFull0 + s], 0, row, head);
 #pragma unroll
                 for (int b = 0; b < C::kVB; ++b)
-                    if (MODE == kModeDkDv) tma_load_head_rows(st + C::kNarrowL + b * (LT * 128), &tm_w1, &bars[bFull0 + s], b * 64, row, head, p.dout_H);
+                    if (MODE == kModeDkDv && p.dout_H) tma_load_4d(st + C::kNarrowL + b * (LT * 128), &tm_w1, &bars[bFull0 + s], b * 64, gh, row, gb);
                     else tma_load_3d(st + C::kNarrowL + b * (LT * 128), &tm_w1, &bars[bFull0 + s], b * 64, row, head);
             };
             if (lead) {
@@ -346,8 +347,8 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd && DV == 64 && LT 
             if (MODE != kModeFwd) {
 #pragma unroll
                 for (int b = 0; b < C::kVB; ++b)
-                    if (MODE == kModeDkDv) tma_load_3d(smem + C::offResW + b * (kTile * 128), &tm_w0, &bars[bRes], b * 64, r0, head);
-                    else tma_load_head_rows(smem + C::offResW + b * (kTile * 128), &tm_w0, &bars[bRes], b * 64, r0, head, p.dout_H);
+                    if (MODE != kModeDkDv && p.dout_H) tma_load_4d(smem + C::offResW + b * (kTile * 128), &tm_w0, &bars[bRes], b * 64, gh, r0, gb);
+                    else tma_load_3d(smem + C::offResW + b * (kTile * 128), &tm_w0, &bars[bRes], b * 64, r0, head);
             }
             if (cross) {
                 mbar_arrive_expect_tx(&bars[bXs], C::kStateTile);

@@ -160,6 +160,7 @@ __global__ void __launch_bounds__(kThreadsR, 1)
             constexpr uint64_t dV = make_smem_desc_base(kTok * 128, 1024, kSwizzle128B);       // A, MN-major: 64-column blocks
             constexpr uint32_t iS = make_idesc_bf16(128, FN, 1, 1);
             constexpr uint32_t iZ = make_idesc_bf16(64, FN, 1, 1);
+            const int gb = KEYS || p.val_H == 0 ? 0 : head / p.val_H, gh = head - gb * p.val_H;     // the head in the coordinates of a dout [B][L][H][d_v]
             auto load = [&](int it) {
                 if (!lead) return;
                 const int s = it % kNSR;
@@ -167,7 +168,8 @@ __global__ void __launch_bounds__(kThreadsR, 1)
                 mbar_arrive_expect_tx(&bars[rFull0 + s], C::kVBytes);
 #pragma unroll
                 for (int b = 0; b < C::kVB; ++b)
-                    tma_load_head_rows(st + b * (kTok * 128), &tm_val, &bars[rFull0 + s], b * 64, tile_of(it) * kTok, head, p.val_H);
+                    if (KEYS || p.val_H == 0) tma_load_3d(st + b * (kTok * 128), &tm_val, &bars[rFull0 + s], b * 64, tile_of(it) * kTok, head);
+                    else tma_load_4d(st + b * (kTok * 128), &tm_val, &bars[rFull0 + s], b * 64, gh, tile_of(it) * kTok, gb);
             };
             for (int it = 0; it < kNSR && it < nit; ++it) load(it);
             int nblk_done = 0;                               // blocks walked so far: the accumulators alternate

@@ -13,8 +13,8 @@ namespace based {
 bool make_rows_map_bf16(CUtensorMap* m, const void* base, int BH, int L, int width, int box_w, int box_rows,
                         CUtensorMapSwizzle sw);
 
-// The same with the head in two coordinates, (x, head % H, row, head / H), of an array that lies [B][L][H][width], the heads of a
-// token side by side (H > 0, BH a multiple of it), or [BH][L][width] (H 0: coordinates x, head, row, 0)
+// The same of an array that lies [B][L][H][width], the heads of a token side by side (H > 0, BH a multiple of it): coordinates x,
+// head % H, row, head / H; H 0: make_rows_map_bf16 (one kind of map for both cost the backward calls up to 1 % there)
 bool make_head_rows_map_bf16(CUtensorMap* m, const void* base, int BH, int H, int L, int width, int box_w, int box_rows,
                              CUtensorMapSwizzle sw);
 
@@ -144,11 +144,6 @@ __device__ __forceinline__ void tma_load_4d(void* smem_dst, const CUtensorMap* m
         "[%6];" ::"r"(smem_u32(smem_dst)),
         "l"(map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(smem_u32(bar))
         : "memory");
-}
-// 64 columns of a row tile through a map of make_head_rows_map_bf16
-__device__ __forceinline__ void tma_load_head_rows(void* smem_dst, const CUtensorMap* map, uint64_t* bar, int x, int row, int head, int H) {
-    const int b = H ? head / H : 0;
-    tma_load_4d(smem_dst, map, bar, x, head - b * H, row, b);
 }
 // untiled bulk copy global -> shared; both addresses 16-byte aligned, bytes a multiple of 16
 __device__ __forceinline__ void bulk_load_1d(void* smem_dst, const void* gsrc, uint32_t bytes, uint64_t* bar) {

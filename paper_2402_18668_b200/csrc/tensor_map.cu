@@ -52,9 +52,10 @@ bool make_rows_map_bf16(CUtensorMap* m, const void* base, int BH, int L, int wid
 
 bool make_head_rows_map_bf16(CUtensorMap* m, const void* base, int BH, int H, int L, int width, int box_w, int box_rows,
                              CUtensorMapSwizzle sw) {
-    const cuuint64_t row = (cuuint64_t)width * 2, heads = H ? H : BH;
-    const cuuint64_t dims[4] = {(cuuint64_t)width, heads, (cuuint64_t)L, (cuuint64_t)(H ? BH / H : 1)};
-    const cuuint64_t strides[3] = {H ? row : L * row, H ? heads * row : row, heads * L * row};
+    if (H == 0) return make_rows_map_bf16(m, base, BH, L, width, box_w, box_rows, sw);
+    const cuuint64_t row = (cuuint64_t)width * 2, heads = H;
+    const cuuint64_t dims[4] = {(cuuint64_t)width, heads, (cuuint64_t)L, (cuuint64_t)(BH / H)};
+    const cuuint64_t strides[3] = {row, heads * row, heads * L * row};
     const cuuint32_t box[4] = {(cuuint32_t)box_w, 1, (cuuint32_t)box_rows, 1};
     return encode_map(m, base, 4, dims, strides, box, sw);
 }

@@ -9,8 +9,11 @@
 // for them, so that what a row warp waits for is its own arithmetic.  Against one group and one set of scores per CTA and four (d_v
 // 128: two) CTAs per SM (backward_tc.cu, kModeFwd): at d_v 128, where a second set was missing most, 59 -> 49 us at d' 32 B4 H16
 // L2048 and 216 -> 164 at d' 24 L4096; with a head alone 20 -> 12 (L2048 d_v 64).  At d_v 64 with every SM busy the two are the same:
-// half of the issue slots are used, 1075 warp instructions per tile of 128 x 64 pairs, and a CTA's start and end, 3.5 per SM and slot
-// at L2048, take a quarter of the time.
+// half of the issue slots are used, 1075 warp instructions per tile of 128 x 64 pairs.  A row warp loads sixteen score columns ahead
+// of the ones it works on: d_v 128 d' 24 47.8 -> 46.9, 64 heads L777 16.7 -> 16.2.  What bounds it is no single part (64 heads L8192 d_v
+// 64, 431 us, parts left out: the rows' work 327, the scores 398, the products 348, both 326, all three 281, the loads too 182): the
+// hand-overs of a tile, and 11 KB of loads for it.  A third row group changes nothing, nor do eight stages for six; 256 queries a CTA,
+// each key tile loaded for two halves, gains 8 % there and loses 5 at L2048 (38 us) and half at few heads.
 #include <math.h>
 
 #include <mutex>
@@ -189,49 +192,69 @@ __global__ void __launch_bounds__(kThreadsQ, 2)
         const int rw = r0 + (int)lane_base;
         const uint64_t k1 = pair_of_f(p.s1, p.s1), k2 = pair_of_f(p.s2, p.s2), one = pair_of_f(1.f, 1.f);
         uint64_t den2[2] = {0, 0};
+        // 16 scores to weights, packed in pairs from w[w0] on; first: the masked form's first column
+        auto weights = [&](auto masked_tag, const uint32_t (&sr)[16], uint32_t (&w)[16], int w0, int first) {
+            constexpr bool MASKED = decltype(masked_tag)::value;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const uint64_t s = pair_of_f(__uint_as_float(sr[2 * i]), __uint_as_float(sr[2 * i + 1]));
+                uint64_t x = fma_pairs(s, fma_pairs(s, k2, k1), one);
+                float lo, hi;
+                if (MASKED) {
+                    const int col = first + 2 * i;
+                    halves_of(x, lo, hi);
+                    x = pair_of_f(col <= row ? lo : 0.f, col + 1 <= row ? hi : 0.f);
+                }
+                den2[i & 1] = add_pairs(den2[i & 1], x);
+                halves_of(x, lo, hi);
+                w[w0 + i] = pack2(lo, hi);
+            }
+        };
+        // (what was loaded is used behind its wait and not before it)
+        auto landed = [&](uint32_t (&r)[16]) {
+            tmem_wait_ld();
+#pragma unroll
+            for (int i = 0; i < 16; ++i) asm volatile("" : "+r"(r[i]));
+        };
+        uint32_t s0[16], s1[16], w[16];
         for (int t = wg; t < n; t += 2) {
             const int si = t % C::kNSet;
             const uint32_t set = tmem_addr(tb, lane_base, si * kLTQ);
             ok = __all_sync(~0u, mbar_wait(&bars[qScore + si], (t / C::kNSet) & 1, abort_flag));
             if (!ok) break;
             tc_fence_after();
-            // 32 columns: scores to weights, packed over the columns before the last ones read
-            auto pass = [&](auto masked_tag, int h) {
-                constexpr bool MASKED = decltype(masked_tag)::value;
-                uint32_t sr[32], w[16];
-                tmem_ld32(set + 32 * h, sr);
-                tmem_wait_ld();
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const uint64_t s = pair_of_f(__uint_as_float(sr[2 * i]), __uint_as_float(sr[2 * i + 1]));
-                    uint64_t x = fma_pairs(s, fma_pairs(s, k2, k1), one);
-                    float lo, hi;
-                    if (MASKED) {
-                        const int col = t * kLTQ + 32 * h + 2 * i;
-                        halves_of(x, lo, hi);
-                        x = pair_of_f(col <= row ? lo : 0.f, col + 1 <= row ? hi : 0.f);
-                    }
-                    den2[i & 1] = add_pairs(den2[i & 1], x);
-                    halves_of(x, lo, hi);
-                    w[i] = pack2(lo, hi);
-                }
-                tmem_st16(set + 16 * h, w);
-            };
             if (t * kLTQ + kLTQ <= rw) {
-                pass(std::false_type{}, 0);
-                pass(std::false_type{}, 1);
+                // sixteen columns at a time, the next ones' load under way; the weights go over columns read before
+                tmem_ld16(set, s0);
+                landed(s0);
+                tmem_ld16(set + 16, s1);
+                weights(std::false_type{}, s0, w, 0, 0);
+                landed(s1);
+                tmem_ld16(set + 32, s0);
+                weights(std::false_type{}, s1, w, 8, 0);
+                tmem_st16(set, w);
+                landed(s0);
+                tmem_ld16(set + 48, s1);
+                weights(std::false_type{}, s0, w, 0, 0);
+                landed(s1);
+                weights(std::false_type{}, s1, w, 8, 0);
+                tmem_st16(set + 16, w);
             } else {
 #pragma unroll 1
                 for (int h = 0; h < 2; ++h) {
                     const int cb = t * kLTQ + 32 * h;
                     if (cb > rw) {                                     // no live pair
-                        uint32_t z[16];
 #pragma unroll
-                        for (int e = 0; e < 16; ++e) z[e] = 0u;
-                        tmem_st16(set + 16 * h, z);
+                        for (int e = 0; e < 16; ++e) w[e] = 0u;
                     } else {
-                        pass(std::true_type{}, h);
+                        tmem_ld16(set + 32 * h, s0);
+                        tmem_ld16(set + 32 * h + 16, s1);
+                        landed(s0);
+                        landed(s1);
+                        weights(std::true_type{}, s0, w, 0, cb);
+                        weights(std::true_type{}, s1, w, 8, cb + 16);
                     }
+                    tmem_st16(set + 16 * h, w);
                 }
             }
             tmem_wait_st();
@@ -264,7 +287,7 @@ __global__ void __launch_bounds__(kThreadsQ, 2)
 #pragma unroll
                 for (int bb = 0; bb < C::kVB; ++bb) tma_store_3d(&tm_out, out_s + bb * (kOwnQ * 128), bb * 64, r0, head);
                 tma_store_commit();
-                tma_store_wait<0>();
+                tma_store_wait_read<0>();
             }
         }
     }

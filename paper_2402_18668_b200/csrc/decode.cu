@@ -45,13 +45,14 @@ static based_status launch_variant(const T* q, const T* k, const T* v, float* kv
 //   deep   18 rows in flight per thread, two CTAs per SM: one wave of up to 296 heads (d_v 128: 128 heads 6.0 against 6.2
 //          wide; 153 rows: 4.2 / 4.7), and again beyond one wave of wide ones (2048 heads 89.9 / 91.4, 800: 36.9 / 39.7);
 //   wide   6 rows, four CTAs per SM: one wave of up to 592 heads (592: 17.5 against 19.2 deep; 400: 12.0 / 15.3);
-//   parts  9 rows, a cluster of two or four CTAs per head (decode_parts).
+//   parts  up to 9 rows, a cluster of two, four or eight CTAs per head (decode_parts).
 template <int DV, typename T, bool SYM>
 static based_status launch_t(const void* q_, const void* k_, const void* v_, float* kv, float* z, void* out_, int BH,
                              int n, cudaStream_t stream) {
     const T *q = static_cast<const T*>(q_), *k = static_cast<const T*>(k_), *v = static_cast<const T*>(v_);
     T* out = static_cast<T*>(out_);
     const int parts = decode_parts<DV, SYM>(BH);
+    if (parts == 8) return launch_variant<DV, T, SYM, 8, 9, 2, false>(q, k, v, kv, z, out, BH, n, stream);
     if (parts == 4) return launch_variant<DV, T, SYM, 4, 9, 2, false>(q, k, v, kv, z, out, BH, n, stream);
     if (parts == 2) return launch_variant<DV, T, SYM, 2, 9, 2, false>(q, k, v, kv, z, out, BH, n, stream);
     if (decode_streams(BH, DV, SYM))
@@ -148,7 +149,7 @@ bool load_kernel(K kernel) {
 }
 template <int DV, typename T, bool SYM>
 bool load_decode_format() {
-    return load_kernel(decode_step_kernel<DV, T, SYM, 4, 9, 2, false>) && load_kernel(decode_step_kernel<DV, T, SYM, 2, 9, 2, false>) &&
+    return load_kernel(decode_step_kernel<DV, T, SYM, 8, 9, 2, false>) && load_kernel(decode_step_kernel<DV, T, SYM, 4, 9, 2, false>) && load_kernel(decode_step_kernel<DV, T, SYM, 2, 9, 2, false>) &&
            load_kernel(decode_step_kernel<DV, T, SYM, 1, 18, 2, false>) && load_kernel(decode_step_kernel<DV, T, SYM, 1, 18, 2, true>) &&
            load_kernel(decode_step_kernel<DV, T, SYM, 1, 6, 4, false>);
 }

@@ -17,7 +17,8 @@ namespace based {
 // UN: rows in flight per thread at most (the rounds are made even).  STREAM: the state of all heads together is larger
 // than L2, so every line is used exactly once per step: evict-first loads and stores (89.9 -> 89.1 us, 51.6 -> 50.4 with SYM).
 // PARTS > 1: the CTAs of a cluster share the head's rows (with few heads one CTA per head leaves most of the chip idle);
-// the partial sums meet in part 0 through distributed shared memory.
+// the others write their sums to part 0's shared memory, signal and leave, and part 0 adds them up (read by part 0 from theirs,
+// which then had to wait for it, a step of 16 heads took 0.35 us more).
 template <int DV, typename T, bool SYM, int PARTS, int UN, bool STREAM>
 __device__ __forceinline__ void decode_step_body(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
                                                  float* __restrict__ kv, float* __restrict__ z, T* __restrict__ out,
@@ -31,11 +32,12 @@ __device__ __forceinline__ void decode_step_body(const T* __restrict__ q, const 
     __shared__ float s_pq[MAXR], s_pk[MAXR];
     __shared__ __align__(16) float s_num[RPP][DV];
     __shared__ float s_den[8];
-    __shared__ float s_part[DV + 1];                             // the part's sums: numerator, denominator
+    __shared__ float s_part[PARTS][DV + 1];                      // the parts' sums: numerator, denominator (PARTS > 1: in part 0 alone)
     const int tid = threadIdx.x, c4 = tid % TPR, rslot = tid / TPR;
     const bool row_thread = rslot < RPP;
     const int r0 = part * ND / PARTS, rows = (part + 1) * ND / PARTS - r0;
 
+    if (PARTS > 1) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");      // part 0 runs: the others may write to it
     float4* S = reinterpret_cast<float4*>(kv + (head * ND + r0) * (size_t)DV) + c4;
     float4 s[UNROLL];
     auto fetch = [&](int p0) {
@@ -104,43 +106,47 @@ __device__ __forceinline__ void decode_step_body(const T* __restrict__ q, const 
     }
     if (row_thread) *reinterpret_cast<float4*>(&s_num[rslot][c4 * 4]) = acc;
     __syncthreads();
+    cg::cluster_group cluster = cg::this_cluster();
+    float* to = PARTS == 1 ? s_part[0] : cluster.map_shared_rank(s_part[part], 0);
+    if (PARTS > 1) asm volatile("barrier.cluster.wait;" ::: "memory");
     if (tid < DV) {
         float num = 0.f;
 #pragma unroll
         for (int r = 0; r < RPP; ++r) num += s_num[r][tid];
-        s_part[tid] = num;
+        to[tid] = num;
     } else if (tid == DV) {
         float den = 0.f;
 #pragma unroll
         for (int w = 0; w < 8; ++w) den += s_den[w];
-        s_part[DV] = den;
+        to[DV] = den;
     }
     if (PARTS == 1) {
         __syncthreads();
-        if (tid < DV) out[head * DV + tid] = from_f32<T>(numerator_only ? s_part[tid] : s_part[tid] / (s_part[DV] + kEps));
-        return;
+    } else {
+        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+        if (part != 0) return;
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
     }
-    cg::cluster_group cluster = cg::this_cluster();
-    cluster.sync();
-    if (part == 0 && tid < DV) {
+    if (tid < DV) {
         float num = 0.f, den = 0.f;
 #pragma unroll
         for (int c = 0; c < PARTS; ++c) {
-            const float* p = cluster.map_shared_rank(s_part, c);
-            num += p[tid];
-            den += p[DV];
+            num += s_part[c][tid];
+            den += s_part[c][DV];
         }
         out[head * DV + tid] = from_f32<T>(numerator_only ? num : num / (den + kEps));
     }
-    cluster.sync();                                              // the parts' sums stay until part 0 has read them
 }
 
-// CTAs per head, by one CTA per SM (us per step on B200, replayed back to back): 16 heads, d_v 128, four 3.6, two 4.4, one
-// 5.2; 74 heads 7.1 / 4.7 / 5.3.  Not where a head's state is small (153 rows x 64: 3.0 / 3.2 / 2.7 at 16 heads).
+// CTAs per head, by one CTA per SM (us per step on B200, replayed back to back on states from memory): d_v 128 with 16 heads eight
+// 4.0, four 4.3, with 2 heads 2.2 / 2.5 (and 2.75 before the parts' sums were pushed); 153 rows 2.9 / 3.0 with 16; d_v 64 2.6 / 2.7;
+// 25 heads four 3.6, two 3.6, one 3.8, 74 heads d_v 128 two 6.7, one 7.6.  Not where a head's state is small (153 rows x 64 with 16
+// heads: 2.6 / 2.4 / 2.5 / 2.3).
 // The sums' order depends on it, so the fused step follows the same rule.
 template <int DV, bool SYM>
 inline int decode_parts(int heads) {
     constexpr int head_kb = (SYM ? kDSym : kD) * DV * 4 / 1024;
+    if (head_kb >= 64 && 8 * heads <= kSMs) return 8;
     if (head_kb >= 64 && 4 * heads <= kSMs) return 4;
     if (head_kb >= 96 && 2 * heads <= kSMs) return 2;
     return 1;

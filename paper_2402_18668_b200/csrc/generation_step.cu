@@ -134,6 +134,7 @@ template <int DV, typename T, bool STREAM, bool SYM, int NPW>
 based_status launch_p(const GenArgs& a, size_t smem, cudaStream_t stream) {
     if constexpr (!STREAM) {
         const int parts = decode_parts<DV, SYM>(a.n_lin);
+        if (parts == 8) return launch_k<DV, T, STREAM, SYM, NPW, 8>(a, smem, stream);
         if (parts == 4) return launch_k<DV, T, STREAM, SYM, NPW, 4>(a, smem, stream);
         if (parts == 2) return launch_k<DV, T, STREAM, SYM, NPW, 2>(a, smem, stream);
     }
@@ -174,7 +175,7 @@ bool load_parts() {
 template <int DV, typename T, bool STREAM, bool SYM, int NPW>
 bool load_one() {
     if (!load_parts<DV, T, STREAM, SYM, NPW, 1>()) return false;
-    if constexpr (!STREAM) return load_parts<DV, T, STREAM, SYM, NPW, 2>() && load_parts<DV, T, STREAM, SYM, NPW, 4>();
+    if constexpr (!STREAM) return load_parts<DV, T, STREAM, SYM, NPW, 2>() && load_parts<DV, T, STREAM, SYM, NPW, 4>() && load_parts<DV, T, STREAM, SYM, NPW, 8>();
     return true;
 }
 template <int DV, typename T>

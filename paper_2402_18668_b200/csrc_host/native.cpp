@@ -176,7 +176,7 @@ Tensor prefill_call(const Tensor& q, const Tensor& k, const Tensor& v, const Ten
                     const Tensor& workspace, void* stream) {
     const int B = size(q, 0), H = size(q, 1), L = size(q, 2), d_feat = size(q, 3), d_v = size(v, 3);
     const based_dtype io = dtype_code(q);
-    if (!out.defined()) out = at::empty_like(v);
+    if (!out.defined()) out = fresh(v);
     size_t need = based_prefill_workspace_bytes(B, H, L, d_feat, d_v, io);
     if (need <= BASED_WORDS_BYTES && !(flags & BASED_STATE_CONTINUE)) need = 0;
     const Workspace ws(workspace, need, q, stream);
@@ -268,7 +268,7 @@ PyObject* decode_step(PyObject* const* a) {
     check_state(kv, z, B, H, d_feat, d_v, flags, true);
     const based_dtype io = dtype_code(q);
     void* stream = stream_of(a[7]);
-    if (!out.defined()) out = at::empty_like(v);
+    if (!out.defined()) out = fresh(v);
     const based_status st = unlocked([&] {
         return based_decode_step_flags(cptr(q), cptr(k), cptr(v), fptr(kv), fptr(z), ptr(out), B, H, d_feat, d_v, io, flags, stream);
     });
@@ -287,7 +287,7 @@ PyObject* swa(PyObject* const* a) {
     const float scale = number(a[5]);
     const based_dtype io = dtype_code(q);
     void* stream = stream_of(a[6]);
-    if (!out.defined()) out = at::empty_like(v);
+    if (!out.defined()) out = fresh(v);
     const based_status st = unlocked([&] {
         return swa_forward(cptr(q), cptr(k), cptr(v), ptr(out), size(q, 0), size(q, 1), size(q, 2), size(q, 3), window, scale, io, stream);
     });
@@ -317,7 +317,7 @@ PyObject* swa_decode(PyObject* const* a) {
     const float scale = number(a[7]);
     const based_dtype io = dtype_code(q);
     void* stream = stream_of(a[8]);
-    if (!out.defined()) out = at::empty_like(v);
+    if (!out.defined()) out = fresh(v);
     const based_status st = unlocked([&] {
         return ragged ? swa_decode_step_ragged(cptr(q), cptr(k), cptr(v), ptr(kc), ptr(vc), ptr(out), B, H, d, window,
                                                static_cast<const int*>(cptr(positions)), scale, io, stream)
@@ -350,8 +350,8 @@ PyObject* generation_step(PyObject* const* a) {
     const float scale = number(a[14]);
     const based_dtype io = dtype_code(q);
     void* stream = stream_of(a[15]);
-    if (!out.defined()) out = at::empty_like(v);
-    if (!out_w.defined()) out_w = at::empty_like(vw);
+    if (!out.defined()) out = fresh(v);
+    if (!out_w.defined()) out_w = fresh(vw);
     const int window = size(kc, 2);
     const based_status st = unlocked([&] {
         return based_generation_step(cptr(q), cptr(k), cptr(v), fptr(kv), fptr(z), ptr(out), cptr(qw), cptr(kw), cptr(vw), ptr(kc),
@@ -471,7 +471,7 @@ PyObject* baseconv(PyObject* const* p) {
         value_error("conv_state must be [B, width-1, C] in the io dtype");
     const based_dtype io = dtype_code(a);
     void* stream = stream_of(p[7]);
-    if (!out.defined()) out = at::empty_like(a);
+    if (!out.defined()) out = fresh(a);
     auto filter = static_cast<const float*>(cptr(h)), bias = static_cast<const float*>(cptr(b2));
     const based_status st = unlocked([&] {
         return step ? baseconv_gate_step(cptr(a), cptr(g), filter, bias, ptr(state), ptr(out), B, C, width, io, stream)

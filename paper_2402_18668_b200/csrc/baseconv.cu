@@ -7,21 +7,21 @@
 // part of this file); h is the depthwise causal filter of width w (the paper suggests 3), h[0]
 // the tap on the current token.
 //
-// The op is one pass over a, g and out: 3 elements of traffic per output element and a dozen
-// flops, so it is bound by HBM bandwidth.  A thread owns 8 consecutive channels (one 16-byte
-// piece of a bf16 row, two of an fp32 row) and walks a run of up to 64 tokens with the last w-1 rows
-// of g in registers, so g is read once (plus w-1 halo rows per run, which the neighbouring run
-// has just brought into L2); a warp covers 256 consecutive channels of a row.  The loop is
-// software-pipelined: the rows of the next four tokens are in flight (kept packed, as loaded)
-// while the current four are converted, combined and stored.
+// The op is one pass over a, g and out: 3 elements of traffic per output element and a dozen flops, so it is bound by HBM
+// bandwidth.  A thread owns 8 consecutive channels (one 16-byte piece of a bf16 row, two of an fp32 row) of 2, 4 or 8
+// consecutive tokens (baseconv_block_kernel): their rows of a and g, and the w - 1 rows of g before them, which a neighbouring
+// block brings into L2 at the same time, are all requested at once, and the blocks sweep the arrays in the order they lie in
+// memory.  That is what HBM rewards: with runs of 64 tokens a thread, the rows of g carried along and the next four tokens' in
+// flight, 2368 blocks were at as many places 1 MB apart.  B8 N4096 C8192 w 3 bf16 261 -> 228 us = 7.06 TB/s (a product a * g by torch
+// over the same arrays: 230), B8 N1024 C8192 72 -> 60, fp32 B8 N2048 C4096 152 -> 123.
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace based {
 
 namespace {
-constexpr int kMaxRun = 64;     // tokens per thread run, at most
-constexpr int kUnroll = 4;      // tokens whose loads are in flight together
-constexpr int kThreadsBC = 128;
+constexpr int kThreadsBC = 128, kThreadsBlock = 64;
 
 template <typename T> struct Row8;
 template <> struct Row8<__nv_bfloat16> {
@@ -29,6 +29,8 @@ template <> struct Row8<__nv_bfloat16> {
     static __device__ __forceinline__ void load_raw(const __nv_bfloat16* p, Raw& r) {
         r.u = __ldcs(reinterpret_cast<const uint4*>(p));
     }
+    // (rows that another block reads too)
+    static __device__ __forceinline__ void load_shared(const __nv_bfloat16* p, Raw& r) { r.u = __ldg(reinterpret_cast<const uint4*>(p)); }
     static __device__ __forceinline__ void unpack(const Raw& r, float (&x)[8]) {
         const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&r.u);
 #pragma unroll
@@ -39,16 +41,6 @@ template <> struct Row8<__nv_bfloat16> {
         }
     }
     static __device__ __forceinline__ void store_raw(__nv_bfloat16* p, const Raw& r) { __stcs(reinterpret_cast<uint4*>(p), r.u); }
-    static __device__ __forceinline__ void load(const __nv_bfloat16* p, float (&x)[8]) {
-        const uint4 u = __ldcs(reinterpret_cast<const uint4*>(p));
-        const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float2 f = __bfloat1622float2(h[i]);
-            x[2 * i] = f.x;
-            x[2 * i + 1] = f.y;
-        }
-    }
     static __device__ __forceinline__ void store(__nv_bfloat16* p, const float (&x)[8]) {
         uint4 u;
         __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&u);
@@ -63,16 +55,16 @@ template <> struct Row8<float> {
         r.a = __ldcs(reinterpret_cast<const float4*>(p));
         r.b = __ldcs(reinterpret_cast<const float4*>(p) + 1);
     }
+    static __device__ __forceinline__ void load_shared(const float* p, Raw& r) {
+        r.a = __ldg(reinterpret_cast<const float4*>(p));
+        r.b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+    }
     static __device__ __forceinline__ void unpack(const Raw& r, float (&x)[8]) {
         x[0] = r.a.x; x[1] = r.a.y; x[2] = r.a.z; x[3] = r.a.w; x[4] = r.b.x; x[5] = r.b.y; x[6] = r.b.z; x[7] = r.b.w;
     }
     static __device__ __forceinline__ void store_raw(float* p, const Raw& r) {
         __stcs(reinterpret_cast<float4*>(p), r.a);
         __stcs(reinterpret_cast<float4*>(p) + 1, r.b);
-    }
-    static __device__ __forceinline__ void load(const float* p, float (&x)[8]) {
-        const float4 a = __ldcs(reinterpret_cast<const float4*>(p)), b = __ldcs(reinterpret_cast<const float4*>(p) + 1);
-        x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
     }
     static __device__ __forceinline__ void store(float* p, const float (&x)[8]) {
         __stcs(reinterpret_cast<float4*>(p), make_float4(x[0], x[1], x[2], x[3]));
@@ -86,6 +78,45 @@ __device__ __forceinline__ void load8(const float* p, float (&x)[8]) {
     x[0] = lo.x; x[1] = lo.y; x[2] = lo.z; x[3] = lo.w; x[4] = hi.x; x[5] = hi.y; x[6] = hi.z; x[7] = hi.w;
 }
 
+// two channels at a time: fp32 pairs, two multiply-adds per instruction
+__device__ __forceinline__ uint32_t& word(uint4& v, int i) { return reinterpret_cast<uint32_t*>(&v)[i]; }
+__device__ __forceinline__ uint32_t word(const uint4& v, int i) { return reinterpret_cast<const uint32_t*>(&v)[i]; }
+__device__ __forceinline__ uint64_t pair_of(float lo, float hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ uint64_t pair_of_bf16(uint32_t w) { return pair_of(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u)); }
+__device__ __forceinline__ uint64_t fma_pairs(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul_pairs(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ void load_pairs(const float* p, uint64_t (&x)[4]) {
+    const ulonglong2 lo = __ldg(reinterpret_cast<const ulonglong2*>(p)), hi = __ldg(reinterpret_cast<const ulonglong2*>(p) + 1);
+    x[0] = lo.x; x[1] = lo.y; x[2] = hi.x; x[3] = hi.y;
+}
+// a SiLU(x) of two channels, rounded to bf16: x / (1 + 2^(-x log2 e)) with the fast exponential and reciprocal
+__device__ __forceinline__ uint32_t gated_pair(uint64_t x, uint64_t a) {
+    float s0, s1;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(s0), "=f"(s1) : "l"(mul_pairs(x, pair_of(-1.4426950408889634f, -1.4426950408889634f))));
+    asm("ex2.approx.ftz.f32 %0, %0;" : "+f"(s0));
+    asm("ex2.approx.ftz.f32 %0, %0;" : "+f"(s1));
+    s0 += 1.0f;
+    s1 += 1.0f;
+    asm("rcp.approx.ftz.f32 %0, %0;" : "+f"(s0));
+    asm("rcp.approx.ftz.f32 %0, %0;" : "+f"(s1));
+    float y0, y1;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(y0), "=f"(y1) : "l"(mul_pairs(a, mul_pairs(x, pair_of(s0, s1)))));
+    const __nv_bfloat162 r = __floats2bfloat162_rn(y0, y1);
+    return *reinterpret_cast<const uint32_t*>(&r);
+}
+
 // SiLU(x) = x * sigmoid(x); the fast exponential and division are exact enough for bf16 outputs,
 // fp32 io takes the accurate ones
 template <bool FAST>
@@ -94,76 +125,81 @@ __device__ __forceinline__ float silu(float x) {
 }
 }  // namespace
 
-template <typename T, int W>
-__global__ void __launch_bounds__(kThreadsBC) baseconv_gate_kernel(const T* __restrict__ a, const T* __restrict__ g,
-                                                                   const float* __restrict__ h,
-                                                                   const float* __restrict__ b2, T* __restrict__ out,
-                                                                   int N, int C, int run) {
+// Blocks per SM: what is in flight on an SM is TOK rows times its threads, so each instance is held to the registers that let one
+// more block in where it is a few above (bf16 w 3: 8 tokens 130 -> 128, seven blocks -> eight, B8 N4096 C8192 241 -> 228 us; 4
+// tokens 102 -> 96, B1 37.6 -> 32.2).
+__host__ __device__ constexpr int blocks_per_sm(int elem, int W, int tok) {
+    if (elem == 4) return tok == 4 ? (W == 1 ? 10 : W < 4 ? 8 : 6) : W == 1 ? 16 : W == 2 ? 11 : W == 3 ? 10 : 8;
+    if (tok == 8) return W == 1 ? 10 : W < 4 ? 8 : 6;
+    if (tok == 4) return W == 1 ? 14 : W == 2 ? 12 : W == 3 ? 10 : 8;
+    return W == 1 ? 18 : W == 2 ? 16 : W == 3 ? 12 : 10;
+}
+// TOK tokens of 8 channels per thread; grid: blocks of 512 channels, of TOK tokens, sequences.  FLAT: the first two in one dimension, for
+// more blocks of tokens than a grid has rows (for all calls, its division cost B8 N4096 C8192 228 -> 239 us).
+template <typename T, int W, int TOK, bool FLAT>
+__global__ void __launch_bounds__(kThreadsBlock, blocks_per_sm(sizeof(T), W, TOK)) baseconv_block_kernel(const T* __restrict__ a, const T* __restrict__ g,
+                                                                       const float* __restrict__ h, const float* __restrict__ b2,
+                                                                       T* __restrict__ out, int N, int C, int gb) {
+    enter_dependent();
     constexpr bool FAST = sizeof(T) == 2;
-    const int c0 = (blockIdx.x * kThreadsBC + threadIdx.x) * 8;
+    const int row = FLAT ? blockIdx.x / gb : blockIdx.y, col = FLAT ? blockIdx.x - row * gb : blockIdx.x;
+    const int c0 = (col * kThreadsBlock + threadIdx.x) * 8;
     if (c0 >= C) return;
-    const int i0 = blockIdx.y * run;
-    const int i1 = min(N, i0 + run);
-    const size_t base = (size_t)blockIdx.z * N * C + c0;
-
-    // prev[j] = g of the token j+1 steps back (zero before the sequence start)
-    float prev[W > 1 ? W - 1 : 1][8];
+    const size_t base = (size_t)(FLAT ? blockIdx.y : blockIdx.z) * N * C + c0;
+    const int i0 = row * TOK;
+    typename Row8<T>::Raw gr[TOK + W - 1], ar[TOK];
 #pragma unroll
-    for (int j = 0; j < W - 1; ++j) {
-        const int i = i0 - 1 - j;
-        if (i >= 0) Row8<T>::load(g + base + (size_t)i * C, prev[j]);
-        else {
-#pragma unroll
-            for (int e = 0; e < 8; ++e) prev[j][e] = 0.f;
-        }
+    for (int u = 0; u < W - 1; ++u) {
+        const int i = i0 + u - (W - 1);
+        if (i >= 0) Row8<T>::load_shared(g + base + (size_t)i * C, gr[u]);
+        else gr[u] = typename Row8<T>::Raw{};                        // before the sequence
     }
-
-    // software pipeline: the loads of the next kUnroll tokens are in flight while these are used
-    typename Row8<T>::Raw gr[kUnroll], ar[kUnroll], gn[kUnroll], an[kUnroll];
-    auto fetch = [&](int i, typename Row8<T>::Raw (&gq)[kUnroll], typename Row8<T>::Raw (&aq)[kUnroll]) {
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-            if (i + u < i1) {
-                Row8<T>::load_raw(g + base + (size_t)(i + u) * C, gq[u]);
-                Row8<T>::load_raw(a + base + (size_t)(i + u) * C, aq[u]);
+    for (int u = 0; u < TOK; ++u)
+        if (i0 + u < N) Row8<T>::load_shared(g + base + (size_t)(i0 + u) * C, gr[u + W - 1]);
+#pragma unroll
+    for (int u = 0; u < TOK; ++u)
+        if (i0 + u < N) Row8<T>::load_raw(a + base + (size_t)(i0 + u) * C, ar[u]);
+    if constexpr (FAST) {
+        uint64_t taps[W][4], bias[4];
+#pragma unroll
+        for (int j = 0; j < W; ++j) load_pairs(h + (size_t)j * C + c0, taps[j]);
+        load_pairs(b2 + c0, bias);
+#pragma unroll
+        for (int u = 0; u < TOK; ++u) {
+            if (i0 + u >= N) break;
+            uint4 y;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                uint64_t acc = bias[e];
+#pragma unroll
+                for (int j = 0; j < W; ++j) acc = fma_pairs(taps[j][e], pair_of_bf16(word(gr[u + W - 1 - j].u, e)), acc);
+                word(y, e) = gated_pair(acc, pair_of_bf16(word(ar[u].u, e)));
             }
+            __stcs(reinterpret_cast<uint4*>(out + base + (size_t)(i0 + u) * C), y);
         }
-    };
-    fetch(i0, gr, ar);
-    float taps[W][8], bias[8];
+    } else {
+        float taps[W][8], bias[8];
 #pragma unroll
-    for (int j = 0; j < W; ++j) load8(h + (size_t)j * C + c0, taps[j]);
-    load8(b2 + c0, bias);
-    for (int i = i0; i < i1; i += kUnroll) {
-        fetch(i + kUnroll, gn, an);
+        for (int j = 0; j < W; ++j) load8(h + (size_t)j * C + c0, taps[j]);
+        load8(b2 + c0, bias);
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-            if (i + u < i1) {
-                float gx[8], ax[8], y[8];
-                Row8<T>::unpack(gr[u], gx);
-                Row8<T>::unpack(ar[u], ax);
+        for (int u = 0; u < TOK; ++u) {
+            if (i0 + u >= N) break;
+            float acc[8], x[8];
+            Row8<T>::unpack(gr[u + W - 1], x);
 #pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    float acc = fmaf(taps[0][e], gx[e], bias[e]);
+            for (int e = 0; e < 8; ++e) acc[e] = fmaf(taps[0][e], x[e], bias[e]);
 #pragma unroll
-                    for (int j = 1; j < W; ++j) acc = fmaf(taps[j][e], prev[j - 1][e], acc);
-                    y[e] = ax[e] * silu<FAST>(acc);
-                }
-                Row8<T>::store(out + base + (size_t)(i + u) * C, y);
+            for (int j = 1; j < W; ++j) {
+                Row8<T>::unpack(gr[u + W - 1 - j], x);
 #pragma unroll
-                for (int j = W - 2; j >= 1; --j)
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) prev[j][e] = prev[j - 1][e];
-                if (W > 1) {
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) prev[0][e] = gx[e];
-                }
+                for (int e = 0; e < 8; ++e) acc[e] = fmaf(taps[j][e], x[e], acc[e]);
             }
-        }
+            Row8<T>::unpack(ar[u], x);
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-            gr[u] = gn[u];
-            ar[u] = an[u];
+            for (int e = 0; e < 8; ++e) x[e] *= silu<FAST>(acc[e]);
+            Row8<T>::store(out + base + (size_t)(i0 + u) * C, x);
         }
     }
 }
@@ -226,10 +262,9 @@ template <typename T, int W>
 static void launch_w(const void* a, const void* g, const float* h, const float* b2, void* state, void* out, int B,
                      int N, int C, bool step, cudaStream_t stream) {
     const int gx = (C / 8 + kThreadsBC - 1) / kThreadsBC;
-    static std::atomic<bool> split[3][64];
+    static std::atomic<bool> split[2][64];
     prefer_l1(baseconv_step_kernel<T, W, 4>, 0, split[0]);       // (a preference only: the launch reports what fails)
     prefer_l1(baseconv_step_kernel<T, W, 1>, 0, split[1]);
-    prefer_l1(baseconv_gate_kernel<T, W>, 0, split[2]);
     // a step is a dependent launch: its blocks come in while the kernel ahead drains (behind the other mixers' steps at batch
     // 128 1.0 us less a token; back to back with itself 0.5 more); four sequences per thread once that still gives every SM a block
     if (step && gx * ((B + 3) / 4) >= kSMs)
@@ -239,16 +274,24 @@ static void launch_w(const void* a, const void* g, const float* h, const float* 
         launch_ex(baseconv_step_kernel<T, W, 1>, dim3(gx, B), dim3(kThreadsBC), 0, 1, true, stream,
             static_cast<const T*>(a), static_cast<const T*>(g), h, b2, static_cast<T*>(state), static_cast<T*>(out), B, C);
     else {
-        // runs of 64 tokens (a halo of width - 1 rows each) while the last wave of blocks is a small part of the grid, 32
-        // below, shorter ones until the grid has a block or two for every SM (us with runs of 64 / 32 / 16 / 8 / 4 tokens:
-        // B3 N128 C5208 12.8 / 7.4 / 5.0 / 4.4 / 5.7, B2 N1024 C2048 12.9 / 7.7 / 6.4 / 6.9 / 7.1, B4 N1024 C8192 width 4
-        // 41 / 37 / 38 / 42 / 51; B8 N4096 C8192 267 / 264 / 270 / 295 / 350, but 276.5 / 277.8 on alternating inputs)
-        auto blocks = [&](int run) { return (long long)gx * ((N + run - 1) / run) * B; };
-        int run = kMaxRun;
-        if (blocks(run) < 2048) run /= 2;
-        while (run > 4 && blocks(run) < 240) run /= 2;
-        baseconv_gate_kernel<T, W><<<dim3(gx, (N + run - 1) / run, B), kThreadsBC, 0, stream>>>(
-            static_cast<const T*>(a), static_cast<const T*>(g), h, b2, static_cast<T*>(out), N, C, run);
+        // Tokens per thread, us with runs of 64 before / 8 / 4 / 2 (bf16): w 3 B8 N4096 C8192 261 / 228 / 233 / 290, B8 N1024 C8192 72 /
+        // 60 / 61 / 75, B4 N3000 C3200 52 / 37 / 38 / 47, B1 N512 C8192 9.4 / 7.7 / 6.8 / 7.7, B3 N200 C1000 5.7 / 4.9 / 5.1 / 5.0; w 4 B8 N4096
+        // C8192 265 / 246 / 262; fp32 w 3 B8 N2048 C4096 152 / - / 123 / 133, B8 N64 C4096 10.6 / - / 8.2 / 7.7.
+        const int gb = (C / 8 + kThreadsBlock - 1) / kThreadsBlock;
+        auto blocks = [&](int tok) { return (long long)gb * ((N + tok - 1) / tok) * B; };
+        auto block = [&](auto tok_tag, auto flat_tag) {
+            constexpr int TOK = decltype(tok_tag)::value;
+            constexpr bool FLAT = decltype(flat_tag)::value;
+            const unsigned rows = (N + TOK - 1) / TOK;
+            launch_ex(baseconv_block_kernel<T, W, TOK, FLAT>, FLAT ? dim3(gb * rows, B) : dim3(gb, rows, B), dim3(kThreadsBlock), 0, 1, true, stream,
+                      static_cast<const T*>(a), static_cast<const T*>(g), h, b2, static_cast<T*>(out), N, C, gb);
+        };
+        using Four = std::integral_constant<int, 4>;
+        using Most = std::integral_constant<int, sizeof(T) == 2 ? 8 : 4>;
+        if (N > 2 * 65535) block(Four{}, std::true_type{});
+        else if (sizeof(T) == 2 && blocks(8) >= 12288) block(Most{}, std::false_type{});
+        else if (blocks(4) >= 2048) block(Four{}, std::false_type{});
+        else block(std::integral_constant<int, 2>{}, std::false_type{});
     }
 }
 

@@ -779,8 +779,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint8_t* sOut = smem + C::offOut;
 
     if (tid == 0) { TRACE(5, 0, 7); TRACE_CTA(0); }     // kernel entry
-    // state pass: the main pass of the same call may be scheduled behind this CTA (see launch_main_after_state)
-    if (STATE_ONLY) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (tid == 0) {
         for (int s = 0; s < NS; ++s) { mbar_init(&bars[kFull0 + s], 1); mbar_init(&bars[kEmpty0 + s], STATE_ONLY ? 1 : 2); }
         mbar_init(&bars[kG1], 1); mbar_init(&bars[kG1b], 1); mbar_init(&bars[kPb], 128); mbar_init(&bars[kG2], 1); mbar_init(&bars[kG2b], 1); mbar_init(&bars[kG4], 1); mbar_init(&bars[kG4b], 1);
@@ -819,12 +817,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    // The recompute-mode kernel is a programmatic dependent launch: a CTA may get here, past its set-up, while the grid
-    // before it in the stream still runs.  It waits for that grid to complete before it touches global memory, and
-    // only then lets the grid behind it be scheduled (a grid is never scheduled before everything two grids back is
-    // complete).  Short calls gain a tenth from it (cfg 2 back to back: 22.9 -> 20.4 us).  Not in the other modes: the
-    // same two instructions in the plain chunk loop's kernel cost it 1-4 %.
-    if (MODE == kModePre) {
+    // The recompute-mode kernel and the state pass are programmatic dependent launches: a CTA may get here, past its set-up,
+    // while the grid before it in the stream still runs.  It waits for that grid to complete before it touches global memory,
+    // and only then lets the grid behind it be scheduled (the state pass: the main pass of the same call, whose first
+    // pieces read the inputs without a wait of their own).  Short calls gain a tenth from it (B4 H16 L2048 back to back: 22.9 ->
+    // 20.4 us; a state pass behind other work 1 to 2 us).  Not in the main mode: the same two instructions in the plain chunk
+    // loop's kernel cost it 1-4 %.
+    if (MODE != kModeMain) {
         asm volatile("griddepcontrol.wait;" ::: "memory");
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     }
@@ -1741,7 +1740,7 @@ based_status launch_dv(const void* q, const void* k, const void* v, void* out, f
         p.pad = 5;
 #endif
         const dim3 grid(plan.balanced + BH - 1, 1);
-        prefill_tc_kernel<DV, kModeState><<<grid, kThreads, C::kSmemBytes, stream>>>(tq, tk, tv, to, p);
+        if (launch_dependent<DV, kModeState>(grid, stream, tq, tk, tv, to, p) != cudaSuccess) return BASED_ERR_CUDA;
         note_launch();
         based_status st = check_launch("prefill_tc_kernel<state, balanced>");
         if (st != BASED_OK) return st;
@@ -1773,7 +1772,7 @@ based_status launch_dv(const void* q, const void* k, const void* v, void* out, f
             st = check_launch("abi_to_slot_kernel");
             if (st != BASED_OK) return st;
         }
-        prefill_tc_kernel<DV, kModeState><<<dim3(nseg - 1, BH), kThreads, C::kSmemBytes, stream>>>(tq, tk, tv, to, p);
+        if (launch_dependent<DV, kModeState>(dim3(nseg - 1, BH), stream, tq, tk, tv, to, p) != cudaSuccess) return BASED_ERR_CUDA;
         note_launch();
         st = check_launch("prefill_tc_kernel<state>");
         if (st != BASED_OK) return st;
@@ -1950,7 +1949,7 @@ static based_status launch_state_dv(const void* k, const void* v, float* kv, flo
         }
     }
     // the q and output maps are not used by the state-update-only pass
-    prefill_tc_kernel<DV, kModeState><<<dim3(plan.nseg, BH), kThreads, C::kSmemBytes, stream>>>(tk, tk, tv, tv, p);
+    if (launch_dependent<DV, kModeState>(dim3(plan.nseg, BH), stream, tk, tk, tv, tv, p) != cudaSuccess) return BASED_ERR_CUDA;
     note_launch();
     based_status st = check_launch("prefill_tc_kernel<state>");
     if (st != BASED_OK) return st;

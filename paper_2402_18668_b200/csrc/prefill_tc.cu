@@ -1754,7 +1754,7 @@ based_status launch_dv(const void* q, const void* k, const void* v, void* out, f
         note_launch();
         return check_launch("prefill_tc_kernel<balanced>");
     }
-    if (nseg > 1 && recompute) {
+    if (recompute) {
         if (continued) p.ticket = new_ticket();
         const cudaError_t e = continued ? launch_dependent<DV, kModePre, true>(dim3(nseg, BH), stream, tq, tk, tv, to, p)
                                              : launch_dependent<DV, kModePre>(dim3(nseg, BH), stream, tq, tk, tv, to, p);
@@ -1864,6 +1864,11 @@ static SegPlan prefill_tc_plan(int BH, int L, int d_v, bool continued = false, s
         if (share >= 16.f && total >= ranges && total <= 14000000 && (size_t)ranges * slot <= ws_limit && cost < 0.95f * best_cost)
             best = {1, nch, false, ranges};
     }
+    // One segment of few chunks: the recompute mode's kernel too, which has no earlier chunks to run then and is a dependent launch
+    // (us, plain chunk loop / this: H16 L100 d_v64 6.3 / 4.9, H2 L16 d_v128 7.1 / 5.4, H100 L256 d_v64 7.9 / 6.9, H256 L300 16.6 / 15.9,
+    // H200 L300 d_v128 20.3 / 19.6, H120 L500 13.3 / 13.2, H200 L700 d_v64 23.5 / 23.6, L1500 38.0 / 39.8; continued H16 L100 10.6 / 9.6, H100
+    // L256 12.3 / 12.1, H256 L300 25.5 / 25.9, at d_v 128 H2 L16 11.6 / 11.0, H200 L128 24.2 / 24.2, H100 L200 14.4 / 15.0)
+    if (best.nseg == 1 && best.balanced == 0 && nch <= (!continued ? 4 : d_v == 64 ? 2 : 1)) best.recompute = true;
 #ifdef BASED_TRACE
     if (const char* e = getenv("BASED_NSEG")) {
         const int v = atoi(e);                      // negative: recompute mode with that many segments

@@ -104,8 +104,6 @@ __global__ void __launch_bounds__(kThreadsS, 2)
     const int head = blockIdx.y, part = blockIdx.x;
     const int nit = (p.L + kTB - 1) / kTB;
 
-    // the outputs' kernel, if one follows, needs nothing of this one: it may take what SMs have left from the start
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (tid == 0) {
         for (int s = 0; s < C::kNS; ++s) mbar_init(&bars[sFull0 + s], 1);
         for (int b = 0; b < 2; ++b) { mbar_init(&bars[sAlu0 + b], kRowThreads / 2); mbar_init(&bars[sMma0 + b], 1); }
@@ -121,6 +119,10 @@ __global__ void __launch_bounds__(kThreadsS, 2)
     tc_fence_after();
     const uint32_t tb = *tmem_base_s;
     bool ok = true;
+    // A dependent launch: set up while the grid ahead drains.  The outputs' kernel, if one follows, needs nothing of this one: it may
+    // take what SMs have left once that grid is complete.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     if (warp == 8) {
         // the whole warp runs this block; one elected lane issues the MMAs, commits and loads (see mma_ss_w)
@@ -336,9 +338,10 @@ based_status launch_state(const void* k, const void* v, float* kv, float* z, int
             configured[dev] = true;
         }
     }
-    generic_state_tc_kernel<DF, DV><<<dim3(C::kParts, BH), kThreadsS, C::kSmem, stream>>>(tv, p);
+    const cudaError_t e = launch_ex(generic_state_tc_kernel<DF, DV>, dim3(C::kParts, BH), dim3(kThreadsS), C::kSmem, 1, true, stream, tv, p);
     note_launch();
-    return check_launch("generic_state_tc_kernel");
+    const based_status st = check_launch("generic_state_tc_kernel");
+    return e == cudaSuccess ? st : BASED_ERR_CUDA;
 }
 }  // namespace
 

@@ -127,6 +127,9 @@ __global__ void __launch_bounds__(kThreadsQ, 2)
     tc_fence_after();
     const uint32_t tb = *tmem_base_s;
     bool ok = true;
+    // (a dependent launch: alone, or beside the state's kernel, which has waited for what is ahead of both)
+    if (!p.overlapped) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     if (warp == 8 || warp == 9) {
         // ============================================================================ MMA warps: scores, products
@@ -319,7 +322,7 @@ based_status launch_forward(const CUtensorMap& q, const CUtensorMap& k, const CU
             configured[dev] = true;
         }
     }
-    const cudaError_t e = launch_ex(quadratic_fwd_tc_kernel<DV>, dim3(grid), dim3(kThreadsQ), C::kSmem, 1, p.overlapped != 0, stream, q, k, v,
+    const cudaError_t e = launch_ex(quadratic_fwd_tc_kernel<DV>, dim3(grid), dim3(kThreadsQ), C::kSmem, 1, true, stream, q, k, v,
                                     out, p);
     note_launch();
     const based_status st = check_launch("quadratic_fwd_tc_kernel");

@@ -311,6 +311,9 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd && DV == 64 && LT 
     tc_fence_after();
     const uint32_t tb = *tmem_base_s;
     bool ok = true;
+    // A dependent launch: set up while the grid ahead drains (the forward beside the state's kernel, which has waited: at once)
+    if (MODE != kModeFwd || !p.overlapped) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     // descriptors: narrow tiles (64-byte rows, SWIZZLE_64B), wide tiles (128-byte rows, SWIZZLE_128B, 64-column blocks)
     constexpr uint64_t dN = make_smem_desc_base(16, 512, kSwizzle64B);                  // K-major, or MN-major one block
@@ -855,6 +858,7 @@ namespace {
 __global__ void __launch_bounds__(256)
     state_scan_kernel(const float* __restrict__ part, const float* __restrict__ zpart, __nv_bfloat16* __restrict__ st,
                       float* __restrict__ sv, int nblk, int per, int suffix) {
+    enter_dependent();
     const int e = blockIdx.x * 256 + threadIdx.x;
     const size_t h0 = (size_t)blockIdx.y * nblk;
     if (e < per) {
@@ -891,18 +895,12 @@ based_status launch_pass(const CUtensorMap& n0, const CUtensorMap& w0, const CUt
             configured[dev] = true;
         }
     }
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(kThreadsB);
-    cfg.dynamicSmemBytes = C::kSmem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = p.overlapped ? 1 : 0;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, backward_tc_kernel<DV, MODE, LT, XB>, n0, w0, n1, w1, st ? *st : n0,
-                                             outm ? *outm : w0, p);
+    // Dependent launches, but not the passes over the queries with more than a CTA per SM: theirs would double up on the SMs that the
+    // grid ahead leaves first (us per backward call, no pass dependent / dk/dv / all: B2 H16 L1000 d_v128 43.9 / 43.0 / 44.8, B8 H12
+    // L300 d_v64 18.7 / 18.8 / 19.3, B1 H8 L300 d_v128 18.8 / 17.8 / 17.0, B4 H16 L2048 d_v64, the keys' states too, 97.6 / 95.9 / 95.1)
+    const bool dependent = MODE == kModeFwd || MODE == kModeDkDv || grid.x <= kSMs;
+    const cudaError_t e = launch_ex(backward_tc_kernel<DV, MODE, LT, XB>, grid, dim3(kThreadsB), C::kSmem, 1, dependent, stream, n0, w0, n1,
+                                    w1, st ? *st : n0, outm ? *outm : w0, p);
     note_launch();
     const based_status s2 = check_launch(what);
     return e == cudaSuccess ? s2 : BASED_ERR_CUDA;
@@ -1023,9 +1021,11 @@ based_status launch_dvb(const void* q, const void* k, const void* v, const void*
             if (running) return launch_block_states_tc(x, val, sts, w.st, w.sv, nullptr, nullptr, BH, val_H, L, W, dvr, rev, stream);
             based_status s2 = launch_block_states_tc(x, val, sts, w.st, w.sv, w.part, w.zpart, BH, val_H, L, W, dvr, rev, stream);
             if (s2 != BASED_OK) return s2;
-            state_scan_kernel<<<dim3((160 * dvr + 255) / 256, BH), 256, 0, stream>>>(w.part, w.zpart, w.st, w.sv, nblk, 160 * dvr, rev);
+            const cudaError_t e = launch_ex(state_scan_kernel, dim3((160 * dvr + 255) / 256, BH), dim3(256), 0, 1, true, stream, w.part,
+                                            w.zpart, w.st, w.sv, nblk, 160 * dvr, rev);
             note_launch();
-            return check_launch("state_scan_kernel");
+            s2 = check_launch("state_scan_kernel");
+            return e == cudaSuccess ? s2 : BASED_ERR_CUDA;
         };
         // states of the keys: S = sum mono(k) v^T, z = sum mono(k), summed over the blocks before each block
         if ((st = states(k, v, nullptr, 0)) != BASED_OK) return st;

@@ -265,12 +265,13 @@ __device__ __forceinline__ void block_rows(uint32_t tb, uint32_t lane_base, cons
 // XB: the block-wise path (merged statistics + dq pass and dk/dv pass, d' = 16); tm_st: the block states,
 // transposed: [BH x nblk][d_v][160] bf16.  tm_out: the wide output (dv, or the forward output), stored by TMA.
 template <int DV, int MODE, int LT, bool XB>
-__global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd && DV == 64 && LT == 64 ? 4 : 2)
+__global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? 4 : 2)
     backward_tc_kernel(const __grid_constant__ CUtensorMap tm_n0, const __grid_constant__ CUtensorMap tm_w0,
                        const __grid_constant__ CUtensorMap tm_n1, const __grid_constant__ CUtensorMap tm_w1,
                        const __grid_constant__ CUtensorMap tm_st, const __grid_constant__ CUtensorMap tm_out,
                        const BParams p) {
     static_assert(!XB || MODE == kModeDqS || MODE == kModeDkDv, "block-wise path: the two passes that use it");
+    static_assert(MODE != kModeFwd || (DV == 64 && LT == 64), "the forward: d_v 64");
     using C = BCfg<DV, MODE, LT, XB>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -661,7 +662,7 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd && DV == 64 && LT 
                 uint32_t sr[32], gr[32];
                 // forward at d_v 64: the second sixteen columns are on their way while the first are worked on (38.3 -> 36.7 us at
                 // B4 H16 L2048 d' 24; at d_v 128, and in the other passes, no gain or 1 to 2 % slower)
-                constexpr bool kHalves = MODE == kModeFwd && DV == 64;
+                constexpr bool kHalves = MODE == kModeFwd;
                 uint32_t (&s0)[16] = *reinterpret_cast<uint32_t (*)[16]>(sr), (&s1)[16] = *reinterpret_cast<uint32_t (*)[16]>(sr + 16);
                 if (kHalves) tmem_ld16(tmem_addr(tb, lane_base, C::colS + blk * 32), s0);
                 else tmem_ld32(tmem_addr(tb, lane_base, C::colS + blk * 32), sr);
@@ -1069,11 +1070,14 @@ based_status launch_dvb(const void* q, const void* k, const void* v, const void*
 // kernel, which takes 16 us alone; the call 55 (one after the other, and both kernels slower, 80 + 61 before).
 based_status launch_quadratic_forward_tc(const void* q, const void* k, const void* v, void* out, int BH, int L,
                                          int d_feat, int d_v, int numerator_only, bool overlapped, cudaStream_t stream) {
-    // Two groups of row warps on one tile after the other (quadratic_fwd_tc.cu) where that is the faster, us, that / this at d' 24: d_v
-    // 128 B4 H16 L2048 49 / 59, L4096 164 / 216, but one key tile, L33, with 1 head 4.5 / 4.4, with 150 5.8 / 5.4, with 600 12.0 / 11.6; d_v
-    // 64 L2048 with 1 head 11.8 / 20.3, L1100 with 16 8.6 / 13.4, L200 5.0 / 5.9, L64 4.1 / 3.9, L2048 with 64 (1024 CTAs) 37.4 / 37.1,
-    // L8192 446 / 441; with the state beside it L128 with 64 9.3 / 8.5
-    if (d_v != 64 ? L > 64 : L > kTile && (long long)((L + kTile - 1) / kTile) * BH <= 2 * kSMs)
+    // Two groups of row warps on one tile after the other (quadratic_fwd_tc.cu) where that is the faster: at d_v 128 always, at d_v 64
+    // where its two CTAs per SM hold every tile, or few heads' long loops leave this kernel's four unfilled (us at d' 24, this / that:
+    // d_v 128 L16 with 1 head 4.5 / 3.6, with 1024 15.4 / 14.3, L64 16.5 / 15.7; d_v 64 with 64 heads L64 3.5 / 3.5, L128 4.3 / 3.9, with
+    // 148 4.9 / 4.2, with 400 7.1 / 8.5, L300 17.0 / 21.7, with 32 L1536 19.4 / 13.9, with 20 L2048 22.2 / 16.6, with 64 L1024 18.0 / 14.3,
+    // L1536 22.5 / 23.6, L4096 113 / 111).  One rule with the state beside it and without, so that the outputs are the same bits (with
+    // it, 64 heads L64 6.9 / 7.4, L128 8.2 / 7.9, L1024 20.4 / 21.4, 32 heads L1536 22.4 / 19.4).
+    const long long tiles = (long long)((L + kTile - 1) / kTile) * BH;
+    if (d_v != 64 || (L > 64 && tiles <= 2 * kSMs) || (L > 11 * kTile && tiles <= 4 * kSMs))
         return launch_quadratic_groups_tc(q, k, v, out, BH, L, d_feat, d_v, numerator_only, overlapped, stream);
     CUtensorMap tq, tk64, tv64, tout;
     const CUtensorMapSwizzle s64 = CU_TENSOR_MAP_SWIZZLE_64B, s128 = CU_TENSOR_MAP_SWIZZLE_128B;
@@ -1093,8 +1097,7 @@ based_status launch_quadratic_forward_tc(const void* q, const void* k, const voi
     const dim3 grid((unsigned)((L + kTile - 1) / kTile) * BH);
     p.heads = BH;
     p.by_length = long_loops_first(BH, L);
-    if (d_v == 64) return launch_pass<64, kModeFwd, 64>(tq, tq, tk64, tv64, p, grid, "quadratic forward (tc)", stream, nullptr, &tout);
-    return launch_pass<128, kModeFwd, 64>(tq, tq, tk64, tv64, p, grid, "quadratic forward (tc)", stream, nullptr, &tout);
+    return launch_pass<64, kModeFwd, 64>(tq, tq, tk64, tv64, p, grid, "quadratic forward (tc)", stream, nullptr, &tout);
 }
 
 int backward_tc_block_tokens(int BH, int L, int d_feat, int d_v, int merged) {

@@ -1571,10 +1571,10 @@ unsigned long long* g_trace = nullptr;
 // the stream has completed, namely once every CTA of that grid has signalled (griddepcontrol.launch_dependents) or
 // left; what they may touch before that grid is complete is the kernel's business (griddepcontrol.wait).  Behind a
 // kernel that never signals, such a launch behaves like a plain one.  Two uses.  The main pass behind a state pass
-// of the same call: every CTA of the state pass signals at its start, so the main pass's CTAs start as SMs come free
-// (they cannot take an SM that a CTA of the state pass still needs, all of those being resident or done by then),
-// and the one group that reads what the state pass wrote waits for its completion.  The recompute-mode kernel behind
-// whatever precedes the call: it waits right after its set-up.
+// of the same call: every CTA of the state pass signals when the grid ahead of it is complete, so the main pass's CTAs start as
+// SMs come free (they cannot take an SM that a CTA of the state pass still needs, all of those being resident or done by
+// then), and the one group that reads what the state pass wrote waits for its completion.  The recompute-mode kernel and
+// the state pass behind whatever precedes the call: they wait right after their set-up.
 template <int DV, int MODE, bool CONT = false>
 cudaError_t launch_dependent(dim3 grid, cudaStream_t stream, const CUtensorMap& tq, const CUtensorMap& tk,
                              const CUtensorMap& tv, const CUtensorMap& to, const Params& p) {
@@ -1991,8 +1991,32 @@ size_t prefill_tc_workspace_bytes(int BH, int L, int d_v) {
     return need;
 }
 
+// Heads left over after whole waves of one CTA per SM, where they are better off in a launch of their own, in segments (recompute
+// mode, no scratch), than one CTA each in a wave that leaves most SMs idle; else 0.  From sixteen chunks on wherever they get two
+// segments (d_v 128: three); below, the second launch's set-up and tail weigh as much as the idle wave unless that wave is the second of
+// two (us, one launch / two, outputs alone: d_v 64 L4096 150 heads 82.9 / 72.3, 208 84.9 / 80.7, L2048 160 heads 46.1 / 41.9, 224, not
+// taken, 48.5 / 50.3, 320 69.8 / 66.7, L1024 150 26.9 / 25.3, 208, not taken, 28.5 / 28.3, L300 192 15.6 / 14.7; d_v 128 L4096 160 heads
+// 128 / 118, L2048 160 69.4 / 66.3, 208, not taken, 71.5 / 72.4, L1024 192, not taken, 45.6 / 46.8 with a new state, L512 160 23.3 / 21.6,
+// 300, not taken, 35.1 / 34.7).  Not continued calls: L2048 d_v 64 160 heads 57.5 / 59.8, the caller's state being read by every segment.
+static int heads_in_segments(int BH, int L, int d_v) {
+    const int nch = (L + kC - 1) / kC, rest = BH % kSMs;
+    if (BH < kSMs || 2 * rest > kSMs || nch < 2) return 0;
+    if (nch >= 16) return (d_v == 64 ? 2 : 3) * rest <= kSMs ? rest : 0;
+    if (BH >= 2 * kSMs) return 0;
+    return nch <= 4 || (d_v == 64 && 3 * rest <= kSMs) ? rest : 0;
+}
+
 based_status launch_prefill_tc(const void* q, const void* k, const void* v, void* out, float* kv, float* z, int BH,
                                int L, int d_v, int flags, void* workspace, cudaStream_t stream, size_t workspace_limit) {
+    if (const int rest = (flags & BASED_STATE_CONTINUE) ? 0 : heads_in_segments(BH, L, d_v)) {
+        const based_status st =
+            launch_prefill_tc(q, k, v, out, kv, z, BH - rest, L, d_v, flags, workspace, stream, workspace_limit);
+        if (st != BASED_OK) return st;
+        const size_t tokens = (size_t)(BH - rest) * L, rows = (size_t)(BH - rest) * ((flags & BASED_STATE_SYM) ? kDSym : kD);
+        auto from = [](auto* p, size_t elements) { return reinterpret_cast<decltype(p)>(reinterpret_cast<uintptr_t>(p) + 2 * elements); };
+        return launch_prefill_tc(from(q, tokens * kDFeat), from(k, tokens * kDFeat), from(v, tokens * d_v), from(out, tokens * d_v),
+                                 kv ? kv + rows * d_v : nullptr, z ? z + rows : nullptr, rest, L, d_v, flags, nullptr, stream, 0);
+    }
     const SegPlan plan = prefill_tc_plan(BH, L, d_v == 112 ? 128 : d_v, (flags & BASED_STATE_CONTINUE) != 0,
                                          workspace ? workspace_limit : 0);
     float* ws = static_cast<float*>(workspace);

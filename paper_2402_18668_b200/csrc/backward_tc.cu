@@ -285,8 +285,18 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? 4 : 2)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int ntiles = (p.L + kTile - 1) / kTile;
     // own tile: the longest loops first (dq, statistics: last query tiles; dk/dv: first key tiles)
-    const int turn = p.by_length ? blockIdx.x / p.heads : blockIdx.x % ntiles;
-    const int head = p.by_length ? blockIdx.x - turn * p.heads : blockIdx.x / ntiles;
+    int turn = p.by_length ? blockIdx.x / p.heads : blockIdx.x % ntiles;
+    int head = p.by_length ? blockIdx.x - turn * p.heads : blockIdx.x / ntiles;
+    if (XB) {
+        // First the tiles that need no block state, all heads': they run beside the states' kernel, on what it leaves of the chip
+        // (us per backward call, after it / beside it: B4 H16 L2048 d_v64 96.2 / 93.0, d_v128 130.1 / 124.5, L4096 245.4 / 238.4, B8 H16
+        // L1024 d_v64 87.1 / 85.7, B4 H8 L2048 67.2 / 66.5; the states' kernel held to the registers that leave room for one of these
+        // CTAs on its own SMs too, at d_v 64: 95.0)
+        const int alone = MODE == kModeDkDv ? ntiles - (p.nblk - 1) * (p.W / kTile) : p.W / kTile, rest = ntiles - alone;
+        const int i = (int)blockIdx.x - p.heads * alone;
+        head = i < 0 ? blockIdx.x / alone : i / rest;
+        turn = i < 0 ? rest + blockIdx.x % alone : i % rest;
+    }
     const int own = MODE == kModeDkDv ? turn : ntiles - 1 - turn;
     const int r0 = own * kTile;
     // looped tiles (LT rows each): keys 0 .. end of the own tile, or queries from the own tile's first row on
@@ -312,8 +322,9 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? 4 : 2)
     tc_fence_after();
     const uint32_t tb = *tmem_base_s;
     bool ok = true;
-    // A dependent launch: set up while the grid ahead drains (the forward beside the state's kernel, which has waited: at once)
-    if (MODE != kModeFwd || !p.overlapped) asm volatile("griddepcontrol.wait;" ::: "memory");
+    // A dependent launch: set up while the grid ahead drains.  Behind a kernel of states, which has waited for everything before it,
+    // the forward and the tiles that need no state start at once.
+    if (MODE == kModeFwd ? !p.overlapped : !XB || cross) asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     // descriptors: narrow tiles (64-byte rows, SWIZZLE_64B), wide tiles (128-byte rows, SWIZZLE_128B, 64-column blocks)
@@ -660,7 +671,7 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? 4 : 2)
             auto pass = [&](auto masked_tag, int blk) {
                 constexpr bool MASKED = decltype(masked_tag)::value;
                 uint32_t sr[32], gr[32];
-                // forward at d_v 64: the second sixteen columns are on their way while the first are worked on (38.3 -> 36.7 us at
+                // forward (d_v 64): the second sixteen columns are on their way while the first are worked on (38.3 -> 36.7 us at
                 // B4 H16 L2048 d' 24; at d_v 128, and in the other passes, no gain or 1 to 2 % slower)
                 constexpr bool kHalves = MODE == kModeFwd;
                 uint32_t (&s0)[16] = *reinterpret_cast<uint32_t (*)[16]>(sr), (&s1)[16] = *reinterpret_cast<uint32_t (*)[16]>(sr + 16);
@@ -896,10 +907,10 @@ based_status launch_pass(const CUtensorMap& n0, const CUtensorMap& w0, const CUt
             configured[dev] = true;
         }
     }
-    // Dependent launches, but not the passes over the queries with more than a CTA per SM: theirs would double up on the SMs that the
-    // grid ahead leaves first (us per backward call, no pass dependent / dk/dv / all: B2 H16 L1000 d_v128 43.9 / 43.0 / 44.8, B8 H12
-    // L300 d_v64 18.7 / 18.8 / 19.3, B1 H8 L300 d_v128 18.8 / 17.8 / 17.0, B4 H16 L2048 d_v64, the keys' states too, 97.6 / 95.9 / 95.1)
-    const bool dependent = MODE == kModeFwd || MODE == kModeDkDv || grid.x <= kSMs;
+    // Dependent launches, but not the tile path's passes over the queries with more than a CTA per SM: theirs would double up on the SMs
+    // that the grid ahead leaves first (us per backward call, no pass dependent / dk/dv / all: B2 H16 L1000 d_v128 43.9 / 43.0 / 44.8, B8
+    // H12 L300 d_v64 18.7 / 18.8 / 19.3, B1 H8 L300 d_v128 18.8 / 17.8 / 17.0, B4 H16 L2048 d_v64, the keys' states too, 97.6 / 95.9 / 95.1)
+    const bool dependent = MODE == kModeFwd || MODE == kModeDkDv || XB || grid.x <= kSMs;
     const cudaError_t e = launch_ex(backward_tc_kernel<DV, MODE, LT, XB>, grid, dim3(kThreadsB), C::kSmem, 1, dependent, stream, n0, w0, n1,
                                     w1, st ? *st : n0, outm ? *outm : w0, p);
     note_launch();
@@ -1062,8 +1073,8 @@ based_status launch_dvb(const void* q, const void* k, const void* v, const void*
 }
 }  // namespace
 
-// Forward of the definition form on the same tiles, for feature dimensions other than 16 (bf16 io,
-// empty initial state): out = (sum_j w_ij v_j) / (sum_j w_ij + eps), w = 1 + s/sqrt(d') + s^2/(2 d').
+// Forward of the definition form, for feature dimensions other than 16 and one chunk of d' 16 (bf16 io,
+// empty initial state); on the same tiles: out = (sum_j w_ij v_j) / (sum_j w_ij + eps), w = 1 + s/sqrt(d') + s^2/(2 d').
 // The weights lie over the scores, so at d_v 64 a CTA takes 128 columns of tensor memory and four share an SM, and tiles off
 // the diagonal evaluate two pairs per instruction: B4 H16 L2048 d_v64 80 -> 48 us (looped tiles of 128 rows: 47), 38 with the
 // longest loops first (36.7 with the scores' second half loaded ahead).  With the state asked for it is launched beside that

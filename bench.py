@@ -52,7 +52,7 @@ NCU_TRAFFIC = {
     "cfg3_1p3b_prefill": 167.85e6 + 102.19e6,     # profiles/prefill_tc_kernel_dv128.md (part of the output still in L2)
     "cfg4_generation": 2 * (144.59e6 + 88.45e6),  # profiles/decode_step_kernel_dv128.md, 1024 -> 2048 heads
     "cfg5_mixer_pair:swa": 2 * (201.37e6 + 43.87e6),  # profiles/swa_tc_kernel.md, 16 -> 32 heads
-    "baseconv": 4 * (272.67e6 + 96.72e6),         # profiles/baseconv_gate_kernel.md, batch 2 -> 8 (part of the writes still in L2)
+    "baseconv": 4 * (268.59e6 + 84.15e6),         # profiles/baseconv_block_kernel.md, batch 2 -> 8 (part of the writes still in L2)
     "swa_decode": 34.36e6,                        # profiles/swa_decode_kernel.md (full size; writes stay in L2)
 }
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
@@ -500,8 +500,8 @@ def bench_swa_decode(w, steps, warmup, torch, based, dist_on, peaks):
 def bench_generation_graph(w, steps, warmup, torch, based, dist_on, peaks):
     """One generated token through the mixer pair at the generation configuration's batch: the
     linear-attention decode step on the 153-row symmetric state plus the window-64 decode step on
-    its rolling cache, captured once as a CUDA graph (paper_2402_18668_b200.generation.DecodeGraph)
-    and replayed per token.  The state (321 MB) is larger than L2; the caches (34 MB) are not, as
+    its rolling cache, set up once (paper_2402_18668_b200.generation.DecodeGraph) and launched
+    per token.  The state (321 MB) is larger than L2; the caches (34 MB) are not, as
     in a real generation loop."""
     from paper_2402_18668_b200.generation import DecodeGraph
     g = torch.Generator(device="cuda").manual_seed(4)
@@ -523,7 +523,7 @@ def bench_generation_graph(w, steps, warmup, torch, based, dist_on, peaks):
     bytes_step = 2.0 * w.B * w.H * based.D_SYM * w.d_v * 4 + 2.0 * w.B * w.H * win * d * esz
     return {
         "workload": f"B{w.B} H{w.H}: decode step on the 153-row state (d_v {w.d_v}) + window-{win} decode step, "
-                    "one fused launch (based_generation_step) replayed as a CUDA graph per token",
+                    "one fused launch (based_generation_step) per token from kept arguments",
         "metric": "generation_tokens_per_s", "value": w.B / t, "unit": "tokens/s", "us_per_token_step": t * 1e6,
         "steps": steps, "kernels_per_replay": 1 if graph.fused else 2,
         "roofline": {"bound": "hbm", "achieved": bytes_step / t / 1e9, "peak": peaks["hbm_gbs"], "unit": "GB/s",
@@ -557,7 +557,7 @@ def bench_baseconv(shape, steps, warmup, torch, based, dist_on, peaks):
         "unit": "tokens/s", "ms_per_step": t * 1e3, "steps": steps, "buffer_sets": n,
         "roofline": {"bound": "hbm", "achieved": per_set / t / 1e9, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                      "frac": per_set / t / 1e9 / peaks["hbm_gbs"], "traffic": NCU_TRAFFIC.get("baseconv"),
-                     "kernel": "baseconv_gate_kernel", "algorithmic_bytes": per_set, "peak_source": peaks["source"]},
+                     "kernel": "baseconv_block_kernel", "algorithmic_bytes": per_set, "peak_source": peaks["source"]},
     }
 
 

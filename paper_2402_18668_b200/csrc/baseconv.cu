@@ -311,7 +311,7 @@ based_status launch_baseconv(const void* a, const void* g, const float* h, const
     if (io == BASED_F32) launch_t<float>(a, g, h, b2, state, out, B, N, C, width, step, stream);
     else launch_t<__nv_bfloat16>(a, g, h, b2, state, out, B, N, C, width, step, stream);
     note_launch();
-    return check_launch(step ? "baseconv_step_kernel" : "baseconv_gate_kernel");
+    return check_launch(step ? "baseconv_step_kernel" : "baseconv_block_kernel");
 }
 
 }  // namespace based

@@ -1,5 +1,5 @@
 // Forward of the definition form (left-hand side of Eq. (2) of Sec. 4.1) on the tensor cores, bf16 io, empty initial state, for the
-// feature dimensions 8, 24 and 32, which the chunked d' = 16 kernel does not cover:
+// feature dimensions 8, 24 and 32, which the chunked d' = 16 kernel does not cover, and for one chunk of d' = 16 without a state:
 //   out = (sum_j w_ij v_j) / (sum_j w_ij + eps),  w = 1 + s/sqrt(d') + s^2/(2 d'),  s = q_i . k_j.
 //
 // One CTA per (head, 128 queries), looping over tiles of 64 keys: S = Q K^T to tensor memory, the rows' threads turn it into weights
@@ -7,7 +7,7 @@
 // CTAs per SM: two groups of four row warps that take the key tiles in turn, one warp each for the scores' MMAs, the products'
 // MMAs and the loads.  Three sets of score columns (two at d_v 128): the scores of the next tiles are there when a group comes
 // for them, so that what a row warp waits for is its own arithmetic.  Against one group and one set of scores per CTA and four (d_v
-// 128: two) CTAs per SM (backward_tc.cu, kModeFwd): at d_v 128, where a second set was missing most, 59 -> 49 us at d' 32 B4 H16
+// 128, then: two) CTAs per SM (backward_tc.cu, kModeFwd): at d_v 128, where a second set was missing most, 59 -> 49 us at d' 32 B4 H16
 // L2048 and 216 -> 164 at d' 24 L4096; with a head alone 20 -> 12 (L2048 d_v 64).  At d_v 64 with every SM busy the two are the same:
 // half of the issue slots are used, 1075 warp instructions per tile of 128 x 64 pairs.  A row warp loads sixteen score columns ahead
 // of the ones it works on: d_v 128 d' 24 47.8 -> 46.9, 64 heads L777 16.7 -> 16.2.  What bounds it is no single part (64 heads L8192 d_v

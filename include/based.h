@@ -252,7 +252,7 @@ size_t based_prefill_backward_workspace_bytes(int B, int H, int L, int d_v, base
  * only: D_i and dout_i . N_i are still recomputed in fp32.  fp32 io ignores out's values.
  * out must not alias a gradient output.
  *
- * Block-wise path (bf16 io, d_feat = 16; L >= 768 at d_v 64, L >= 1024 to 1536 at d_v 112 / 128): O(L) per
+ * Block-wise path (bf16 io, d_feat = 16; L >= 768 to 1025 at d_v 64, L >= 1024 to 1536 at d_v 112 / 128): O(L) per
  * head, the recurrent view of Sec. 4.1 applied to the gradients.  The sequence is cut into blocks of
  * W = 256 tokens (512 for long sequences of few heads at d_v 128).  Pairs inside a block go through
  * the tiles above.  All earlier blocks reach a query through their summed state S = sum_j phi(k_j) v_j^T, z = sum_j phi(k_j):

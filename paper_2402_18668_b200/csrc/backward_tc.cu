@@ -925,8 +925,10 @@ based_status launch_pass(const CUtensorMap& n0, const CUtensorMap& w0, const CUt
 //   64 heads: d_v 64 L 768 34 / 47, L 1024 52 / 54, L 1280 73 / 66; d_v 128 L 768 50 / 59, L 1024 74 / 72
 //   16 heads: d_v 64 L 768 29 / 36, L 1024 36 / 37, L 1536 51 / 42; d_v 128 L 1280 46 / 52, L 1536 53 / 54, L 2048 70 / 55
 //   32 heads: d_v 64 L 1280 46 / 61, L 1536 56 / 66, L 2048 82 / 70; d_v 128 L 1536 74 / 91, L 2048 112 / 101
-// The line at L 768 (d_v 64) is older than these figures, which put the crossing between 768 and 1024 at 128 heads, at 1024
-// at 16 and between 1024 and 1280 at 64: from 768 up to there the tile path would be 2 to 13 us faster.
+// And, since both paths' passes are dependent launches, at d_v 64: 64 heads L 768 32 / 48, L 800 41 / 48 (blocks there all the same),
+// 80 L 768 43 / 49, 128 62 / 66, L 769 74.4 / 74.1, L 897 93 / 83; 8 heads L 769 28 / 34, L 1024 34 / 35, L 1025 36 / 35; 16 29 / 36, 34 / 35,
+// 36 / 36; 24 30 / 36, 36 / 37, 38 / 37; 32 L 769 32 / 38, L 897 37.4 / 37.8, L 1024 39.2 / 37.9; 2 (where the line stays) L 768 26 / 28, L 769
+// 28.0 / 28.8, L 897 31 / 29.  The tile path is also the more precise (2.3e-3 against 2.4e-3 of fp64 gradients), so no line moves below where it was.
 // Below 64 heads one CTA per head and block sums the states, and a second short wave of those costs as much as a full one:
 // there the line lies later once the blocks are more than one wave (24 heads are not at L 1536: 54 / 44, 60 / 56).
 // With them at d_v 128 blocks of 512 tokens are the faster from 64 k rows on (256 / 512 tokens: 16 heads L 8192 217 / 206,
@@ -938,9 +940,9 @@ based_status launch_pass(const CUtensorMap& n0, const CUtensorMap& w0, const CUt
 int backward_block_len(int L, int df, bool merged, int d_v, int BH) {
     if (df != 16) return 0;
     int from;
-    if (BH >= 64) from = !merged ? 1280 : d_v == 64 ? 768 : 1024;
+    if (BH >= 64) from = !merged ? 1280 : d_v == 64 ? 769 : 1024;
     else if (BH * ((L + 255) / 256) > kSMs) from = 2048;
-    else from = d_v == 64 ? (merged ? 768 : 1024) : 1536;
+    else from = d_v != 64 ? 1536 : !merged ? 1024 : BH <= 4 ? 768 : BH < 32 ? 1025 : 897;
     if (L < from) return 0;
     return BH < 64 && d_v != 64 && L >= 4096 && (long long)BH * L >= 65536 ? 512 : 256;
 }

@@ -32,3 +32,19 @@ def test_tiles_beside_the_states(d_v, BH, L, flags):
         assert (np.abs(a - b).max(axis=(0, 2, 3)) <= TOL_BF16 * np.abs(b).max(axis=(0, 2, 3))).all()
     assert all(torch.equal(a, b) for r in runs[1:] for a, b in zip(r, runs[0]))
     assert based.based_poll_error() == based.BASED_OK
+
+
+@pytest.mark.parametrize("BH,L,block", [(64, 768, 0), (64, 769, 256), (16, 1024, 0), (16, 1025, 256), (3, 767, 0), (3, 768, 256), (33, 896, 0),
+                                        (33, 897, 256)])
+def test_lines_between_the_paths(BH, L, block):
+    assert based.binding.lib().based_prefill_backward_block_tokens(1, BH, L, 16, 64, based.BASED_BF16, 0, 1) == block
+    gen = wl.generator(BH * 1000 + L)
+    w = wl.Workload("lines", 1, BH, L, 16, 64, "bf16", 0.5)
+    q, k, v = wl.prefill_inputs(w, gen)
+    g = torch.randn(1, BH, L, 64, generator=gen).bfloat16()
+    heads = sorted({0, BH - 1})
+    want = oracle.linattn_backward(*(wl.to_f64(t[:, heads]) for t in (q, k, v, g)))
+    x = [t.cuda() for t in (q, k, v, g)]
+    for a, b in zip(based.based_prefill_backward(*x, out=based.based_prefill(*x[:3])), want):
+        a = wl.to_f64(a[:, heads])
+        assert (np.abs(a - b).max(axis=(0, 2, 3)) <= TOL_BF16 * np.abs(b).max(axis=(0, 2, 3))).all()

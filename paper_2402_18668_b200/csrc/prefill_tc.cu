@@ -506,10 +506,11 @@ template <int DV>
 __device__ __forceinline__ void write_state(float* kv, float* z, int dv, const short2* s_abi, uint32_t tb, int part, float* stage) {
     using C = Cfg<DV>;
     constexpr int kQ = DV / 4, kPer = 128 / kQ;                      // 16-byte words of a row, rows per pass
-    // (read afresh: the kernel's own copy would have to live through the role loops; us, that / this, outputs alone: B1 H2
-    // L3000 20.0 / 19.4, H100 L1024 15.5 / 15.1, B4 H16 L2048 19.6 / 19.4, H200 L700 23.5 / 22.9, with a new state 26.2 / 25.8)
-    int tx;
-    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tx));
+    // (d_v 64: read afresh, the kernel's own copy would have to live through the role loops; us, that / this, outputs alone: B1 H2
+    // L3000 20.0 / 19.4, H100 L1024 15.5 / 15.1, B4 H16 L2048 19.6 / 19.4, H200 L700 23.5 / 22.9, with a new state 26.2 / 25.8.  At d_v 128
+    // the loops come out better with the copy: B3 H16 L777 d_v112 continued 18.2 / 18.4, B8 H16 L4096 71.4 / 72.0)
+    int tx = threadIdx.x;
+    if (DV == 64) asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tx));
     const int warp = tx >> 5, lane = tx & 31, tid = tx & 127;
     const uint32_t lane_base = (uint32_t)(warp & 3) * 32u;
     const int t = ((warp & 3) << 5) + lane;                              // lane of S^T

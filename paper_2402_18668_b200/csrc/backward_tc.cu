@@ -1118,7 +1118,8 @@ int backward_tc_block_tokens(int BH, int L, int d_feat, int d_v, int merged) {
 }
 
 size_t backward_tc_workspace_bytes(int BH, int L, int d_v) {
-    const int W = backward_block_len(L, 16, true, d_v, BH);
+    // with the forward output or without: neither line lies below the other everywhere (5 to 31 heads, d_v 64: 1025 with, 1024 without)
+    const int with = backward_block_len(L, 16, true, d_v, BH), W = with ? with : backward_block_len(L, 16, false, d_v, BH);
     if (W > 0) return block_ws(nullptr, BH, L, d_v, (L + W - 1) / W).bytes;         // statistics, block states
     return (size_t)BH * L * 2 * sizeof(float);                 // (1 / D, b) per row
 }

@@ -283,6 +283,10 @@ static void launch_w(const void* a, const void* g, const float* h, const float* 
             constexpr int TOK = decltype(tok_tag)::value;
             constexpr bool FLAT = decltype(flat_tag)::value;
             const unsigned rows = (N + TOK - 1) / TOK;
+            // (behind a kernel that left the SM to shared memory, us without / with the preference, B8 N1024 C8192 59 alone: behind the
+            // sliding window 102 / 62, a prefill 89 / 59; B8 N4096 227 alone: 385 / 230, 343 / 226; B1 N512 4.8 alone: 8.3 / 5.4, 6.9 / 5.5)
+            static std::atomic<bool> split_block[64];
+            prefer_l1(baseconv_block_kernel<T, W, TOK, FLAT>, 0, split_block);
             launch_ex(baseconv_block_kernel<T, W, TOK, FLAT>, FLAT ? dim3(gb * rows, B) : dim3(gb, rows, B), dim3(kThreadsBlock), 0, 1, true, stream,
                       static_cast<const T*>(a), static_cast<const T*>(g), h, b2, static_cast<T*>(out), N, C, gb);
         };

@@ -152,7 +152,7 @@ static based_status prefill_impl(const void* q, const void* k, const void* v, vo
         if (!workspace) workspace_bytes = 0;
     }
     // One chunk and no state to write: the chunk's pairs are all there is, and the definition form's kernels, the same sums of the same
-    // bf16 weights, have less to set up (us, chunked / this: d_v 64, 16 heads L64 4.8 / 3.4, L128 5.7 / 3.8, 200 heads L64 10.6 / 4.0;
+    // bf16 weights in the same order (the outputs are the bits that a call with a state gives), have less to set up (us, chunked / this: d_v 64, 16 heads L64 4.8 / 3.4, L128 5.7 / 3.8, 200 heads L64 10.6 / 4.0;
     // d_v 128, 16 heads L64 5.9 / 3.8, 400 heads L128 23 / 9).  Longer calls would be faster so up to L 1500 with 16 heads (L1024 10.2 /
     // 7.2), but the chunked form holds what is before the chunk more precisely (2.25e-3 against 2.29e-3 of 64-bit results).
     if (io == BASED_BF16 && !kv_state && L <= 128)

@@ -82,7 +82,10 @@ __device__ __forceinline__ bool all_rows(bool pred) {
 }
 }  // namespace
 
-template <int DV>
+// IN_ORDER: one chunk of d' 16.  The first group takes both key tiles, and a row's weights are summed as the chunked kernel sums them
+// (the even columns, the odd ones, then both; so does kModeFwd), so that the outputs are the bits that the chunked kernel gives beside a
+// state (us, both groups / this: L128, 16 heads d_v 64 3.24 / 3.36, d_v 128 3.72 / 3.82, 200 heads d_v 128 5.18 / 5.01, 400 8.34 / 8.43).
+template <int DV, bool IN_ORDER>
 __global__ void __launch_bounds__(kThreadsQ, 2)
     quadratic_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                             const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_out, const FParams p) {
@@ -208,7 +211,8 @@ __global__ void __launch_bounds__(kThreadsQ, 2)
                     halves_of(x, lo, hi);
                     x = pair_of_f(col <= row ? lo : 0.f, col + 1 <= row ? hi : 0.f);
                 }
-                den2[i & 1] = add_pairs(den2[i & 1], x);
+                uint64_t& den = den2[IN_ORDER ? 0 : i & 1];
+                den = add_pairs(den, x);
                 halves_of(x, lo, hi);
                 w[w0 + i] = pack2(lo, hi);
             }
@@ -220,7 +224,7 @@ __global__ void __launch_bounds__(kThreadsQ, 2)
             for (int i = 0; i < 16; ++i) asm volatile("" : "+r"(r[i]));
         };
         uint32_t s0[16], s1[16], w[16];
-        for (int t = wg; t < n; t += 2) {
+        for (int t = !IN_ORDER ? wg : wg == 0 ? 0 : n; t < n; t += IN_ORDER ? 1 : 2) {
             const int si = t % C::kNSet;
             const uint32_t set = tmem_addr(tb, lane_base, si * kLTQ);
             ok = __all_sync(~0u, mbar_wait(&bars[qScore + si], (t / C::kNSet) & 1, abort_flag));
@@ -307,7 +311,7 @@ __global__ void __launch_bounds__(kThreadsQ, 2)
 }
 
 namespace {
-template <int DV>
+template <int DV, bool IN_ORDER>
 based_status launch_forward(const CUtensorMap& q, const CUtensorMap& k, const CUtensorMap& v, const CUtensorMap& out, const FParams& p,
                             unsigned grid, cudaStream_t stream) {
     using C = FCfg<DV>;
@@ -317,12 +321,12 @@ based_status launch_forward(const CUtensorMap& q, const CUtensorMap& k, const CU
         if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return BASED_ERR_CUDA;
         std::lock_guard<std::mutex> lock(setup_mutex());
         if (!configured[dev]) {
-            if (cudaFuncSetAttribute(quadratic_fwd_tc_kernel<DV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::kSmem) != cudaSuccess)
+            if (cudaFuncSetAttribute(quadratic_fwd_tc_kernel<DV, IN_ORDER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::kSmem) != cudaSuccess)
                 return BASED_ERR_CUDA;
             configured[dev] = true;
         }
     }
-    const cudaError_t e = launch_ex(quadratic_fwd_tc_kernel<DV>, dim3(grid), dim3(kThreadsQ), C::kSmem, 1, true, stream, q, k, v,
+    const cudaError_t e = launch_ex(quadratic_fwd_tc_kernel<DV, IN_ORDER>, dim3(grid), dim3(kThreadsQ), C::kSmem, 1, true, stream, q, k, v,
                                     out, p);
     note_launch();
     const based_status st = check_launch("quadratic_fwd_tc_kernel");
@@ -349,7 +353,9 @@ based_status launch_quadratic_groups_tc(const void* q, const void* k, const void
     p.overlapped = overlapped;
     const long long ctas = (long long)((L + kOwnQ - 1) / kOwnQ) * BH;
     p.by_length = ctas > kSMs;
-    return d_v == 64 ? launch_forward<64>(tq, tk, tv, to, p, (unsigned)ctas, stream) : launch_forward<128>(tq, tk, tv, to, p, (unsigned)ctas, stream);
+    const bool in_order = d_feat == kDFeat;
+    if (d_v == 64) return in_order ? launch_forward<64, true>(tq, tk, tv, to, p, (unsigned)ctas, stream) : launch_forward<64, false>(tq, tk, tv, to, p, (unsigned)ctas, stream);
+    return in_order ? launch_forward<128, true>(tq, tk, tv, to, p, (unsigned)ctas, stream) : launch_forward<128, false>(tq, tk, tv, to, p, (unsigned)ctas, stream);
 }
 
 }  // namespace based

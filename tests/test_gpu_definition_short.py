@@ -34,6 +34,20 @@ def test_one_chunk(d_v, BH, L, flags):
     assert based.based_poll_error() == based.BASED_OK
 
 
+@pytest.mark.parametrize("d_v", [64, 112, 128])
+@pytest.mark.parametrize("BH", [1, 16, 296, 297, 700])
+@pytest.mark.parametrize("flags", [0, based.BASED_NUMERATOR_ONLY])
+def test_one_chunk_same_bits_beside_a_state(d_v, BH, flags):
+    """The outputs do not depend on whether the state is asked for (up to L 128 another kernel gives them then)."""
+    for L in (1, 17, 32, 33, 64, 65, 97, 100, 127, 128, 129):
+        gen = torch.Generator(device="cuda").manual_seed(BH * 1000 + L)
+        q, k = (torch.randn(1, BH, L, 16, generator=gen, device="cuda").mul(0.5).bfloat16() for _ in range(2))
+        v = torch.randn(1, BH, L, d_v, generator=gen, device="cuda").bfloat16()
+        kv, z = based.new_state(1, BH, d_v)
+        assert torch.equal(based.based_prefill(q, k, v, flags=flags), based.based_prefill(q, k, v, kv_state=kv, z_state=z, flags=flags)), L
+    assert based.based_poll_error() == based.BASED_OK
+
+
 @pytest.mark.parametrize("BH,L", [(64, 64), (64, 65), (296, 100), (297, 100), (37, 1024), (38, 1024), (49, 1408), (49, 1409), (50, 1409),
                                   (5, 4096)])
 def test_lines_between_the_kernels(BH, L):

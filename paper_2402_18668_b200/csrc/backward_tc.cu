@@ -53,6 +53,9 @@ namespace {
 constexpr int kTile = 128;
 constexpr int kThreadsB = 160;
 constexpr int kModeStats = 0, kModeDq = 1, kModeDkDv = 2, kModeFwd = 3, kModeDqS = 4;
+// the forward with the rounded weights' sums, for one chunk of d' 16, which gives the bits of prefill_tc_kernel's ROUNDED
+constexpr int kModeFwdRounded = 5;
+__host__ __device__ constexpr int base_mode(int mode) { return mode == kModeFwdRounded ? kModeFwd : mode; }
 constexpr uint32_t kQKTile = kTile * 64;                 // [128][32] bf16, 64-byte rows, SWIZZLE_64B
 
 // LT: rows of the tiles the CTA loops over (columns of the accumulators): 64 where that lets two CTAs
@@ -264,12 +267,13 @@ __device__ __forceinline__ void block_rows(uint32_t tb, uint32_t lane_base, cons
 // tm_n1 / tm_w1: of the tiles it loops over.
 // XB: the block-wise path (merged statistics + dq pass and dk/dv pass, d' = 16); tm_st: the block states,
 // transposed: [BH x nblk][d_v][160] bf16.  tm_out: the wide output (dv, or the forward output), stored by TMA.
-template <int DV, int MODE, int LT, bool XB>
-__global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? 4 : 2)
+template <int DV, int KIND, int LT, bool XB>
+__global__ void __launch_bounds__(kThreadsB, base_mode(KIND) == kModeFwd ? 4 : 2)
     backward_tc_kernel(const __grid_constant__ CUtensorMap tm_n0, const __grid_constant__ CUtensorMap tm_w0,
                        const __grid_constant__ CUtensorMap tm_n1, const __grid_constant__ CUtensorMap tm_w1,
                        const __grid_constant__ CUtensorMap tm_st, const __grid_constant__ CUtensorMap tm_out,
                        const BParams p) {
+    constexpr int MODE = base_mode(KIND);
     static_assert(!XB || MODE == kModeDqS || MODE == kModeDkDv, "block-wise path: the two passes that use it");
     static_assert(MODE != kModeFwd || (DV == 64 && LT == 64), "the forward: d_v 64");
     using C = BCfg<DV, MODE, LT, XB>;
@@ -705,7 +709,7 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? 4 : 2)
                     if (MODE != kModeDq) w = masked(fma_f32x2(sv, fma_f32x2(sv, k2, k1), one));
                     if (MODE == kModeDq || MODE == kModeDqS || MODE == kModeDkDv) dw = fma_f32x2(sv, k22, k1);
                     if (MODE == kModeDqS) dw = masked(dw);
-                    if (MODE == kModeFwd || MODE == kModeStats || MODE == kModeDqS) den2 = add_f32x2(den2, w);
+                    if ((MODE == kModeFwd && KIND != kModeFwdRounded) || MODE == kModeStats || MODE == kModeDqS) den2 = add_f32x2(den2, w);
                     if (MODE == kModeStats || MODE == kModeDqS) en2 = fma_f32x2(w, gv, en2);
                     if (MODE == kModeDqS) {
                         ds = mul_f32x2(dw, add_f32x2(gv, negm));             // first tile: w' (gv - m); second: w'
@@ -722,6 +726,7 @@ __global__ void __launch_bounds__(kThreadsB, MODE == kModeFwd ? 4 : 2)
                     float lo, hi;
                     split_f32x2(w, lo, hi);
                     pw[i] = pack_bf16x2(lo, hi);
+                    if (KIND == kModeFwdRounded) den2 = add_f32x2(den2, f32x2(__uint_as_float(pw[i] << 16), __uint_as_float(pw[i] & 0xffff0000u)));
                     split_f32x2(ds, lo, hi);
                     pd[i] = pack_bf16x2(lo, hi);
                 }
@@ -890,10 +895,11 @@ __global__ void __launch_bounds__(256)
         }
     }
 }
-template <int DV, int MODE, int LT, bool XB = false>
+template <int DV, int KIND, int LT, bool XB = false>
 based_status launch_pass(const CUtensorMap& n0, const CUtensorMap& w0, const CUtensorMap& n1, const CUtensorMap& w1,
                          const BParams& p, dim3 grid, const char* what, cudaStream_t stream,
                          const CUtensorMap* st = nullptr, const CUtensorMap* outm = nullptr) {
+    constexpr int MODE = base_mode(KIND);
     using C = BCfg<DV, MODE, LT, XB>;
     static bool configured[64] = {};
     int dev = 0;
@@ -901,7 +907,7 @@ based_status launch_pass(const CUtensorMap& n0, const CUtensorMap& w0, const CUt
     {
         std::lock_guard<std::mutex> lock(setup_mutex());
         if (!configured[dev]) {
-            if (cudaFuncSetAttribute(backward_tc_kernel<DV, MODE, LT, XB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            if (cudaFuncSetAttribute(backward_tc_kernel<DV, KIND, LT, XB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)C::kSmem) != cudaSuccess)
                 return BASED_ERR_CUDA;
             configured[dev] = true;
@@ -911,7 +917,7 @@ based_status launch_pass(const CUtensorMap& n0, const CUtensorMap& w0, const CUt
     // that the grid ahead leaves first (us per backward call, no pass dependent / dk/dv / all: B2 H16 L1000 d_v128 43.9 / 43.0 / 44.8, B8
     // H12 L300 d_v64 18.7 / 18.8 / 19.3, B1 H8 L300 d_v128 18.8 / 17.8 / 17.0, B4 H16 L2048 d_v64, the keys' states too, 97.6 / 95.9 / 95.1)
     const bool dependent = MODE == kModeFwd || MODE == kModeDkDv || XB || grid.x <= kSMs;
-    const cudaError_t e = launch_ex(backward_tc_kernel<DV, MODE, LT, XB>, grid, dim3(kThreadsB), C::kSmem, 1, dependent, stream, n0, w0, n1,
+    const cudaError_t e = launch_ex(backward_tc_kernel<DV, KIND, LT, XB>, grid, dim3(kThreadsB), C::kSmem, 1, dependent, stream, n0, w0, n1,
                                     w1, st ? *st : n0, outm ? *outm : w0, p);
     note_launch();
     const based_status s2 = check_launch(what);
@@ -1110,6 +1116,7 @@ based_status launch_quadratic_forward_tc(const void* q, const void* k, const voi
     const dim3 grid((unsigned)((L + kTile - 1) / kTile) * BH);
     p.heads = BH;
     p.by_length = long_loops_first(BH, L);
+    if (d_feat == 16) return launch_pass<64, kModeFwdRounded, 64>(tq, tq, tk64, tv64, p, grid, "quadratic forward (tc)", stream, nullptr, &tout);
     return launch_pass<64, kModeFwd, 64>(tq, tq, tk64, tv64, p, grid, "quadratic forward (tc)", stream, nullptr, &tout);
 }
 

@@ -135,7 +135,8 @@ enum Bar {
 };
 
 // segments per head, chunks per segment (the last one takes the rest), mode
-struct SegPlan { int nseg; int per; bool recompute; int balanced; };   // balanced > 0: that many equal chunk ranges over all heads
+// (balanced > 0: that many equal chunk ranges over all heads; rounded: recompute mode in the plain chunk loop's place, see ROUNDED)
+struct SegPlan { int nseg; int per; bool recompute; int balanced; bool rounded = false; };
 
 struct Params {
     float* kv_abi;        // [BH, 273, DV] or null
@@ -714,7 +715,12 @@ __device__ __noinline__ void find_piece(Piece* piece, int* s_rest, int balanced,
 }
 
 // CONT: the piece starts from the caller's state (an instance of its own: what it adds stays out of the others' registers).
-template <int DV, int MODE, bool CONT = false>
+// ROUNDED: the row sums are those of the rounded weights, the ones that multiply V, as in the plain chunk loop at d_v 64, whose
+// row sums are the tensor cores'.  With small scores the weights of a row are alike and so are their roundings, which cancel between
+// sum and products: an instance for the calls that would run that loop but for their length (error against 64 bits at input
+// scale 0.25, plain loop / sums of what was rounded / of the rounded: L33 2.0e-3 / 2.2e-3 / 2.0e-3, L65 2.05e-3 / 2.4e-3 / 2.05e-3; scale 1,
+// where the plain loop's 16-bit polynomial counts, L128 2.6e-3 / 2.2e-3 / 2.05e-3).
+template <int DV, int MODE, bool CONT = false, bool ROUNDED = false>
 __global__ void __launch_bounds__(kThreads, 1)
     prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                       const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o,
@@ -1466,10 +1472,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                             for (int i = 0; i < 16; ++i) {
                                 const uint64_t s2 = f32x2(sc[2 * i], sc[2 * i + 1]);
                                 const uint64_t w2 = fma2(s2, fma2(s2, k2, k1), k0);
-                                den2 = add2(den2, w2);
                                 float w0, w1;
                                 f32x2_split(w2, w0, w1);
                                 pk[i] = pack_bf16(w0, w1);
+                                den2 = add2(den2, ROUNDED ? f32x2(pk[i] << 16, pk[i] & 0xffff0000u) : w2);
                             }
                             f32x2_split(den2, den0, den1);
                         } else {                         // the batch that holds the diagonal
@@ -1480,9 +1486,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                                 f32x2_split(fma2(s2, fma2(s2, k2, k1), k0), w0, w1);
                                 w0 = (2 * i <= lane) ? w0 : 0.f;
                                 w1 = (2 * i + 1 <= lane) ? w1 : 0.f;
-                                den0 += w0;
-                                den1 += w1;
                                 pk[i] = pack_bf16(w0, w1);
+                                den0 += ROUNDED ? __uint_as_float(pk[i] << 16) : w0;
+                                den1 += ROUNDED ? __uint_as_float(pk[i] & 0xffff0000u) : w1;
                             }
                         }
                     }
@@ -1580,7 +1586,7 @@ unsigned long long* g_trace = nullptr;
 // SMs come free (they cannot take an SM that a CTA of the state pass still needs, all of those being resident or done by
 // then), and the one group that reads what the state pass wrote waits for its completion.  The recompute-mode kernel and
 // the state pass behind whatever precedes the call: they wait right after their set-up.
-template <int DV, int MODE, bool CONT = false>
+template <int DV, int MODE, bool CONT = false, bool ROUNDED = false>
 cudaError_t launch_dependent(dim3 grid, cudaStream_t stream, const CUtensorMap& tq, const CUtensorMap& tk,
                              const CUtensorMap& tv, const CUtensorMap& to, const Params& p) {
     cudaLaunchConfig_t cfg = {};
@@ -1593,7 +1599,7 @@ cudaError_t launch_dependent(dim3 grid, cudaStream_t stream, const CUtensorMap& 
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, prefill_tc_kernel<DV, MODE, CONT>, tq, tk, tv, to, p);
+    return cudaLaunchKernelEx(&cfg, prefill_tc_kernel<DV, MODE, CONT, ROUNDED>, tq, tk, tv, to, p);
 }
 
 // The caller's state of a continued call, folded into the internal basis, as the first workspace slot of each head
@@ -1718,17 +1724,14 @@ based_status launch_dv(const void* q, const void* k, const void* v, void* out, f
         if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return BASED_ERR_CUDA;
         std::lock_guard<std::mutex> lock(setup_mutex());
         if (!configured[dev]) {
-            if (cudaFuncSetAttribute(prefill_tc_kernel<DV, kModeMain>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)C::kSmemBytes) != cudaSuccess ||
-                cudaFuncSetAttribute(prefill_tc_kernel<DV, kModeState>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)C::kSmemBytes) != cudaSuccess ||
-                cudaFuncSetAttribute(prefill_tc_kernel<DV, kModePre>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)C::kSmemBytes) != cudaSuccess ||
-                cudaFuncSetAttribute(prefill_tc_kernel<DV, kModeMain, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)C::kSmemBytes) != cudaSuccess ||
-                cudaFuncSetAttribute(prefill_tc_kernel<DV, kModePre, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)C::kSmemBytes) != cudaSuccess)
+            auto room = [](auto kernel) {
+                return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::kSmemBytes) == cudaSuccess;
+            };
+            if (!room(prefill_tc_kernel<DV, kModeMain>) || !room(prefill_tc_kernel<DV, kModeState>) || !room(prefill_tc_kernel<DV, kModePre>) ||
+                !room(prefill_tc_kernel<DV, kModeMain, true>) || !room(prefill_tc_kernel<DV, kModePre, true>))
                 return BASED_ERR_CUDA;
+            if constexpr (DV == 64)
+                if (!room(prefill_tc_kernel<DV, kModePre, false, true>) || !room(prefill_tc_kernel<DV, kModePre, true, true>)) return BASED_ERR_CUDA;
             configured[dev] = true;
         }
     }
@@ -1761,8 +1764,14 @@ based_status launch_dv(const void* q, const void* k, const void* v, void* out, f
     }
     if (recompute) {
         if (continued) p.ticket = new_ticket();
-        const cudaError_t e = continued ? launch_dependent<DV, kModePre, true>(dim3(nseg, BH), stream, tq, tk, tv, to, p)
-                                             : launch_dependent<DV, kModePre>(dim3(nseg, BH), stream, tq, tk, tv, to, p);
+        auto launch = [&](auto rounded) {
+            constexpr bool R = decltype(rounded)::value;
+            return continued ? launch_dependent<DV, kModePre, true, R>(dim3(nseg, BH), stream, tq, tk, tv, to, p)
+                             : launch_dependent<DV, kModePre, false, R>(dim3(nseg, BH), stream, tq, tk, tv, to, p);
+        };
+        cudaError_t e;
+        if constexpr (DV == 64) e = plan.rounded ? launch(std::true_type{}) : launch(std::false_type{});
+        else e = launch(std::false_type{});
         if (e != cudaSuccess) return BASED_ERR_CUDA;
         note_launch();
         return check_launch("prefill_tc_kernel<pre>");
@@ -2013,20 +2022,21 @@ static int heads_in_segments(int BH, int L, int d_v) {
 
 based_status launch_prefill_tc(const void* q, const void* k, const void* v, void* out, float* kv, float* z, int BH,
                                int L, int d_v, int flags, void* workspace, cudaStream_t stream, size_t workspace_limit) {
-    if (const int rest = (flags & BASED_STATE_CONTINUE) ? 0 : heads_in_segments(BH, L, d_v)) {
-        const based_status st =
-            launch_prefill_tc(q, k, v, out, kv, z, BH - rest, L, d_v, flags, workspace, stream, workspace_limit);
-        if (st != BASED_OK) return st;
-        const size_t tokens = (size_t)(BH - rest) * L, rows = (size_t)(BH - rest) * ((flags & BASED_STATE_SYM) ? kDSym : kD);
+    // heads `first` .. of the call, n of them
+    auto heads = [&](int first, int n, void* scratch, size_t limit) {
+        SegPlan plan = prefill_tc_plan(n, L, d_v == 112 ? 128 : d_v, (flags & BASED_STATE_CONTINUE) != 0, scratch ? limit : 0);
+        plan.rounded = plan.recompute && (plan.nseg == 1 || first > 0);
+        const size_t tokens = (size_t)first * L, rows = (size_t)first * ((flags & BASED_STATE_SYM) ? kDSym : kD);
         auto from = [](auto* p, size_t elements) { return reinterpret_cast<decltype(p)>(reinterpret_cast<uintptr_t>(p) + 2 * elements); };
-        return launch_prefill_tc(from(q, tokens * kDFeat), from(k, tokens * kDFeat), from(v, tokens * d_v), from(out, tokens * d_v),
-                                 kv ? kv + rows * d_v : nullptr, z ? z + rows : nullptr, rest, L, d_v, flags, nullptr, stream, 0);
-    }
-    const SegPlan plan = prefill_tc_plan(BH, L, d_v == 112 ? 128 : d_v, (flags & BASED_STATE_CONTINUE) != 0,
-                                         workspace ? workspace_limit : 0);
-    float* ws = static_cast<float*>(workspace);
-    if (d_v == 64) return launch_dv<64>(q, k, v, out, kv, z, BH, L, 64, flags, ws, plan, stream);
-    return launch_dv<128>(q, k, v, out, kv, z, BH, L, d_v, flags, ws, plan, stream);      // 112 or 128
+        const void *qh = from(q, tokens * kDFeat), *kh = from(k, tokens * kDFeat), *vh = from(v, tokens * d_v);
+        void* oh = from(out, tokens * d_v);
+        float *kvh = kv ? kv + rows * d_v : nullptr, *zh = z ? z + rows : nullptr, *ws = static_cast<float*>(scratch);
+        if (d_v == 64) return launch_dv<64>(qh, kh, vh, oh, kvh, zh, n, L, 64, flags, ws, plan, stream);
+        return launch_dv<128>(qh, kh, vh, oh, kvh, zh, n, L, d_v, flags, ws, plan, stream);      // 112 or 128
+    };
+    const int rest = (flags & BASED_STATE_CONTINUE) ? 0 : heads_in_segments(BH, L, d_v);
+    const based_status st = heads(0, BH - rest, workspace, workspace_limit);
+    return st != BASED_OK || rest == 0 ? st : heads(BH - rest, rest, nullptr, 0);
 }
 
 }  // namespace based

@@ -85,6 +85,7 @@ __device__ __forceinline__ bool all_rows(bool pred) {
 // IN_ORDER: one chunk of d' 16.  The first group takes both key tiles, and a row's weights are summed as the chunked kernel sums them
 // (the even columns, the odd ones, then both; so does kModeFwd), so that the outputs are the bits that the chunked kernel gives beside a
 // state (us, both groups / this: L128, 16 heads d_v 64 3.24 / 3.36, d_v 128 3.72 / 3.82, 200 heads d_v 128 5.18 / 5.01, 400 8.34 / 8.43).
+// At d_v 64 the rounded weights, as there (prefill_tc_kernel's ROUNDED): 16 heads L128 3.66 -> 3.81, 600 8.6 -> 9.0.
 template <int DV, bool IN_ORDER>
 __global__ void __launch_bounds__(kThreadsQ, 2)
     quadratic_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
@@ -211,10 +212,11 @@ __global__ void __launch_bounds__(kThreadsQ, 2)
                     halves_of(x, lo, hi);
                     x = pair_of_f(col <= row ? lo : 0.f, col + 1 <= row ? hi : 0.f);
                 }
-                uint64_t& den = den2[IN_ORDER ? 0 : i & 1];
-                den = add_pairs(den, x);
                 halves_of(x, lo, hi);
-                w[w0 + i] = pack2(lo, hi);
+                const uint32_t packed = pack2(lo, hi);
+                w[w0 + i] = packed;
+                uint64_t& den = den2[IN_ORDER ? 0 : i & 1];
+                den = add_pairs(den, IN_ORDER && DV == 64 ? pair_of_f(__uint_as_float(packed << 16), __uint_as_float(packed & 0xffff0000u)) : x);
             }
         };
         // (what was loaded is used behind its wait and not before it)

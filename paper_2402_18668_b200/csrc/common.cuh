@@ -59,6 +59,15 @@ cudaError_t launch_ex(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, 
     cfg.numAttrs = n;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
+// Whether the definition form's forward, `tiles` CTAs of up to n = `per_head` turns of its loop each on the chip's `slots`, is a dependent
+// launch.  One that nearly fills the slots once is not: its first CTAs, the longest, would double up on the SMs that the grid ahead
+// leaves first (us repeated, dependent / plain.  d' 8 d_v 64, two CTAs per SM: 16 heads L2048 16.3 / 14.1, 20 L1409 12.6 / 11.2, 10 L4096 29 /
+// 24; four: 64 L777 14.3 / 12.5, 64 L1100 19.6 / 16.4, 20 L4096 55 / 45; d_v 128: 16 L2048 19.9 / 18.4, 10 L4096 35.6 / 31.6).  Otherwise the
+// set-up beside that grid pays: few tiles (16 L1024 7.5 / 8.1), short loops (128 L200 5.3 / 6.1, 100 L777 15.8 / 17.0), more than a wave (the
+// longer the loops the later: 32 L2048 19.8 / 21.5, 64 L2048 34 / 36, 28 L4096 53.5 / 52.6).
+inline bool dependent_forward(long long tiles, int per_head, int slots) {
+    return per_head < 7 || 3 * tiles <= 2 * slots || 64 * (tiles - slots) > (long long)(per_head - 4) * slots;
+}
 // Splits an SM's 256 KB between L1 and shared memory for a kernel that streams through L1: loads in flight take L1 lines, and
 // without a preference a kernel runs with whatever split the one before it left (decode step, 2048 heads, d_v 128: 91 us
 // with a quarter for shared memory or no preference alone, 113 with all of it).  Once per kernel and device.

@@ -328,8 +328,8 @@ based_status launch_forward(const CUtensorMap& q, const CUtensorMap& k, const CU
             configured[dev] = true;
         }
     }
-    const cudaError_t e = launch_ex(quadratic_fwd_tc_kernel<DV, IN_ORDER>, dim3(grid), dim3(kThreadsQ), C::kSmem, 1, true, stream, q, k, v,
-                                    out, p);
+    const cudaError_t e = launch_ex(quadratic_fwd_tc_kernel<DV, IN_ORDER>, dim3(grid), dim3(kThreadsQ), C::kSmem, 1,
+                                    p.overlapped || dependent_forward(grid, grid / p.heads, 2 * kSMs), stream, q, k, v, out, p);
     note_launch();
     const based_status st = check_launch("quadratic_fwd_tc_kernel");
     return e == cudaSuccess ? st : BASED_ERR_CUDA;

@@ -1,0 +1,56 @@
+"""Times of calls that follow one another, each as a dependent launch where that pays: a call does not slow the next one down."""
+import pytest
+import torch
+
+import paper_2402_18668_b200 as based
+
+pytestmark = pytest.mark.gpu
+
+
+def microseconds(*steps):
+    """Each step's time, repeated in a graph; the least of ten turns, the steps in turn."""
+    graphs = []
+    for step in steps:
+        step()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            for _ in range(20):
+                step()
+        graphs.append(graph)
+    best = [float("inf")] * len(steps)
+    for _ in range(10):
+        for i, graph in enumerate(graphs):
+            start, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            start.record()
+            graph.replay()
+            end.record()
+            end.synchronize()
+            best[i] = min(best[i], start.elapsed_time(end) * 50)
+    return best
+
+
+def inputs(BH, L, d, d_v):
+    g = torch.Generator(device="cuda").manual_seed(BH + L)
+    q, k = (torch.randn(1, BH, L, d, generator=g, device="cuda").mul(0.25).bfloat16() for _ in range(2))
+    return q, k, torch.randn(1, BH, L, d_v, generator=g, device="cuda").bfloat16()
+
+
+def prefill(BH, L, d, d_v, state=False):
+    q, k, v = inputs(BH, L, d, d_v)
+    out = torch.empty_like(v)
+    kw = dict(zip(("kv_state", "z_state"), based.new_state(1, BH, d_v, d_feat=d))) if state else {}
+    return lambda: based.based_prefill(q, k, v, out=out, **kw)
+
+
+@pytest.mark.parametrize("d,d_v,BH,L,state", [(24, 64, 20, 4096, False), (8, 64, 40, 2048, False), (24, 64, 10, 4096, False)])
+def test_behind_itself(d, d_v, BH, L, state):
+    """Behind itself a call takes no longer than behind a small kernel, that one's time included (1.04 to 1.16 times as long where its
+    long CTAs share the SMs that the call before leaves first)."""
+    call, small = prefill(BH, L, d, d_v, state), torch.empty(256, device="cuda")
+
+    def both():
+        small.zero_()
+        call()
+
+    alone, behind = microseconds(call, both)
+    assert alone <= 1.02 * behind

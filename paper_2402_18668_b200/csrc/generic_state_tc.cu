@@ -338,7 +338,16 @@ based_status launch_state(const void* k, const void* v, float* kv, float* z, int
             configured[dev] = true;
         }
     }
-    const cudaError_t e = launch_ex(generic_state_tc_kernel<DF, DV>, dim3(C::kParts, BH), dim3(kThreadsS), C::kSmem, 1, true, stream, tv, p);
+    // A dependent launch, but not at d' 32 with two tiles of values (five CTAs per head, the longest walks) where these CTAs would share the
+    // SMs that the outputs' CTAs of a call before leave first, and each have one to itself behind the end of that call: too many of both for
+    // the chip at once, but few outputs' tiles beyond (us repeated, dependent / plain, with the outputs, d_v 112: 16 heads L1409 24.5 /
+    // 20.8, 24 L1024 19.6 / 17.4, 16 L2048 30.4 / 26.7, 10 L4096 52 / 45.6; d_v 128, dependent by plain: 20 L300 1.06, 18 L300 0.89, 32 L300
+    // 0.95, 14 L1024 0.94, 20 L1024 1.11, 28 L1024 0.99, 13 L1409 0.96, 24 L1409 0.96, 10 L2048 0.96, 13 L4096 0.98)
+    const int tiles = (L + 127) / 128, ctas = BH * (C::kParts + tiles);
+    const bool one_each = DF == 32 && DV == 128 && BH * C::kParts <= kSMs && ctas > kSMs + 8 * ((tiles < 14 ? tiles : 14) - 2) &&
+                          ctas <= 330 + 4 * tiles;
+    const cudaError_t e =
+        launch_ex(generic_state_tc_kernel<DF, DV>, dim3(C::kParts, BH), dim3(kThreadsS), C::kSmem, 1, !one_each, stream, tv, p);
     note_launch();
     const based_status st = check_launch("generic_state_tc_kernel");
     return e == cudaSuccess ? st : BASED_ERR_CUDA;

@@ -42,7 +42,8 @@ def prefill(BH, L, d, d_v, state=False):
     return lambda: based.based_prefill(q, k, v, out=out, **kw)
 
 
-@pytest.mark.parametrize("d,d_v,BH,L,state", [(24, 64, 20, 4096, False), (8, 64, 40, 2048, False), (24, 64, 10, 4096, False)])
+@pytest.mark.parametrize("d,d_v,BH,L,state", [(24, 64, 20, 4096, False), (8, 64, 40, 2048, False), (24, 64, 10, 4096, False),
+                                              (32, 112, 10, 4096, True), (32, 112, 16, 2048, True)])
 def test_behind_itself(d, d_v, BH, L, state):
     """Behind itself a call takes no longer than behind a small kernel, that one's time included (1.04 to 1.16 times as long where its
     long CTAs share the SMs that the call before leaves first)."""

@@ -1042,7 +1042,11 @@ based_status launch_dvb(const void* q, const void* k, const void* v, const void*
             if (running) return launch_block_states_tc(x, val, sts, w.st, w.sv, nullptr, nullptr, BH, val_H, L, W, dvr, rev, stream);
             based_status s2 = launch_block_states_tc(x, val, sts, w.st, w.sv, w.part, w.zpart, BH, val_H, L, W, dvr, rev, stream);
             if (s2 != BASED_OK) return s2;
-            const cudaError_t e = launch_ex(state_scan_kernel, dim3((160 * dvr + 255) / 256, BH), dim3(256), 0, 1, true, stream, w.part,
+            // (dependent with many heads, and with one: with a few the pass behind it, a dependent launch itself, comes in while the scan's blocks
+            // are being placed; us per backward call, dependent / plain: d_v 128 2 heads L3000 49.4 / 42.7, 6 L2048 49.3 / 42.6, 8 L1536 48.3 / 44.1,
+            // 12 L2048 47.7 / 48.3, d_v 64 1 L1024 27.9 / 30.1, 4 L2048 35.4 / 32.1, 12 L1536 37.5 / 34.7, 16 L3000 61.5 / 62.2, 32 L2048 66.4 / 67.2)
+            const bool dependent = BH == 1 || BH >= (DV == 64 ? 16 : 12);
+            const cudaError_t e = launch_ex(state_scan_kernel, dim3((160 * dvr + 255) / 256, BH), dim3(256), 0, 1, dependent, stream, w.part,
                                             w.zpart, w.st, w.sv, nblk, 160 * dvr, rev);
             note_launch();
             s2 = check_launch("state_scan_kernel");

@@ -913,11 +913,13 @@ based_status launch_pass(const CUtensorMap& n0, const CUtensorMap& w0, const CUt
             configured[dev] = true;
         }
     }
-    // Dependent launches, but not the tile path's passes over the queries with more than a CTA per SM: theirs would double up on the SMs
-    // that the grid ahead leaves first (us per backward call, no pass dependent / dk/dv / all: B2 H16 L1000 d_v128 43.9 / 43.0 / 44.8, B8
-    // H12 L300 d_v64 18.7 / 18.8 / 19.3, B1 H8 L300 d_v128 18.8 / 17.8 / 17.0, B4 H16 L2048 d_v64, the keys' states too, 97.6 / 95.9 / 95.1)
+    // Dependent launches, but not the tile path's passes over the queries with more than a CTA per SM (d_v 112 / 128: per two SMs): theirs
+    // would double up on the SMs that the grid ahead leaves first (us per backward call, no pass dependent / dk/dv / all: B2 H16 L1000
+    // d_v128 43.9 / 43.0 / 44.8, B8 H12 L300 d_v64 18.7 / 18.8 / 19.3, B1 H8 L300 d_v128 18.8 / 17.8 / 17.0, B4 H16 L2048 d_v64, the keys' states
+    // too, 97.6 / 95.9 / 95.1; dk/dv / all at d_v 128, 12 heads L1024 36.7 / 38.7, 16 37.2 / 39.6, 24 L768 30.9 / 32.3, 8 L1024 36.5 / 35.7, 16 L512
+    // 22.4 / 21.6, at d_v 64 16 L1024 34.3 / 33.7)
     const bool dependent = MODE == kModeFwd ? p.overlapped || dependent_forward(grid.x, grid.x / p.heads, 4 * kSMs)
-                                            : MODE == kModeDkDv || XB || grid.x <= kSMs;
+                                            : MODE == kModeDkDv || XB || grid.x <= (DV == 64 ? kSMs : kSMs / 2);
     const cudaError_t e = launch_ex(backward_tc_kernel<DV, KIND, LT, XB>, grid, dim3(kThreadsB), C::kSmem, 1, dependent, stream, n0, w0, n1,
                                     w1, st ? *st : n0, outm ? *outm : w0, p);
     note_launch();

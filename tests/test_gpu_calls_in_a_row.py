@@ -58,13 +58,20 @@ def test_behind_itself(d, d_v, BH, L, state):
     assert alone <= 1.02 * behind
 
 
+def backward(BH, L, d_v):
+    q, k, v = inputs(BH, L, 16, d_v)
+    out = based.based_prefill(q, k, v)
+    dout = torch.randn_like(v)
+    return lambda: based.based_prefill_backward(q, k, v, dout, out=out)
+
+
 def test_backward_of_fewer_heads():
     """Two heads' block-wise backward is well below twelve heads' (0.95 of it while the scan of the block states was a dependent launch)."""
-    def step(BH):
-        q, k, v = inputs(BH, 3000, 16, 128)
-        out = based.based_prefill(q, k, v)
-        dout = torch.randn_like(v)
-        return lambda: based.based_prefill_backward(q, k, v, dout, out=out)
-
-    two, twelve = microseconds(step(2), step(12))
+    two, twelve = microseconds(backward(2, 3000, 128), backward(12, 3000, 128))
     assert two <= 0.9 * twelve
+
+
+def test_backward_with_a_tile_for_every_sm():
+    """128 tiles take little longer than 64, each an SM of its own (1.11 times where they share the SMs that are left first)."""
+    half, whole = microseconds(backward(8, 1024, 128), backward(16, 1024, 128))
+    assert whole <= 1.075 * half

@@ -1881,8 +1881,11 @@ static SegPlan prefill_tc_plan(int BH, int L, int d_v, bool continued = false, s
     // One segment of few chunks: the recompute mode's kernel too, which has no earlier chunks to run then and is a dependent launch
     // (us, plain chunk loop / this: H16 L100 d_v64 6.3 / 4.9, H2 L16 d_v128 7.1 / 5.4, H100 L256 d_v64 7.9 / 6.9, H256 L300 16.6 / 15.9,
     // H200 L300 d_v128 20.3 / 19.6, H120 L500 13.3 / 13.2, H200 L700 d_v64 23.5 / 23.6, L1500 38.0 / 39.8; continued H16 L100 10.6 / 9.6, H100
-    // L256 12.3 / 12.1, H256 L300 25.5 / 25.9, at d_v 128 H2 L16 11.6 / 11.0, H200 L128 24.2 / 24.2, H100 L200 14.4 / 15.0)
-    if (best.nseg == 1 && best.balanced == 0 && nch <= (!continued ? 4 : d_v == 64 ? 2 : 1)) best.recompute = true;
+    // L256 12.3 / 12.1, H256 L300 25.5 / 25.9, at d_v 128 H2 L16 11.6 / 11.0, H200 L128 24.2 / 24.2, H100 L200 14.4 / 15.0).  With more than two
+    // waves of CTAs the loop counts for more (d_v 64 H297 L512 25.6 / 26.3, H450 L400 33.2 / 34.3, H1000 L512 64.9 / 68.2, L300 54.3 / 56.1, L256 45.4 /
+    // 45.6; d_v 128 H297 L512 33.2 / 34.8, H450 L400 45.0 / 45.9, H370 L300 29.7 / 29.1).
+    const int most = continued ? (d_v == 64 ? 2 : 1) : BH <= 2 * kSMs ? 4 : d_v == 64 ? 2 : 3;
+    if (best.nseg == 1 && best.balanced == 0 && nch <= most) best.recompute = true;
 #ifdef BASED_TRACE
     if (const char* e = getenv("BASED_NSEG")) {
         const int v = atoi(e);                      // negative: recompute mode with that many segments

@@ -2010,17 +2010,20 @@ size_t prefill_tc_workspace_bytes(int BH, int L, int d_v) {
 
 // Heads left over after whole waves of one CTA per SM, where they are better off in a launch of their own, in segments (recompute
 // mode, no scratch), than one CTA each in a wave that leaves most SMs idle; else 0.  From sixteen chunks on wherever they get two
-// segments (d_v 128: three); below, the second launch's set-up and tail weigh as much as the idle wave unless that wave is the second of
-// two (us, one launch / two, outputs alone: d_v 64 L4096 150 heads 82.9 / 72.3, 208 84.9 / 80.7, L2048 160 heads 46.1 / 41.9, 224, not
-// taken, 48.5 / 50.3, 320 69.8 / 66.7, L1024 150 26.9 / 25.3, 208, not taken, 28.5 / 28.3, L300 192 15.6 / 14.7; d_v 128 L4096 160 heads
-// 128 / 118, L2048 160 69.4 / 66.3, 208, not taken, 71.5 / 72.4, L1024 192, not taken, 45.6 / 46.8 with a new state, L512 160 23.3 / 21.6,
-// 300, not taken, 35.1 / 34.7).  Not continued calls: L2048 d_v 64 160 heads 57.5 / 59.8, the caller's state being read by every segment.
+// segments and a few SMs to spare (d_v 128: three), from the third wave on four; below, the second launch's set-up and tail weigh as much
+// as the idle wave unless that wave is the second of two and, from five chunks on at d_v 64, its heads are few (us, one launch / two,
+// outputs alone: d_v 64 L4096 150 heads 82.9 / 72.3, 208 84.9 / 80.7, L2048 160 heads 46.1 / 41.9, 320 69.8 / 66.7, L1024 150 26.9 / 25.3, L300 192
+// 15.6 / 14.7; d_v 128 L4096 160 heads 128 / 118, L2048 160 69.4 / 66.3, L512 160 23.3 / 21.6.  Not taken: d_v 64 L4096 222 85.0 / 84.5, L2048 222 48.3
+// / 49.8, 345 69.5 / 70.7, 370 70.5 / 72.4, L1024 208 28.5 / 28.3, 196 27.6 / 27.7, L640 172 20.2 / 20.4, 197 20.6 / 21.7; d_v 128 L2048 208 71.5 / 72.4,
+// 345 107.8 / 109.8, L1024 192 with a new state 45.6 / 46.8, L512 300 35.1 / 34.7).  Not continued calls: L2048 d_v 64 160 heads 57.5 / 59.8, the
+// caller's state being read by every segment.
 static int heads_in_segments(int BH, int L, int d_v) {
     const int nch = (L + kC - 1) / kC, rest = BH % kSMs;
     if (BH < kSMs || 2 * rest > kSMs || nch < 2) return 0;
-    if (nch >= 16) return (d_v == 64 ? 2 : 3) * rest <= kSMs ? rest : 0;
-    if (BH >= 2 * kSMs) return 0;
-    return nch <= 4 || (d_v == 64 && 3 * rest <= kSMs) ? rest : 0;
+    bool apart;
+    if (nch >= 16) apart = BH >= 2 * kSMs ? 4 * rest <= kSMs : d_v == 64 ? 7 * rest <= 3 * kSMs : 3 * rest <= kSMs;
+    else apart = BH < 2 * kSMs && (nch <= 4 || (d_v == 64 && 3 * rest <= kSMs && rest <= 9 * (nch - 4)));
+    return apart ? rest : 0;
 }
 
 based_status launch_prefill_tc(const void* q, const void* k, const void* v, void* out, float* kv, float* z, int BH,

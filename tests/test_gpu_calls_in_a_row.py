@@ -75,3 +75,9 @@ def test_backward_with_a_tile_for_every_sm():
     """128 tiles take little longer than 64, each an SM of its own (1.11 times where they share the SMs that are left first)."""
     half, whole = microseconds(backward(8, 1024, 128), backward(16, 1024, 128))
     assert whole <= 1.075 * half
+
+
+def test_heads_after_a_wave():
+    """49 heads after a wave of 148 take no longer than 74 (1.04 of it in segments, with five chunks)."""
+    fewer, more = microseconds(prefill(197, 640, 16, 64), prefill(222, 640, 16, 64))
+    assert fewer <= 1.02 * more

@@ -252,10 +252,11 @@ size_t based_prefill_backward_workspace_bytes(int B, int H, int L, int d_v, base
  * only: D_i and dout_i . N_i are still recomputed in fp32.  fp32 io ignores out's values.
  * out must not alias a gradient output.
  *
- * Block-wise path (bf16 io, d_feat = 16; L >= 768 to 1025 at d_v 64, L >= 1024 to 1536 at d_v 112 / 128): O(L) per
- * head, the recurrent view of Sec. 4.1 applied to the gradients.  The sequence is cut into blocks of
- * W = 256 tokens (512 for long sequences of few heads at d_v 128).  Pairs inside a block go through
- * the tiles above.  All earlier blocks reach a query through their summed state S = sum_j phi(k_j) v_j^T, z = sum_j phi(k_j):
+ * Block-wise path (bf16 io, d_feat = 16; from 768 to 2048 tokens on, by d_v, the number of heads and whether out is given:
+ * based_prefill_backward_block_tokens says which path a call takes): O(L) per head, the recurrent view of Sec. 4.1 applied to
+ * the gradients.  The sequence is cut into blocks of W = 256 tokens (512 for long sequences of few heads at d_v 128).  Pairs
+ * inside a block go through the tiles above.  All earlier blocks reach a query through their summed state
+ * S = sum_j phi(k_j) v_j^T, z = sum_j phi(k_j):
  *   sum_j w'_ij (dout_i.v_j - m_i) k_j = J(q_i)^T (S dout_i - m_i z),   D_i += phi(q_i) . z
  * (J the Jacobian of phi), and all later blocks reach a key through R = sum_i phi(q_i) (dout_i / D_i)^T
  * and R_b = sum_i b_i phi(q_i):  dk_j += J(k_j)^T (R v_j + R_b),  dv_j += R^T phi(k_j).
@@ -400,8 +401,8 @@ based_status based_generation_step(const void* q, const void* k, const void* v, 
  * aligned, read in stream order like any launch's inputs; overlapping neither another input's buffer nor anything that the
  * step writes: the outputs, the state, the caches, the position) leaves a copy in them, a step with six NULLs runs on what they
  * hold.  All other pointers are fixed at creation and must outlive the graph.  Creation launches nothing; call
- * based_preload_decode first.  Steps of one graph may come from several threads and on any streams of its device: each runs
- * behind the one before it.  Not on a stream under capture (BASED_ERR_CUDA).
+ * based_preload_decode first.  Steps of one graph may come from several threads and on any streams of its device, which is
+ * the current one at creation and at every step: each runs behind the one before it.  Not on a stream under capture (BASED_ERR_CUDA).
  */
 typedef struct based_generation_graph based_generation_graph;
 based_status based_generation_graph_create(void* q, void* k, void* v, float* kv_state, float* z_state, void* out, void* qw,

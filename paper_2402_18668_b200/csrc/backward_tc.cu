@@ -934,8 +934,8 @@ based_status launch_pass(const CUtensorMap& n0, const CUtensorMap& w0, const CUt
 //   64 heads: d_v 64 L 768 34 / 47, L 1024 52 / 54, L 1280 73 / 66; d_v 128 L 768 50 / 59, L 1024 74 / 72
 //   16 heads: d_v 64 L 768 29 / 36, L 1024 36 / 37, L 1536 51 / 42; d_v 128 L 1280 46 / 52, L 1536 53 / 54, L 2048 70 / 55
 //   32 heads: d_v 64 L 1280 46 / 61, L 1536 56 / 66, L 2048 82 / 70; d_v 128 L 1536 74 / 91, L 2048 112 / 101
-// And, since both paths' passes are dependent launches, at d_v 64: 64 heads L 768 32 / 48, L 800 41 / 48 (blocks there all the same),
-// 80 L 768 43 / 49, 128 62 / 66, L 769 74.4 / 74.1, L 897 93 / 83; 8 heads L 769 28 / 34, L 1024 34 / 35, L 1025 36 / 35; 16 29 / 36, 34 / 35,
+// And, since both paths' passes are dependent launches, at d_v 64: 64 heads L 768 32 / 48, L 800 41 / 48 (blocks there all the same:
+// the line of 64 heads and more is 128 heads'; up to some 110 heads and 1024 tokens tiles would be the faster), 80 L 768 43 / 49, 128 62 / 66, L 769 74.4 / 74.1, L 897 93 / 83; 8 heads L 769 28 / 34, L 1024 34 / 35, L 1025 36 / 35; 16 29 / 36, 34 / 35,
 // 36 / 36; 24 30 / 36, 36 / 37, 38 / 37; 32 L 769 32 / 38, L 897 37.4 / 37.8, L 1024 39.2 / 37.9; 2 (where the line stays) L 768 26 / 28, L 769
 // 28.0 / 28.8, L 897 31 / 29.  The tile path is also the more precise (2.3e-3 against 2.4e-3 of fp64 gradients), so no line moves below where it was.
 // Below 64 heads one CTA per head and block sums the states, and a second short wave of those costs as much as a full one:

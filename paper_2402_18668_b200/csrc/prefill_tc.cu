@@ -509,7 +509,8 @@ __device__ __forceinline__ void write_state(float* kv, float* z, int dv, const s
     constexpr int kQ = DV / 4, kPer = 128 / kQ;                      // 16-byte words of a row, rows per pass
     // (d_v 64: read afresh, the kernel's own copy would have to live through the role loops; us, that / this, outputs alone: B1 H2
     // L3000 20.0 / 19.4, H100 L1024 15.5 / 15.1, B4 H16 L2048 19.6 / 19.4, H200 L700 23.5 / 22.9, with a new state 26.2 / 25.8.  At d_v 128
-    // the loops come out better with the copy: B3 H16 L777 d_v112 continued 18.2 / 18.4, B8 H16 L4096 71.4 / 72.0)
+    // the loops come out better with the copy: B3 H16 L777 d_v112 continued 18.2 / 18.4, B8 H16 L4096 71.4 / 72.0; which of the two is the
+    // better is this compiler's register allocation and nothing else)
     int tx = threadIdx.x;
     if (DV == 64) asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tx));
     const int warp = tx >> 5, lane = tx & 31, tid = tx & 127;
@@ -571,8 +572,9 @@ __device__ __forceinline__ void write_state(float* kv, float* z, int dv, const s
 // made here: a segment that has read the state stores the call's ticket in its word of the workspace, and the last one
 // waits for the others' words before it writes (in practice they were stored long since: the last segment runs longest).
 // It clears them for a replay of the same launch; a ticket is a 64-bit number that no other launch uses, so whatever lay
-// in the workspace before is not one.  The CTAs of such a call are at most one per SM and need nothing of one another
-// to start and to read, so the wait ends; it is bounded all the same.
+// in the workspace before is not one.  A call of two or more segments has at most one CTA per SM, and they need nothing of
+// one another to start and to read, so the wait ends (with one segment per head, of any number of heads, there is no word to
+// wait for); it is bounded all the same.
 // (blockIdx: segment, head.  All from special registers and constants, and out of line: values kept in registers for it
 // through the role loops cost them spills, and B3 H16 L777 d_v112 1 to 2 us; this way 19.7 -> 20.0, d_v 128 19.2 -> 19.7, d_v 64
 // nothing.)
